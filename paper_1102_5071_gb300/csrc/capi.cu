@@ -57,6 +57,8 @@ struct cfet_ctx {
   OpCsr csr{};
   OpCsrFx csr_fx{};
   OpCsrC csr_c{};
+  std::vector<int> csr_rp;     // host copy of rp until the row split is made (cfet_create)
+  int* d_csr_rb = nullptr;     // row split over the CTAs [grid + 1]
   void* d_csr = nullptr;       // one allocation: rp | col | vr | vi | VR | VI | vr32 | vi32
   // interaction picture: host copies of the chain (stage weight tables)
   double ip_J = 0.0, ip_Delta = 0.0;
@@ -202,6 +204,7 @@ void free_ctx(cfet_ctx* c) {
   cudaFree(c->d_pauli_dtab);
   cudaFree(c->d_tmaps);
   cudaFree(c->d_csr);
+  cudaFree(c->d_csr_rb);
   if (c->h_st) cudaFreeHost(c->h_st);
   if (c->h_scal) cudaFreeHost(c->h_scal);
   delete c;
@@ -579,7 +582,7 @@ const char* csr_check(const cfet_op& o, int dim) {
 cfet_status csr_upload(cfet_ctx* ctx, const cfet_op* H0, int nV, const cfet_op* V) {
   const int dim = ctx->dim;
   const int nops = 1 + nV;
-  bool cplx = false;
+  unsigned cplx = 0;  // bit o: operator o has complex values
   std::vector<int> rp((size_t)nops * (dim + 1));
   size_t nnz = 0;
   for (int k = -1; k < nV; ++k) {
@@ -587,7 +590,8 @@ cfet_status csr_upload(cfet_ctx* ctx, const cfet_op* H0, int nV, const cfet_op* 
     const int64_t n = o.row_ptr[dim];
     for (int r = 0; r <= dim; ++r) rp[(size_t)(k + 1) * (dim + 1) + r] = (int)(nnz + o.row_ptr[r]);
     if (o.csr_im)
-      for (int64_t e = 0; e < n; ++e) cplx = cplx || o.csr_im[e] != 0.0;
+      for (int64_t e = 0; e < n; ++e)
+        if (o.csr_im[e] != 0.0) { cplx |= 1u << (k + 1); break; }
     nnz += (size_t)n;
   }
   const size_t n1 = nnz > 0 ? nnz : 1;
@@ -663,8 +667,49 @@ cfet_status csr_upload(cfet_ctx* ctx, const cfet_op* H0, int nV, const cfet_op* 
   fx.VR = reinterpret_cast<const long long*>(b + o_VR);
   fx.VI = cplx ? reinterpret_cast<const long long*>(b + o_VI) : nullptr;
   ctx->csr_c = OpCsrC{nops, d_rp, d_col, reinterpret_cast<const float*>(b + o_v32),
-                      cplx ? reinterpret_cast<const float*>(b + o_i32) : nullptr};
+                      cplx ? reinterpret_cast<const float*>(b + o_i32) : nullptr, nullptr, 0};
+  fx.rb = nullptr;
+  // threads per row of the fixed-point and complex64 applies
+  // eight or more entries of a row of one operator per thread (mean over the
+  // rows): with 10 entries two threads a row take 35.2 us per Lanczos iteration
+  // of 60 001 rows, one 46.5, four 36.2 and eight 47.7
+  const double per = (double)nnz / ((double)dim * nops);
+  int lb = 0;
+  while (lb < 4 && per >= 8.0 * (1 << lb)) ++lb;
+  fx.cplx = ctx->csr_c.cplx = cplx;
+  fx.lane_bits = ctx->csr_c.lane_bits = lb;
+  ctx->csr_rp.swap(rp);
   return CFET_OK;
+}
+
+// Rows of the CTAs: contiguous ranges of about equal work, a row costing its
+// stored entries (all operators) plus kCsrRowCost for the vector passes, and at
+// most `cap` rows each (cap * grid >= dim).
+constexpr long long kCsrRowCost = 8;
+std::vector<int> csr_row_split(const std::vector<int>& rp, int nops, int dim, int grid, long long cap) {
+  auto work = [&](int r) {
+    long long w = kCsrRowCost;
+    for (int o = 0; o < nops; ++o) {
+      const int* p = rp.data() + (size_t)o * (dim + 1) + r;
+      w += p[1] - p[0];
+    }
+    return w;
+  };
+  long long total = 0;
+  for (int r = 0; r < dim; ++r) total += work(r);
+  std::vector<int> rb(grid + 1, dim);
+  rb[0] = 0;
+  long long done = 0;
+  int r = 0;
+  for (int b = 0; b < grid; ++b) {
+    const long long goal = (total * (b + 1) + grid - 1) / grid;  // work of rows [0, rb[b + 1])
+    const long long least = (long long)dim - cap * (grid - 1 - b);  // rows that the later CTAs cannot take
+    const int r0 = r;
+    while (r < dim && r - r0 < cap && (r < least || done + work(r) / 2 < goal)) done += work(r++);
+    rb[b + 1] = r;
+  }
+  rb[grid] = dim;
+  return rb;
 }
 
 }  // namespace
@@ -1191,7 +1236,9 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
   }
   // element threads per CTA (the fixed-point kernel adds one control warp)
   const int workers = ctl_warp ? ctx->block - 32 : ctx->block;
+  int lane_bits = ctl_warp && family == kFamilyCsr ? ctx->csr_fx.lane_bits : 0;  // 2^lane_bits threads per element
   int want = (dim + workers - 1) / workers;
+  if (want > 1) want = (int)std::min((((long long)dim << lane_bits) + workers - 1) / workers, 1LL << 30);
   if (o.grid_size > 0) want = o.grid_size;
   ctx->grid = want < maxg ? want : maxg;
   if (ctl_warp && ctx->grid > kMaxCtlGrid) ctx->grid = kMaxCtlGrid;  // record exchange limit
@@ -1202,7 +1249,7 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
     const size_t sb = fx_small_smem_bytes(dim, o.m_max);
     if (sb > 0 && fx_small_prepare(sb) == 0) {
       ctx->small_fx = true;
-      ctx->small_block = 32 + std::min(ctx->block - 32, (dim + 31) / 32 * 32);
+      ctx->small_block = 32 + std::min(ctx->block - 32, ((dim << lane_bits) + 31) / 32 * 32);
     }
   }
   if (ctx->precision == CFET_PREC_FX)  // basis q_1..q_{m_max+1}; the Chebyshev kernel's three vectors
@@ -1227,6 +1274,17 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
       return fail(nullptr, CFET_EINVAL, "fixed-point precision: dimension too large for the grid, use CFET_PREC_F64");
     }
   }
+  if (ctl_warp && family == kFamilyCsr) {
+    // exact sums: a thread takes at most 4096 rows
+    auto cap = [&] { return (4096LL * workers >> lane_bits) * (ctx->precision == CFET_PREC_FX ? 1 : 1 << 20); };
+    while (lane_bits > 0 && cap() * ctx->grid < dim) --lane_bits;
+    ctx->csr_fx.lane_bits = ctx->csr_c.lane_bits = lane_bits;
+    const std::vector<int> rb = csr_row_split(ctx->csr_rp, 1 + nV, dim, ctx->grid, cap());
+    CKC(cudaMalloc(&ctx->d_csr_rb, rb.size() * sizeof(int)), "cudaMalloc(row split)");
+    CKC(cudaMemcpy(ctx->d_csr_rb, rb.data(), rb.size() * sizeof(int), cudaMemcpyHostToDevice), "upload row split");
+    ctx->csr_fx.rb = ctx->csr_c.rb = ctx->d_csr_rb;
+  }
+  std::vector<int>().swap(ctx->csr_rp);
   CKC(cudaMalloc(&ctx->d_partials, partial_words_per_cta(ctx) * (size_t)ctx->grid * sizeof(double)),
       "cudaMalloc(partials)");
   CKC(cudaMalloc(&ctx->d_bar, 2 * sizeof(unsigned)), "cudaMalloc(barrier)");

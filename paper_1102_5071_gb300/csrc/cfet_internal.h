@@ -150,6 +150,9 @@ struct OpCsrFx {
   const long long* VI;    // [nnz] or NULL (real operators)
   int E_op[1 + kMaxDrives];
   double maxrow[1 + kMaxDrives];  // max over rows of sum (|re| + |im|), real units
+  const int* rb;          // [grid + 1]: rows [rb[b], rb[b + 1]) belong to CTA b (csr_row_split)
+  int lane_bits;          // 2^lane_bits neighbouring threads share a row in the apply
+  unsigned cplx;          // bit o: operator o has complex values
 };
 
 // Mixed-precision forms (see kernels_c64.cu): FP32 operator data.
@@ -178,6 +181,9 @@ struct OpCsrC {
   const int* col;
   const float* vr;
   const float* vi;        // NULL for real operators
+  const int* rb;          // as OpCsrFx
+  int lane_bits;
+  unsigned cplx;
 };
 
 struct PropParams {

@@ -298,47 +298,59 @@ __device__ __forceinline__ longlong2 fx_apply_dia(const longlong2* q, const long
 // (complex values: re = sum VR w.x - VI w.y, im = sum VR w.y + VI w.x; the row
 // sums of |VR| + |VI| stay below 2^62 and |q| < 2^57, so no sum overflows),
 // then one rounded product with the operator's scalar mantissa as for DIA.
-__device__ __forceinline__ longlong2 fx_apply_csr(const longlong2* q, const longlong2* qm, int r, int dim,
+// 2^op.lane_bits neighbouring threads (all of them in the call, `on` false past
+// the CTA's rows) share the row r: each takes every 2^lane_bits-th entry and the
+// exact partial sums are added by shuffles, so the result does not depend on
+// the split; the first of them returns it.
+// Bound by the gathers: every entry fetches a 32-byte sector of q at random from
+// L2 besides its 20 B of matrix data.  60 001 rows of 20 entries (random complex
+// H0, banded real V) take 15.5 us per apply on 152 CTAs, 3.9 TB/s of those
+// bytes; more loads in flight per thread (unrolled by 4, or batches of 4 and 6
+// entries loaded before their use) measured 18-21 us.  One thread per row over
+// equal row counts, as before, took 22.5 us in the mean CTA and 48 in the last.
+__device__ __forceinline__ void fx_lane_sum128(__int128& a, int lane_bits) {
+  for (int b = 0; b < lane_bits; ++b) {
+    const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)a, 1 << b);
+    const long long hi = __shfl_xor_sync(0xffffffffu, (long long)(a >> 64), 1 << b);
+    a += ((__int128)hi << 64) | lo;
+  }
+}
+__device__ __forceinline__ longlong2 fx_apply_csr(const longlong2* q, const longlong2* qm, int r, bool on, int dim,
                                                   const OpCsrFx& op, const FxConstA& c) {
+  const int T = 1 << op.lane_bits, sub = threadIdx.x & (T - 1);
   long long ur = 0, ui = 0;
   for (int o = 0; o < op.nops; ++o) {
     const int* rp = op.rp + (size_t)o * (dim + 1);
-    const int e0 = __ldg(rp + r), e1 = __ldg(rp + r + 1);
+    const int e0 = on ? __ldg(rp + r) + sub : 0, e1 = on ? __ldg(rp + r + 1) : 0;
     __int128 ar = 0, ai = 0;
-    if (op.VI) {
-      for (int e = e0; e < e1; ++e) {
+    if ((op.cplx >> o) & 1u) {
+#pragma unroll 2
+      for (int e = e0; e < e1; e += T) {
         const long long a = __ldg(op.VR + e), b = __ldg(op.VI + e);
         const longlong2 w = q[__ldg(op.col + e)];
         ar += (__int128)a * w.x - (__int128)b * w.y;
         ai += (__int128)a * w.y + (__int128)b * w.x;
       }
     } else {
-      for (int e = e0; e < e1; ++e) {
+#pragma unroll 2
+      for (int e = e0; e < e1; e += T) {
         const long long a = __ldg(op.VR + e);
         const longlong2 w = q[__ldg(op.col + e)];
         ar += (__int128)a * w.x;
         ai += (__int128)a * w.y;
       }
     }
+    fx_lane_sum128(ar, op.lane_bits);
+    fx_lane_sum128(ai, op.lane_bits);
     ur += fx_mulhi(c.m_op[o], fx_shr128(ar, c.sh_pre[o]));
     ui += fx_mulhi(c.m_op[o], fx_shr128(ai, c.sh_pre[o]));
   }
-  if (c.use_prev) {
+  if (c.use_prev && on && sub == 0) {
     const longlong2 w = qm[r];
     ur += fx_mulhi(c.m_p, w.x << c.pp);
     ui += fx_mulhi(c.m_p, w.y << c.pp);
   }
   return make_longlong2(ur, ui);
-}
-
-// The two stored-matrix families behind one name (DIA, CSR).
-__device__ __forceinline__ longlong2 fx_apply_sparse(const longlong2* q, const longlong2* qm, int r, int dim,
-                                                     const OpDiaFx& op, const FxConstA& c) {
-  return fx_apply_dia(q, qm, r, dim, op, c);
-}
-__device__ __forceinline__ longlong2 fx_apply_sparse(const longlong2* q, const longlong2* qm, int r, int dim,
-                                                     const OpCsrFx& op, const FxConstA& c) {
-  return fx_apply_csr(q, qm, r, dim, op, c);
 }
 
 }  // namespace cfet

@@ -216,13 +216,15 @@ __device__ __forceinline__ void cheb_rot(int k, long long yr, long long yi, long
   }
 }
 
+// (CSR: 2^lane_bits threads share row x, all of them in the call, `on` false past the CTA's rows.)
 template <int FAMILY, class Op>
-__device__ __forceinline__ longlong2 cheb_apply1(const longlong2* cur, const longlong2* prev, int x, int dim,
+__device__ __forceinline__ longlong2 cheb_apply1(const longlong2* cur, const longlong2* prev, int x, bool on, int dim,
                                                  const Op& op, const FxConstA& c, const long long* mb, long long m_s) {
   longlong2 y;
   if constexpr (FAMILY == kFamilySpin) y = fx_apply_spin(cur, prev, x, op, c, mb);
-  else y = fx_apply_sparse(cur, prev, x, dim, op, c);
-  if (m_s != 0) {
+  else if constexpr (FAMILY == kFamilyDia) y = fx_apply_dia(cur, prev, x, dim, op, c);
+  else y = fx_apply_csr(cur, prev, x, on, dim, op, c);
+  if (m_s != 0 && on) {
     const longlong2 v = cur[x];
     y.x += fx_mulhi(m_s, v.x << c.pk);
     y.y += fx_mulhi(m_s, v.y << c.pk);
@@ -275,11 +277,20 @@ __device__ __forceinline__ void cheb_pass(const SmemCheb& S, const Op& op, const
       }
     }
   };
-  int x = wx0;
-  for (; x < wxe; x += wstep) {
-    longlong2 y = make_longlong2(0, 0);
-    if (APPLY) y = cheb_apply1<FAMILY>(cur, prev, x, dim, op, S.c, S.mb, S.m_s);
-    elem(x, y);
+  if constexpr (FAMILY == kFamilyCsr && APPLY) {
+    const int lb = op.lane_bits, t = threadIdx.x;
+    for (int r0 = wx0 - t; r0 < wxe; r0 += wstep >> lb) {
+      const int r = r0 + (t >> lb);
+      const bool on = r < wxe;
+      const longlong2 y = cheb_apply1<FAMILY>(cur, prev, r, on, dim, op, S.c, S.mb, S.m_s);
+      if (on && (t & ((1 << lb) - 1)) == 0) elem(r, y);
+    }
+  } else {
+    for (int x = wx0; x < wxe; x += wstep) {
+      longlong2 y = make_longlong2(0, 0);
+      if (APPLY) y = cheb_apply1<FAMILY>(cur, prev, x, true, dim, op, S.c, S.mb, S.m_s);
+      elem(x, y);
+    }
   }
 }
 
@@ -294,8 +305,12 @@ __global__ void __launch_bounds__(kChebThreads, 1) k_cheb_fx(PropParams p, Op op
   const int G = gridDim.x;
   const int chunk = (dim + G - 1) / G;
   const int wstep = blockDim.x;
-  const int wx0 = blockIdx.x * chunk + tid;
-  const int wxe = min(dim, (blockIdx.x + 1) * chunk);
+  int wx0 = blockIdx.x * chunk + tid;
+  int wxe = min(dim, (blockIdx.x + 1) * chunk);
+  if constexpr (FAMILY == kFamilyCsr) {  // rows split by their work, not their number (csr_row_split)
+    wx0 = __ldg(op.rb + blockIdx.x) + tid;
+    wxe = __ldg(op.rb + blockIdx.x + 1);
+  }
   const int ncoef = 1 + p.nV;
   const unsigned tag0 = (unsigned)ld_volatile_i32((const int*)&p.st->tag_base);
   unsigned gen = 0;

@@ -468,8 +468,12 @@ __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_fx(PropPa
   // neighbours of low-bit flips (and short band offsets) are found in L1
   const int chunk = (dim + G - 1) / G;
   const int wstep = NW * 32;
-  const int wx0 = blockIdx.x * chunk + tid;  // workers only
-  const int wxe = min(dim, (blockIdx.x + 1) * chunk);
+  int wx0 = blockIdx.x * chunk + tid;  // workers only
+  int wxe = min(dim, (blockIdx.x + 1) * chunk);
+  if constexpr (FAMILY == kFamilyCsr) {  // rows split by their work, not their number (csr_row_split)
+    wx0 = __ldg(op.rb + blockIdx.x) + tid;
+    wxe = __ldg(op.rb + blockIdx.x + 1);
+  }
   const int ncoef = 1 + p.nV;
   // record exchange: three slots (phase A, phase B, reconstruction) of six
   // tagged words per CTA; two uses of one slot are always separated by an
@@ -685,10 +689,25 @@ __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_fx(PropPa
                 mx = max(mx, max(fx_absmax(h1.x, h1.y), fx_absmax(h2.x, h2.y)));
               }
             }
+            if constexpr (FAMILY == kFamilyCsr) {
+              const int lb = op.lane_bits;
+              for (int r0 = wx0 - tid; r0 < wxe; r0 += wstep >> lb) {
+                const int r = r0 + (tid >> lb);
+                const bool on = r < wxe;
+                const longlong2 hv = fx_apply_csr(q, qm, r, on, dim, op, c);
+                if (on && (tid & ((1 << lb) - 1)) == 0) {
+                  u[r] = hv;
+                  const longlong2 v = q[r];
+                  a2 += (__int128)v.x * hv.x + (__int128)v.y * hv.y;
+                  mx = max(mx, fx_absmax(hv.x, hv.y));
+                }
+              }
+              x = wxe;
+            }
             for (; x < wxe; x += wstep) {
-              longlong2 hv;
+              longlong2 hv = make_longlong2(0, 0);
               if constexpr (FAMILY == kFamilySpin) hv = fx_apply_spin(q, qm, x, op, c, S.mb);
-              else hv = fx_apply_sparse(q, qm, x, dim, op, c);
+              else if constexpr (FAMILY == kFamilyDia) hv = fx_apply_dia(q, qm, x, dim, op, c);
               u[x] = hv;
               const longlong2 v = q[x];
               a2 += (__int128)v.x * hv.x + (__int128)v.y * hv.y;
