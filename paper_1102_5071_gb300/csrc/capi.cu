@@ -142,10 +142,8 @@ struct cfet_ctx {
 namespace {
 
 // Reduction / exchange scratch per CTA (8-byte words): the FP64 kernel uses 3
-// partials, the control-warp kernels slots of tagged words: the two-pass
-// fixed-point and complex64 kernels 3 slots of at most 8 words, the one-pass
-// fixed-point kernel two 16-word slots and three 8-word slots.
-constexpr size_t kPartialWordsPerCta = 56;
+// partials, the control-warp kernels the two slots of the record exchange.
+constexpr size_t kPartialWordsPerCta = 8;
 constexpr int kMaxCtlGrid = 256;  // 32 lanes x 8 records per lane of the exchange
 // FP64 kernel with full re-orthogonalisation: 3 slots + 2 m_max Gram-Schmidt coefficients per CTA
 static size_t partial_words_per_cta(const cfet_ctx* ctx) {
@@ -1826,10 +1824,11 @@ cfet_status cfet_selftest_wait_timeout(int32_t which, double timeout_s, int32_t*
   unsigned long long* rec = nullptr;
   unsigned* bar = nullptr;
   int* st = nullptr;
-  cudaError_t e = cudaMalloc(&rec, 2 * sizeof(unsigned long long));
+  constexpr size_t rec_words = 2 * kPartialWordsPerCta;  // two CTAs
+  cudaError_t e = cudaMalloc(&rec, rec_words * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMalloc(&bar, 2 * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMalloc(&st, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(rec, 0, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMemset(rec, 0, rec_words * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMemset(bar, 0, 2 * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMemset(st, 0, sizeof(int));
   if (e == cudaSuccess) e = (cudaError_t)launch_wait_selftest(which, rec, bar, st, (long long)(timeout_s * 1e9));

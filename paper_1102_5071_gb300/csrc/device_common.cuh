@@ -70,41 +70,48 @@ static __device__ bool warp_grid_barrier(unsigned* bar, unsigned& gen, int* stat
 // ------------------------------------------------------------------ tagged exchange
 // Grid-wide exchange of small per-CTA records, executed by one warp of each
 // CTA; it is the grid barrier of the kernels with a control warp.  A record is
-// W 32-bit payload words, each published as one 64-bit word
-// (tag << 32 | payload), so that a reader sees a payload together with its tag
-// (aligned 64-bit stores are single-copy atomic); readers wait until the words
-// of every CTA carry `tag`.  No atomics and no last-arriver step: one store and
-// one round of loads per exchange.  Records of up to 8 words are stored
-// contiguously (word w of CTA i at rec[i S + w], S = W rounded up to 8 for
-// 5..8 words, so that no record straddles two 64-byte halves of a line);
-// wider ones word-major (rec[w G + i]), so that a warp's load of one word of
-// 32 consecutive CTAs touches two 128-byte lines: a 16-word exchange of 152
-// CTAs took 11.1 us contiguous and 4.0 us word-major, while the 4- and 6-word
-// records of the Krylov kernels were 3-10 % faster contiguous (measured both
-// ways); a 6-word exchange took 6.2 us at stride 6 and 4.5 us at stride 8.
-// Lane l reads the records of CTAs l, l + 32, ..., l + 32 (kExchMaxPerLane - 1)
-// in that order and passes each to acc.add(); acc.reset() starts every polling
-// round.  `fence` orders the CTA's earlier global stores before its record
-// (writer) and the records before the CTA's later loads (reader); it is needed
-// when other CTAs will read vectors written before the exchange.  Returns false
-// in every lane when the wait limit expired (CFET_ETIMEOUT recorded) or another
-// CTA reported an error.  A slot of W words per CTA needs S G words.
+// W <= 6 32-bit payload words, published in pairs of 64-bit words that hold three
+// payload words and 16 bits of the exchange's tag each
+//   tag << 48 | payload[3j] | low half of payload[3j + 1] << 32,
+//   tag << 48 | high half of payload[3j + 1] | payload[3j + 2] << 16,
+// so that a reader sees every payload bit together with its tag (an aligned
+// 64-bit element of a 16-byte store or load is single-copy atomic); readers wait
+// until the words of every CTA carry `tag`.  No atomics and no last-arriver step:
+// one store and one round of loads per exchange.  Two slots alternate by the
+// parity of the tag, which counts the exchanges of a call from 1, so a stale
+// word always carries the tag of two exchanges before (the slots are cleared
+// per call), and a slot is rewritten only after every CTA has published in the
+// other one, that is, has read this one.  Lane l reads the records of CTAs l,
+// l + 32, ..., l + 32 (kExchMaxPerLane - 1); the loads of a polling round (one
+// or two 16-byte loads per record) are all in flight together, and only the
+// complete round is passed to acc.add(), in that order.  (One tagged 64-bit word
+// per payload word, six 8-byte loads per record accumulated inside the polling
+// loop, took 4.0 us per exchange of six words over 152 CTAs where registers were
+// plentiful and 6.4 us where they were not.)
+// `fence` orders the CTA's earlier global stores before its record (writer) and
+// the records before the CTA's later loads (reader); it is needed when other
+// CTAs will read vectors written before the exchange.  Returns false in every
+// lane when the wait limit expired (CFET_ETIMEOUT recorded) or another CTA
+// reported an error.  The two slots need kExchWords G words.
 constexpr int kExchMaxPerLane = 8;  // grids of at most 256 CTAs
+constexpr int kExchHeld = 5;        // records per lane kept in registers (grids of at most 160 CTAs)
+constexpr int kExchWords = 8;
 
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+__device__ __forceinline__ void st_relaxed_v2(unsigned long long* p, unsigned long long a, unsigned long long b) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
 }
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+__device__ __forceinline__ ulonglong2 ld_relaxed_v2(const unsigned long long* p) {
+  ulonglong2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
   return v;
 }
 
 template <int W, class Acc>
-static __device__ bool ctl_exchange(unsigned long long* rec, const unsigned (&mine)[W], unsigned tag, bool fence,
-                                    int* status, long long timeout_ns, long long& spin, Acc& acc) {
-  constexpr bool kWordMajor = W > 8;
-  constexpr int kStride = (W > 4 && W <= 8) ? 8 : W;  // contiguous records: words per CTA
+static __device__ __forceinline__ bool ctl_exchange(unsigned long long* rec, const unsigned (&mine)[W], unsigned tag,
+                                                    bool fence, int* status, long long timeout_ns, long long& spin,
+                                                    Acc& acc) {
+  static_assert(W >= 1 && W <= 6, "two pairs of words hold six payload words");
+  constexpr int NP = (W + 2) / 3;
   const int lane = threadIdx.x & 31;
   const int G = gridDim.x;
   if (G == 1) {  // a single CTA: its own record is the total; nothing to publish or wait for
@@ -113,50 +120,85 @@ static __device__ bool ctl_exchange(unsigned long long* rec, const unsigned (&mi
     return true;
   }
   const long long c0 = sm_clock();
+  rec += (size_t)(tag & 1u) * (kExchWords / 2) * G;
+  const unsigned t16 = tag & 0xffffu;
   if (lane == 0) {
     if (fence) __threadfence();
 #pragma unroll
-    for (int w = 0; w < W; ++w)
-      st_relaxed_u64(kWordMajor ? rec + (size_t)w * G + blockIdx.x : rec + (size_t)blockIdx.x * kStride + w,
-                     ((unsigned long long)tag << 32) | mine[w]);
+    for (int j = 0; j < NP; ++j) {
+      const unsigned v0 = mine[3 * j], v1 = 3 * j + 1 < W ? mine[3 * j + 1 < W ? 3 * j + 1 : 0] : 0u;
+      const unsigned v2 = 3 * j + 2 < W ? mine[3 * j + 2 < W ? 3 * j + 2 : 0] : 0u;
+      const unsigned long long t = (unsigned long long)t16 << 48;
+      st_relaxed_v2(rec + (size_t)blockIdx.x * 4 + 2 * j, t | ((unsigned long long)(v1 & 0xffffu) << 32) | v0,
+                    t | ((unsigned long long)v2 << 16) | (v1 >> 16));
+    }
   }
   __syncwarp();
   int ok = 1;
   const long long t0 = global_timer_ns();
   unsigned rounds = 0;
+  unsigned long long x0[kExchHeld], x1[kExchHeld], x2[kExchHeld], x3[kExchHeld];
   while (true) {
-    acc.reset();
-    int ready = 1;
+    unsigned bad = 0;
 #pragma unroll
-    for (int j = 0; j < kExchMaxPerLane; ++j) {
-      const int i = lane + 32 * j;
-      if (i < G) {
-        unsigned v[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-          const unsigned long long x =
-              ld_relaxed_u64(kWordMajor ? rec + (size_t)w * G + i : rec + (size_t)i * kStride + w);
-          v[w] = (unsigned)x;
-          ready &= (unsigned)(x >> 32) == tag;
+    for (int k = 0; k < kExchHeld; ++k) {
+      x0[k] = x1[k] = x2[k] = x3[k] = (unsigned long long)t16 << 48;
+      if (32 * k < G) {  // (uniform)
+        const int i = lane + 32 * k < G ? lane + 32 * k : 0;  // (past the end: record 0, not passed on)
+        const ulonglong2 v = ld_relaxed_v2(rec + (size_t)i * 4);
+        x0[k] = v.x;
+        x1[k] = v.y;
+        if constexpr (NP > 1) {
+          const ulonglong2 w = ld_relaxed_v2(rec + (size_t)i * 4 + 2);
+          x2[k] = w.x;
+          x3[k] = w.y;
         }
-        acc.add(v);
       }
     }
-    if (__all_sync(0xffffffffu, ready)) break;
+#pragma unroll
+    for (int k = 0; k < kExchHeld; ++k)
+      bad |= ((unsigned)(x0[k] >> 48) ^ t16) | ((unsigned)(x1[k] >> 48) ^ t16) | ((unsigned)(x2[k] >> 48) ^ t16) |
+             ((unsigned)(x3[k] >> 48) ^ t16);
+#pragma unroll 1
+    for (int i = lane + 32 * kExchHeld; i < G; i += 32) {
+      const ulonglong2 v = ld_relaxed_v2(rec + (size_t)i * 4), w = NP > 1 ? ld_relaxed_v2(rec + (size_t)i * 4 + 2) : v;
+      bad |= ((unsigned)(v.x >> 48) ^ t16) | ((unsigned)(v.y >> 48) ^ t16) | ((unsigned)(w.x >> 48) ^ t16) |
+             ((unsigned)(w.y >> 48) ^ t16);
+    }
+    if (__all_sync(0xffffffffu, bad == 0)) break;
     if ((++rounds & 15u) == 0u) {
-      int bad = 0;
+      int give_up = 0;
       if (lane == 0) {
         if (ld_volatile_i32(status) != 0) {
-          bad = 1;
+          give_up = 1;
         } else if (global_timer_ns() - t0 > timeout_ns) {
           atomicCAS(status, 0, (int)CFET_ETIMEOUT);
-          bad = 1;
+          give_up = 1;
         }
       }
-      if (__shfl_sync(0xffffffffu, bad, 0)) {
+      if (__shfl_sync(0xffffffffu, give_up, 0)) {
         ok = 0;
         break;
       }
+    }
+  }
+  acc.reset();
+  auto take = [&](unsigned long long a0, unsigned long long a1, unsigned long long a2, unsigned long long a3) {
+    const unsigned v[6] = {(unsigned)a0, ((unsigned)(a0 >> 32) & 0xffffu) | ((unsigned)a1 << 16), (unsigned)(a1 >> 16),
+                           (unsigned)a2, ((unsigned)(a2 >> 32) & 0xffffu) | ((unsigned)a3 << 16), (unsigned)(a3 >> 16)};
+    unsigned w[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) w[i] = v[i];
+    acc.add(w);
+  };
+  if (ok) {
+#pragma unroll
+    for (int k = 0; k < kExchHeld; ++k)
+      if (lane + 32 * k < G) take(x0[k], x1[k], x2[k], x3[k]);
+#pragma unroll 1
+    for (int i = lane + 32 * kExchHeld; i < G; i += 32) {  // complete: the words no longer change
+      const ulonglong2 v = ld_relaxed_v2(rec + (size_t)i * 4), w = NP > 1 ? ld_relaxed_v2(rec + (size_t)i * 4 + 2) : v;
+      take(v.x, v.y, w.x, w.y);
     }
   }
   if (fence) __threadfence();
@@ -317,7 +359,14 @@ __constant__ double kInvN[kSmallTaylorTerms + 1] = {
     0.0, 1.0, 1.0 / 2, 1.0 / 3, 1.0 / 4, 1.0 / 5, 1.0 / 6, 1.0 / 7, 1.0 / 8, 1.0 / 9, 1.0 / 10,
     1.0 / 11, 1.0 / 12, 1.0 / 13, 1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17, 1.0 / 18};
 
-static __device__ void small_expm_e1(int k, const double* a, const double* b, double ts, double* yr, double* yi,
+// (Out of line, with rolled loops, like every cold or long function of the
+// control path: the persistent kernels' code was over 500 KB with them inlined
+// at each use, and the control warps spent microseconds per iteration on
+// instruction fetches.)
+static __device__ __noinline__ void sincos_call(double x, double* sn, double* cs) { sincos(x, sn, cs); }
+static __device__ __noinline__ double div_call(double a, double b) { return a / b; }
+
+static __device__ __noinline__ void small_expm_e1(int k, const double* a, const double* b, double ts, double* yr, double* yi,
                                      double* tr, double* ti) {
   const int lane = threadIdx.x & 31;
   // Spectral interval of T_k from FP32 Gershgorin bounds of the truncated
@@ -327,6 +376,7 @@ static __device__ void small_expm_e1(int k, const double* a, const double* b, do
   GershAcc g;
   sb_gersh_init(g);
   int bad = 0;
+#pragma unroll 1
   for (int r = lane; r < k; r += 32) {
     sb_gersh_row(g, r, k, a, b);
     bad |= sb_nonfinite(a[r]) | (r < k - 1 ? sb_nonfinite(b[r]) : 0);
@@ -354,7 +404,7 @@ static __device__ void small_expm_e1(int k, const double* a, const double* b, do
   int S = 1;
   if (!bad) S = sr32 < 65536.0f ? (int)ceilf(sr32) : 65536;
   if (S < 1) S = 1;
-  const double hstep = S == 1 ? ts : ts / S;
+  const double hstep = S == 1 ? ts : div_call(ts, S);
   const float x = bad ? 1.0f : sr32 / (float)S;
   const int nterms = x > 0.5f ? kSmallTaylorTerms : (x > 0.25f ? 15 : (x > 0.1f ? 12 : 10));
   // rows owned by this lane: shifted diagonal and couplings in registers
@@ -365,7 +415,7 @@ static __device__ void small_expm_e1(int k, const double* a, const double* b, do
   const double bl1 = on1 ? b[r1 - 1] : 0.0, br1 = (on1 && r1 < k - 1) ? b[r1] : 0.0;
   if (!bad && !noshift && sr32 > (float)kChebyshevFrom && sr32 < 4096.0f) {
     const double rho = sb_f2d(rho32), sr = fabs(ts) * rho;
-    const double a_ = sr, inv_a = 1.0 / a_, inv_rho = 1.0 / rho;
+    const double a_ = sr, inv_a = div_call(1.0, a_), inv_rho = div_call(1.0, rho);
     const bool neg = ts < 0.0;  // (-i s)^n with s = sign(ts)
     const double x0 = d0 * inv_rho, xl0 = bl0 * inv_rho, xr0 = br0 * inv_rho;
     const double x1 = d1 * inv_rho, xl1 = bl1 * inv_rho, xr1 = br1 * inv_rho;
@@ -373,6 +423,7 @@ static __device__ void small_expm_e1(int k, const double* a, const double* b, do
     double jn1 = 0.0, jn = 1e-200, norm = 0.0;  // J_{n+1}, J_n (unscaled)
     // Clenshaw state b_{n+1}, b_{n+2} (real and imaginary parts) of each row
     double pr0 = 0, qr0 = 0, pi0 = 0, qi0 = 0, pr1 = 0, qr1 = 0, pi1 = 0, qi1 = 0;
+#pragma unroll 1
     for (int n = nstart; n >= 1; --n) {
       // coefficient 2 (-i s)^n J_n: the phase (-i)^m, m = n or -n mod 4
       const int m = neg ? ((4 - (n & 3)) & 3) : (n & 3);
@@ -423,9 +474,9 @@ static __device__ void small_expm_e1(int k, const double* a, const double* b, do
       si1 = fma(xr1, ri, fma(xl1, li, x1 * pi1)) - qi1;
     }
     __syncwarp();
-    const double inv_norm = 1.0 / norm;
+    const double inv_norm = div_call(1.0, norm);
     double sn, cs;
-    sincos(ts * sig, &sn, &cs);
+    sincos_call(ts * sig, &sn, &cs);
     // y = e^{-i ts sig} S / norm, e^{-i ts sig} = cs - i sn
     if (on0) { yr[r0] = (sr0 * cs + si0 * sn) * inv_norm; yi[r0] = (si0 * cs - sr0 * sn) * inv_norm; }
     if (on1) { yr[r1] = (sr1 * cs + si1 * sn) * inv_norm; yi[r1] = (si1 * cs - sr1 * sn) * inv_norm; }
@@ -434,25 +485,28 @@ static __device__ void small_expm_e1(int k, const double* a, const double* b, do
   }
   if (k <= 16) {
     // Rows on half-warps: lane l holds the real (l < 16) or the imaginary part
-    // (l >= 16) of row l & 15, neighbours by shuffles within each half.  The
-    // same expressions as the two-rows-per-lane form below (bit-identical
-    // results) with half the FP64 instructions per term.
+    // (l >= 16) of row l & 15, neighbours by shuffles within each half: half the
+    // FP64 instructions per term of the two-rows-per-lane form below.  The
+    // Taylor polynomial is summed by Horner's rule, y <- y_0 + (-i h T / n) y
+    // with h T formed once: four FP64 instructions per term instead of the six
+    // of the running sum (the pipe takes 64 cycles for each).
     const int r = lane & 15;
     const bool imag = lane >= 16, on = r < k;
-    const double d = on ? a[r] - sig : 0.0;
-    const double bl = (on && r > 0) ? b[r - 1] : 0.0, br = (on && r < k - 1) ? b[r] : 0.0;
+    const double d = on ? hstep * (a[r] - sig) : 0.0;
+    const double bl = (on && r > 0) ? hstep * b[r - 1] : 0.0, br = (on && r < k - 1) ? hstep * b[r] : 0.0;
     double acc = (r == 0 && !imag) ? 1.0 : 0.0;  // current y
+#pragma unroll 1
     for (int sidx = 0; sidx < S; ++sidx) {
       double t = acc;
-      for (int n = 1; n <= nterms; ++n) {
-        const double c = hstep * kInvN[n];
+#pragma unroll 1
+      for (int n = nterms; n >= 1; --n) {
         const double tl = __shfl_up_sync(0xffffffffu, t, 1, 16);    // row r - 1 (own value at r = 0: bl = 0)
         const double tn = __shfl_down_sync(0xffffffffu, t, 1, 16);  // row r + 1 (own value at r = 15: br = 0)
         const double z = fma(br, tn, fma(bl, tl, d * t));
         const double zo = __shfl_xor_sync(0xffffffffu, z, 16);       // the other part of the same row
-        t = imag ? -c * zo : c * zo;                                 // (-i c) z
-        acc += t;
+        t = fma(imag ? -kInvN[n] : kInvN[n], zo, acc);               // acc + (-i / n) z
       }
+      acc = t;
     }
     if (noshift) {
       if (on) (imag ? yi : yr)[r] = acc;
@@ -460,7 +514,7 @@ static __device__ void small_expm_e1(int k, const double* a, const double* b, do
       return;
     }
     double sn, cs;
-    sincos(ts * sig, &sn, &cs);
+    sincos_call(ts * sig, &sn, &cs);
     const double ao = __shfl_xor_sync(0xffffffffu, acc, 16);
     // multiply by e^{-i ts sig} = cs - i sn
     if (on) {
@@ -471,11 +525,13 @@ static __device__ void small_expm_e1(int k, const double* a, const double* b, do
     return;
   }
   double ar0 = (r0 == 0) ? 1.0 : 0.0, ai0 = 0.0, ar1 = 0.0, ai1 = 0.0;  // current y
+#pragma unroll 1
   for (int sidx = 0; sidx < S; ++sidx) {
     double t_r0 = ar0, t_i0 = ai0, t_r1 = ar1, t_i1 = ai1;
     if (on0) { tr[r0] = t_r0; ti[r0] = t_i0; }
     if (on1) { tr[r1] = t_r1; ti[r1] = t_i1; }
     __syncwarp();
+#pragma unroll 1
     for (int n = 1; n <= nterms; ++n) {
       const double c = hstep * kInvN[n];
       double zr0 = 0, zi0 = 0, zr1 = 0, zi1 = 0;
@@ -502,7 +558,7 @@ static __device__ void small_expm_e1(int k, const double* a, const double* b, do
     }
   }
   double sn = 0.0, cs = 1.0;
-  if (!noshift) sincos(ts * sig, &sn, &cs);
+  if (!noshift) sincos_call(ts * sig, &sn, &cs);
   // multiply by e^{-i ts sig} = cs - i sn
   if (on0) { yr[r0] = ar0 * cs + ai0 * sn; yi[r0] = ai0 * cs - ar0 * sn; }
   if (on1) { yr[r1] = ar1 * cs + ai1 * sn; yi[r1] = ai1 * cs - ar1 * sn; }
@@ -523,7 +579,7 @@ __constant__ float kInvNf[kSmallTaylorTerms + 1] = {
 // True only when err exceeds thr even after that bound is taken off: the FP64
 // evaluation (same series, same number of terms) would then reject k too, so
 // the FP64 small exponential can be skipped.  Warp-uniform result.
-static __device__ bool small_expm_rejects32(int k, const double* a, const double* b, double ts, double scale,
+static __device__ __noinline__ bool small_expm_rejects32(int k, const double* a, const double* b, double ts, double scale,
                                             double thr) {
   if (k < 1 || k > 16 || !(thr >= 0.0)) return false;
   const unsigned full = 0xffffffffu;
@@ -546,6 +602,7 @@ static __device__ bool small_expm_rejects32(int k, const double* a, const double
   const float d = on ? (float)(ad - (double)sig) : 0.f, ad_ = fabsf(d), abl = fabsf(bl), abr = fabsf(br);
   const float tsf = (float)ts;
   float t = (r == 0 && !imag) ? 1.f : 0.f, acc = t, m = t, msum = 0.f;
+#pragma unroll 2
   for (int n = 1; n <= nterms; ++n) {
     const float c = tsf * kInvNf[n];
     const float tl = __shfl_up_sync(full, t, 1, 16), tn = __shfl_down_sync(full, t, 1, 16);
@@ -570,9 +627,10 @@ static __device__ bool small_expm_rejects32(int k, const double* a, const double
 
 // Gershgorin width of T (max of a_r + radius minus min of a_r - radius), an
 // upper bound of its eigenvalue spread; warp-uniform result.
-static __device__ double gersh_width(int k, const double* a, const double* b) {
+static __device__ __noinline__ double gersh_width(int k, const double* a, const double* b) {
   const int lane = threadIdx.x & 31;
   double lo = 1e300, hi = -1e300;
+#pragma unroll 1
   for (int r = lane; r < k; r += 32) {
     const double rad = (r > 0 ? fabs(b[r - 1]) : 0.0) + (r < k - 1 ? fabs(b[r]) : 0.0);
     lo = fmin(lo, a[r] - rad);
@@ -593,6 +651,7 @@ static __device__ bool gersh_gate(int k, const double* a, const double* b, doubl
   const int lane = threadIdx.x & 31;
   GershAcc s;
   sb_gersh_init(s);
+#pragma unroll 1
   for (int r = lane; r < k; r += 32) sb_gersh_row(s, r, k, a, b);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -616,6 +675,7 @@ static __device__ bool krylov_lead_rejects(int k, const double* a, const double*
   const int lane = threadIdx.x & 31;
   LeadAcc s;
   sb_lead_init(s);
+#pragma unroll 1
   for (int r = lane; r < k; r += 32) sb_lead_row(s, r, k, a, b);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {

@@ -116,18 +116,24 @@ __device__ __forceinline__ long long fx_absmax(long long a, long long b) {
 }
 
 // ------------------------------------------------------------------ exact reductions
-// Sum over a warp of (lo, hi) 128-bit values and max of an int64 (lane 0 result).
+// Sum over a warp of (lo, hi) 128-bit values and max of a non-negative int64,
+// results in every lane.  The sum goes through five 26-bit limbs (the top one
+// signed, |value| < 2^122), each one warp reduction instruction: shorter than
+// five levels of six shuffles with carries.
 __device__ __forceinline__ void fx_warp_reduce(unsigned long long& lo, long long& hi, long long& mx) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long lo2 = __shfl_down_sync(0xffffffffu, lo, o);
-    const long long hi2 = __shfl_down_sync(0xffffffffu, hi, o);
-    const long long mx2 = __shfl_down_sync(0xffffffffu, mx, o);
-    const unsigned long long s = lo + lo2;
-    hi = hi + hi2 + (s < lo ? 1 : 0);
-    lo = s;
-    mx = mx > mx2 ? mx : mx2;
-  }
+  constexpr unsigned kM26 = (1u << 26) - 1u, kAll = 0xffffffffu;
+  const unsigned r0 = __reduce_add_sync(kAll, (unsigned)lo & kM26);
+  const unsigned r1 = __reduce_add_sync(kAll, (unsigned)(lo >> 26) & kM26);
+  const unsigned r2 = __reduce_add_sync(kAll, ((unsigned)(lo >> 52) | ((unsigned)hi << 12)) & kM26);
+  const unsigned r3 = __reduce_add_sync(kAll, (unsigned)(hi >> 14) & kM26);
+  const int r4 = __reduce_add_sync(kAll, (int)(hi >> 40));
+  const unsigned mh = (unsigned)((unsigned long long)mx >> 32);
+  const unsigned xh = __reduce_max_sync(kAll, mh);
+  const unsigned xl = __reduce_max_sync(kAll, mh == xh ? (unsigned)mx : 0u);
+  const unsigned long long t = (unsigned long long)r0 + ((unsigned long long)r1 << 26);
+  lo = t + ((unsigned long long)r2 << 52);
+  hi = (long long)(r2 >> 12) + (lo < t ? 1 : 0) + ((long long)r3 << 14) + ((long long)r4 << 40);
+  mx = (long long)(((unsigned long long)xh << 32) | xl);
 }
 // (hi 2^64 + lo) 2^kRedShift rounded to the nearest double, by integer operations.
 __device__ __forceinline__ double fx_i128_to_double(unsigned long long lo, long long hi) {
@@ -137,10 +143,18 @@ __device__ __forceinline__ double fx_i128_to_double(unsigned long long lo, long 
 
 // ------------------------------------------------------------------ apply constants
 struct FxConstA {
-  // spin
-  long long m_cz, m_hop, m_x, m_p;
+  // spin: mantissas of the diagonal, hop, uniform field and q_{k-1} terms with
+  // their product shifts folded in, and the normalising shifts of their inputs
+  // (by name, or by term number)
+  union {
+    struct { long long m_cz, m_hop, m_x, m_p; };
+    long long m4[4];
+  };
+  union {
+    struct { int pk, ph, px, pp; };
+    int p4[4];
+  };
   int s_d, s_diag, s_hop, s_x, s_p, s_nu;
-  int pk, ph, px, pp;
   int use_prev;
   int Eu;
   // dia: per operator P_o = shr128(sum VAL q, sh_pre[o]); term = fx_mul(m_op[o], P_o, s_op[o])
@@ -150,6 +164,11 @@ struct FxConstA {
 };
 
 // ------------------------------------------------------------------ applies
+// WIDE (chains of at most kWideSites sites, vectors in shared memory): the
+// neighbour loops are unrolled whole, so that all loads of an element are in
+// flight at once; one warp per scheduler has nothing else to hide them behind.
+constexpr int kWideSites = 10;
+template <bool WIDE>
 __device__ __forceinline__ longlong2 fx_apply_spin(const longlong2* q, const longlong2* qm, int x,
                                                    const OpSpinFx& op, const FxConstA& c, const long long* mb) {
   const int N = op.N, L = op.lo_bits;
@@ -161,8 +180,9 @@ __device__ __forceinline__ longlong2 fx_apply_spin(const longlong2* q, const lon
   long long ui = fx_mulhi(Dp, v.y << c.pk);
   long long hr = 0, hi = 0;
   const unsigned anti = ((unsigned)x ^ ((unsigned)x >> 1)) & ((1u << (N - 1)) - 1u);
-#pragma unroll 4
-  for (int i = 0; i < N - 1; ++i) {  // antiparallel bonds only (predicated)
+  constexpr int kUnroll = WIDE ? kWideSites : 4;
+#pragma unroll kUnroll
+  for (int i = 0; i < (WIDE ? kWideSites : N - 1); ++i) {  // antiparallel bonds only (predicated)
     if ((anti >> i) & 1u) {
       const longlong2 w = q[x ^ (3 << i)];
       hr += w.x;
@@ -173,8 +193,9 @@ __device__ __forceinline__ longlong2 fx_apply_spin(const longlong2* q, const lon
   ui += fx_mulhi(c.m_hop, hi << c.ph);
   if (op.uniform) {
     long long xr = 0, xi = 0;
-#pragma unroll 4
-    for (int i = 0; i < N; ++i) {
+#pragma unroll kUnroll
+    for (int i = 0; i < (WIDE ? kWideSites : N); ++i) {
+      if (WIDE && i >= N) break;
       const longlong2 w = q[x ^ (1 << i)];
       xr += w.x;
       xi += w.y;
@@ -182,8 +203,9 @@ __device__ __forceinline__ longlong2 fx_apply_spin(const longlong2* q, const lon
     ur += fx_mulhi(c.m_x, xr << c.px);
     ui += fx_mulhi(c.m_x, xi << c.px);
   } else {
-#pragma unroll 4
-    for (int i = 0; i < N; ++i) {
+#pragma unroll kUnroll
+    for (int i = 0; i < (WIDE ? kWideSites : N); ++i) {
+      if (WIDE && i >= N) break;
       const longlong2 w = q[x ^ (1 << i)];
       ur += fx_mulhi(mb[i], w.x << c.pk);
       ui += fx_mulhi(mb[i], w.y << c.pk);

@@ -74,7 +74,10 @@ __device__ __forceinline__ void ff_warp_sum(float& s, float& c) {
 // ------------------------------------------------------------------ shared state
 struct CConst {
   // phase A: u = s_k H_j q_k - beta_{k-1} s_{k-1} q_{k-1}
-  float cz, ch, cx, cp;          // spin: c0 s_k, 2 J c0 s_k, uniform field s_k, -beta s_{k-1}
+  union {                        // spin: c0 s_k, 2 J c0 s_k, uniform field s_k, -beta s_{k-1}
+    struct { float cz, ch, cx, cp; };
+    float c4[4];
+  };
   float co[1 + kMaxDrives];      // dia: c_o s_k per operator
   int use_prev;
 };
@@ -88,16 +91,32 @@ struct SmemC {
   double tr[kMaxKrylov], ti[kMaxKrylov];
   float cr[kMaxKrylov], ci[kMaxKrylov];  // reconstruction coefficients
   double scal[1 + kMaxDrives];
+  double cst[3];                 // spin: c_0, 2 J c_0, b_0 of the stage
   double bsite_raw[kMaxSites];
   float bx[kMaxSites];           // non-uniform fields: b_i s_k
   CConst ca;
   float am;                      // phase B: -alpha_k s_k
   double wnorm2;                 // ||w||^2 of the current iteration (from the phase-A sums)
   double qnorm2[kMaxKrylov + 3]; // ||q_i||^2 of the stored vectors (reduced after they are written)
-  int abort_flag, stop_prev, accept_now, pend, y_ready, acc_h;
+  // commands to the workers
+  int cmd, it;                   // CCmd; the iteration, or the number of basis vectors (kCRec)
+  int final_rec;
+  // control flow (in shared memory: a register spill would go to local memory,
+  // whose lines the workers' loops sweep out of L1)
+  long long e, fpos;             // stage exponential of the launch; next forced decision
+  double remaining;              // of the stage exponential
+  double acc_err;                // estimate of the accepted substep
+  int nsub_e;                    // substeps of the stage exponential
+  int y_ready, acc_h;
   int tma_fail;                  // tiled apply: a tile wait gave up
-  double err_now, err_prev;
   double beta0;
+  // trace (cfet_stats.phase_ns; slots 0, 2, 4, 7 by thread 0, the others by the
+  // control lane 0) and, by the control lane 0, the run's counters
+  long long tacc[8];
+  long long twe;                 // thread 0: end of its last element loop
+  long long n_app, n_sub, rpos;
+  int max_k;
+  double max_err;
   LeadAcc lead;                  // running FP32 bounds of the current T_k for the estimate's screens
   GershAcc gfull;                // rows whose couplings are all known
 };
@@ -317,7 +336,7 @@ struct FFAcc {
 // Keeping the chain in FP32 pairs avoids long dependent sequences on the
 // 1/64-rate FP64 units.  NS = 0: a pure grid barrier.
 template <int NS>
-__device__ bool c_ctl_reduce(SmemC& S, int NW, unsigned long long* part, unsigned tag, bool fence, int* status,
+__device__ __forceinline__ bool c_ctl_reduce(SmemC& S, int NW, unsigned long long* part, unsigned tag, bool fence, int* status,
                              long long timeout_ns, double* sum, long long& spin) {
   const int lane = threadIdx.x & 31;
   constexpr int W = NS > 0 ? 2 * NS : 1;
@@ -347,33 +366,55 @@ __device__ bool c_ctl_reduce(SmemC& S, int NW, unsigned long long* part, unsigne
   return true;
 }
 
-// Phase-A constants for iteration `it` (lane 0 scalars, per-site table over lanes).
-template <int FAMILY, class Op>
-__device__ void c_const_a(SmemC& S, const Op& op, int it) {
-  const int lane = threadIdx.x & 31;
-  const double sk = S.scale[it];
-  if (lane == 0) {
-    CConst& c = S.ca;
-    if constexpr (FAMILY == kFamilySpin) {
-      const double cz = S.scal[0] * sk;
-      c.cz = (float)cz;
-      c.ch = (float)(cz * op.J2);
-      c.cx = (float)(S.bsite_raw[0] * sk);
-    } else {
-      for (int o = 0; o < op.nops; ++o) c.co[o] = (float)(S.scal[o] * sk);
-    }
-    c.cp = it > 1 ? (float)(-S.beta[it - 1] * S.scale[it - 1]) : 0.f;
-    c.use_prev = it > 1;
+// One sum out of line, for the passes that run once per launch or substep: the
+// norm of the new q_1.
+__device__ __noinline__ bool c_ctl_reduce_cold(SmemC& S, int NW, unsigned long long* part, unsigned tag, int* status,
+                                               long long timeout_ns) {
+  double sum[1];
+  const bool ok = c_ctl_reduce<1>(S, NW, part, tag, true, status, timeout_ns, sum, S.tacc[5]);
+  if (ok && (threadIdx.x & 31) == 0) {
+    S.beta0 = sqrt(sum[0]);
+    S.qnorm2[1] = sum[0];
   }
+  __syncwarp();
+  return ok;
+}
+
+// Phase-A constants for iteration `it`, one scalar per lane: a product and a
+// conversion of the FP64 units (64 and 190 cycles) for all of them at once.
+// spin: the stage scalars c_0, 2 J c_0 and b_0 times s_k, and -beta s_{k-1};
+// DIA, CSR: one operator scalar per lane, then -beta s_{k-1}.
+template <int FAMILY, class Op>
+__device__ __forceinline__ void c_const_a(SmemC& S, const Op& op, int it) {
+  const int lane = threadIdx.x & 31;
+  CConst& c = S.ca;
+  const double sk = S.scale[it];
+  const int np = FAMILY == kFamilySpin ? 3 : 1 + kMaxDrives;  // lane of the q_{k-1} coefficient
+  double a = 0.0, f = sk;
   if constexpr (FAMILY == kFamilySpin) {
+    if (lane < 3) a = S.cst[lane];
+  } else {
+    if (lane < op.nops) a = S.scal[lane];
+  }
+  if (lane == np && it > 1) {
+    a = -S.beta[it - 1];
+    f = S.scale[it - 1];
+  }
+  const float v = (float)(a * f);
+  if constexpr (FAMILY == kFamilySpin) {
+    if (lane < 4) c.c4[lane] = v;
     if (!op.uniform)
       for (int i = lane; i < op.N; i += 32) S.bx[i] = (float)(S.bsite_raw[i] * sk);
+  } else {
+    if (lane < op.nops) c.co[lane] = v;
+    if (lane == np) c.cp = v;
   }
+  if (lane == 0) c.use_prev = it > 1;
 }
 
 // Error estimate of iteration k (control warp), with the FP32 screen of
 // fx_estimate: above thr without the FP64 small exponential when it can.
-__device__ double c_estimate(SmemC& S, int k, double ts, double thr) {
+__device__ __noinline__ double c_estimate(SmemC& S, int k, double ts, double thr) {
   const int dec = krylov_lead_decide(S.lead, k, ts, S.beta0, S.beta[k], thr);
   if (dec == 0) return 2.0 * thr + 1e-300;
   const double scale = S.beta0 * S.beta[k];
@@ -642,73 +683,253 @@ __device__ void c_tiled_pass(const TmaPass& T, const OpSpinC& op, const CConst& 
   workers_sync(nworkers);
 }
 
+// Halves the step on the basis of iteration it until the estimate meets the
+// proportional tolerance (control warp): S.acc_h, 0 when no step does.
+__device__ __noinline__ void c_halve(SmemC& S, int it, double tol, double tau) {
+  const double remaining = S.remaining;
+  int hh = 0;
+  double err = 0.0;
+  const double width = gersh_width(it, S.alpha + 1, S.beta + 1);
+#pragma unroll 1
+  for (int h = 1; h <= 40; ++h) {
+    const double ts = ldexp(remaining, -h);
+    if (!(fabs(ts) * width <= 2.0 * it)) continue;
+    err = c_estimate(S, it, ts, tol * ts / tau);
+    if (err <= tol * ts / tau) { hh = h; break; }
+  }
+  if ((threadIdx.x & 31) == 0) { S.acc_h = hh; S.acc_err = err; S.y_ready = hh > 0; }
+  __syncwarp();
+}
+
+// Estimate of iteration it against the proportional tolerance (control warp):
+// 1 (accepted, S.yr / S.yi hold y) or 0; the estimate in S.acc_err.
+__device__ __noinline__ int c_check(SmemC& S, int it, double tol, double tau) {
+  const double thr = tol * S.remaining / tau;
+  const double err = c_estimate(S, it, S.remaining, thr);
+  const int acc = err <= thr;
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) {
+    S.acc_err = err;
+    S.y_ready = acc;
+  }
+  __syncwarp();
+  return acc;
+}
+
+// Reconstruction coefficients of the accepted (k, ts) into S (control warp).
+__device__ __noinline__ void c_rec_consts(SmemC& S, int acc_k, double ts) {
+  const int lane = threadIdx.x & 31;
+  if (!S.y_ready) small_expm_e1(acc_k, S.alpha + 1, S.beta + 1, ts, S.yr, S.yi, S.tr, S.ti);
+  __syncwarp();
+#pragma unroll 1
+  for (int i = lane; i < acc_k; i += 32) {
+    const double f = S.beta0 * S.scale[i + 1];
+    S.cr[i] = (float)(f * S.yr[i]);
+    S.ci[i] = (float)(f * S.yi[i]);
+  }
+}
+
 // ------------------------------------------------------------------ the kernel
+// Worker and control warps run separate loops, as in kernels_fx.cu (fx_worker,
+// fx_control): the control warp publishes one element pass at a time.
+enum CCmd { kCExit = 0, kCConvert, kCApply, kCOrth, kCRec };
+
 // TILED: the window-tiled apply of long spin chains (a separate instantiation,
 // so that the element-wise kernel carries none of its code).
-template <int FAMILY, class Op, bool TILED = false>
-__global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_c64(PropParams p, Op op) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  SmemC& S = *reinterpret_cast<SmemC*>(smem_raw);
-  const int tid = threadIdx.x;
-  const int NW = (int)(blockDim.x >> 5) - 1;
-  const bool ctl = (tid >> 5) == NW;
-  const int lane = tid & 31;
-  const bool lead = ctl && lane == 0;
+template <int FAMILY, class Op, bool TILED>
+__device__ __forceinline__ void c_worker(const PropParams& p, const Op& op, SmemC& S, unsigned char* tiles_base,
+                                         int wstep) {
+  const int tid = threadIdx.x, lane = tid & 31;
   const int dim = p.dim;
-  const int G = gridDim.x;
-  const int chunk = (dim + G - 1) / G;  // one contiguous chunk per CTA
-  const int wstep = NW * 32;
-  int wx0 = blockIdx.x * chunk + tid;
-  int wxe = min(dim, (blockIdx.x + 1) * chunk);
+  int wx0, wxe;  // one contiguous chunk per CTA
   if constexpr (FAMILY == kFamilyCsr) {  // rows split by their work, not their number (csr_row_split)
     wx0 = __ldg(op.rb + blockIdx.x) + tid;
     wxe = __ldg(op.rb + blockIdx.x + 1);
+  } else {
+    const int chunk = (dim + gridDim.x - 1) / gridDim.x;
+    wx0 = blockIdx.x * chunk + tid;
+    wxe = min(dim, ((int)blockIdx.x + 1) * chunk);
   }
-  const int ncoef = 1 + p.nV;
-  // record exchange: three slots (phase A, phase B, reconstruction) of one
-  // float-float pair (two tagged words) per CTA; tags continue across launches
-  const unsigned tag0 = (unsigned)ld_volatile_i32((const int*)&p.st->tag_base);
-  unsigned gen = 0;
-  unsigned long long* partA = reinterpret_cast<unsigned long long*>(p.partials);  // 3 sums: 6 words (stride 8)
-  unsigned long long* partB = partA + 8 * G;                                        // 1 sum: 2 words
-  unsigned long long* partR = partA + 16 * G;                                       // 1 sum: 2 words
-  unsigned long long* partW = partA + 24 * G;  // window barriers of the tiled apply: two 1-word slots
-  // tiled apply: windows and the tile buffers behind SmemC
+  auto Q = [&](int i) -> float2* { return p.qbasis32 + (size_t)(i - 1) * dim; };
   TileWin win[kTiledMaxWindows] = {};
   int nwin = 1;
-  if constexpr (TILED) {
-    nwin = tiled_windows<kTileBits>(op.N, win);
-  }
-  // tiled apply: the stages' mbarriers and tile buffers behind SmemC
-  unsigned char* tiles_base = smem_raw + ((sizeof(SmemC) + 127) & ~size_t(127));
+  if constexpr (TILED) nwin = tiled_windows<kTileBits>(op.N, win);
   unsigned tph = 0;  // parities of the stages' mbarriers (the same in every worker)
-  const TmaPass TP{p.tmaps, reinterpret_cast<unsigned long long*>(tiles_base),
-                   reinterpret_cast<float2*>(tiles_base + 128), &S.tma_fail, &tph, &p.st->status, p.timeout_ns};
-  if constexpr (TILED) {
-    if (tid == 0) {  // ordered before any use by the CTA barriers of the conversion pass
-      for (int s2 = 0; s2 < kTmaStages; ++s2) mbar_init(TP.bar + s2, 1);
-      S.tma_fail = 0;
-      mbar_init_fence();
-    }
-  }
-  int wslot = 0;
-  DevStatus* st = p.st;
-  const bool glead = (blockIdx.x == 0) && lead;
-  long long tacc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  long long twe = 0;  // thread 0: end of its last worker loop
-  const bool fixed_k = p.tol <= 0.0;
-  const bool forced = p.f_nsub != nullptr;
-  long long fpos = st->forced_pos;
-  long long rpos = st->rec_pos;
-  long long n_app = 0, n_sub = 0;
-  int max_k = 0;
-  double max_err = 0.0;
-
-  auto Q = [&](int i) -> float2* { return p.qbasis32 + (size_t)(i - 1) * dim; };
-
-  // ---------------- psi (complex128) -> q_1 (complex64), ||q_1||^2, finiteness
-  {
-    if (!ctl) {
+  if (tid == 0) S.twe = 0;
+  while (true) {
+    __syncthreads();  // the command and its constants are set
+    const int cmd = S.cmd;
+    if (tid == 0 && S.twe) S.tacc[7] += sm_clock() - S.twe;
+    if (cmd == kCExit) break;
+    const long long tw0 = sm_clock();
+    if (cmd == kCApply) {
+      // -------- phase A: u = s H q_it - beta s q_{it-1}.  <q,u> and ||u||^2: with
+      // ||q||^2 (reduced when q was written) they give alpha and
+      // ||u - alpha s q||^2, so the decisions need not wait for the
+      // orthogonalisation pass
+      const int it = S.it;
+      const CConst& c = S.ca;
+      const float2* q = Q(it);
+      const float2* qm = it > 1 ? Q(it - 1) : q;
+      float2* u = Q(it + 1);
+      float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f, s2 = 0.f, c2 = 0.f;
+      int x = wx0;
+      if constexpr (TILED) {  // window passes, grid exchanges between them (control warp)
+        const TmaPass TP{p.tmaps, reinterpret_cast<unsigned long long*>(tiles_base),
+                         reinterpret_cast<float2*>(tiles_base + 128), &S.tma_fail, &tph, &p.st->status, p.timeout_ns};
+        for (int w = 0; w < nwin; ++w) {
+          // basis indices: q_it is vector it - 1, q_{it-1} vector it - 2, u vector it
+          // (from it = 2 on, window 0 first turns u_{it-1} in vector
+          // it - 1 into q_it = u_{it-1} - alpha s q_{it-1}: ORTH)
+          const int iq = it - 1, ia = w == 0 ? (it > 1 ? it - 2 : 0) : it, iu = it;
+          if (w == 0) {
+            const float am = S.am;
+            if (nwin == 1) {
+              if (it > 1)
+                c_tiled_pass<true, true, true>(TP, op, c, S.bx, iq, ia, iu, win[0], 0, wstep, s0, c0, s1, c1, am, &s2,
+                                               &c2);
+              else
+                c_tiled_pass<true, true>(TP, op, c, S.bx, iq, ia, iu, win[0], 0, wstep, s0, c0, s1, c1);
+            } else {
+              if (it > 1)
+                c_tiled_pass<true, false, true>(TP, op, c, S.bx, iq, ia, iu, win[0], 0, wstep, s0, c0, s1, c1, am, &s2,
+                                                &c2);
+              else
+                c_tiled_pass<true, false>(TP, op, c, S.bx, iq, ia, iu, win[0], 0, wstep, s0, c0, s1, c1);
+            }
+          } else if (w == nwin - 1) {
+            c_tiled_pass<false, true>(TP, op, c, S.bx, iq, ia, iu, win[w], w, wstep, s0, c0, s1, c1);
+          } else {
+            c_tiled_pass<false, false>(TP, op, c, S.bx, iq, ia, iu, win[w], w, wstep, s0, c0, s1, c1);
+          }
+          if (w + 1 < nwin) {
+            window_written_sync();    // all threads: window w written
+            window_exchanged_sync();  // all threads: the grid exchange passed
+          }
+        }
+      } else {
+        // spin apply on two elements per thread and loop iteration (twice the
+        // independent neighbour loads per warp)
+        if constexpr (FAMILY == kFamilySpin) {
+          for (; x + wstep < wxe; x += 2 * wstep) {
+            float2 h1, h2;
+            c_apply_spin2(q, qm, x, x + wstep, op, c, S.bx, h1, h2);
+            u[x] = h1;
+            u[x + wstep] = h2;
+            const float2 v1 = q[x], v2 = q[x + wstep];
+            ff_add_prod(s0, c0, v1.x, h1.x);
+            ff_add_prod(s0, c0, v1.y, h1.y);
+            ff_add_prod(s0, c0, v2.x, h2.x);
+            ff_add_prod(s0, c0, v2.y, h2.y);
+            ff_add_prod(s1, c1, h1.x, h1.x);
+            ff_add_prod(s1, c1, h1.y, h1.y);
+            ff_add_prod(s1, c1, h2.x, h2.x);
+            ff_add_prod(s1, c1, h2.y, h2.y);
+          }
+        }
+        if constexpr (FAMILY == kFamilyCsr) {
+          const int lb = op.lane_bits;
+          for (int r0 = wx0 - tid; r0 < wxe; r0 += wstep >> lb) {
+            const int r = r0 + (tid >> lb);
+            const bool on = r < wxe;
+            const float2 hv = c_apply_csr(q, qm, r, on, dim, op, c);
+            if (on && (tid & ((1 << lb) - 1)) == 0) {
+              u[r] = hv;
+              const float2 v = q[r];
+              ff_add_prod(s0, c0, v.x, hv.x);
+              ff_add_prod(s0, c0, v.y, hv.y);
+              ff_add_prod(s1, c1, hv.x, hv.x);
+              ff_add_prod(s1, c1, hv.y, hv.y);
+            }
+          }
+        } else {
+          for (; x < wxe; x += wstep) {
+            float2 hv;
+            if constexpr (FAMILY == kFamilySpin) hv = c_apply_spin(q, qm, x, op, c, S.bx);
+            else hv = c_apply_dia(q, qm, x, dim, op, c);
+            u[x] = hv;
+            const float2 v = q[x];
+            ff_add_prod(s0, c0, v.x, hv.x);
+            ff_add_prod(s0, c0, v.y, hv.y);
+            ff_add_prod(s1, c1, hv.x, hv.x);
+            ff_add_prod(s1, c1, hv.y, hv.y);
+          }
+        }
+      }
+      c_worker_partial(S, s0, c0, 0);
+      c_worker_partial(S, s1, c1, 1);
+      if constexpr (TILED) c_worker_partial(S, s2, c2, 2);  // ||q_it||^2 of the w stored in window 0
+      if (tid == 0) S.tacc[0] += (S.twe = sm_clock()) - tw0;
+    } else if (cmd == kCOrth) {
+      // -------- phase B: w = u - alpha s q_it, ||w||^2 of the stored w for the
+      // next iteration (the tiled form does it in the next window 0)
+      const int it = S.it;
+      const float am = S.am;
+      const float2* q = Q(it);
+      float2* u = Q(it + 1);
+      float s0 = 0.f, c0 = 0.f;
+      int x = wx0;
+      // four elements per step with every load issued first (more bytes
+      // in flight per thread); the sums keep the order of the plain loop
+      for (; x + 3 * wstep < wxe; x += 4 * wstep) {
+        float2 v[4], uu[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          v[j] = q[x + j * wstep];
+          uu[j] = u[x + j * wstep];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float2 w = make_float2(fmaf(am, v[j].x, uu[j].x), fmaf(am, v[j].y, uu[j].y));
+          u[x + j * wstep] = w;
+          ff_add_prod(s0, c0, w.x, w.x);
+          ff_add_prod(s0, c0, w.y, w.y);
+        }
+      }
+      for (; x < wxe; x += wstep) {
+        const float2 v = q[x];
+        const float2 uu = u[x];
+        const float2 w = make_float2(fmaf(am, v.x, uu.x), fmaf(am, v.y, uu.y));
+        u[x] = w;
+        ff_add_prod(s0, c0, w.x, w.x);
+        ff_add_prod(s0, c0, w.y, w.y);
+      }
+      c_worker_partial(S, s0, c0, 0);
+      if (tid == 0) S.tacc[2] += (S.twe = sm_clock()) - tw0;
+    } else if (cmd == kCRec) {
+      // -------- reconstruct q_1 <- beta0 sum_i y_i s_i q_i
+      const int acc_k = S.it;
+      const bool final_rec = S.final_rec;
+      float s = 0.f, cc = 0.f;
+      for (int x = wx0; x < wxe; x += wstep) {
+        float re = 0.f, im = 0.f;
+        int i = 0;
+        for (; i + 3 < acc_k; i += 4) {  // four basis loads in flight before their use (same order)
+          float2 v[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[j] = Q(i + j + 1)[x];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float cr = S.cr[i + j], ci = S.ci[i + j];
+            re = fmaf(cr, v[j].x, fmaf(-ci, v[j].y, re));
+            im = fmaf(cr, v[j].y, fmaf(ci, v[j].x, im));
+          }
+        }
+        for (; i < acc_k; ++i) {
+          const float2 v = Q(i + 1)[x];
+          const float cr = S.cr[i], ci = S.ci[i];
+          re = fmaf(cr, v.x, fmaf(-ci, v.y, re));
+          im = fmaf(cr, v.y, fmaf(ci, v.x, im));
+        }
+        Q(1)[x] = make_float2(re, im);
+        if (final_rec) p.psi[x] = make_double2((double)re, (double)im);
+        ff_add_prod(s, cc, re, re);
+        ff_add_prod(s, cc, im, im);
+      }
+      c_worker_partial(S, s, cc);
+      if (tid == 0) S.tacc[4] += (S.twe = sm_clock()) - tw0;
+    } else {
+      // -------- psi (complex128) -> q_1 (complex64), ||q_1||^2, finiteness
       float s = 0.f, c = 0.f;
       int bad = 0;
       for (int x = wx0; x < wxe; x += wstep) {
@@ -719,210 +940,124 @@ __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_c64(PropP
         ff_add_prod(s, c, f.x, f.x);
         ff_add_prod(s, c, f.y, f.y);
       }
-      if (__any_sync(0xffffffffu, bad) && lane == 0) atomicCAS(&st->status, 0, (int)CFET_ENAN);
+      if (__any_sync(0xffffffffu, bad) && lane == 0) atomicCAS(&p.st->status, 0, (int)CFET_ENAN);
       c_worker_partial(S, s, c);
     }
-    __syncthreads();
-    if (ctl) {
-      double sum[1];
-      if (!c_ctl_reduce<1>(S, NW, partR, tag0 + (++gen), true, &st->status, p.timeout_ns, sum, tacc[5])) {
-        if (lane == 0) S.abort_flag = 1;
-      } else if (lane == 0) {
-        S.abort_flag = ld_volatile_i32(&st->status) != 0;
-        S.beta0 = sqrt(sum[0]);
-        S.qnorm2[1] = sum[0];
-      }
-    }
-    __syncthreads();
-    if (S.abort_flag) return;
+    __syncthreads();  // the pass is done
   }
+}
 
-  for (long long e = 0; e < p.nexp; ++e) {
-    if (tid < ncoef) S.scal[tid] = p.scal[e * ncoef + tid];
+template <int FAMILY, class Op, bool TILED>
+__device__ __forceinline__ void c_control(const PropParams& p, const Op& op, SmemC& S, int NW) {
+  const int lane = threadIdx.x & 31;
+  const int G = gridDim.x;
+  const int ncoef = 1 + p.nV;
+  DevStatus* const st = p.st;
+  // record exchange (ctl_exchange): tags continue across launches
+  unsigned tag = (unsigned)ld_volatile_i32((const int*)&st->tag_base);
+  unsigned long long* const rec = reinterpret_cast<unsigned long long*>(p.partials);
+  const bool glead = blockIdx.x == 0 && lane == 0;
+  const bool fixed_k = p.tol <= 0.0;
+  const bool forced = p.f_nsub != nullptr;
+  if (lane == 0) {
+    for (int i = 0; i < 8; ++i) S.tacc[i] = 0;
+    S.n_app = S.n_sub = 0;
+    S.rpos = st->rec_pos;
+    S.fpos = st->forced_pos;
+    S.max_k = 0;
+    S.max_err = 0.0;
+    S.e = 0;
+  }
+  auto start = [&](int cmd, int it) {  // one element pass of the workers
+    if (lane == 0) {
+      S.cmd = cmd;
+      S.it = it;
+    }
+    __syncwarp();
     __syncthreads();
+  };
+
+  // ---------------- psi (complex128) -> q_1 (complex64)
+  start(kCConvert, 0);
+  __syncthreads();
+  if (!c_ctl_reduce_cold(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
+  if (ld_volatile_i32(&st->status) != 0) return;
+
+  while (S.e < p.nexp) {
+    if (lane < ncoef) S.scal[lane] = p.scal[S.e * ncoef + lane];
+    if (lane == 0) {
+      S.remaining = p.tau;
+      S.nsub_e = 0;
+    }
+    __syncwarp();
     if constexpr (FAMILY == kFamilySpin) {
-      if (ctl && lane < op.N) {
+      if (lane < op.N) {
         double bi = 0.0;
         for (int k = 0; k < p.nV; ++k) bi = fma(S.scal[1 + k], __ldg(op.xf + k * op.N + lane), bi);
         S.bsite_raw[lane] = bi;
+        if (lane == 0) {
+          S.cst[0] = S.scal[0];
+          S.cst[1] = S.scal[0] * op.J2;
+          S.cst[2] = bi;
+        }
       }
-      __syncthreads();
+      __syncwarp();
     }
-    const long long eg = p.exp_base + e;
-    const bool last_exp = (e == p.nexp - 1);
-    const int nforced = forced ? p.f_nsub[eg] : 0;
-    double remaining = p.tau;
-    int nsub_e = 0;
     while (true) {
-      if (nsub_e >= p.max_substeps || (forced && nsub_e >= nforced)) {
+      if (S.nsub_e >= p.max_substeps || (forced && S.nsub_e >= p.f_nsub[p.exp_base + S.e])) {
         if (glead) atomicCAS(&st->status, 0, (int)CFET_EKRYLOV);
         return;
       }
-      int kf = -1, hf = 0;
-      if (forced) {
-        kf = p.f_k[fpos];
-        hf = p.f_h[fpos];
-      }
-      const double beta0 = S.beta0;
+      const int klimit = forced ? p.f_k[S.fpos] : p.m_max;
       int acc_k = 0, acc_h = 0;
-      double acc_err = 0.0;
-      if (beta0 != 0.0) {
-        const int klimit = forced ? kf : p.m_max;
-        if (lead) {
-          S.scale[1] = 1.0 / beta0;
-          S.pend = 0;
-          S.stop_prev = 0;
-          S.accept_now = 0;
+      if (lane == 0) S.acc_err = 0.0;
+      if (S.beta0 != 0.0) {
+        if (lane == 0) {
+          S.scale[1] = div_call(1.0, S.beta0);
           S.y_ready = 0;
         }
-        if (ctl) {
-          __syncwarp();
-          c_const_a<FAMILY>(S, op, 1);
-        }
-        __syncthreads();
+        __syncwarp();
+        c_const_a<FAMILY>(S, op, 1);
+        bool accepted = false, pend = false;
         int it = 1;
         for (;; ++it) {
-          // -------- phase A(it); deferred estimate of it-1 on the control warp
-          const int pend = S.pend;
-          if (!ctl) {
-            const CConst& c = S.ca;
-            const float2* q = Q(it);
-            const float2* qm = it > 1 ? Q(it - 1) : q;
-            float2* u = Q(it + 1);
-            // <q,u> and ||u||^2: with ||q||^2 (reduced when q was written) they
-            // give alpha and ||u - alpha s q||^2, so the decisions need not wait
-            // for the orthogonalisation pass
-            float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f, s2 = 0.f, c2 = 0.f;
-            const long long tw0 = sm_clock();
-            int x = wx0;
-            if constexpr (TILED) {
-              {  // window passes, grid exchanges between them (control warp)
-                for (int w = 0; w < nwin; ++w) {
-                  // basis indices: q_it is vector it - 1, q_{it-1} vector it - 2, u vector it
-                  // (from it = 2 on, window 0 first turns u_{it-1} in vector
-                  // it - 1 into q_it = u_{it-1} - alpha s q_{it-1}: ORTH)
-                  const int iq = it - 1, ia = w == 0 ? (it > 1 ? it - 2 : 0) : it, iu = it;
-                  if (w == 0) {
-                    const float am = S.am;
-                    if (nwin == 1) {
-                      if (it > 1)
-                        c_tiled_pass<true, true, true>(TP, op, c, S.bx, iq, ia, iu, win[0], 0, wstep, s0, c0, s1, c1,
-                                                       am, &s2, &c2);
-                      else
-                        c_tiled_pass<true, true>(TP, op, c, S.bx, iq, ia, iu, win[0], 0, wstep, s0, c0, s1, c1);
-                    } else {
-                      if (it > 1)
-                        c_tiled_pass<true, false, true>(TP, op, c, S.bx, iq, ia, iu, win[0], 0, wstep, s0, c0, s1, c1,
-                                                        am, &s2, &c2);
-                      else
-                        c_tiled_pass<true, false>(TP, op, c, S.bx, iq, ia, iu, win[0], 0, wstep, s0, c0, s1, c1);
-                    }
-                  } else if (w == nwin - 1) {
-                    c_tiled_pass<false, true>(TP, op, c, S.bx, iq, ia, iu, win[w], w, wstep, s0, c0, s1, c1);
-                  } else {
-                    c_tiled_pass<false, false>(TP, op, c, S.bx, iq, ia, iu, win[w], w, wstep, s0, c0, s1, c1);
-                  }
-                  if (w + 1 < nwin) {
-                    window_written_sync();    // all threads: window w written
-                    window_exchanged_sync();  // all threads: the grid exchange passed
-                  }
-                }
-                x = wxe;  // nothing left for the element loops
-              }
+          // -------- phase A(it) on the workers; deferred estimate of it-1 here
+          start(kCApply, it);
+          bool stop_prev = false;
+          if (pend) {
+            const long long te0 = sm_clock();
+            stop_prev = c_check(S, it - 1, p.tol, p.tau) != 0;
+            if (lane == 0) S.tacc[6] += sm_clock() - te0;
+          }
+          if constexpr (TILED) {  // grid exchanges between the window passes of the workers
+            TileWin win[kTiledMaxWindows] = {};
+            const int nwin = tiled_windows<kTileBits>(op.N, win);
+            bool ok = true;
+            for (int w = 0; w + 1 < nwin; ++w) {
+              window_written_sync();
+              double none[1];
+              ok = ok && c_ctl_reduce<0>(S, NW, rec, ++tag, true, &st->status, p.timeout_ns, none, S.tacc[5]);
+              window_exchanged_sync();
             }
-            // spin apply on two elements per thread and loop iteration (twice the
-            // independent neighbour loads per warp)
-            if constexpr (FAMILY == kFamilySpin) {
-              for (; x + wstep < wxe; x += 2 * wstep) {
-                float2 h1, h2;
-                c_apply_spin2(q, qm, x, x + wstep, op, c, S.bx, h1, h2);
-                u[x] = h1;
-                u[x + wstep] = h2;
-                const float2 v1 = q[x], v2 = q[x + wstep];
-                ff_add_prod(s0, c0, v1.x, h1.x);
-                ff_add_prod(s0, c0, v1.y, h1.y);
-                ff_add_prod(s0, c0, v2.x, h2.x);
-                ff_add_prod(s0, c0, v2.y, h2.y);
-                ff_add_prod(s1, c1, h1.x, h1.x);
-                ff_add_prod(s1, c1, h1.y, h1.y);
-                ff_add_prod(s1, c1, h2.x, h2.x);
-                ff_add_prod(s1, c1, h2.y, h2.y);
-              }
-            }
-            if constexpr (FAMILY == kFamilyCsr) {
-              const int lb = op.lane_bits;
-              for (int r0 = wx0 - tid; r0 < wxe; r0 += wstep >> lb) {
-                const int r = r0 + (tid >> lb);
-                const bool on = r < wxe;
-                const float2 hv = c_apply_csr(q, qm, r, on, dim, op, c);
-                if (on && (tid & ((1 << lb) - 1)) == 0) {
-                  u[r] = hv;
-                  const float2 v = q[r];
-                  ff_add_prod(s0, c0, v.x, hv.x);
-                  ff_add_prod(s0, c0, v.y, hv.y);
-                  ff_add_prod(s1, c1, hv.x, hv.x);
-                  ff_add_prod(s1, c1, hv.y, hv.y);
-                }
-              }
-              x = wxe;
-            }
-            for (; x < wxe; x += wstep) {
-              float2 hv = make_float2(0.f, 0.f);
-              if constexpr (FAMILY == kFamilySpin) hv = c_apply_spin(q, qm, x, op, c, S.bx);
-              else if constexpr (FAMILY == kFamilyDia) hv = c_apply_dia(q, qm, x, dim, op, c);
-              u[x] = hv;
-              const float2 v = q[x];
-              ff_add_prod(s0, c0, v.x, hv.x);
-              ff_add_prod(s0, c0, v.y, hv.y);
-              ff_add_prod(s1, c1, hv.x, hv.x);
-              ff_add_prod(s1, c1, hv.y, hv.y);
-            }
-            c_worker_partial(S, s0, c0, 0);
-            c_worker_partial(S, s1, c1, 1);
-            if constexpr (TILED) c_worker_partial(S, s2, c2, 2);  // ||q_it||^2 of the w stored in window 0
-            if (tid == 0) {
-              twe = sm_clock();
-              tacc[0] += twe - tw0;
-            }
-          } else {
-            if (pend) {
-              const long long te0 = sm_clock();
-              const double err = c_estimate(S, it - 1, remaining, p.tol * remaining / p.tau);
-              if (lane == 0) {
-                S.err_prev = err;
-                S.stop_prev = err <= p.tol * remaining / p.tau;
-                S.y_ready = S.stop_prev;
-                tacc[6] += sm_clock() - te0;
-              }
-              __syncwarp();
-            }
-            if constexpr (TILED) {
-              {  // grid exchanges between the window passes of the workers
-                for (int w = 0; w + 1 < nwin; ++w) {
-                  window_written_sync();
-                  double none[1];
-                  const bool ok = !S.abort_flag && c_ctl_reduce<0>(S, NW, partW + (size_t)wslot * G, tag0 + (++gen),
-                                                                   true, &st->status, p.timeout_ns, none, tacc[5]);
-                  __syncwarp();
-                  if (!ok && lane == 0) S.abort_flag = 1;
-                  wslot ^= 1;
-                  window_exchanged_sync();
-                }
-              }
+            if (!ok) {
+              __syncthreads();
+              return;
             }
           }
           __syncthreads();
-          if (ctl) {
-            const long long tc0 = sm_clock(), sp0 = tacc[5];
+          {
+            const long long sp0 = S.tacc[5];
             double sum[3];
             // (the tiled apply leaves u written by other CTAs: fence; it also
             // carries ||q_it||^2 of the w that its window 0 stored)
-            constexpr bool kMayTile = TILED;
-            if ((kMayTile && S.abort_flag) ||
-                !c_ctl_reduce<TILED ? 3 : 2>(S, NW, partA, tag0 + (++gen), kMayTile, &st->status, p.timeout_ns,
-                                             sum, tacc[5])) {
-              if (lane == 0) S.abort_flag = 1;
-            } else if (lane == 0 && !S.stop_prev) {
+            if (!c_ctl_reduce<TILED ? 3 : 2>(S, NW, rec, ++tag, TILED, &st->status, p.timeout_ns, sum, S.tacc[5]))
+              return;
+            if (stop_prev) {  // the deferred estimate accepted it-1
+              it -= 1;
+              accepted = true;
+              break;
+            }
+            if (lane == 0) {
               if (TILED && it > 1) S.qnorm2[it] = sum[2];
               // q_it holds the Lanczos vector v_it times 1/scale[it]:
               // alpha = <v, u>,  ||w||^2 = ||u - alpha v||^2
@@ -934,61 +1069,17 @@ __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_c64(PropP
               S.alpha[it] = alpha;
               S.am = (float)(-alpha * s_it);
               S.wnorm2 = sum[1] - alpha * alpha * (2.0 - s_it * s_it * S.qnorm2[it]);
+              S.tacc[1] += sm_clock() - S.twe - (S.tacc[5] - sp0);
             }
-            if (lane == 0) tacc[1] += sm_clock() - tc0 - (tacc[5] - sp0);
-          }
-          __syncthreads();
-          if (tid == 0) tacc[7] += sm_clock() - twe;
-          if (S.abort_flag) return;
-          if (S.stop_prev) {  // the deferred estimate accepted it-1
-            it -= 1;
-            acc_err = S.err_prev;
-            break;
           }
           // -------- phase B(it): w = u - alpha s_it q_it on the workers (the
           // tiled form does it in the next iteration's window 0); beta (known
           // from the phase-A sums), the decisions and the next iteration's
-          // constants on the control warp at the same time
-          if (!ctl) {
-            if constexpr (!TILED) {
-              const float am = S.am;
-              const float2* q = Q(it);
-              float2* u = Q(it + 1);
-              float s0 = 0.f, c0 = 0.f;  // ||w||^2 of the stored w, for the next iteration
-              const long long tw0 = sm_clock();
-              int x = wx0;
-              // four elements per step with every load issued first (more bytes
-              // in flight per thread); the sums keep the order of the plain loop
-              for (; x + 3 * wstep < wxe; x += 4 * wstep) {
-                float2 v[4], uu[4];
-  #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  v[j] = q[x + j * wstep];
-                  uu[j] = u[x + j * wstep];
-                }
-  #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  const float2 w = make_float2(fmaf(am, v[j].x, uu[j].x), fmaf(am, v[j].y, uu[j].y));
-                  u[x + j * wstep] = w;
-                  ff_add_prod(s0, c0, w.x, w.x);
-                  ff_add_prod(s0, c0, w.y, w.y);
-                }
-              }
-              for (; x < wxe; x += wstep) {
-                const float2 v = q[x];
-                const float2 uu = u[x];
-                const float2 w = make_float2(fmaf(am, v.x, uu.x), fmaf(am, v.y, uu.y));
-                u[x] = w;
-                ff_add_prod(s0, c0, w.x, w.x);
-                ff_add_prod(s0, c0, w.y, w.y);
-              }
-              c_worker_partial(S, s0, c0, 0);
-              if (tid == 0) {
-                twe = sm_clock();
-                tacc[2] += twe - tw0;
-              }
-            }
-          } else {
+          // constants here at the same time
+          if constexpr (!TILED) start(kCOrth, it);
+          else __syncwarp();
+          bool acc = false;
+          {
             const long long tc0 = sm_clock();
             // beta and 1/beta from one reciprocal square root (a rounding-level
             // negative ||w||^2 is an exact breakdown)
@@ -999,195 +1090,138 @@ __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_c64(PropP
             const bool breakdown =
                 sb_no_breakdown(b, S.alpha[it], prev_b) != 1 && b <= 1e-13 * (fabs(S.alpha[it]) + prev_b + 1.0);
             int gate = -1;
+            __syncwarp();
             if (lane == 0) {
               S.beta[it] = b;
               S.scale[it + 1] = rb;
-              gate = krylov_bounds_update(S, it, remaining);
+              gate = krylov_bounds_update(S, it, S.remaining);
+              S.acc_err = 0.0;
             }
             gate = __shfl_sync(0xffffffffu, gate, 0);
             __syncwarp();
-            int acc_flag = 0, pend_next = 0;
-            double err = 0.0;
+            pend = false;
             if (forced) {
-              acc_flag = (it == kf);
+              acc = it == klimit;
             } else if (fixed_k) {
-              acc_flag = (it == p.m_max) || breakdown;
+              acc = it == p.m_max || breakdown;
             } else if (breakdown) {
-              acc_flag = 1;
+              acc = true;
             } else if (it >= p.m_min &&
                        (gate >= 0 ? gate == 1
-                                  : fabs(remaining) * gersh_width(it, S.alpha + 1, S.beta + 1) <= 2.0 * it)) {
-              if (it < klimit) {
-                pend_next = 1;  // estimate runs during the next apply
-              } else {
-                err = c_estimate(S, it, remaining, p.tol * remaining / p.tau);
-                acc_flag = err <= p.tol * remaining / p.tau;
-              }
+                                  : fabs(S.remaining) * gersh_width(it, S.alpha + 1, S.beta + 1) <= 2.0 * it)) {
+              if (it < klimit) pend = true;  // the estimate runs during the next apply
+              else acc = c_check(S, it, p.tol, p.tau) != 0;
             }
-            if (lane == 0) {
-              S.accept_now = acc_flag;
-              S.pend = pend_next;
-              S.err_now = err;
-              S.y_ready = acc_flag && !forced && !fixed_k && !breakdown;
-            }
-            __syncwarp();
-            if (!acc_flag && it < klimit) c_const_a<FAMILY>(S, op, it + 1);
-            if (lane == 0) tacc[3] += sm_clock() - tc0;
+            if (!acc && it < klimit) c_const_a<FAMILY>(S, op, it + 1);
+            if (lane == 0) S.tacc[3] += sm_clock() - tc0;
           }
-          __syncthreads();
-          const bool last_it = S.accept_now || it >= klimit;
-          if (!TILED && !last_it) {
-            // every CTA's w must be visible before the next apply reads it; the
-            // exchange also carries ||w||^2 of the stored w
-            if (ctl) {
-              double wsum[1];
-              if (!c_ctl_reduce<1>(S, NW, partB, tag0 + (++gen), true, &st->status, p.timeout_ns, wsum, tacc[5])) {
-                if (lane == 0) S.abort_flag = 1;
-              } else if (lane == 0) {
-                S.qnorm2[it + 1] = wsum[0];
-              }
-            }
+          if constexpr (!TILED) {
             __syncthreads();
+            if (!acc && it < klimit) {
+              // every CTA's w must be visible before the next apply reads it; the
+              // exchange also carries ||w||^2 of the stored w
+              double wsum[1];
+              if (!c_ctl_reduce<1>(S, NW, rec, ++tag, true, &st->status, p.timeout_ns, wsum, S.tacc[5])) return;
+              if (lane == 0) S.qnorm2[it + 1] = wsum[0];
+            }
           }
-          if (tid == 0) tacc[7] += sm_clock() - twe;
-          if (S.abort_flag) return;
-          if (S.accept_now) {
-            acc_err = S.err_now;
+          __syncwarp();
+          if (acc) {
+            accepted = true;
             break;
           }
           if (it >= klimit) break;
         }
         acc_k = it;
-        const bool accepted = S.accept_now || S.stop_prev;
-        acc_h = 0;
         if (forced) {
-          acc_h = hf;
+          acc_h = p.f_h[S.fpos];
         } else if (!accepted) {
           // halve the substep on the same basis until the estimate meets the
-          // proportional tolerance (control warp)
-          if (ctl) {
-            int hh = 0;
-            double err = 0.0;
-            const double width = gersh_width(it, S.alpha + 1, S.beta + 1);
-            for (int h = 1; h <= 40; ++h) {
-              const double ts = ldexp(remaining, -h);
-              if (!(fabs(ts) * width <= 2.0 * it)) continue;
-              err = c_estimate(S, it, ts, p.tol * ts / p.tau);
-              if (err <= p.tol * ts / p.tau) { hh = h; break; }
-            }
-            if (lane == 0) { S.acc_h = hh; S.err_now = err; S.y_ready = hh > 0; }
-          }
-          __syncthreads();
+          // proportional tolerance
+          c_halve(S, it, p.tol, p.tau);
           acc_h = S.acc_h;
-          acc_err = S.err_now;
           if (acc_h == 0) {
             if (glead) atomicCAS(&st->status, 0, (int)CFET_EKRYLOV);
             return;
           }
         }
-        n_app += acc_k;
-      }
-      const double ts = ldexp(remaining, -acc_h);
-      const bool final_rec = last_exp && acc_h == 0;
-      if (acc_k > 0) {
         // -------- reconstruct q_1 <- beta0 sum_i y_i s_i q_i
-        if (ctl) {
+        {
           const long long tr0 = sm_clock();
-          if (!S.y_ready) small_expm_e1(acc_k, S.alpha + 1, S.beta + 1, ts, S.yr, S.yi, S.tr, S.ti);
-          __syncwarp();
-          for (int i = lane; i < acc_k; i += 32) {
-            const double f = beta0 * S.scale[i + 1];
-            S.cr[i] = (float)(f * S.yr[i]);
-            S.ci[i] = (float)(f * S.yi[i]);
-          }
-          if (lane == 0) tacc[6] += sm_clock() - tr0;
-        }
-        __syncthreads();
-        if (!ctl) {
-          float s = 0.f, cc = 0.f;
-          const long long tw0 = sm_clock();
-          for (int x = wx0; x < wxe; x += wstep) {
-            float re = 0.f, im = 0.f;
-            int i = 0;
-            for (; i + 3 < acc_k; i += 4) {  // four basis loads in flight before their use (same order)
-              float2 v[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) v[j] = Q(i + j + 1)[x];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const float cr = S.cr[i + j], ci = S.ci[i + j];
-                re = fmaf(cr, v[j].x, fmaf(-ci, v[j].y, re));
-                im = fmaf(cr, v[j].y, fmaf(ci, v[j].x, im));
-              }
-            }
-            for (; i < acc_k; ++i) {
-              const float2 v = Q(i + 1)[x];
-              const float cr = S.cr[i], ci = S.ci[i];
-              re = fmaf(cr, v.x, fmaf(-ci, v.y, re));
-              im = fmaf(cr, v.y, fmaf(ci, v.x, im));
-            }
-            Q(1)[x] = make_float2(re, im);
-            if (final_rec) p.psi[x] = make_double2((double)re, (double)im);
-            ff_add_prod(s, cc, re, re);
-            ff_add_prod(s, cc, im, im);
-          }
-          c_worker_partial(S, s, cc);
-          if (tid == 0) {
-              twe = sm_clock();
-              tacc[4] += twe - tw0;
-            }
-        }
-        __syncthreads();
-        if (ctl) {
-          double sum[1];
-          if (!c_ctl_reduce<1>(S, NW, partR, tag0 + (++gen), true, &st->status, p.timeout_ns, sum, tacc[5])) {
-            if (lane == 0) S.abort_flag = 1;
-          } else if (lane == 0) {
-            S.beta0 = sqrt(sum[0]);
-            S.qnorm2[1] = sum[0];
+          c_rec_consts(S, acc_k, ldexp(S.remaining, -acc_h));
+          if (lane == 0) {
+            S.final_rec = S.e == p.nexp - 1 && acc_h == 0;
+            S.tacc[6] += sm_clock() - tr0;
           }
         }
+        start(kCRec, acc_k);
         __syncthreads();
-        if (tid == 0) tacc[7] += sm_clock() - twe;
-        if (S.abort_flag) return;
+        if (!c_ctl_reduce_cold(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
       }
-      if (glead && p.r_k != nullptr) {
-        if (rpos < p.r_cap) {
-          p.r_k[rpos] = acc_k;
-          p.r_h[rpos] = acc_h;
-        } else {
-          st->rec_overflow = 1;
+      if (lane == 0) {
+        if (glead && p.r_k != nullptr) {
+          if (S.rpos < p.r_cap) {
+            p.r_k[S.rpos] = acc_k;
+            p.r_h[S.rpos] = acc_h;
+          } else {
+            st->rec_overflow = 1;
+          }
         }
+        S.rpos += 1;
+        S.n_sub += 1;
+        S.n_app += acc_k;
+        if (acc_k > S.max_k) S.max_k = acc_k;
+        if (S.acc_err > S.max_err) S.max_err = S.acc_err;
+        if (forced) S.fpos += 1;
+        S.nsub_e += 1;
+        S.remaining -= ldexp(S.remaining, -acc_h);
       }
-      rpos += 1;
-      if (forced) fpos += 1;
-      n_sub += 1;
-      nsub_e += 1;
-      if (acc_k > max_k) max_k = acc_k;
-      if (acc_err > max_err) max_err = acc_err;
+      __syncwarp();
       if (acc_h == 0) break;
-      remaining -= ts;
     }
-    if (glead && p.r_nsub != nullptr) p.r_nsub[eg] = nsub_e;
+    if (glead && p.r_nsub != nullptr) p.r_nsub[p.exp_base + S.e] = S.nsub_e;
+    if (lane == 0) S.e += 1;
+    __syncwarp();
   }
   if (glead) {
-    st->tag_base = tag0 + gen;
-    st->forced_pos = fpos;
-    st->rec_pos = rpos;
+    st->tag_base = tag;
+    st->forced_pos = S.fpos;
+    st->rec_pos = S.rpos;
     st->n_exp += p.nexp;
-    st->n_sub += n_sub;
-    st->n_app += n_app;
-    if (max_k > st->max_k) st->max_k = max_k;
-    if (max_err > st->max_err) st->max_err = max_err;
+    st->n_sub += S.n_sub;
+    st->n_app += S.n_app;
+    if (S.max_k > st->max_k) st->max_k = S.max_k;
+    if (S.max_err > st->max_err) st->max_err = S.max_err;
   }
-  if (tid == 0 || lead) {  // every CTA: mean and max of its phase times
-    // thread 0 holds the worker slots 0, 2, 4, 7; the control lane 1, 3, 5, 6
-    const int mine[2][4] = {{0, 2, 4, 7}, {1, 3, 5, 6}};
-    for (int j = 0; j < 4; ++j) {
-      const int i = mine[tid == 0 ? 0 : 1][j];
-      atomicAdd((unsigned long long*)&st->phase_ns[i], (unsigned long long)(tacc[i] / G));
-      atomicMax(&st->phase_max_ns[i], tacc[i]);
+  if (lane < 8) {  // every CTA: mean and max of its phase times (see cfet_stats.phase_ns), SM clock cycles
+    const long long t = S.tacc[lane];
+    atomicAdd((unsigned long long*)&st->phase_ns[lane], (unsigned long long)(t / G));
+    atomicMax(&st->phase_max_ns[lane], t);
+  }
+}
+
+template <int FAMILY, class Op, bool TILED = false>
+__global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_c64(PropParams p, Op op) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SmemC& S = *reinterpret_cast<SmemC*>(smem_raw);
+  const int NW = (int)(blockDim.x >> 5) - 1;
+  // tiled apply: the stages' mbarriers and tile buffers behind SmemC
+  unsigned char* const tiles_base = smem_raw + ((sizeof(SmemC) + 127) & ~size_t(127));
+  if constexpr (TILED) {
+    if (threadIdx.x == 0) {  // ordered before any use by the CTA barriers of the conversion pass
+      for (int s2 = 0; s2 < kTmaStages; ++s2) mbar_init(reinterpret_cast<unsigned long long*>(tiles_base) + s2, 1);
+      S.tma_fail = 0;
+      mbar_init_fence();
     }
+  }
+  if ((int)(threadIdx.x >> 5) < NW) {
+    c_worker<FAMILY, Op, TILED>(p, op, S, tiles_base, NW * 32);
+  } else {
+    c_control<FAMILY, Op, TILED>(p, op, S, NW);
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) S.cmd = kCExit;  // also after an error
+    __syncwarp();
+    __syncthreads();
   }
 }
 

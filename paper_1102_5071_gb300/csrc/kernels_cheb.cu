@@ -221,7 +221,7 @@ template <int FAMILY, class Op>
 __device__ __forceinline__ longlong2 cheb_apply1(const longlong2* cur, const longlong2* prev, int x, bool on, int dim,
                                                  const Op& op, const FxConstA& c, const long long* mb, long long m_s) {
   longlong2 y;
-  if constexpr (FAMILY == kFamilySpin) y = fx_apply_spin(cur, prev, x, op, c, mb);
+  if constexpr (FAMILY == kFamilySpin) y = fx_apply_spin<false>(cur, prev, x, op, c, mb);
   else if constexpr (FAMILY == kFamilyDia) y = fx_apply_dia(cur, prev, x, dim, op, c);
   else y = fx_apply_csr(cur, prev, x, on, dim, op, c);
   if (m_s != 0 && on) {
@@ -314,7 +314,6 @@ __global__ void __launch_bounds__(kChebThreads, 1) k_cheb_fx(PropParams p, Op op
   const int ncoef = 1 + p.nV;
   const unsigned tag0 = (unsigned)ld_volatile_i32((const int*)&p.st->tag_base);
   unsigned gen = 0;
-  int slot = 0;  // exchange slot, alternating: two uses of a slot are separated by the other
   unsigned long long* rec = reinterpret_cast<unsigned long long*>(p.partials);
   DevStatus* st = p.st;
   const bool glead = blockIdx.x == 0 && tid == 0;
@@ -345,7 +344,7 @@ __global__ void __launch_bounds__(kChebThreads, 1) k_cheb_fx(PropParams p, Op op
       }
       const unsigned mine[4] = {(unsigned)cy, (unsigned)(cy >> 32), (unsigned)ca, (unsigned)(ca >> 32)};
       ChebMax2 acc;
-      const bool ok = ctl_exchange<4>(rec + (size_t)slot * 4 * G, mine, tag0 + (++gen), fence, &st->status,
+      const bool ok = ctl_exchange<4>(rec, mine, tag0 + (++gen), fence, &st->status,
                                       p.timeout_ns, t_wait, acc);
       unsigned long long ty = acc.a, ta = acc.b;
 #pragma unroll
@@ -359,7 +358,6 @@ __global__ void __launch_bounds__(kChebThreads, 1) k_cheb_fx(PropParams p, Op op
     } else {
       ++gen;
     }
-    slot ^= 1;
     return true;
   };
 

@@ -58,40 +58,60 @@ struct SmemFx {
   // Lanczos scalars (FP64) and vector metadata
   double alpha[kMaxKrylov + 2];
   double beta[kMaxKrylov + 2];
-  double scale[kMaxKrylov + 3];  // 1 / ||q_i||, real units
-  double A[kMaxKrylov + 3];      // max stored |M| of q_i
+  double nq[kMaxKrylov + 3];     // ||q_i||^2, in [1, 4) (or 0)
+  double scale[kMaxKrylov + 3];  // 1 / ||q_i||
+  double rn[kMaxKrylov + 3];     // 1 / ||q_i||^2
+  double cprev[kMaxKrylov + 3];  // coefficient of q_{i-1} in the recurrence of q_{i+1}
+  long long A[kMaxKrylov + 3];   // max stored |M| of q_i
   int E[kMaxKrylov + 3];         // exponent of q_i
+  int pw[kMaxKrylov + 3];        // q_{i+1} = w_i 2^-pw[i]
   double yr[kMaxKrylov], yi[kMaxKrylov];
   double tr[kMaxKrylov], ti[kMaxKrylov];
   // reconstruction constants
   long long crm[kMaxKrylov], cim[kMaxKrylov];
-  int csr[kMaxKrylov], csi[kMaxKrylov], cp[kMaxKrylov];
-  // stage data
+  int cp[kMaxKrylov];
+  // stage data: the scalars' mantissas, fixed for the exponential
   double scal[1 + kMaxDrives];
-  double bsite_raw[kMaxSites];
-  double bsum_raw, bmax_raw;  // sum and max over sites of |bsite_raw|
-  int eb;                     // exponent of the per-site table mb
-  long long mb[kMaxSites];
+  Mant mcz, mh, mx;           // c_0, 2 J c_0, the uniform field
+  Mant mop[1 + kMaxDrives];   // DIA, CSR: operator scalars
+  UpB hbound;                 // bound of |H q| / max|q|
+  UpB rowb[1 + kMaxDrives];   // DIA, CSR: maxrow of each operator
+  int eb;                     // exponent of the per-site table mbraw
+  long long mbraw[kMaxSites]; // per-site fields, fixed for the exponential
+  long long mb[kMaxSites];    // the same with the iteration's product shift
   FxConstA ca;
   // phase B constants
   long long m_a;
-  int s_a, sh_u, pk_b;
+  int sh_u, pk_b;
   int Eu, Ew, Epsi;
-  // control flags
-  int abort_flag;     // leave the kernel
-  int stop_prev;      // the deferred check accepted the previous iteration
-  int accept_now;     // accepted at the current iteration
-  int pend;           // a check of the current iteration is deferred
+  // commands to the workers
+  int cmd, it;                // FxCmd; the iteration, or the number of basis vectors (kFxRec)
+  int final_rec;
+  // control flow (in shared memory: what a register spill would take to local
+  // memory, whose lines the workers' loops sweep out of L1)
+  long long e, fpos;  // stage exponential of the launch; next forced decision
+  double remaining;   // of the stage exponential
+  double acc_err;     // estimate of the accepted substep
+  int nsub_e;         // substeps of the stage exponential
   int y_ready;        // yr/yi hold exp(-i ts T_k) e_1 for the accepted (k, ts)
   int acc_h;
-  int final_rec;
-  double err_now, err_prev;
   double beta0;
+  double rsum;  // fx_ctl_reduce_cold
+  long long rmx;
+  double nsum;  // ||q_1||^2 in units of 2^(2 E[1])
   // running FP32 bounds of the current T_k for the estimate's screens
   LeadAcc lead;
   GershAcc gfull;  // rows whose couplings are all known
   int gate_it;     // FP32 gate of the current iteration (1, 0, -1: FP64 needed)
   int tma_fail;    // tiled apply: a tile wait gave up
+  // kept here, not in registers (the element loops need those): the trace
+  // (cfet_stats.phase_ns; slots 0, 2, 4, 7 by thread 0, the others by the
+  // control lane 0) and, by the control lane 0, the run's counters
+  long long tacc[8];
+  long long twe;      // thread 0: end of its last element loop
+  long long n_app, n_sub, rpos;
+  int max_k;
+  double max_err;
 };
 
 // ------------------------------------------------------------------ control-warp helpers
@@ -114,17 +134,20 @@ struct FxAcc {
 
 // Control warp: combine the workers' per-warp partials into this CTA's record,
 // exchange records with every CTA (the grid barrier), and return the exact
-// global sum (as FP64) and the global max to all lanes.
-__device__ bool fx_ctl_reduce(SmemFx& S, int NW, unsigned long long* part, unsigned tag, bool fence, int* status,
+// global sum (as FP64) and the global max to all lanes.  ONE: the only CTA.
+template <bool ONE>
+__device__ __forceinline__ bool fx_ctl_reduce(SmemFx& S, int NW, unsigned long long* part, unsigned tag, bool fence, int* status,
                               long long timeout_ns, double& sum, long long& mxi, long long& spin) {
   const int lane = threadIdx.x & 31;
   unsigned long long lo = 0;
   long long hi = 0, m = 0;
   if (lane < NW) { lo = S.wlo[lane]; hi = S.whi[lane]; m = S.wmx[lane]; }
   fx_warp_reduce(lo, hi, m);
-  lo = __shfl_sync(0xffffffffu, lo, 0);
-  hi = __shfl_sync(0xffffffffu, hi, 0);
-  m = __shfl_sync(0xffffffffu, m, 0);
+  if constexpr (ONE) {
+    sum = fx_i128_to_double(lo, hi);
+    mxi = m;
+    return true;
+  }
   const unsigned mine[6] = {(unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi,
                             (unsigned)((unsigned long long)hi >> 32), (unsigned)m,
                             (unsigned)((unsigned long long)m >> 32)};
@@ -134,12 +157,25 @@ __device__ bool fx_ctl_reduce(SmemFx& S, int NW, unsigned long long* part, unsig
   hi = acc.hi;
   m = acc.m;
   fx_warp_reduce(lo, hi, m);
-  lo = __shfl_sync(0xffffffffu, lo, 0);
-  hi = __shfl_sync(0xffffffffu, hi, 0);
-  m = __shfl_sync(0xffffffffu, m, 0);
   sum = fx_i128_to_double(lo, hi);
   mxi = m;
   return true;
+}
+
+// The same out of line, for the passes that run once per launch or substep:
+// results in S.rsum and S.rmx.
+template <bool ONE>
+__device__ __noinline__ bool fx_ctl_reduce_cold(SmemFx& S, int NW, unsigned long long* part, unsigned tag, int* status,
+                                                long long timeout_ns) {
+  double sum;
+  long long mxi;
+  const bool ok = fx_ctl_reduce<ONE>(S, NW, part, tag, true, status, timeout_ns, sum, mxi, S.tacc[5]);
+  if (ok && (threadIdx.x & 31) == 0) {
+    S.rsum = sum;
+    S.rmx = mxi;
+  }
+  __syncwarp();
+  return ok;
 }
 
 // Worker warps: per-warp reduction of (int128 sum, int64 max) into shared memory.
@@ -351,94 +387,147 @@ __device__ void fx_tiled_pass(const FxTma& T, const OpSpinFx& op, const FxConstA
   workers_sync(nworkers);
 }
 
-// Scalar part of the phase-A constants (one lane).
+// The Krylov basis is built by the unnormalised three-term recurrence
+//   u_k = H q_k - c_k q_{k-1},  w_k = u_k - alpha_k q_k,  q_{k+1} = w_k 2^-p_k,
+//   alpha_k = <q_k, u_k> / ||q_k||^2,  c_k = beta_{k-1}^2 2^-p_{k-1}
+//           = 2^p_{k-1} ||q_k||^2 / ||q_{k-1}||^2,
+// v_k = q_k / ||q_k|| being the Lanczos vectors of Sec. 8.1 and p_k the power
+// of two that brings ||q_{k+1}||^2 into [1, 4) (only the exponent of the stored
+// vector changes).  The stage scalars then enter every apply with the same
+// mantissas and only shifts depend on the iteration, and between the reduction
+// of ||w_k||^2 and the next apply stands one FP64 product: on this GPU a
+// dependent FP64 instruction of the control warp costs 64 cycles, a reciprocal
+// square root 370.  beta_k, 1 / ||q_{k+1}|| and the tests that need them are
+// taken while the workers already apply H (fx_close_iteration and the deferred
+// estimate).  With the normalised recurrence (scalars times 1 / beta in every
+// iteration) the control warp held the workers 2.5 us after every phase B and
+// 1.05 us after every phase A.
+
+// Per-exponential constants (whole control warp; S.scal is set).
 template <int FAMILY, class Op>
-__device__ void fx_const_a_scalars(SmemFx& S, const Op& op, int it) {
-  FxConstA& c = S.ca;
-  const double sk = S.scale[it];
-  const int Ek = S.E[it];
-  const double Ak = S.A[it];
-  const double Akr = fx_scale2(Ak, Ek);
-  const double bp = it > 1 ? S.beta[it - 1] * S.scale[it - 1] : 0.0;
-  const double Apr = it > 1 ? fx_scale2(S.A[it - 1], S.E[it - 1]) : 0.0;
-  c.pk = fx_norm_shift(Ak);
-  double B = fabs(bp) * Apr;
+__device__ __noinline__ void fx_stage_consts(SmemFx& S, const Op& op, int nV) {
+  const int lane = threadIdx.x & 31;
   if constexpr (FAMILY == kFamilySpin) {
-    const double cz = S.scal[0] * sk;
-    const double ch = cz * op.J2;
-    // sum and max of |b_i s_k| from the per-stage sums of |b_i|
-    const double bsum = fabs(sk) * S.bsum_raw, bmax = fabs(sk) * S.bmax_raw;
-    B += (fabs(cz) * op.maxdz + fabs(ch) * op.nbond + bsum) * Akr;
-    const int Eu = fx_exp_for(B, kFxBits);
-    const Mant mcz = fx_mant(cz);
-    const int ED = fx_exp_for(fabs(cz) * op.maxdz, 59);
-    c.m_cz = mcz.m;
-    c.s_d = ED - mcz.e - (op.E_dz - 1) - 64;
-    c.s_diag = Eu - (ED - 3) - (Ek - c.pk) - 64;
-    c.m_cz = fx_fold(mcz.m, c.s_d + c.s_diag);
-    const Mant mh = fx_mant(ch);
-    c.ph = fx_norm_shift((op.N > 1 ? op.nbond : 1.0) * Ak);
-    c.m_hop = mh.m;
-    c.s_hop = Eu - mh.e - (Ek - c.ph) - 64;
-    c.m_hop = fx_fold(c.m_hop, c.s_hop);
-    if (op.uniform) {
-      const Mant mx = fx_mant(S.bsite_raw[0] * sk);
-      c.px = fx_norm_shift(op.nsite * Ak);
-      c.m_x = mx.m;
-      c.s_x = Eu - mx.e - (Ek - c.px) - 64;
-      c.m_x = fx_fold(c.m_x, c.s_x);
-    } else {
-      const int eb = fx_exp_for(bmax, 62);
-      c.s_nu = Eu - eb - (Ek - c.pk) - 64;
-      S.eb = eb;
+    double bi = 0.0;  // per-site transverse fields of this stage (N <= 30 lanes)
+    if (lane < op.N)
+      for (int k = 0; k < nV; ++k) bi = fma(S.scal[1 + k], __ldg(op.xf + k * op.N + lane), bi);
+    double bs = fabs(bi), bm = fabs(bi);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      bs += __shfl_xor_sync(0xffffffffu, bs, o);
+      bm = fmax(bm, __shfl_xor_sync(0xffffffffu, bm, o));
     }
-    c.Eu = Eu;
+    if (!op.uniform) {
+      const int eb = fx_exp_for(bm, 62);
+      if (lane < op.N) S.mbraw[lane] = __double2ll_rn(fx_scale2(bi, -eb));
+      if (lane == 0) S.eb = eb;
+    }
+    if (lane == 0) {
+      const double cz = S.scal[0], ch = cz * op.J2, db = fabs(cz) * op.maxdz;
+      S.mcz = fx_mant(cz);
+      S.mh = fx_mant(ch);
+      S.mx = fx_mant(bi);
+      S.hbound = sb_upb(db + fabs(ch) * op.nbond + bs);
+    }
   } else {
-    for (int o = 0; o < op.nops; ++o) B += fabs(S.scal[o] * sk) * op.maxrow[o] * Akr;
-    const int Eu = fx_exp_for(B, kFxBits);
-    c.Eu = Eu;
-    for (int o = 0; o < op.nops; ++o) {
-      const int Epre = fx_exp_for(op.maxrow[o] * Akr, 62);  // |P_o| < 2^62
-      c.sh_pre[o] = Epre - op.E_op[o] - Ek;
-      const Mant m = fx_mant(S.scal[o] * sk);
-      c.m_op[o] = m.m;
-      c.s_op[o] = Eu - m.e - Epre - 64;
-      c.m_op[o] = fx_fold(c.m_op[o], c.s_op[o]);
+    if (lane == 0) {
+      double hb = 0.0;
+      for (int o = 0; o < op.nops; ++o) {
+        S.mop[o] = fx_mant(S.scal[o]);
+        S.rowb[o] = sb_upb(op.maxrow[o]);
+        hb += fabs(S.scal[o]) * op.maxrow[o];
+      }
+      S.hbound = sb_upb(hb);
     }
   }
-  const Mant mp = fx_mant(-bp);
-  c.pp = it > 1 ? fx_norm_shift(S.A[it - 1]) : 0;
-  c.m_p = mp.m;
-  c.s_p = c.Eu - mp.e - (it > 1 ? S.E[it - 1] - c.pp : 0) - 64;
-  c.m_p = fx_fold(c.m_p, c.s_p);
-  c.use_prev = it > 1;
-  S.Eu = c.Eu;
+  if (lane == 0) S.hbound = sb_upb_mul(S.hbound, UpB{1.0f + 0x1p-20f, 0});  // FP64 rounding of the sums above
+  __syncwarp();
 }
 
-// Phase-A constants (called by the whole control warp: lane 0 computes the
-// scalars, the per-site table is split over the lanes): result exponent of
-// u = s_k H q_k - beta_{k-1} s_{k-1} q_{k-1} from the bound of every term,
-// normalising shifts and product shifts.
+// Phase-A constants of iteration it (called by the whole control warp): result
+// exponent of u = H q_it - c q_{it-1} from the bound of every term (in every
+// lane), then one lane per term: value m 2^e times a sum of cnt entries of a
+// vector with maximum A at exponent E takes the normalising shift p and the
+// product shift Eu - e - (E - p) - 64.
 template <int FAMILY, class Op>
-__device__ void fx_const_a(SmemFx& S, const Op& op, int it) {
+__device__ __forceinline__ void fx_const_a(SmemFx& S, const Op& op, int it) {
   const int lane = threadIdx.x & 31;
   FxConstA& c = S.ca;
-  if (lane == 0) fx_const_a_scalars<FAMILY>(S, op, it);
-  __syncwarp();
+  const long long Ak = S.A[it], Ap = it > 1 ? S.A[it - 1] : 0;
+  const int Ek = S.E[it], Ep = it > 1 ? S.E[it - 1] : 0;
+  const double cp = it > 1 ? S.cprev[it] : 0.0;
+  const UpB Akr = sb_upb_scale2(sb_upb_ll(Ak), Ek);
+  const UpB B = sb_upb_add(sb_upb_mul(S.hbound, Akr), sb_upb_mul(sb_upb(cp), sb_upb_scale2(sb_upb_ll(Ap), Ep)));
+  const int Eu = sb_upb_exp_for(B, kFxBits);
+  if (lane == 0) {
+    c.use_prev = it > 1;
+    c.Eu = Eu;
+    S.Eu = Eu;
+  }
   if constexpr (FAMILY == kFamilySpin) {
+    // terms: diagonal (c_0 times the table at 2^E_dz), hops, uniform field, q_{it-1}
+    if (lane < 4) {
+      const Mant m = lane == 0 ? S.mcz : (lane == 1 ? S.mh : (lane == 2 ? S.mx : fx_mant(-cp)));
+      const int e = lane == 0 ? m.e + op.E_dz + 60 : m.e;
+      const int cnt = lane == 1 ? (op.N > 1 ? op.N - 1 : 1) : (lane == 2 ? op.N : 1);
+      const int ps = sb_norm_shift_ll(cnt * (lane == 3 ? Ap : Ak));
+      c.p4[lane] = ps;
+      c.m4[lane] = fx_fold(m.m, Eu - e - ((lane == 3 ? Ep : Ek) - ps) - 64);
+    }
     if (!op.uniform) {
-      const double sk = S.scale[it];
-      for (int i = lane; i < op.N; i += 32)
-        S.mb[i] = fx_fold(__double2ll_rn(fx_scale2(S.bsite_raw[i] * sk, -S.eb)), c.s_nu);
+      const int s_nu = Eu - S.eb - (Ek - sb_norm_shift_ll(Ak)) - 64;
+      for (int i = lane; i < op.N; i += 32) S.mb[i] = fx_fold(S.mbraw[i], s_nu);
+    }
+  } else {
+    if (lane < op.nops) {
+      const int Epre = sb_upb_exp_for(sb_upb_mul(S.rowb[lane], Akr), 62);  // |P_o| < 2^62
+      const Mant m = S.mop[lane];
+      c.sh_pre[lane] = Epre - op.E_op[lane] - Ek;
+      c.m_op[lane] = fx_fold(m.m, Eu - m.e - Epre - 64);
+    } else if (lane == op.nops) {
+      const Mant m = fx_mant(-cp);
+      c.pp = sb_norm_shift_ll(Ap);
+      c.m_p = fx_fold(m.m, Eu - m.e - (Ep - c.pp) - 64);
     }
   }
+}
+
+template <int FAMILY, class Op>
+__device__ __noinline__ void fx_const_a_cold(SmemFx& S, const Op& op, int it) {  // once per substep
+  fx_const_a<FAMILY>(S, op, it);
+}
+
+// Squared norm `sum` 2^(2E) of a vector stored at exponent E: the power of two
+// p that brings it into [1, 4), and the scaled value (0 and 0 for sum = 0).
+__device__ __forceinline__ double fx_norm_pow(double sum, int E, int& p) {
+  if (!(__double_as_longlong(sum) > 0)) {
+    p = 0;
+    return 0.0;
+  }
+  p = (fx_ilog2(sum) + 2 * E) >> 1;
+  return fx_scale2(sum, 2 * (E - p));
+}
+
+// What iteration it leaves for later (one lane): 1 / ||q_{it+1}||, its square
+// and beta_it = ||q_{it+1}|| 2^p / ||q_it||.
+__device__ void fx_close_iteration(SmemFx& S, int it) {
+  const double n = S.nq[it + 1];
+  const double rs = __double_as_longlong(n) > 0 ? rsqrt(n) : 0.0;
+  S.scale[it + 1] = rs;
+  S.rn[it + 1] = rs * rs;
+  S.beta[it] = fx_scale2(n * rs * S.scale[it], S.pw[it]);
+}
+// Lanczos breakdown at iteration it (closed).
+__device__ __forceinline__ bool fx_breakdown(const SmemFx& S, int it) {
+  const double b = S.beta[it], prev_b = it > 1 ? S.beta[it - 1] : 0.0;
+  return sb_no_breakdown(b, S.alpha[it], prev_b) != 1 && b <= 1e-13 * (fabs(S.alpha[it]) + prev_b + 1.0);
 }
 
 // Error estimate of iteration k (control warp): err = beta0 beta_k |y_k| with
 // y = exp(-i ts T_k) e_1 left in S.yr/S.yi.  When the FP32 screen shows that
 // err exceeds the threshold thr, the FP64 evaluation is skipped and a value
 // above thr is returned (S.yr/S.yi then stay untouched).
-__device__ double fx_estimate(SmemFx& S, int k, double ts, double thr) {
+__device__ __noinline__ double fx_estimate(SmemFx& S, int k, double ts, double thr) {
   const int dec = krylov_lead_decide(S.lead, k, ts, S.beta0, S.beta[k], thr);
   if (dec == 0) return 2.0 * thr + 1e-300;
   const double scale = S.beta0 * S.beta[k];
@@ -448,87 +537,217 @@ __device__ double fx_estimate(SmemFx& S, int k, double ts, double thr) {
   return scale * sqrt(fma(yr, yr, yi * yi));
 }
 
+// Halves the step on the basis of iteration it until the estimate meets the
+// proportional tolerance (control warp): S.acc_h, 0 when no step does.
+__device__ __noinline__ void fx_halve(SmemFx& S, int it, double tol, double tau) {
+  const double remaining = S.remaining;
+  int hh = 0;
+  double err = 0.0;
+  const double width = gersh_width(it, S.alpha + 1, S.beta + 1);
+#pragma unroll 1
+  for (int h = 1; h <= 40; ++h) {
+    const double ts = fx_scale2(remaining, -h);
+    if (!(fabs(ts) * width <= 2.0 * it)) continue;
+    err = fx_estimate(S, it, ts, tol * ts / tau);
+    if (err <= tol * ts / tau) { hh = h; break; }
+  }
+  if ((threadIdx.x & 31) == 0) { S.acc_h = hh; S.acc_err = err; S.y_ready = hh > 0; }
+}
+
 // ------------------------------------------------------------------ the kernel
+// Worker and control warps run separate loops: the control warp publishes one
+// command (an element pass) at a time with its constants in shared memory, a CTA
+// barrier starts the pass, a second one ends it.  Keeping the two apart halves
+// the registers live in either: with one common control flow the control warp's
+// scalars were spilled, and a spill reloaded after the workers' loops have
+// swept L1 costs an L2 round trip (0.5 to 1 us on the critical path of every
+// phase of a multi-CTA launch).
+enum FxCmd { kFxExit = 0, kFxMax, kFxConvert, kFxApply, kFxOrth, kFxRec };
+
+__device__ __forceinline__ void fx_cta_sync() { __syncthreads(); }  // by workers and control warp, each from its loop
+
 // TILED: the window-tiled apply of long spin chains (a separate instantiation,
 // so that the element-wise kernel carries none of its code).  SMALL: one CTA
 // with the Krylov basis in shared memory (separate too, so that the other
 // instantiations keep global-memory loads for the vectors).
-template <int FAMILY, class Op, bool TILED = false, bool SMALL = false>
-__global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_fx(PropParams p, Op op) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  SmemFx& S = *reinterpret_cast<SmemFx*>(smem_raw);
+template <int FAMILY, class Op, bool TILED, bool SMALL>
+__device__ __forceinline__ void fx_worker(const PropParams& p, const Op& op, SmemFx& S, unsigned char* tiles_base,
+                                          int wstep) {
   const int tid = threadIdx.x;
-  const int NW = (int)(blockDim.x >> 5) - 1;   // worker warps
-  const bool ctl = (tid >> 5) == NW;            // control warp
-  const int lane = tid & 31;
-  const bool lead = ctl && lane == 0;
   const int dim = p.dim;
-  const int G = gridDim.x;
   // each CTA walks one contiguous chunk of the vectors, so that the
   // neighbours of low-bit flips (and short band offsets) are found in L1
-  const int chunk = (dim + G - 1) / G;
-  const int wstep = NW * 32;
-  int wx0 = blockIdx.x * chunk + tid;  // workers only
-  int wxe = min(dim, (blockIdx.x + 1) * chunk);
+  int wx0, wxe;
   if constexpr (FAMILY == kFamilyCsr) {  // rows split by their work, not their number (csr_row_split)
     wx0 = __ldg(op.rb + blockIdx.x) + tid;
     wxe = __ldg(op.rb + blockIdx.x + 1);
+  } else {
+    const int chunk = (dim + gridDim.x - 1) / gridDim.x;
+    wx0 = blockIdx.x * chunk + tid;
+    wxe = min(dim, ((int)blockIdx.x + 1) * chunk);
   }
-  const int ncoef = 1 + p.nV;
-  // record exchange: three slots (phase A, phase B, reconstruction) of six
-  // tagged words per CTA; two uses of one slot are always separated by an
-  // exchange on another slot; tags continue across launches
-  const unsigned tag0 = (unsigned)ld_volatile_i32((const int*)&p.st->tag_base);
-  unsigned gen = 0;
-  unsigned long long* partA = reinterpret_cast<unsigned long long*>(p.partials);
-  unsigned long long* partB = partA + 8 * G;
-  unsigned long long* partR = partA + 16 * G;
-  unsigned long long* partW = partA + 24 * G;  // window exchanges of the tiled apply: two 1-word slots
-  // tiled apply: windows and the tile buffers behind SmemFx
+  // one-CTA launches of small problems keep the basis in shared memory
+  longlong2* const qb = SMALL ? reinterpret_cast<longlong2*>(tiles_base) : p.qbasis;
+  auto Q = [&](int i) -> longlong2* { return qb + (size_t)(i - 1) * dim; };
   TileWin win[kTiledMaxWindows] = {};
   int nwin = 1;
-  if constexpr (TILED) {
-    nwin = tiled_windows<kFxTileBits>(op.N, win);
-  }
-  // behind SmemFx: the shared-memory basis of one-CTA launches, or the tiled
-  // apply's stage mbarriers (128 bytes) and tile buffers
-  unsigned char* const tiles_base = smem_raw + ((sizeof(SmemFx) + 127) & ~size_t(127));
-  longlong2* tbuf = reinterpret_cast<longlong2*>(tiles_base);
+  if constexpr (TILED) nwin = tiled_windows<kFxTileBits>(op.N, win);
   unsigned tph = 0;  // parities of the stages' mbarriers (the same in every worker)
-  const FxTma TP{p.tmaps, reinterpret_cast<unsigned long long*>(tiles_base),
-                 reinterpret_cast<longlong2*>(tiles_base + 128), &S.tma_fail, &tph, &p.st->status, p.timeout_ns};
-  if constexpr (TILED) {
-    if (tid == 0) {  // ordered before any use by the CTA barriers of the conversion pass
-      for (int s2 = 0; s2 < kTmaStages; ++s2) mbar_init(TP.bar + s2, 1);
-      S.tma_fail = 0;
-      mbar_init_fence();
-    }
-  }
-  int wslot = 0;
-  DevStatus* st = p.st;
-  const bool glead = (blockIdx.x == 0) && lead;
-  // trace (see cfet_stats.phase_ns): worker loop times by thread 0, control
-  // own-time and barrier waits by the control lane 0, in SM clock cycles
-  long long tacc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  long long twe = 0;  // thread 0: end of its last worker loop
-  const bool fixed_k = p.tol <= 0.0;
-  const bool forced = p.f_nsub != nullptr;
-
-  long long fpos = st->forced_pos;
-  long long rpos = st->rec_pos;
-  long long n_app = 0, n_sub = 0;
-  int max_k = 0;
-  double max_err = 0.0;
-
-  // one-CTA launches of small problems keep the basis in shared memory (a
-  // separate instantiation: the others keep global-memory loads)
-  longlong2* const qb = SMALL ? tbuf : p.qbasis;
-  auto Q = [&](int i) -> longlong2* { return qb + (size_t)(i - 1) * dim; };
-
-  // ---------------- psi (complex128) -> q_1
-  // pass 1: max |component| (as ordered bit patterns of |v|) and NaN/Inf detection
-  {
-    if (!ctl) {
+  if (tid == 0) S.twe = 0;
+  while (true) {
+    fx_cta_sync();  // the command and its constants are set
+    const int cmd = S.cmd;
+    if (tid == 0 && S.twe) S.tacc[7] += sm_clock() - S.twe;
+    if (cmd == kFxExit) break;
+    const long long tw0 = sm_clock();
+    if (cmd == kFxApply) {
+      // -------- phase A: u = H q_it - c q_{it-1}, <q, u>
+      const int it = S.it;
+      const FxConstA& c = S.ca;
+      const longlong2* q = Q(it);
+      const longlong2* qm = it > 1 ? Q(it - 1) : q;
+      longlong2* u = Q(it + 1);
+      __int128 a2 = 0;
+      long long mx = 0;
+      int x = wx0;
+      if constexpr (TILED) {  // window passes, grid exchanges between them (control warp)
+        const FxTma TP{p.tmaps, reinterpret_cast<unsigned long long*>(tiles_base),
+                       reinterpret_cast<longlong2*>(tiles_base + 128), &S.tma_fail, &tph, &p.st->status,
+                       p.timeout_ns};
+        for (int w = 0; w < nwin; ++w) {
+          // basis indices: q_it is vector it - 1, q_{it-1} vector it - 2, u vector it
+          const int iq = it - 1, ia = w == 0 ? (it > 1 ? it - 2 : 0) : it, iu = it;
+          if (w == 0) {
+            if (nwin == 1)
+              fx_tiled_pass<true, true>(TP, op, c, S.mb, iq, ia, iu, win[0], 0, wstep, a2, mx);
+            else
+              fx_tiled_pass<true, false>(TP, op, c, S.mb, iq, ia, iu, win[0], 0, wstep, a2, mx);
+          } else if (w == nwin - 1) {
+            fx_tiled_pass<false, true>(TP, op, c, S.mb, iq, ia, iu, win[w], w, wstep, a2, mx);
+          } else {
+            fx_tiled_pass<false, false>(TP, op, c, S.mb, iq, ia, iu, win[w], w, wstep, a2, mx);
+          }
+          if (w + 1 < nwin) {
+            window_written_sync();    // all threads: window w written
+            window_exchanged_sync();  // all threads: the grid exchange passed
+          }
+        }
+      } else {
+        if constexpr (FAMILY == kFamilySpin) {
+          for (; x + wstep < wxe; x += 2 * wstep) {
+            longlong2 h1, h2;
+            fx_apply_spin2(q, qm, x, x + wstep, op, c, S.mb, h1, h2);
+            u[x] = h1;
+            u[x + wstep] = h2;
+            const longlong2 v1 = q[x], v2 = q[x + wstep];
+            a2 += (__int128)v1.x * h1.x + (__int128)v1.y * h1.y;
+            a2 += (__int128)v2.x * h2.x + (__int128)v2.y * h2.y;
+            mx = max(mx, max(fx_absmax(h1.x, h1.y), fx_absmax(h2.x, h2.y)));
+          }
+        }
+        if constexpr (FAMILY == kFamilyCsr) {
+          const int lb = op.lane_bits;
+          for (int r0 = wx0 - tid; r0 < wxe; r0 += wstep >> lb) {
+            const int r = r0 + (tid >> lb);
+            const bool on = r < wxe;
+            const longlong2 hv = fx_apply_csr(q, qm, r, on, dim, op, c);
+            if (on && (tid & ((1 << lb) - 1)) == 0) {
+              u[r] = hv;
+              const longlong2 v = q[r];
+              a2 += (__int128)v.x * hv.x + (__int128)v.y * hv.y;
+              mx = max(mx, fx_absmax(hv.x, hv.y));
+            }
+          }
+        } else {
+          for (; x < wxe; x += wstep) {
+            longlong2 hv;
+            if constexpr (FAMILY == kFamilySpin)
+              hv = SMALL && op.N <= kWideSites ? fx_apply_spin<true>(q, qm, x, op, c, S.mb)
+                                               : fx_apply_spin<false>(q, qm, x, op, c, S.mb);
+            else
+              hv = fx_apply_dia(q, qm, x, dim, op, c);
+            u[x] = hv;
+            const longlong2 v = q[x];
+            a2 += (__int128)v.x * hv.x + (__int128)v.y * hv.y;
+            mx = max(mx, fx_absmax(hv.x, hv.y));
+          }
+        }
+      }
+      fx_worker_partial(S, a2, mx);
+      if (tid == 0) S.tacc[0] += (S.twe = sm_clock()) - tw0;
+    } else if (cmd == kFxOrth) {
+      // -------- phase B: w = u - alpha q_it, ||w||^2
+      const int sh_u = S.sh_u, pk = S.pk_b, it = S.it;
+      const long long m_a = S.m_a;
+      const longlong2* q = Q(it);
+      longlong2* u = Q(it + 1);
+      __int128 b2 = 0;
+      long long mx = 0;
+      int x = wx0;
+      // two elements per step with every load issued first (exact sums:
+      // the order does not matter)
+      for (; x + wstep < wxe; x += 2 * wstep) {
+        const longlong2 v0 = q[x], v1 = q[x + wstep];
+        const longlong2 u0 = u[x], u1 = u[x + wstep];
+        const long long wr0 = fx_rshr(u0.x, sh_u) + fx_mulhi(m_a, v0.x << pk);
+        const long long wi0 = fx_rshr(u0.y, sh_u) + fx_mulhi(m_a, v0.y << pk);
+        const long long wr1 = fx_rshr(u1.x, sh_u) + fx_mulhi(m_a, v1.x << pk);
+        const long long wi1 = fx_rshr(u1.y, sh_u) + fx_mulhi(m_a, v1.y << pk);
+        u[x] = make_longlong2(wr0, wi0);
+        u[x + wstep] = make_longlong2(wr1, wi1);
+        b2 += (__int128)wr0 * wr0 + (__int128)wi0 * wi0;
+        b2 += (__int128)wr1 * wr1 + (__int128)wi1 * wi1;
+        mx = max(mx, max(fx_absmax(wr0, wi0), fx_absmax(wr1, wi1)));
+      }
+      for (; x < wxe; x += wstep) {
+        const longlong2 v = q[x];
+        const longlong2 uu = u[x];
+        const long long wr = fx_rshr(uu.x, sh_u) + fx_mulhi(m_a, v.x << pk);
+        const long long wi = fx_rshr(uu.y, sh_u) + fx_mulhi(m_a, v.y << pk);
+        u[x] = make_longlong2(wr, wi);
+        b2 += (__int128)wr * wr + (__int128)wi * wi;
+        mx = max(mx, fx_absmax(wr, wi));
+      }
+      fx_worker_partial(S, b2, mx);
+      if (tid == 0) S.tacc[2] += (S.twe = sm_clock()) - tw0;
+    } else if (cmd == kFxRec) {
+      // -------- reconstruct q_1 <- beta0 sum_i y_i s_i q_i
+      const int acc_k = S.it;
+      const bool final_rec = S.final_rec;
+      const double outscale = fx_scale2(1.0, S.Epsi);
+      __int128 a2 = 0;
+      long long mx = 0;
+      // (cr + i ci)(vr + i vi) with three products; the sums (< 2^63) are
+      // halved to stay in fx_mulhi's operand range
+      auto term = [&](int i, const longlong2 v, long long& re, long long& im) {
+        const int pi = S.cp[i];
+        const long long cr = S.crm[i], ci = S.cim[i];
+        const long long vr = v.x << pi, vi = v.y << pi;
+        const long long p1 = fx_mulhi(cr, vr), p2 = fx_mulhi(ci, vi);
+        const long long p3 = fx_mulhi((cr + ci) >> 1, (vr + vi) >> 1) << 2;
+        re += p1 - p2;
+        im += p3 - p1 - p2;
+      };
+      for (int x = wx0; x < wxe; x += wstep) {
+        long long re = 0, im = 0;
+        int i = 0;
+        for (; i + 3 < acc_k; i += 4) {  // four basis loads in flight before their use
+          longlong2 v[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[j] = Q(i + j + 1)[x];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) term(i + j, v[j], re, im);
+        }
+        for (; i < acc_k; ++i) term(i, Q(i + 1)[x], re, im);
+        Q(1)[x] = make_longlong2(re, im);
+        if (final_rec) p.psi[x] = make_double2(__ll2double_rn(re) * outscale, __ll2double_rn(im) * outscale);
+        a2 += (__int128)re * re + (__int128)im * im;
+        mx = max(mx, fx_absmax(re, im));
+      }
+      fx_worker_partial(S, a2, mx);
+      if (tid == 0) S.tacc[4] += (S.twe = sm_clock()) - tw0;
+    } else if (cmd == kFxMax) {
+      // -------- max |component| of psi (as ordered bit patterns of |v|; finds NaN and Inf too)
       long long mx = 0;
       for (int x = wx0; x < wxe; x += wstep) {
         const double2 v = p.psi[x];
@@ -537,28 +756,8 @@ __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_fx(PropPa
         mx = max(mx, max(a, b));
       }
       fx_worker_partial(S, 0, mx);
-    }
-    __syncthreads();
-    if (ctl) {
-      // the max bit pattern is reduced in the int64 max lane
-      double sum;
-      long long bits;
-      if (!fx_ctl_reduce(S, NW, partA, tag0 + (++gen), false, &st->status, p.timeout_ns, sum, bits, tacc[5])) {
-        if (lane == 0) S.abort_flag = 1;
-      } else if (lane == 0) {
-        S.abort_flag = 0;
-        if (bits >= 0x7FF0000000000000LL) {
-          atomicCAS(&st->status, 0, (int)CFET_ENAN);
-          S.abort_flag = 1;
-        } else {
-          S.E[1] = fx_exp_for(__longlong_as_double(bits), kFxBits);
-        }
-      }
-    }
-    __syncthreads();
-    if (S.abort_flag) return;
-    // pass 2: convert and take ||q_1||^2, max |M|
-    if (!ctl) {
+    } else {
+      // -------- psi (complex128) -> q_1, ||q_1||^2, max |M|
       const double sc = fx_scale2(1.0, -S.E[1]);
       __int128 a2 = 0;
       long long mx = 0;
@@ -571,482 +770,350 @@ __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_fx(PropPa
       }
       fx_worker_partial(S, a2, mx);
     }
-    __syncthreads();
-    if (ctl) {
-      double sum;
-      long long mxi;
-      if (!fx_ctl_reduce(S, NW, partB, tag0 + (++gen), true, &st->status, p.timeout_ns, sum, mxi, tacc[5])) {
-        if (lane == 0) S.abort_flag = 1;
-      } else if (lane == 0) {
-        S.beta0 = fx_scale2(sqrt(sum), S.E[1]);
-        S.A[1] = __ll2double_ru(mxi);
-      }
-    }
-    __syncthreads();
-    if (S.abort_flag) return;
+    fx_cta_sync();  // the pass is done
   }
+}
 
-  for (long long e = 0; e < p.nexp; ++e) {
-    if (tid < ncoef) S.scal[tid] = p.scal[e * ncoef + tid];
-    __syncthreads();
-    if constexpr (FAMILY == kFamilySpin) {
-      if (ctl) {  // per-site transverse fields of this stage (N <= 30 lanes)
-        double bi = 0.0;
-        if (lane < op.N) {
-          for (int k = 0; k < p.nV; ++k) bi = fma(S.scal[1 + k], __ldg(op.xf + k * op.N + lane), bi);
-          S.bsite_raw[lane] = bi;
-        }
-        double bs = fabs(bi), bm = fabs(bi);
+// Reconstruction coefficients of the accepted (k, ts) into S (control warp).
+__device__ __noinline__ void fx_rec_consts(SmemFx& S, int acc_k, double ts) {
+  const int lane = threadIdx.x & 31;
+  if (!S.y_ready) small_expm_e1(acc_k, S.alpha + 1, S.beta + 1, ts, S.yr, S.yi, S.tr, S.ti);
+  __syncwarp();
+  double bnd = 0.0;
+#pragma unroll 1
+  for (int i = lane; i < acc_k; i += 32) {
+    const double f = S.beta0 * S.scale[i + 1];
+    const double cr = f * S.yr[i], ci = f * S.yi[i];
+    S.yr[i] = cr;
+    S.yi[i] = ci;
+    bnd += (fabs(cr) + fabs(ci)) * fx_scale2(sb_ll_to_double_up(S.A[i + 1]), S.E[i + 1]);
+  }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          bs += __shfl_xor_sync(0xffffffffu, bs, o);
-          bm = fmax(bm, __shfl_xor_sync(0xffffffffu, bm, o));
-        }
-        if (lane == 0) {
-          S.bsum_raw = bs;
-          S.bmax_raw = bm;
-        }
-      }
-      __syncthreads();
+  for (int o = 16; o > 0; o >>= 1) bnd += __shfl_xor_sync(0xffffffffu, bnd, o);
+  const int Ep = fx_exp_for(bnd, kFxBits);
+#pragma unroll 1
+  for (int i = lane; i < acc_k; i += 32) {
+    const Mant mr = fx_mant(S.yr[i]), mi = fx_mant(S.yi[i]);
+    const int pi = sb_norm_shift_ll(S.A[i + 1]);
+    S.cp[i] = pi;
+    S.crm[i] = fx_fold(mr.m, Ep - mr.e - (S.E[i + 1] - pi) - 64);
+    S.cim[i] = fx_fold(mi.m, Ep - mi.e - (S.E[i + 1] - pi) - 64);
+  }
+  if (lane == 0) S.Epsi = Ep;
+}
+
+// Full check of iteration it on the control warp: breakdown, then the gate and
+// the estimate (err, into S.acc_err).  Returns 1 (accepted) or 0; y_ready is set
+// when S.yr / S.yi hold y for the accepted (it, remaining).
+__device__ __noinline__ int fx_check(SmemFx& S, int it, double tol, double tau, int m_min, bool estimate) {
+  const int lane = threadIdx.x & 31;
+  const double remaining = S.remaining, thr = tol * remaining / tau;
+  int acc = 0, have_y = 0;
+  double err = 0.0;
+  if (fx_breakdown(S, it)) {
+    acc = 1;
+  } else if (estimate && it >= m_min) {
+    const int gate = S.gate_it;
+    if (gate >= 0 ? gate == 1 : fabs(remaining) * gersh_width(it, S.alpha + 1, S.beta + 1) <= 2.0 * it) {
+      err = fx_estimate(S, it, remaining, thr);
+      acc = have_y = err <= thr;
     }
-    const long long eg = p.exp_base + e;
-    const bool last_exp = (e == p.nexp - 1);
-    const int nforced = forced ? p.f_nsub[eg] : 0;
-    double remaining = p.tau;
-    int nsub_e = 0;
+  }
+  __syncwarp();
+  if (lane == 0) {
+    S.acc_err = err;
+    S.y_ready = have_y;
+  }
+  __syncwarp();
+  return acc;
+}
+
+template <int FAMILY, class Op, bool TILED, bool SMALL>
+__device__ __forceinline__ void fx_control(const PropParams& p, const Op& op, SmemFx& S, int NW) {
+  const int lane = threadIdx.x & 31;
+  const int G = gridDim.x;
+  const int ncoef = 1 + p.nV;
+  // record exchange (ctl_exchange): tags continue across launches
+  DevStatus* const st = p.st;
+  unsigned tag = (unsigned)ld_volatile_i32((const int*)&st->tag_base);
+  unsigned long long* const rec = reinterpret_cast<unsigned long long*>(p.partials);
+  const bool glead = blockIdx.x == 0 && lane == 0;
+  const bool fixed_k = p.tol <= 0.0;
+  const bool forced = p.f_nsub != nullptr;
+  if (lane == 0) {
+    for (int i = 0; i < 8; ++i) S.tacc[i] = 0;
+    S.n_app = S.n_sub = 0;
+    S.rpos = st->rec_pos;
+    S.fpos = st->forced_pos;
+    S.max_k = 0;
+    S.max_err = 0.0;
+  }
+  // one element pass of the workers: start (command and constants set by lane
+  // 0 or the warp) and end
+  auto start = [&](int cmd, int it) {
+    if (lane == 0) {
+      S.cmd = cmd;
+      S.it = it;
+    }
+    __syncwarp();
+    fx_cta_sync();
+  };
+  double sum;
+  long long mxi;
+
+  // ---------------- psi (complex128) -> q_1
+  start(kFxMax, 0);
+  fx_cta_sync();
+  if (!fx_ctl_reduce_cold<SMALL>(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
+  if (S.rmx >= 0x7FF0000000000000LL) {
+    if (lane == 0) atomicCAS(&st->status, 0, (int)CFET_ENAN);
+    return;
+  }
+  if (lane == 0) S.E[1] = fx_exp_for(__longlong_as_double(S.rmx), kFxBits);
+  start(kFxConvert, 0);
+  fx_cta_sync();
+  if (!fx_ctl_reduce_cold<SMALL>(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
+  if (lane == 0) {
+    S.nsum = S.rsum;
+    S.A[1] = S.rmx;
+  }
+  __syncwarp();
+
+  if (lane == 0) S.e = 0;
+  __syncwarp();
+  while (S.e < p.nexp) {
+    if (lane < ncoef) S.scal[lane] = p.scal[S.e * ncoef + lane];
+    if (lane == 0) {
+      S.remaining = p.tau;
+      S.nsub_e = 0;
+    }
+    __syncwarp();
+    fx_stage_consts<FAMILY>(S, op, p.nV);
     while (true) {
-      if (nsub_e >= p.max_substeps || (forced && nsub_e >= nforced)) {
+      if (S.nsub_e >= p.max_substeps || (forced && S.nsub_e >= p.f_nsub[p.exp_base + S.e])) {
         if (glead) atomicCAS(&st->status, 0, (int)CFET_EKRYLOV);
         return;
       }
-      int kf = -1, hf = 0;
-      if (forced) {
-        kf = p.f_k[fpos];
-        hf = p.f_h[fpos];
-      }
-      const double beta0 = S.beta0;
+      const int klimit = forced ? p.f_k[S.fpos] : p.m_max;
       int acc_k = 0, acc_h = 0;
-      double acc_err = 0.0;
-      if (beta0 != 0.0) {
-        const int klimit = forced ? kf : p.m_max;
-        if (lead) {
-          S.scale[1] = 1.0 / beta0;
-          S.pend = 0;
-          S.stop_prev = 0;
-          S.accept_now = 0;
+      if (lane == 0) S.acc_err = 0.0;
+      if (__double_as_longlong(S.nsum) != 0) {  // (a zero state stays zero)
+        if (lane == 0) {
+          int p0;
+          const double n = fx_norm_pow(S.nsum, S.E[1], p0), rs = rsqrt(n);
+          S.E[1] -= p0;
+          S.nq[1] = n;
+          S.scale[1] = rs;
+          S.rn[1] = rs * rs;
+          S.beta0 = fx_scale2(n * rs, p0);
           S.y_ready = 0;
         }
-        if (ctl) {
-          __syncwarp();
-          fx_const_a<FAMILY>(S, op, 1);
-        }
-        __syncthreads();
+        __syncwarp();
+        fx_const_a_cold<FAMILY>(S, op, 1);
+        bool accepted = false, pend = false;
         int it = 1;
         for (;; ++it) {
-          // -------- phase A(it) on the workers; deferred estimate of it-1 on the control warp
-          const int pend = S.pend;
-          if (!ctl) {
-            const FxConstA& c = S.ca;
-            const longlong2* q = Q(it);
-            const longlong2* qm = it > 1 ? Q(it - 1) : q;
-            longlong2* u = Q(it + 1);
-            __int128 a2 = 0;
-            long long mx = 0;
-            const long long tw0 = sm_clock();
-            int x = wx0;
-            if constexpr (TILED) {
-              {  // window passes, grid exchanges between them (control warp)
-                for (int w = 0; w < nwin; ++w) {
-                  // basis indices: q_it is vector it - 1, q_{it-1} vector it - 2, u vector it
-                  const int iq = it - 1, ia = w == 0 ? (it > 1 ? it - 2 : 0) : it, iu = it;
-                  if (w == 0) {
-                    if (nwin == 1)
-                      fx_tiled_pass<true, true>(TP, op, c, S.mb, iq, ia, iu, win[0], 0, wstep, a2, mx);
-                    else
-                      fx_tiled_pass<true, false>(TP, op, c, S.mb, iq, ia, iu, win[0], 0, wstep, a2, mx);
-                  } else if (w == nwin - 1) {
-                    fx_tiled_pass<false, true>(TP, op, c, S.mb, iq, ia, iu, win[w], w, wstep, a2, mx);
-                  } else {
-                    fx_tiled_pass<false, false>(TP, op, c, S.mb, iq, ia, iu, win[w], w, wstep, a2, mx);
-                  }
-                  if (w + 1 < nwin) {
-                    window_written_sync();    // all threads: window w written
-                    window_exchanged_sync();  // all threads: the grid exchange passed
-                  }
-                }
-                x = wxe;  // nothing left for the element loops
-              }
-            }
-            if constexpr (FAMILY == kFamilySpin) {
-              for (; x + wstep < wxe; x += 2 * wstep) {
-                longlong2 h1, h2;
-                fx_apply_spin2(q, qm, x, x + wstep, op, c, S.mb, h1, h2);
-                u[x] = h1;
-                u[x + wstep] = h2;
-                const longlong2 v1 = q[x], v2 = q[x + wstep];
-                a2 += (__int128)v1.x * h1.x + (__int128)v1.y * h1.y;
-                a2 += (__int128)v2.x * h2.x + (__int128)v2.y * h2.y;
-                mx = max(mx, max(fx_absmax(h1.x, h1.y), fx_absmax(h2.x, h2.y)));
-              }
-            }
-            if constexpr (FAMILY == kFamilyCsr) {
-              const int lb = op.lane_bits;
-              for (int r0 = wx0 - tid; r0 < wxe; r0 += wstep >> lb) {
-                const int r = r0 + (tid >> lb);
-                const bool on = r < wxe;
-                const longlong2 hv = fx_apply_csr(q, qm, r, on, dim, op, c);
-                if (on && (tid & ((1 << lb) - 1)) == 0) {
-                  u[r] = hv;
-                  const longlong2 v = q[r];
-                  a2 += (__int128)v.x * hv.x + (__int128)v.y * hv.y;
-                  mx = max(mx, fx_absmax(hv.x, hv.y));
-                }
-              }
-              x = wxe;
-            }
-            for (; x < wxe; x += wstep) {
-              longlong2 hv = make_longlong2(0, 0);
-              if constexpr (FAMILY == kFamilySpin) hv = fx_apply_spin(q, qm, x, op, c, S.mb);
-              else if constexpr (FAMILY == kFamilyDia) hv = fx_apply_dia(q, qm, x, dim, op, c);
-              u[x] = hv;
-              const longlong2 v = q[x];
-              a2 += (__int128)v.x * hv.x + (__int128)v.y * hv.y;
-              mx = max(mx, fx_absmax(hv.x, hv.y));
-            }
-            fx_worker_partial(S, a2, mx);
-            if (tid == 0) {
-              twe = sm_clock();
-              tacc[0] += twe - tw0;
-            }
-          } else {
+          // -------- phase A(it) on the workers; what iteration it-1 left here
+          start(kFxApply, it);
+          bool stop_prev = false;
+          if (it > 1) {
+            const long long te0 = sm_clock();
+            if (lane == 0) fx_close_iteration(S, it - 1);
+            __syncwarp();
             if (pend) {
-              const long long te0 = sm_clock();
-              const double err = fx_estimate(S, it - 1, remaining, p.tol * remaining / p.tau);
-              if (lane == 0) {
-                S.err_prev = err;
-                S.stop_prev = err <= p.tol * remaining / p.tau;
-                S.y_ready = S.stop_prev;
-                tacc[6] += sm_clock() - te0;
-              }
-              __syncwarp();
+              stop_prev = fx_check(S, it - 1, p.tol, p.tau, p.m_min, !fixed_k) != 0;
             }
-            if constexpr (TILED) {
-              {  // grid exchanges between the window passes of the workers
-                for (int w = 0; w + 1 < nwin; ++w) {
-                  window_written_sync();
-                  const bool ok = !S.abort_flag && fx_ctl_barrier(partW + (size_t)wslot * G, tag0 + (++gen),
-                                                                  &st->status, p.timeout_ns, tacc[5]);
-                  __syncwarp();
-                  if (!ok && lane == 0) S.abort_flag = 1;
-                  wslot ^= 1;
-                  window_exchanged_sync();
-                }
-              }
+            if (lane == 0) S.tacc[6] += sm_clock() - te0;
+          }
+          if constexpr (TILED) {  // grid exchanges between the window passes of the workers
+            TileWin win[kTiledMaxWindows] = {};
+            const int nwin = tiled_windows<kFxTileBits>(op.N, win);
+            bool ok = true;
+            for (int w = 0; w + 1 < nwin; ++w) {
+              window_written_sync();
+              ok = ok && fx_ctl_barrier(rec, ++tag, &st->status, p.timeout_ns, S.tacc[5]);
+              window_exchanged_sync();
+            }
+            if (!ok) {
+              fx_cta_sync();
+              return;
             }
           }
-          __syncthreads();
-          if (ctl) {
-            const long long tc0 = sm_clock(), sp0 = tacc[5];
-            double sum;
-            long long mxi;
+          fx_cta_sync();
+          {
+            const long long sp0 = S.tacc[5];
             // (the tiled apply leaves u written by other CTAs: fence)
-            constexpr bool kMayTile = TILED;
-            if ((kMayTile && S.abort_flag) ||
-                !fx_ctl_reduce(S, NW, partA, tag0 + (++gen), kMayTile, &st->status, p.timeout_ns,
-                               sum, mxi, tacc[5])) {
-              if (lane == 0) S.abort_flag = 1;
-            } else if (lane == 0 && !S.stop_prev) {
-              const double s_it = S.scale[it];
-              const double alpha = fx_scale2(sum, S.E[it] + S.Eu) * s_it;
+            if (!fx_ctl_reduce<SMALL>(S, NW, rec, ++tag, TILED, &st->status, p.timeout_ns, sum, mxi, S.tacc[5]))
+              return;
+            if (stop_prev) {  // the deferred check accepted it-1
+              it -= 1;
+              accepted = true;
+              break;
+            }
+            if (mxi >= (1LL << 60)) {  // fixed-point range exceeded (not expected)
+              if (lane == 0) atomicCAS(&st->status, 0, (int)CFET_ENAN);
+              return;
+            }
+            if (lane == 0) {
+              const int Eu = S.Eu, Ek = S.E[it];
+              const double alpha = fx_scale2(sum, Ek + Eu) * S.rn[it];
               S.alpha[it] = alpha;
-              // phase-B constants: w = u - alpha s_it q_it
-              const double am = alpha * s_it;
-              const double Bw = fx_scale2(sb_ll_to_double_up(mxi), S.Eu) + fabs(am) * fx_scale2(S.A[it], S.E[it]);
-              const int Ew = fx_exp_for(Bw, kFxBits);
-              const Mant ma = fx_mant(-am);
-              const int pk = fx_norm_shift(S.A[it]);
+              // phase-B constants: w = u - alpha q_it
+              const long long Ak = S.A[it];
+              const UpB Bw = sb_upb_add(sb_upb_scale2(sb_upb_ll(mxi), Eu),
+                                        sb_upb_mul(sb_upb(alpha), sb_upb_scale2(sb_upb_ll(Ak), Ek)));
+              const int Ew = sb_upb_exp_for(Bw, kFxBits);
+              const Mant ma = fx_mant(-alpha);
+              const int pk = sb_norm_shift_ll(Ak);
               S.Ew = Ew;
-              S.sh_u = Ew - S.Eu;
-              S.m_a = ma.m;
+              S.sh_u = Ew - Eu;
               S.pk_b = pk;
-              S.s_a = Ew - ma.e - (S.E[it] - pk) - 64;
-              S.m_a = fx_fold(ma.m, S.s_a);
-              if (mxi >= (1LL << 60)) {  // fixed-point range exceeded (not expected)
-                atomicCAS(&st->status, 0, (int)CFET_ENAN);
-                S.abort_flag = 1;
-              }
+              S.m_a = fx_fold(ma.m, Ew - ma.e - (Ek - pk) - 64);
+              S.tacc[1] += sm_clock() - S.twe - (S.tacc[5] - sp0);
             }
-            if (lane == 0) tacc[1] += sm_clock() - tc0 - (tacc[5] - sp0);
           }
-          __syncthreads();
-          if (tid == 0) tacc[7] += sm_clock() - twe;
-          if (S.abort_flag) return;
-          if (S.stop_prev) {  // the deferred estimate accepted it-1
-            it -= 1;
-            acc_err = S.err_prev;
-            break;
-          }
-          // -------- phase B(it): w = u - alpha s_it q_it, beta = ||w||
-          if (!ctl) {
-            const int sh_u = S.sh_u, pk = S.pk_b;
-            const long long m_a = S.m_a;
-            const longlong2* q = Q(it);
-            longlong2* u = Q(it + 1);
-            __int128 b2 = 0;
-            long long mx = 0;
-            const long long tw0 = sm_clock();
-            int x = wx0;
-            // two elements per step with every load issued first (exact sums:
-            // the order does not matter)
-            for (; x + wstep < wxe; x += 2 * wstep) {
-              const longlong2 v0 = q[x], v1 = q[x + wstep];
-              const longlong2 u0 = u[x], u1 = u[x + wstep];
-              const long long wr0 = fx_rshr(u0.x, sh_u) + fx_mulhi(m_a, v0.x << pk);
-              const long long wi0 = fx_rshr(u0.y, sh_u) + fx_mulhi(m_a, v0.y << pk);
-              const long long wr1 = fx_rshr(u1.x, sh_u) + fx_mulhi(m_a, v1.x << pk);
-              const long long wi1 = fx_rshr(u1.y, sh_u) + fx_mulhi(m_a, v1.y << pk);
-              u[x] = make_longlong2(wr0, wi0);
-              u[x + wstep] = make_longlong2(wr1, wi1);
-              b2 += (__int128)wr0 * wr0 + (__int128)wi0 * wi0;
-              b2 += (__int128)wr1 * wr1 + (__int128)wi1 * wi1;
-              mx = max(mx, max(fx_absmax(wr0, wi0), fx_absmax(wr1, wi1)));
+          // -------- phase B(it) on the workers; running bounds of T_it (alpha_it
+          // and beta_{it-1} are known) and the FP32 gate of its estimate here
+          start(kFxOrth, it);
+          if (lane == 0) S.gate_it = krylov_bounds_update(S, it, S.remaining);
+          __syncwarp();
+          fx_cta_sync();
+          {
+            const long long sp0 = S.tacc[5];
+            if (!fx_ctl_reduce<SMALL>(S, NW, rec, ++tag, true, &st->status, p.timeout_ns, sum, mxi,
+                                      S.tacc[5]))
+              return;
+            if (lane == 0) {
+              int pw;
+              const double n = fx_norm_pow(sum, S.Ew, pw);
+              S.nq[it + 1] = n;
+              S.pw[it] = pw;
+              S.E[it + 1] = S.Ew - pw;
+              S.A[it + 1] = mxi;
+              S.cprev[it + 1] = fx_scale2(n * S.rn[it], pw);
             }
-            for (; x < wxe; x += wstep) {
-              const longlong2 v = q[x];
-              const longlong2 uu = u[x];
-              const long long wr = fx_rshr(uu.x, sh_u) + fx_mulhi(m_a, v.x << pk);
-              const long long wi = fx_rshr(uu.y, sh_u) + fx_mulhi(m_a, v.y << pk);
-              u[x] = make_longlong2(wr, wi);
-              b2 += (__int128)wr * wr + (__int128)wi * wi;
-              mx = max(mx, fx_absmax(wr, wi));
-            }
-            fx_worker_partial(S, b2, mx);
-            if (tid == 0) {
-              twe = sm_clock();
-              tacc[2] += twe - tw0;
-            }
-          } else if (lane == 0) {
-            // meanwhile: running bounds of T_it (alpha_it and beta_{it-1} are
-            // known) and the FP32 gate of its estimate
-            S.gate_it = krylov_bounds_update(S, it, remaining);
-          }
-          __syncthreads();
-          if (ctl) {
-            const long long tc0 = sm_clock(), sp0 = tacc[5];
-            double sum;
-            long long mxi;
-            if (!fx_ctl_reduce(S, NW, partB, tag0 + (++gen), true, &st->status, p.timeout_ns, sum, mxi, tacc[5])) {
-              if (lane == 0) S.abort_flag = 1;
+            __syncwarp();
+            // the tests of this iteration run during the next apply (deferred
+            // check) unless it is the last one or w vanished
+            const bool zero = !(__double_as_longlong(sum) > 0);
+            bool acc = false;
+            pend = false;
+            if (forced) {
+              acc = it == klimit;
+            } else if (fixed_k && it == klimit) {
+              acc = true;
+            } else if (zero || it == klimit) {
+              if (lane == 0) fx_close_iteration(S, it);
+              __syncwarp();
+              acc = fx_check(S, it, p.tol, p.tau, p.m_min, !zero) != 0 || zero;
             } else {
-              // beta and 1/beta from one reciprocal square root
-              const double rb = __double_as_longlong(sum) > 0 ? rsqrt(sum) : 0.0;
-              const double b = fx_scale2(sum * rb, S.Ew);
-              const double prev_b = it > 1 ? S.beta[it - 1] : 0.0;
-              const bool breakdown =
-                  sb_no_breakdown(b, S.alpha[it], prev_b) != 1 && b <= 1e-13 * (fabs(S.alpha[it]) + prev_b + 1.0);
-              const int gate = S.gate_it;
-              if (lane == 0) {
-                S.beta[it] = b;
-                S.scale[it + 1] = fx_scale2(rb, -S.Ew);
-                S.E[it + 1] = S.Ew;
-                S.A[it + 1] = sb_ll_to_double_up(mxi);
-              }
-              __syncwarp();
-              int acc_flag = 0, pend_next = 0;
-              double err = 0.0;
-              if (forced) {
-                acc_flag = (it == kf);
-              } else if (fixed_k) {
-                acc_flag = (it == p.m_max) || breakdown;
-              } else if (breakdown) {
-                acc_flag = 1;
-              } else if (it >= p.m_min &&
-                         (gate >= 0 ? gate == 1
-                                    : fabs(remaining) * gersh_width(it, S.alpha + 1, S.beta + 1) <= 2.0 * it)) {
-                if (it < klimit) {
-                  pend_next = 1;  // estimate runs during the next apply
-                } else {
-                  err = fx_estimate(S, it, remaining, p.tol * remaining / p.tau);
-                  acc_flag = err <= p.tol * remaining / p.tau;
-                }
-              }
-              if (lane == 0) {
-                S.accept_now = acc_flag;
-                S.pend = pend_next;
-                S.err_now = err;
-                S.y_ready = acc_flag && !forced && !fixed_k && !breakdown;
-              }
-              __syncwarp();
-              if (!acc_flag && it < klimit) fx_const_a<FAMILY>(S, op, it + 1);
+              pend = true;
             }
-            if (lane == 0) tacc[3] += sm_clock() - tc0 - (tacc[5] - sp0);
+            if (acc) {
+              accepted = true;
+              break;
+            }
+            if (it >= klimit) break;
+            fx_const_a<FAMILY>(S, op, it + 1);
+            if (lane == 0) S.tacc[3] += sm_clock() - S.twe - (S.tacc[5] - sp0);
           }
-          __syncthreads();
-          if (tid == 0) tacc[7] += sm_clock() - twe;
-          if (S.abort_flag) return;
-          if (S.accept_now) {
-            acc_err = S.err_now;
-            break;
-          }
-          if (it >= klimit) break;
         }
         acc_k = it;
-        const bool accepted = S.accept_now || S.stop_prev;
-        acc_h = 0;
         if (forced) {
-          acc_h = hf;
+          acc_h = p.f_h[S.fpos];
         } else if (!accepted) {
-          // halve the substep on the same basis until the estimate meets the
-          // proportional tolerance (control warp)
-          if (ctl) {
-            int hh = 0;
-            double err = 0.0;
-            const double width = gersh_width(it, S.alpha + 1, S.beta + 1);
-            for (int h = 1; h <= 40; ++h) {
-              const double ts = fx_scale2(remaining, -h);
-              if (!(fabs(ts) * width <= 2.0 * it)) continue;
-              err = fx_estimate(S, it, ts, p.tol * ts / p.tau);
-              if (err <= p.tol * ts / p.tau) { hh = h; break; }
-            }
-            if (lane == 0) { S.acc_h = hh; S.err_now = err; S.y_ready = hh > 0; }
-          }
-          __syncthreads();
+          fx_halve(S, it, p.tol, p.tau);
+          __syncwarp();
           acc_h = S.acc_h;
-          acc_err = S.err_now;
           if (acc_h == 0) {
             if (glead) atomicCAS(&st->status, 0, (int)CFET_EKRYLOV);
             return;
           }
         }
-        n_app += acc_k;
-      }
-      const double ts = fx_scale2(remaining, -acc_h);
-      const bool final_rec = last_exp && acc_h == 0;
-      if (acc_k > 0) {
         // -------- reconstruct q_1 <- beta0 sum_i y_i s_i q_i
-        if (ctl) {
+        {
           const long long tr0 = sm_clock();
-          if (!S.y_ready) small_expm_e1(acc_k, S.alpha + 1, S.beta + 1, ts, S.yr, S.yi, S.tr, S.ti);
-          __syncwarp();
-          double bnd = 0.0;
-          for (int i = lane; i < acc_k; i += 32) {
-            const double f = beta0 * S.scale[i + 1];
-            const double cr = f * S.yr[i], ci = f * S.yi[i];
-            S.yr[i] = cr;
-            S.yi[i] = ci;
-            bnd += (fabs(cr) + fabs(ci)) * fx_scale2(S.A[i + 1], S.E[i + 1]);
-          }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) bnd += __shfl_xor_sync(0xffffffffu, bnd, o);
-          const int Ep = fx_exp_for(bnd, kFxBits);
-          for (int i = lane; i < acc_k; i += 32) {
-            const Mant mr = fx_mant(S.yr[i]), mi = fx_mant(S.yi[i]);
-            const int pi = fx_norm_shift(S.A[i + 1]);
-            S.crm[i] = mr.m;
-            S.cim[i] = mi.m;
-            S.cp[i] = pi;
-            S.csr[i] = Ep - mr.e - (S.E[i + 1] - pi) - 64;
-            S.csi[i] = Ep - mi.e - (S.E[i + 1] - pi) - 64;
-            S.crm[i] = fx_fold(mr.m, S.csr[i]);
-            S.cim[i] = fx_fold(mi.m, S.csi[i]);
-          }
+          fx_rec_consts(S, acc_k, fx_scale2(S.remaining, -acc_h));
           if (lane == 0) {
-            S.Epsi = Ep;
-            tacc[6] += sm_clock() - tr0;
+            S.final_rec = S.e == p.nexp - 1 && acc_h == 0;
+            S.tacc[6] += sm_clock() - tr0;
           }
         }
-        __syncthreads();
-        if (!ctl) {
-          const double outscale = fx_scale2(1.0, S.Epsi);
-          __int128 a2 = 0;
-          long long mx = 0;
-          const long long tw0 = sm_clock();
-          // (cr + i ci)(vr + i vi) with three products; the sums (< 2^63) are
-          // halved to stay in fx_mulhi's operand range
-          auto term = [&](int i, const longlong2 v, long long& re, long long& im) {
-            const int pi = S.cp[i];
-            const long long cr = S.crm[i], ci = S.cim[i];
-            const long long vr = v.x << pi, vi = v.y << pi;
-            const long long p1 = fx_mulhi(cr, vr), p2 = fx_mulhi(ci, vi);
-            const long long p3 = fx_mulhi((cr + ci) >> 1, (vr + vi) >> 1) << 2;
-            re += p1 - p2;
-            im += p3 - p1 - p2;
-          };
-          for (int x = wx0; x < wxe; x += wstep) {
-            long long re = 0, im = 0;
-            int i = 0;
-            for (; i + 3 < acc_k; i += 4) {  // four basis loads in flight before their use
-              longlong2 v[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) v[j] = Q(i + j + 1)[x];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) term(i + j, v[j], re, im);
-            }
-            for (; i < acc_k; ++i) term(i, Q(i + 1)[x], re, im);
-            Q(1)[x] = make_longlong2(re, im);
-            if (final_rec) p.psi[x] = make_double2(__ll2double_rn(re) * outscale, __ll2double_rn(im) * outscale);
-            a2 += (__int128)re * re + (__int128)im * im;
-            mx = max(mx, fx_absmax(re, im));
-          }
-          fx_worker_partial(S, a2, mx);
-          if (tid == 0) {
-              twe = sm_clock();
-              tacc[4] += twe - tw0;
-            }
+        start(kFxRec, acc_k);
+        fx_cta_sync();
+        if (!fx_ctl_reduce_cold<SMALL>(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
+        if (lane == 0) {
+          S.nsum = S.rsum;
+          S.E[1] = S.Epsi;
+          S.A[1] = S.rmx;
         }
-        __syncthreads();
-        if (ctl) {
-          double sum;
-          long long mxi;
-          if (!fx_ctl_reduce(S, NW, partR, tag0 + (++gen), true, &st->status, p.timeout_ns, sum, mxi, tacc[5])) {
-            if (lane == 0) S.abort_flag = 1;
-          } else if (lane == 0) {
-            S.beta0 = fx_scale2(sqrt(sum), S.Epsi);
-            S.E[1] = S.Epsi;
-            S.A[1] = __ll2double_ru(mxi);
-          }
-        }
-        __syncthreads();
-        if (tid == 0) tacc[7] += sm_clock() - twe;
-        if (S.abort_flag) return;
+        __syncwarp();
       }
-      if (glead && p.r_k != nullptr) {
-        if (rpos < p.r_cap) {
-          p.r_k[rpos] = acc_k;
-          p.r_h[rpos] = acc_h;
-        } else {
-          st->rec_overflow = 1;
+      if (lane == 0) {
+        if (glead && p.r_k != nullptr) {
+          if (S.rpos < p.r_cap) {
+            p.r_k[S.rpos] = acc_k;
+            p.r_h[S.rpos] = acc_h;
+          } else {
+            st->rec_overflow = 1;
+          }
         }
+        S.rpos += 1;
+        S.n_sub += 1;
+        S.n_app += acc_k;
+        if (acc_k > S.max_k) S.max_k = acc_k;
+        if (S.acc_err > S.max_err) S.max_err = S.acc_err;
+        if (forced) S.fpos += 1;
+        S.nsub_e += 1;
+        S.remaining -= fx_scale2(S.remaining, -acc_h);
       }
-      rpos += 1;
-      if (forced) fpos += 1;
-      n_sub += 1;
-      nsub_e += 1;
-      if (acc_k > max_k) max_k = acc_k;
-      if (acc_err > max_err) max_err = acc_err;
+      __syncwarp();
       if (acc_h == 0) break;
-      remaining -= ts;
     }
-    if (glead && p.r_nsub != nullptr) p.r_nsub[eg] = nsub_e;
+    if (glead && p.r_nsub != nullptr) p.r_nsub[p.exp_base + S.e] = S.nsub_e;
+    if (lane == 0) S.e += 1;
+    __syncwarp();
   }
   if (glead) {
-    st->tag_base = tag0 + gen;
-    st->forced_pos = fpos;
-    st->rec_pos = rpos;
+    st->tag_base = tag;
+    st->forced_pos = S.fpos;
+    st->rec_pos = S.rpos;
     st->n_exp += p.nexp;
-    st->n_sub += n_sub;
-    st->n_app += n_app;
-    if (max_k > st->max_k) st->max_k = max_k;
-    if (max_err > st->max_err) st->max_err = max_err;
+    st->n_sub += S.n_sub;
+    st->n_app += S.n_app;
+    if (S.max_k > st->max_k) st->max_k = S.max_k;
+    if (S.max_err > st->max_err) st->max_err = S.max_err;
   }
-  if (tid == 0 || lead) {  // every CTA: mean and max of its phase times
-    // thread 0 holds the worker slots 0, 2, 4, 7; the control lane 1, 3, 5, 6
-    const int mine[2][4] = {{0, 2, 4, 7}, {1, 3, 5, 6}};
-    for (int j = 0; j < 4; ++j) {
-      const int i = mine[tid == 0 ? 0 : 1][j];
-      atomicAdd((unsigned long long*)&st->phase_ns[i], (unsigned long long)(tacc[i] / G));
-      atomicMax(&st->phase_max_ns[i], tacc[i]);
+  if (lane < 8) {  // every CTA: mean and max of its phase times (see cfet_stats.phase_ns), SM clock cycles
+    const long long t = S.tacc[lane];
+    atomicAdd((unsigned long long*)&st->phase_ns[lane], (unsigned long long)(t / G));
+    atomicMax(&st->phase_max_ns[lane], t);
+  }
+}
+
+template <int FAMILY, class Op, bool TILED = false, bool SMALL = false>
+__global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_fx(PropParams p, Op op) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SmemFx& S = *reinterpret_cast<SmemFx*>(smem_raw);
+  const int NW = (int)(blockDim.x >> 5) - 1;  // worker warps
+  // behind SmemFx: the shared-memory basis of one-CTA launches, or the tiled
+  // apply's stage mbarriers (128 bytes) and tile buffers
+  unsigned char* const tiles_base = smem_raw + ((sizeof(SmemFx) + 127) & ~size_t(127));
+  if constexpr (TILED) {
+    if (threadIdx.x == 0) {  // ordered before any use by the CTA barriers of the conversion pass
+      for (int s2 = 0; s2 < kTmaStages; ++s2) mbar_init(reinterpret_cast<unsigned long long*>(tiles_base) + s2, 1);
+      S.tma_fail = 0;
+      mbar_init_fence();
     }
+  }
+  if ((int)(threadIdx.x >> 5) < NW) {
+    fx_worker<FAMILY, Op, TILED, SMALL>(p, op, S, tiles_base, NW * 32);
+  } else {
+    fx_control<FAMILY, Op, TILED, SMALL>(p, op, S, NW);
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) S.cmd = kFxExit;  // also after an error
+    __syncwarp();
+    fx_cta_sync();
   }
 }
 

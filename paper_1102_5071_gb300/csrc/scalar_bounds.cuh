@@ -338,6 +338,64 @@ __host__ __device__ __forceinline__ int sb_gersh_gate(const GershAcc& s, int k, 
   return -1;
 }
 
+// ------------------------------------------------------------------ upper bounds m 2^e
+// Non-negative upper bounds with an FP32 mantissa and an integer exponent
+// (m = 0, or 1 <= m < 2 up to the operations' own normalisation): the
+// fixed-point exponents only need bounds, and FP64 arithmetic for them costs 64
+// cycles per operation on the control warp.  Every operation rounds up; one
+// loses at most 2^-22 relative.
+struct UpB {
+  float m;
+  int e;
+};
+__host__ __device__ __forceinline__ UpB sb_upb_norm(float m, int e) {  // m >= 0 finite, normal or 0
+  const unsigned b = sb_fbits(m);
+  if (b < 0x00800000u) return UpB{0.f, 0};
+  return UpB{sb_float((b & 0x007FFFFFu) | 0x3F800000u), e + (int)(b >> 23) - 127};
+}
+// |v| (finite; a subnormal v counts as 2^-1022).
+__host__ __device__ __forceinline__ UpB sb_upb(double v) {
+  const unsigned long long b = (unsigned long long)sb_bits(v) & 0x7FFFFFFFFFFFFFFFULL;
+  if (b == 0) return UpB{0.f, 0};
+  if (b < 0x0010000000000000ULL) return UpB{1.f, -1022};
+  const unsigned f = (unsigned)((b >> 29) & 0x7FFFFFULL) + ((b & 0x1FFFFFFFULL) ? 1u : 0u);  // may carry to 2
+  return UpB{sb_float(0x3F800000u + f), (int)(b >> 52) - 1023};
+}
+// v >= 0.
+__host__ __device__ __forceinline__ UpB sb_upb_ll(long long v) {
+  if (v <= 0) return UpB{0.f, 0};
+  const int lz = sb_clz64((unsigned long long)v);
+  const unsigned long long n = (unsigned long long)v << lz;  // leading one at bit 63
+  const unsigned f = (unsigned)((n >> 40) & 0x7FFFFFULL) + ((n & 0xFFFFFFFFFFULL) ? 1u : 0u);
+  return UpB{sb_float(0x3F800000u + f), 63 - lz};
+}
+__host__ __device__ __forceinline__ UpB sb_upb_mul(UpB a, UpB b) {
+  const float m = a.m * b.m;  // 0 or in [1, 4]
+  return sb_upb_norm(m * (1.0f + 0x1p-22f), a.e + b.e);
+}
+__host__ __device__ __forceinline__ UpB sb_upb_add(UpB a, UpB b) {
+  if (a.m == 0.f) return b;
+  if (b.m == 0.f) return a;
+  const bool sw = b.e > a.e;
+  const UpB x = sw ? b : a, y = sw ? a : b;
+  const int d = x.e - y.e;
+  const float t = d > 40 ? 0x1p-40f : y.m * sb_float((unsigned)(127 - d) << 23);
+  return sb_upb_norm((x.m + t) * (1.0f + 0x1p-22f), x.e);
+}
+__host__ __device__ __forceinline__ UpB sb_upb_scale2(UpB a, int e) { return UpB{a.m, a.e + e}; }
+// Exponent E with a < 2^(bits + E); -960 for zero and outside 2^-963 .. 2^963.
+__host__ __device__ __forceinline__ int sb_upb_exp_for(UpB a, int bits) {
+  const UpB n = sb_upb_norm(a.m, a.e);
+  if (n.m == 0.f || n.e < -963 || n.e > 963) return -960;
+  return n.e - (bits - 1);
+}
+// Left shift that brings an int64 of magnitude <= v to below 2^62.
+__host__ __device__ __forceinline__ int sb_norm_shift_ll(long long v) {
+  if (v <= 0) return 0;
+  const int p = sb_clz64((unsigned long long)v) - 2;
+  return p < 0 ? 0 : p;
+}
+
 // ------------------------------------------------------------------ breakdown test
 // Lanczos breakdown: beta <= 1e-13 (|alpha| + beta_prev + 1).  1: no
 // breakdown for certain; -1: undecided.
