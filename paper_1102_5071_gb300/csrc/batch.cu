@@ -81,6 +81,7 @@ struct BParams {
   const int* f_nsub; const int* f_k; const int* f_h;
   int* r_nsub; int* r_k; int* r_h;
   BStat* stat;
+  int stage_bytes;      // shared memory behind SmemB for the staged vector, per CTA
 };
 
 // ------------------------------------------------------------------ number formats
@@ -100,6 +101,8 @@ struct FmtF64 {
     return Acc{__shfl_down_sync(0xffffffffu, a.s, o)};
   }
   static __device__ __forceinline__ double value(const Acc& a) { return a.s; }
+  static __device__ __forceinline__ void ld2(const V* p, V& a, V& b) { a = p[0]; b = p[1]; }
+  static __device__ __forceinline__ void st2(V* p, V a, V b) { p[0] = a; p[1] = b; }
 };
 
 // complex64 vectors; per-thread Dot2 (error-free product and sum), float-float
@@ -134,6 +137,15 @@ struct FmtC64 {
     return Acc{__shfl_down_sync(0xffffffffu, a.s, o), __shfl_down_sync(0xffffffffu, a.c, o)};
   }
   static __device__ __forceinline__ double value(const Acc& a) { return (double)a.s + (double)a.c; }
+  // element pairs (even index): one 16-byte access
+  static __device__ __forceinline__ void ld2(const V* p, V& a, V& b) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    a = make_float2(v.x, v.y);
+    b = make_float2(v.z, v.w);
+  }
+  static __device__ __forceinline__ void st2(V* p, V a, V b) {
+    *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+  }
 };
 
 template <class Fmt>
@@ -154,7 +166,19 @@ struct SmemB {
   int accept_now, acc_h, y_ready;
   double err_now;
   int item;
+  // the running instance (in shared memory, like its counters: registers are for
+  // the element passes)
+  BInst inst;
+  long long n_app, n_sub, fpos, rpos;
+  double remaining, max_err;
+  int max_k;
 };
+
+// Offset of the staged vector behind SmemB.
+template <class Fmt>
+__host__ __device__ constexpr int stage_offset() { return ((int)sizeof(SmemB<Fmt>) + 127) & ~127; }
+constexpr int kBatchStageMax = 200 * 1024;   // staged bytes of one CTA, at most
+constexpr int kBatchStageHalf = 100 * 1024;  // two CTAs per SM
 
 // ------------------------------------------------------------------ reductions
 // Sum over the CTA (and over the cluster when coop) of per-thread partials;
@@ -240,31 +264,216 @@ __device__ __forceinline__ typename Fmt::V batch_apply(const typename Fmt::V* __
   return Fmt::make(ur, ui);
 }
 
+// ------------------------------------------------------------------ scalar work (warp 0, out of line:
+// the element passes keep few enough registers for two CTAs of 512 threads per SM)
+// beta and the decision of iteration it.  kf: the forced Krylov dimension, 0 for none.
+template <class Fmt>
+__device__ __noinline__ void batch_decide(SmemB<Fmt>& S, int it, double bsum, double beta0, const BParams& P, int kf) {
+  const double remaining = S.remaining;
+  const int lane = threadIdx.x & 31;
+  const double b = sqrt(bsum);
+  const double prev_b = it > 1 ? S.beta[it - 1] : 0.0;
+  const bool breakdown =
+      sb_no_breakdown(b, S.alpha[it], prev_b) != 1 && b <= 1e-13 * (fabs(S.alpha[it]) + prev_b + 1.0);
+  const bool fixed_k = P.tol <= 0.0;
+  if (lane == 0) {
+    S.beta[it] = b;
+    S.scale[it + 1] = div_call(1.0, b);
+  }
+  __syncwarp();
+  int acc_flag = 0;
+  double err = 0.0;
+  if (kf > 0) {
+    acc_flag = (it == kf);
+  } else if (fixed_k) {
+    acc_flag = (it == P.m_max) || breakdown;
+  } else if (breakdown) {
+    acc_flag = 1;
+  } else if (it >= P.m_min && gersh_gate(it, S.alpha + 1, S.beta + 1, remaining)) {
+    const double thr = P.tol * remaining / P.tau;
+    if (krylov_lead_rejects(it, S.alpha + 1, S.beta + 1, remaining, beta0 * b, thr)) {
+      err = 2.0 * thr + 1e-300;
+    } else {
+      small_expm_e1(it, S.alpha + 1, S.beta + 1, remaining, S.yr, S.yi, S.tr, S.ti);
+      err = beta0 * b * hypot(S.yr[it - 1], S.yi[it - 1]);
+      acc_flag = err <= thr;
+    }
+  }
+  if (lane == 0) {
+    S.accept_now = acc_flag;
+    S.err_now = err;
+    S.y_ready = acc_flag && kf == 0 && !fixed_k && !breakdown;
+  }
+}
+
+template <class Fmt>
+__device__ __noinline__ void batch_halve(SmemB<Fmt>& S, int it, double beta0, double tol, double tau) {
+  const double remaining = S.remaining;
+  int hh = 0;
+  double err = 0.0;
+  const double width = gersh_width(it, S.alpha + 1, S.beta + 1);
+#pragma unroll 1
+  for (int h = 1; h <= 40; ++h) {
+    const double ts = ldexp(remaining, -h);
+    if (!(fabs(ts) * width <= 2.0 * it)) continue;
+    small_expm_e1(it, S.alpha + 1, S.beta + 1, ts, S.yr, S.yi, S.tr, S.ti);
+    err = beta0 * S.beta[it] * hypot(S.yr[it - 1], S.yi[it - 1]);
+    if (err <= tol * ts / tau) { hh = h; break; }
+  }
+  if ((threadIdx.x & 31) == 0) { S.acc_h = hh; S.err_now = err; S.y_ready = hh > 0; }
+}
+
+template <class Fmt>
+__device__ __noinline__ void batch_rec_consts(SmemB<Fmt>& S, int acc_k, double ts, double beta0) {
+  const int lane = threadIdx.x & 31;
+  if (!S.y_ready) small_expm_e1(acc_k, S.alpha + 1, S.beta + 1, ts, S.yr, S.yi, S.tr, S.ti);
+  __syncwarp();
+#pragma unroll 1
+  for (int i = lane; i < acc_k; i += 32) {
+    const double f = beta0 * S.scale[i + 1];
+    S.cr[i] = (typename Fmt::T)(f * S.yr[i]);
+    S.ci[i] = (typename Fmt::T)(f * S.yi[i]);
+  }
+}
+
+// Element pair (x, x + 1), x = part 2^lc + j even, of an instance whose applied
+// vector is staged in shared memory: sq holds this CTA's 2^lc elements, the other
+// parts are the same buffers of the cluster's CTAs.  A flip or hop of any bit
+// above bit 0 maps a pair onto a pair, so one access serves both elements; bits
+// below lc stay in this CTA, the flips and hops of the part's own bits read the
+// same j in another CTA (the part is uniform over the CTA, so these are whole
+// warps reading consecutive pairs over distributed shared memory).
+template <class Fmt>
+__device__ __forceinline__ void batch_apply2(const typename Fmt::V* sq, const typename Fmt::V* __restrict__ qm, int j,
+                                             int part, int lc, int N, int L, int uniform,
+                                             const typename Fmt::T* dz_lo, const typename Fmt::T* dz_hi,
+                                             const SmemB<Fmt>& S, cg::cluster_group& cl, typename Fmt::V& v0,
+                                             typename Fmt::V& v1, typename Fmt::V& r0, typename Fmt::V& r1) {
+  using T = typename Fmt::T;
+  using V = typename Fmt::V;
+  const int x = (part << lc) | j;
+  V p0 = Fmt::make(0, 0), p1 = p0;
+  if (S.use_prev) Fmt::ld2(qm + x, p0, p1);  // issued ahead of the neighbour sums
+  const T d0 = S.cz * (dz_lo[x & ((1 << L) - 1)] + dz_hi[x >> (L - 1)]);
+  const T d1 = S.cz * (dz_lo[(x + 1) & ((1 << L) - 1)] + dz_hi[(x + 1) >> (L - 1)]);
+  Fmt::ld2(sq + j, v0, v1);
+  T ur0 = d0 * v0.x, ui0 = d0 * v0.y, ur1 = d1 * v1.x, ui1 = d1 * v1.y;
+  T hr0 = 0, hi0 = 0, hr1 = 0, hi1 = 0;
+  auto hop = [&](const V* q) {
+    V a, b;
+    Fmt::ld2(q, a, b);
+    hr0 += a.x;
+    hi0 += a.y;
+    hr1 += b.x;
+    hi1 += b.y;
+  };
+  const unsigned anti = ((unsigned)x ^ ((unsigned)x >> 1)) & ((1u << (N - 1)) - 1u);
+  if (N > 1) {  // bond (0, 1): one element of the pair j ^ 2
+    V a, b;
+    Fmt::ld2(sq + (j ^ 2), a, b);
+    if ((j >> 1) & 1) {
+      hr0 += b.x;
+      hi0 += b.y;
+    } else {
+      hr1 += a.x;
+      hi1 += a.y;
+    }
+  }
+#pragma unroll 4
+  for (int i = 1; i < lc - 1; ++i)
+    if ((anti >> i) & 1u) hop(sq + (j ^ (3 << i)));
+  if (lc < N) {
+    if ((anti >> (lc - 1)) & 1u) hop(cl.map_shared_rank(const_cast<V*>(sq), part ^ 1) + (j ^ (1 << (lc - 1))));
+    for (int i = lc; i < N - 1; ++i)
+      if ((anti >> i) & 1u) hop(cl.map_shared_rank(const_cast<V*>(sq), part ^ (3 << (i - lc))) + j);
+  }
+  ur0 = fma(S.ch, hr0, ur0);
+  ui0 = fma(S.ch, hi0, ui0);
+  ur1 = fma(S.ch, hr1, ur1);
+  ui1 = fma(S.ch, hi1, ui1);
+  if (uniform) {
+    T xr0 = v1.x, xi0 = v1.y, xr1 = v0.x, xi1 = v0.y;  // bit 0 swaps the pair
+    auto flip = [&](const V* q) {
+      V a, b;
+      Fmt::ld2(q, a, b);
+      xr0 += a.x;
+      xi0 += a.y;
+      xr1 += b.x;
+      xi1 += b.y;
+    };
+#pragma unroll 4
+    for (int i = 1; i < lc; ++i) flip(sq + (j ^ (1 << i)));
+    for (int i = lc; i < N; ++i) flip(cl.map_shared_rank(const_cast<V*>(sq), part ^ (1 << (i - lc))) + j);
+    ur0 = fma(S.cx, xr0, ur0);
+    ui0 = fma(S.cx, xi0, ui0);
+    ur1 = fma(S.cx, xr1, ur1);
+    ui1 = fma(S.cx, xi1, ui1);
+  } else {
+    auto flip = [&](const V* q, T b_) {
+      V a, b;
+      Fmt::ld2(q, a, b);
+      ur0 = fma(b_, a.x, ur0);
+      ui0 = fma(b_, a.y, ui0);
+      ur1 = fma(b_, b.x, ur1);
+      ui1 = fma(b_, b.y, ui1);
+    };
+    ur0 = fma(S.bx[0], v1.x, ur0);
+    ui0 = fma(S.bx[0], v1.y, ui0);
+    ur1 = fma(S.bx[0], v0.x, ur1);
+    ui1 = fma(S.bx[0], v0.y, ui1);
+#pragma unroll 4
+    for (int i = 1; i < lc; ++i) flip(sq + (j ^ (1 << i)), S.bx[i]);
+    for (int i = lc; i < N; ++i) flip(cl.map_shared_rank(const_cast<V*>(sq), part ^ (1 << (i - lc))) + j, S.bx[i]);
+  }
+  if (S.use_prev) {
+    ur0 = fma(S.cp, p0.x, ur0);
+    ui0 = fma(S.cp, p0.y, ui0);
+    ur1 = fma(S.cp, p1.x, ur1);
+    ui1 = fma(S.cp, p1.y, ui1);
+  }
+  r0 = Fmt::make(ur0, ui0);
+  r1 = Fmt::make(ur1, ui1);
+}
+
 // ------------------------------------------------------------------ one instance
+// The applied vector q_it is staged in shared memory when a CTA's part of it fits
+// (every pass that forms it writes it there and to the basis): the neighbour sums
+// then read shared memory instead of gathering through L1 from L2, which served
+// most of a large instance's flips and hops.
 template <class Fmt>
 __device__ void run_instance(const BParams& P, int ii, int part, int nparts, bool coop, SmemB<Fmt>& S,
                              cg::cluster_group& cl) {
   using V = typename Fmt::V;
   using T = typename Fmt::T;
   using Acc = typename Fmt::Acc;
-  const BInst I = P.inst[ii];
+  if (threadIdx.x == 0) {
+    S.inst = P.inst[ii];
+    S.n_app = S.n_sub = S.fpos = S.rpos = 0;
+    S.max_k = 0;
+    S.max_err = 0.0;
+  }
+  __syncthreads();
+  const BInst& I = S.inst;
   const int tid = threadIdx.x, lane = tid & 31;
   const bool w0 = tid < 32;                   // scalar warp
   const bool lead = (tid == 0) && part == 0;  // writes results of the instance
   const int dim = I.dim, N = I.N;
-  const int chunk = (((dim + nparts - 1) / nparts) + 31) & ~31;
+  // parts of 2^lc elements (at least 64 of them: with more parts than that the last stay empty)
+  int lc = N - (31 - __clz(nparts));
+  if (lc < 6) lc = min(N, 6);
+  const int chunk = 1 << lc;
+  const bool staged = chunk * (int)sizeof(V) <= P.stage_bytes;
   const int x0 = part * chunk + tid, xe = min(dim, (part + 1) * chunk);
   const int step = blockDim.x;
+  const int jn = part * chunk < dim ? chunk : 0;  // staged passes: pairs j = 2 tid, 2 tid + 2 step, ...
+  V* const sq = reinterpret_cast<V*>(reinterpret_cast<unsigned char*>(&S) + stage_offset<Fmt>());
+  const int xb = part * chunk;
   const T* dz_lo = reinterpret_cast<const T*>(I.dz);
   const T* dz_hi = dz_lo + (1 << I.L);
   V* basis = reinterpret_cast<V*>(I.basis);
   auto Q = [&](int i) -> V* { return basis + (size_t)(i - 1) * dim; };
-  const bool fixed_k = P.tol <= 0.0;
   const bool forced = I.f_nsub >= 0;
-  long long fpos = 0, rpos = 0;
-  long long n_app = 0, n_sub = 0;
-  int max_k = 0, status = 0;
-  double max_err = 0.0;
+  int status = 0;
   int slot = 0;
 
   // psi (complex128) -> q_1, ||q_1||^2 (non-finite input gives a non-finite sum)
@@ -274,6 +483,7 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
     for (int x = x0; x < xe; x += step) {
       const V f = Fmt::from64(I.psi[x]);
       Q(1)[x] = f;
+      if (staged) sq[x - xb] = f;
       Fmt::add_prod(a, f.x, f.x);
       Fmt::add_prod(a, f.y, f.y);
     }
@@ -288,7 +498,8 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
     __syncthreads();
     const bool last_exp = (e == P.nexp - 1);
     const int nforced = forced ? P.f_nsub[I.f_nsub + e] : 0;
-    double remaining = P.tau;
+    if (tid == 0) S.remaining = P.tau;
+    __syncthreads();
     int nsub_e = 0;
     while (true) {
       if (nsub_e >= P.max_substeps || (forced && nsub_e >= nforced)) {
@@ -297,8 +508,8 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
       }
       int kf = -1, hf = 0;
       if (forced) {
-        kf = P.f_k[I.f_kh + fpos];
-        hf = P.f_h[I.f_kh + fpos];
+        kf = P.f_k[I.f_kh + S.fpos];
+        hf = P.f_h[I.f_kh + S.fpos];
       }
       int acc_k = 0, acc_h = 0;
       double acc_err = 0.0;
@@ -325,6 +536,17 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
             const V* q = Q(it);
             const V* qm = it > 1 ? Q(it - 1) : q;
             V* u = Q(it + 1);
+            if (staged) {
+              for (int j = 2 * tid; j < jn; j += 2 * step) {
+                V v0, v1, h0, h1;
+                batch_apply2<Fmt>(sq, qm, j, part, lc, N, I.L, I.uniform, dz_lo, dz_hi, S, cl, v0, v1, h0, h1);
+                Fmt::st2(u + xb + j, h0, h1);
+                Fmt::add_prod(a, v0.x, h0.x);
+                Fmt::add_prod(a, v0.y, h0.y);
+                Fmt::add_prod(a, v1.x, h1.x);
+                Fmt::add_prod(a, v1.y, h1.y);
+              }
+            } else
             for (int x = x0; x < xe; x += step) {
               const V hv = batch_apply<Fmt>(q, qm, x, N, I.L, I.uniform, dz_lo, dz_hi, S);
               u[x] = hv;
@@ -345,6 +567,21 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
             const T am = S.am;
             const V* q = Q(it);
             V* u = Q(it + 1);
+            if (staged) {
+              for (int j = 2 * tid; j < jn; j += 2 * step) {
+                V v0, v1, u0, u1;
+                Fmt::ld2(sq + j, v0, v1);
+                Fmt::ld2(u + xb + j, u0, u1);
+                const V w0_ = Fmt::make(fma(am, v0.x, u0.x), fma(am, v0.y, u0.y));
+                const V w1_ = Fmt::make(fma(am, v1.x, u1.x), fma(am, v1.y, u1.y));
+                Fmt::st2(u + xb + j, w0_, w1_);
+                Fmt::st2(sq + j, w0_, w1_);
+                Fmt::add_prod(a, w0_.x, w0_.x);
+                Fmt::add_prod(a, w0_.y, w0_.y);
+                Fmt::add_prod(a, w1_.x, w1_.x);
+                Fmt::add_prod(a, w1_.y, w1_.y);
+              }
+            } else
             for (int x = x0; x < xe; x += step) {
               const V v = q[x];
               const V uu = u[x];
@@ -355,40 +592,7 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
             }
           }
           const double bsum = batch_reduce<Fmt>(S, a, slot, coop, cl);
-          if (w0) {
-            const double b = sqrt(bsum);
-            const double prev_b = it > 1 ? S.beta[it - 1] : 0.0;
-            const bool breakdown =
-                sb_no_breakdown(b, S.alpha[it], prev_b) != 1 && b <= 1e-13 * (fabs(S.alpha[it]) + prev_b + 1.0);
-            if (lane == 0) {
-              S.beta[it] = b;
-              S.scale[it + 1] = 1.0 / b;
-            }
-            __syncwarp();
-            int acc_flag = 0;
-            double err = 0.0;
-            if (forced) {
-              acc_flag = (it == kf);
-            } else if (fixed_k) {
-              acc_flag = (it == P.m_max) || breakdown;
-            } else if (breakdown) {
-              acc_flag = 1;
-            } else if (it >= P.m_min && gersh_gate(it, S.alpha + 1, S.beta + 1, remaining)) {
-              const double thr = P.tol * remaining / P.tau;
-              if (krylov_lead_rejects(it, S.alpha + 1, S.beta + 1, remaining, beta0 * b, thr)) {
-                err = 2.0 * thr + 1e-300;
-              } else {
-                small_expm_e1(it, S.alpha + 1, S.beta + 1, remaining, S.yr, S.yi, S.tr, S.ti);
-                err = beta0 * b * hypot(S.yr[it - 1], S.yi[it - 1]);
-                acc_flag = err <= thr;
-              }
-            }
-            if (lane == 0) {
-              S.accept_now = acc_flag;
-              S.err_now = err;
-              S.y_ready = acc_flag && !forced && !fixed_k && !breakdown;
-            }
-          }
+          if (w0) batch_decide<Fmt>(S, it, bsum, beta0, P, forced ? kf : 0);
           __syncthreads();
           if (S.accept_now) {
             accepted = true;
@@ -401,19 +605,7 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
         if (forced) {
           acc_h = hf;
         } else if (!accepted) {
-          if (w0) {
-            int hh = 0;
-            double err = 0.0;
-            const double width = gersh_width(it, S.alpha + 1, S.beta + 1);
-            for (int h = 1; h <= 40; ++h) {
-              const double ts = ldexp(remaining, -h);
-              if (!(fabs(ts) * width <= 2.0 * it)) continue;
-              small_expm_e1(it, S.alpha + 1, S.beta + 1, ts, S.yr, S.yi, S.tr, S.ti);
-              err = beta0 * S.beta[it] * hypot(S.yr[it - 1], S.yi[it - 1]);
-              if (err <= P.tol * ts / P.tau) { hh = h; break; }
-            }
-            if (lane == 0) { S.acc_h = hh; S.err_now = err; S.y_ready = hh > 0; }
-          }
+          if (w0) batch_halve<Fmt>(S, it, beta0, P.tol, P.tau);
           __syncthreads();
           acc_h = S.acc_h;
           acc_err = S.err_now;
@@ -422,20 +614,11 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
             break;
           }
         }
-        n_app += acc_k;
       }
-      const double ts = ldexp(remaining, -acc_h);
+      const double ts = ldexp(S.remaining, -acc_h);
       if (acc_k > 0) {
         // reconstruct q_1 <- beta0 sum_i y_i s_i q_i
-        if (w0) {
-          if (!S.y_ready) small_expm_e1(acc_k, S.alpha + 1, S.beta + 1, ts, S.yr, S.yi, S.tr, S.ti);
-          __syncwarp();
-          for (int i = lane; i < acc_k; i += 32) {
-            const double f = beta0 * S.scale[i + 1];
-            S.cr[i] = (T)(f * S.yr[i]);
-            S.ci[i] = (T)(f * S.yi[i]);
-          }
-        }
+        if (w0) batch_rec_consts<Fmt>(S, acc_k, ts, beta0);
         __syncthreads();
         const bool final_rec = last_exp && acc_h == 0;
         Acc a = Fmt::zero();
@@ -448,38 +631,44 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
             im = fma(cr, v.y, fma(ci, v.x, im));
           }
           Q(1)[x] = Fmt::make(re, im);
+          if (staged) sq[x - xb] = Fmt::make(re, im);
           if (final_rec) I.psi[x] = make_double2((double)re, (double)im);
           Fmt::add_prod(a, re, re);
           Fmt::add_prod(a, im, im);
         }
         beta0 = sqrt(batch_reduce<Fmt>(S, a, slot, coop, cl));
       }
-      if (lead && I.r_kh >= 0) {
-        if (rpos < I.r_cap) {
-          P.r_k[I.r_kh + rpos] = acc_k;
-          P.r_h[I.r_kh + rpos] = acc_h;
-        } else {
-          P.stat[ii].rec_overflow = 1;
+      __syncthreads();  // everyone has read the step's state
+      if (tid == 0) {
+        if (lead && I.r_kh >= 0) {
+          if (S.rpos < I.r_cap) {
+            P.r_k[I.r_kh + S.rpos] = acc_k;
+            P.r_h[I.r_kh + S.rpos] = acc_h;
+          } else {
+            P.stat[ii].rec_overflow = 1;
+          }
         }
+        S.rpos += 1;
+        if (forced) S.fpos += 1;
+        S.n_sub += 1;
+        S.n_app += acc_k;
+        if (acc_k > S.max_k) S.max_k = acc_k;
+        if (acc_err > S.max_err) S.max_err = acc_err;
+        S.remaining -= ts;
       }
-      rpos += 1;
-      if (forced) fpos += 1;
-      n_sub += 1;
+      __syncthreads();
       nsub_e += 1;
-      if (acc_k > max_k) max_k = acc_k;
-      if (acc_err > max_err) max_err = acc_err;
       if (acc_h == 0) break;
-      remaining -= ts;
     }
     if (lead && I.r_nsub >= 0) P.r_nsub[I.r_nsub + e] = nsub_e;
   }
   if (lead) {
     BStat& st = P.stat[ii];
     st.n_exp = P.nexp;
-    st.n_sub = n_sub;
-    st.n_app = n_app;
-    st.max_k = max_k;
-    st.max_err = max_err;
+    st.n_sub = S.n_sub;
+    st.n_app = S.n_app;
+    st.max_k = S.max_k;
+    st.max_err = S.max_err;
     st.status = status;
   }
   __syncthreads();
@@ -487,7 +676,7 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
 
 // ------------------------------------------------------------------ the kernel
 template <class Fmt>
-__global__ void __launch_bounds__(512) k_batch_propagate(BParams P) {
+__global__ void __launch_bounds__(512, 2) k_batch_propagate(BParams P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmemB<Fmt>& S = *reinterpret_cast<SmemB<Fmt>*>(smem_raw);
   cg::cluster_group cl = cg::this_cluster();
@@ -513,7 +702,7 @@ int launch_batch(const BParams& p, int clusters, int cluster_size, int threads, 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(clusters * cluster_size);
   cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = sizeof(SmemB<Fmt>);
+  cfg.dynamicSmemBytes = stage_offset<Fmt>() + p.stage_bytes;
   cfg.stream = (cudaStream_t)stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -526,11 +715,16 @@ int launch_batch(const BParams& p, int clusters, int cluster_size, int threads, 
 }
 
 template <class Fmt>
-int max_clusters(int cluster_size, int threads) {
+int max_clusters(int cluster_size, int threads, int stage_bytes) {
+  if (cudaFuncSetAttribute(k_batch_propagate<Fmt>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           stage_offset<Fmt>() + kBatchStageMax) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cluster_size);
   cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = sizeof(SmemB<Fmt>);
+  cfg.dynamicSmemBytes = stage_offset<Fmt>() + stage_bytes;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = cluster_size;
@@ -651,6 +845,57 @@ std::vector<BItem> make_items(const cfet_batch* b, const cfet_batch_plan& pl) {
   std::vector<BItem> out;
   for (int i : idx) out.push_back(items[i]);
   return out;
+}
+
+// Shared memory of a CTA for the staged vector under plan pl: the largest part
+// of an instance (as run_instance splits it) within kBatchStageMax; parts above
+// kBatchStageHalf, which leave room for one CTA per SM only, count when they are
+// at least half of the work that can be staged.
+int stage_bytes_for(const cfet_batch* b, const cfet_batch_plan& pl) {
+  const int esz = b->precision == CFET_PREC_C64 ? (int)sizeof(float2) : (int)sizeof(double2);
+  int lg = 0;
+  while ((1 << lg) < pl.cluster_size) ++lg;
+  long long most = 0, most_half = 0;
+  double big = 0.0, all = 0.0;
+  for (int i = 0; i < b->n; ++i) {
+    const int N = b->chains[i].nsites;
+    const bool coop = pl.cluster_size > 1 && N >= pl.coop_min_sites;
+    int lc = coop ? N - lg : N;
+    if (lc < 6) lc = std::min(N, 6);
+    const long long bytes = (1LL << lc) * esz;
+    if (bytes > kBatchStageMax) continue;
+    most = std::max(most, bytes);
+    if (bytes <= kBatchStageHalf) most_half = std::max(most_half, bytes);
+    else big += b->dims[i];
+    all += b->dims[i];
+  }
+  return ((int)(2.0 * big >= all ? most : most_half) + 127) & ~127;
+}
+
+// Plan before any tuning, by what the instances are (256 chains of 10..16 sites,
+// CF6:5Opt, two steps; kernel time).  complex64: clusters of 8, instances from 14
+// sites spread over one (a smaller one's vector, at most 64 KB, is staged by a
+// single CTA): 7.1 ms; from 13 or 15 sites 7.5 and 11.2; clusters of 4 8.1 at
+// best, of 2 11.7; the former default (clusters of 4 CTAs of 256 threads, only
+// the largest size spread) 20.9, and 21.2 before vectors were staged.  FP64
+// (bound by the FP64 units, vectors twice as large): clusters of 4 from 13
+// sites, 25.9 ms a step (31.4 with the former default, 31.4 with clusters of 8).
+// CTAs of 256 threads where the spread instances give each SM more than two
+// CTAs of short parts (100 chains of 12..14 sites: 1.93 against 2.34 ms); the
+// part of a spread instance is at least 256 elements.
+cfet_batch_plan default_plan(const cfet_batch* b) {
+  const bool c64 = b->precision == CFET_PREC_C64;
+  int nmax = 0;
+  for (int i = 0; i < b->n; ++i) nmax = std::max(nmax, b->chains[i].nsites);
+  cfet_batch_plan pl{};
+  pl.cluster_size = c64 ? 8 : 4;
+  pl.coop_min_sites = std::max(11, std::min(c64 ? 14 : 13, nmax - 1));
+  long long spread = 0;
+  for (int i = 0; i < b->n; ++i) spread += b->chains[i].nsites >= pl.coop_min_sites;
+  const bool short_parts = (1LL << nmax) / pl.cluster_size < 4096;
+  pl.threads = short_parts && spread * pl.cluster_size > 304 ? 256 : 512;
+  pl.tuned_ms = 0.f;
+  return pl;
 }
 
 cfet_status ensure_scal(cfet_batch* b, size_t n) {
@@ -782,8 +1027,10 @@ cfet_status run_batch(cfet_batch* b, const cfet_batch_plan& pl, double2* const* 
     inst[i].r_cap = r_cap[i];
   }
   const std::vector<BItem> items = make_items(b, pl);
-  const int maxc = b->precision == CFET_PREC_C64 ? max_clusters<FmtC64>(pl.cluster_size, pl.threads)
-                                                 : max_clusters<FmtF64>(pl.cluster_size, pl.threads);
+  const int stage = stage_bytes_for(b, pl);
+  p.stage_bytes = stage;
+  const int maxc = b->precision == CFET_PREC_C64 ? max_clusters<FmtC64>(pl.cluster_size, pl.threads, stage)
+                                                 : max_clusters<FmtF64>(pl.cluster_size, pl.threads, stage);
   if (maxc < 1) return bfail(b, CFET_EINVAL, "plan cannot be launched (no cluster fits on the device)");
   const int clusters = std::min<int>((int)items.size(), maxc);
   // the previous launch may still read the tables: order on the stream
@@ -989,14 +1236,7 @@ cfet_status cfet_batch_create(cfet_batch** out, int32_t n, const cfet_chain* cha
     b->chains[i].h = b->h[i].data();
     b->chains[i].a = b->a[i].data();
   }
-  // default plan: clusters of 4 CTAs of 256 threads, instances of the
-  // largest size present (when more than 12 sites) spread over a cluster
-  int nmax = 0;
-  for (int i = 0; i < n; ++i) nmax = std::max(nmax, chains[i].nsites);
-  b->plan.cluster_size = 4;
-  b->plan.threads = 256;
-  b->plan.coop_min_sites = nmax > 12 ? nmax : kBatchMaxSites + 1;
-  b->plan.tuned_ms = 0.f;
+  b->plan = default_plan(b);
 #undef BCKC
   *out = b;
   return CFET_OK;
@@ -1093,7 +1333,7 @@ cfet_status cfet_batch_tune(cfet_batch* b, double t0, double dt, int32_t order, 
         cands.push_back(cfet_batch_plan{cs, th, kBatchMaxSites + 1, 0.f});
         continue;
       }
-      for (int thr : {nmax - 1, nmax, kBatchMaxSites + 1}) {
+      for (int thr : {nmax - 2, nmax - 1, nmax, kBatchMaxSites + 1}) {
         if (thr < 1) continue;
         cands.push_back(cfet_batch_plan{cs, th, thr, 0.f});
       }
