@@ -1915,11 +1915,15 @@ cfet_status cfet_fidelity_grad(cfet_ctx* ctx, const void* psi0, const void* phi,
   }
   if (!ctx->d_adj_vec) {
     CK(cudaMalloc(&ctx->d_adj_vec, (size_t)(2 + 2 * kAdjMaxK) * dim * sizeof(double2)), "cudaMalloc(adjoint)");
-    int g = max_coresident_blocks_adjoint(256);
+    int g = max_coresident_blocks_adjoint();
     if (g < 1) return fail(ctx, CFET_ECUDA, "occupancy query failed for the adjoint kernel");
-    const int want = (dim + 255) / 256;
+    int nsm = 0;
+    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device), "device attribute");
+    g = std::min(g, std::min(kMaxCtlGrid, nsm));
+    // one CTA per SM; at least half of its threads get an element
+    const int want = (dim + kAdjThreads / 2 - 1) / (kAdjThreads / 2);
     ctx->adj_grid = want < g ? want : g;
-    CK(cudaMalloc(&ctx->d_adj_part, 2 * (2 * kAdjMaxK + 2) * (size_t)ctx->adj_grid * sizeof(double)),
+    CK(cudaMalloc(&ctx->d_adj_part, kPartialWordsPerCta * (size_t)ctx->adj_grid * sizeof(double)),
        "cudaMalloc(adjoint partials)");
   }
   const int nql = 6 + 12 + 24 + 48;
@@ -2016,6 +2020,8 @@ cfet_status cfet_fidelity_grad(cfet_ctx* ctx, const void* psi0, const void* phi,
   // ---- backward sweep, one launch per checkpoint interval
   CK(cudaMemsetAsync(ctx->d_adj_acc, 0, (2 * (size_t)nseg + 4) * sizeof(double), st), "gradient reset");
   CK(cudaMemsetAsync(ctx->d_st, 0, sizeof(DevStatus), st), "status reset");
+  CK(cudaMemsetAsync(ctx->d_adj_part, 0, kPartialWordsPerCta * (size_t)ctx->adj_grid * sizeof(double), st),
+     "exchange reset");
   for (long long c = nch - 1; c >= 0; --c) {
     const long long n0 = c * checkpoint_every;
     const long long n1 = (n0 + checkpoint_every) < nsteps ? (n0 + checkpoint_every) : nsteps;
@@ -2046,11 +2052,9 @@ cfet_status cfet_fidelity_grad(cfet_ctx* ctx, const void* psi0, const void* phi,
     p.grad = ctx->d_adj_acc;
     p.out = ctx->d_adj_acc + 2 * nseg;
     p.partials = ctx->d_adj_part;
-    p.bar = ctx->d_bar;
     p.st = ctx->d_st;
     p.timeout_ns = (long long)(ctx->opt.barrier_timeout_s * 1e9);
-    CK(cudaMemsetAsync(ctx->d_bar, 0, 2 * sizeof(unsigned), st), "barrier reset");
-    const int e = launch_adjoint_spin(p, ctx->spin, ctx->adj_grid, 256, st);
+    const int e = launch_adjoint_spin(p, ctx->spin, ctx->adj_grid, st);
     if (e != cudaSuccess) return cuda_fail(ctx, (cudaError_t)e, "adjoint kernel launch");
   }
   CK(cudaEventRecord(e2, st), "event");

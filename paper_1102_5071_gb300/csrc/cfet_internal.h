@@ -246,6 +246,7 @@ int cheb_threads(int workers);  // threads per CTA of the Chebyshev kernel for `
 
 // Backward (adjoint) sweep of the fidelity gradient (see adjoint.cu).
 constexpr int kAdjMaxK = 16;     // Krylov dimension limit of the adjoint sweep
+constexpr int kAdjThreads = 512;
 constexpr int kAdjMaxNodes = 48; // Gauss-Legendre nodes of the stage integral
 
 struct AdjParams {
@@ -270,8 +271,7 @@ struct AdjParams {
   const double* glw;
   double* grad;            // [2 nseg]: accumulated d<phi|psi(T)>/dA_k (re, im)
   double* out;             // [4]: re, im of the overlap (first launch), max drift, n_applies
-  double* partials;        // [2 slots x 34 values x grid]
-  unsigned* bar;
+  double* partials;        // record exchange: kExchWords words per CTA, cleared once per call
   DevStatus* st;
   long long timeout_ns;
 };
@@ -319,12 +319,12 @@ constexpr int kFxTileBits = 11;    // fixed-point tiled apply: tiles of 2^11 int
 constexpr int kFxTiledMinSites = 23;
 constexpr int kTiledMinSites = 13;  // tiles of up to 2^12 elements
 constexpr int kTiledMaxSites = 30;  // four windows cover 32 sites at 2^11-element tiles
-int launch_adjoint_spin(const AdjParams& p, const OpSpin& op, int grid, int block, void* stream);
+int launch_adjoint_spin(const AdjParams& p, const OpSpin& op, int grid, void* stream);
 int launch_wait_selftest(int which, unsigned long long* rec, unsigned* bar, int* status, long long timeout_ns);
 constexpr int kDiffBlocks = 152;  // blocks (partials) of the difference norm
 int launch_diff_norm2(const double2* a, const double2* b, int n, double* part, int nblk, void* stream);
 int launch_copy_probe(void* a, void* b, long long n16, int reps, int grid, void* stream);
-int max_coresident_blocks_adjoint(int block);
+int max_coresident_blocks_adjoint();
 int max_coresident_blocks(int family, int block);  // per device, for the persistent kernel
 size_t propagate_smem_bytes(int block);
 
