@@ -154,13 +154,11 @@ struct FxConstA {
     struct { int pk, ph, px, pp; };
     int p4[4];
   };
-  int s_d, s_diag, s_hop, s_x, s_p, s_nu;
   int use_prev;
   int Eu;
   // dia: per operator P_o = shr128(sum VAL q, sh_pre[o]); term = fx_mul(m_op[o], P_o, s_op[o])
   long long m_op[1 + kMaxDrives];
   int sh_pre[1 + kMaxDrives];
-  int s_op[1 + kMaxDrives];
 };
 
 // ------------------------------------------------------------------ applies
@@ -173,7 +171,7 @@ __device__ __forceinline__ longlong2 fx_apply_spin(const longlong2* q, const lon
                                                    const OpSpinFx& op, const FxConstA& c, const long long* mb) {
   const int N = op.N, L = op.lo_bits;
   const long long dz = __ldg(op.DZ_lo + (x & ((1 << L) - 1))) + __ldg(op.DZ_hi + (x >> (L - 1)));
-  // D = c0 s_k dz(x) 2^-s_diag (m_cz carries both shifts), then D * q_k[x]
+  // D = c0 s_k dz(x) (m_cz carries the shift), then D * q_k[x]
   const long long Dp = fx_mulhi(c.m_cz, dz << 1) << 3;
   const longlong2 v = q[x];
   long long ur = fx_mulhi(Dp, v.x << c.pk);

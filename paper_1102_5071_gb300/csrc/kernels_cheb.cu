@@ -44,6 +44,8 @@ namespace cfet {
 #endif
 constexpr int kChebThreads = CFET_CHEB_THREADS;
 
+constexpr int kChebHeld = 32;  // expansion coefficients loaded at a time
+
 struct SmemCheb {
   // constants of the current term
   FxConstA c;
@@ -54,6 +56,7 @@ struct SmemCheb {
   int sa;                         // right shift of the stored sum before this term's addition
   int E_acc;                      // exponent of the sum after this term
   int E_out;                      // exponent of this term's output
+  double rk[kChebHeld];           // coefficients of the terms k with k / kChebHeld equal to the current one's
   long long m_cs, m_sn;           // conversion of the sum to v_0: cos(tau b), -sin(tau b)
   int L_rot;
   // per exponential
@@ -63,9 +66,10 @@ struct SmemCheb {
   // per exponential and kind of term (0: first, Htilde; 1: later, 2 Htilde):
   // mantissas of the scalars and the coefficient sum of the output bound
   struct TermScalars {
-    double csum;                 // B = A_prev + csum * A_k (real units)
+    UpB csum;                    // B = A_prev + csum * A_k (real units)
     Mant mcz, mh, mx, ms;        // c0 g, c0 g 2J, b_0 g (uniform fields), -g b
-    int ED, eb;                  // exponent of the diagonal bound; of the per-site table
+    UpB rowb[1 + kMaxDrives];    // DIA, CSR: maxrow of each operator
+    int eb;                      // exponent of the per-site table
     Mant mop[1 + kMaxDrives];    // DIA: scal[o] g
     long long mbraw[kMaxSites];  // per-site table before the product shift
   } ts[2];
@@ -117,7 +121,6 @@ __device__ void cheb_exp_scalars(SmemCheb& S, int slot, const Op& op, double g, 
       const double ch = cz * op.J2;
       cs += fabs(cz) * op.maxdz + fabs(ch) * (op.N - 1) + fabs(g) * S.bsum;
       T.mcz = fx_mant(cz);
-      T.ED = fx_exp_for(fabs(cz) * op.maxdz, 59);
       T.mh = fx_mant(ch);
       if (op.uniform) T.mx = fx_mant(S.bsite[0] * g);
       else T.eb = fx_exp_for(fabs(g) * S.bmax, 62);
@@ -125,9 +128,10 @@ __device__ void cheb_exp_scalars(SmemCheb& S, int slot, const Op& op, double g, 
       for (int o = 0; o < op.nops; ++o) {
         cs += fabs(S.scal[o] * g) * op.maxrow[o];
         T.mop[o] = fx_mant(S.scal[o] * g);
+        T.rowb[o] = sb_upb(op.maxrow[o]);
       }
     }
-    T.csum = cs;
+    T.csum = sb_upb_mul(sb_upb(cs), UpB{1.0f + 0x1p-20f, 0});  // (FP64 rounding of the sum)
   }
   if constexpr (FAMILY == kFamilySpin) {
     if (!op.uniform) {
@@ -141,61 +145,61 @@ __device__ void cheb_exp_scalars(SmemCheb& S, int slot, const Op& op, double g, 
 
 // Constants of the term  y = g H_j v - g b v - use_prev * v_prev  (warp 0):
 // v has measured max |mantissa| Ak at exponent Ek, v_prev Apr at Epr; y gets
-// the exponent of the rigorous bound B of its terms (returned in real units),
-// as in the Krylov kernel (kernels_fx.cu).  Uses the per-exponential scalars
-// of cheb_exp_scalars; only shifts and folds depend on the term.
+// the exponent of the rigorous bound B of its terms (returned to every lane), as
+// in the Krylov kernel (fx_const_a): bounds in FP32 mantissa and integer
+// exponent, one lane per term.  Uses the per-exponential scalars of
+// cheb_exp_scalars; only shifts and folds depend on the term.  (With FP64 bounds
+// and one lane for all terms this took 1.4 us per term on the critical path.)
 template <int FAMILY, class Op>
-__device__ double cheb_term_const(SmemCheb& S, int slot, const Op& op, int use_prev, long long Ak, int Ek,
-                                  long long Apr, int Epr) {
+__device__ UpB cheb_term_const(SmemCheb& S, int slot, const Op& op, int use_prev, long long Ak, int Ek, long long Apr,
+                               int Epr) {
   const int lane = threadIdx.x & 31;
   FxConstA& c = S.c;
   const SmemCheb::TermScalars& T = S.ts[slot];
-  double B = 0.0;
+  const UpB Akr = sb_upb_scale2(sb_upb_ll(Ak), Ek);
+  UpB B = sb_upb_mul(T.csum, Akr);
+  if (use_prev) B = sb_upb_add(B, sb_upb_scale2(sb_upb_ll(Apr), Epr));
+  const int Eu = sb_upb_exp_for(B, kFxBits);
+  const Mant mprev{use_prev ? -(1LL << 61) : 0, -61};  // -1
   if (lane == 0) {
-    const double A = (double)Ak;
-    const double Akr = fx_scale2(A, Ek);
-    c.pk = fx_norm_shift(A);
-    B = (use_prev ? fx_scale2((double)Apr, Epr) : 0.0) + T.csum * Akr;
-    const int Eu = fx_exp_for(B, kFxBits);
     c.Eu = Eu;
-    if constexpr (FAMILY == kFamilySpin) {
-      c.s_d = T.ED - T.mcz.e - (op.E_dz - 1) - 64;
-      c.s_diag = Eu - (T.ED - 3) - (Ek - c.pk) - 64;
-      c.m_cz = fx_fold(T.mcz.m, c.s_d + c.s_diag);
-      c.ph = fx_norm_shift((op.N > 1 ? op.N - 1 : 1) * A);
-      c.s_hop = Eu - T.mh.e - (Ek - c.ph) - 64;
-      c.m_hop = fx_fold(T.mh.m, c.s_hop);
-      if (op.uniform) {
-        c.px = fx_norm_shift(op.N * A);
-        c.s_x = Eu - T.mx.e - (Ek - c.px) - 64;
-        c.m_x = fx_fold(T.mx.m, c.s_x);
-      } else {
-        c.s_nu = Eu - T.eb - (Ek - c.pk) - 64;
-      }
-    } else {
-      for (int o = 0; o < op.nops; ++o) {
-        const int Epre = fx_exp_for(op.maxrow[o] * Akr, 62);  // |P_o| < 2^62
-        c.sh_pre[o] = Epre - op.E_op[o] - Ek;
-        c.s_op[o] = Eu - T.mop[o].e - Epre - 64;
-        c.m_op[o] = fx_fold(T.mop[o].m, c.s_op[o]);
-      }
-    }
-    // -v_prev: mantissa of -1 is -2^61 at exponent -61
-    c.pp = use_prev ? fx_norm_shift((double)Apr) : 0;
-    c.s_p = Eu + 61 - (Epr - c.pp) - 64;
-    c.m_p = use_prev ? fx_fold(-(1LL << 61), c.s_p) : 0;
     c.use_prev = use_prev;
-    S.m_s = T.ms.m == 0 ? 0 : fx_fold(T.ms.m, Eu - T.ms.e - (Ek - c.pk) - 64);
   }
   if constexpr (FAMILY == kFamilySpin) {
+    // diagonal (the table at 2^E_dz), hops, uniform field, v_prev, shift term
+    if (lane < 5) {
+      const Mant m = lane == 0 ? T.mcz : (lane == 1 ? T.mh : (lane == 2 ? T.mx : (lane == 3 ? mprev : T.ms)));
+      const int e = lane == 0 ? m.e + op.E_dz + 60 : m.e;
+      const int cnt = lane == 1 ? (op.N > 1 ? op.N - 1 : 1) : (lane == 2 ? op.N : 1);
+      const int ps = sb_norm_shift_ll(cnt * (lane == 3 ? Apr : Ak));
+      const long long f = fx_fold(m.m, Eu - e - ((lane == 3 ? Epr : Ek) - ps) - 64);
+      if (lane < 4) {
+        c.p4[lane] = ps;
+        c.m4[lane] = f;
+      } else {
+        S.m_s = f;
+      }
+    }
     if (!op.uniform) {
-      __syncwarp();
-      const int s_nu = c.s_nu;
+      const int s_nu = Eu - T.eb - (Ek - sb_norm_shift_ll(Ak)) - 64;
       for (int i = lane; i < op.N; i += 32) S.mb[i] = fx_fold(T.mbraw[i], s_nu);
+    }
+  } else {
+    if (lane < op.nops) {
+      const int Epre = sb_upb_exp_for(sb_upb_mul(T.rowb[lane], Akr), 62);  // |P_o| < 2^62
+      const Mant m = T.mop[lane];
+      c.sh_pre[lane] = Epre - op.E_op[lane] - Ek;
+      c.m_op[lane] = fx_fold(m.m, Eu - m.e - Epre - 64);
+    } else if (lane == op.nops) {
+      c.pp = sb_norm_shift_ll(Apr);
+      c.m_p = fx_fold(mprev.m, Eu - mprev.e - (Epr - c.pp) - 64);
+    } else if (lane == op.nops + 1) {
+      c.pk = sb_norm_shift_ll(Ak);
+      S.m_s = fx_fold(T.ms.m, Eu - T.ms.e - (Ek - c.pk) - 64);
     }
   }
   __syncwarp();
-  return __shfl_sync(0xffffffffu, B, 0);
+  return B;
 }
 
 // fx_mulhi(fold(mant(r)), x << p) = r * x * 2^(Ex - Eout) for x at exponent Ex
@@ -447,33 +451,39 @@ __global__ void __launch_bounds__(kChebThreads, 1) k_cheb_fx(PropParams p, Op op
       // ---- constants of this term (warp 0)
       if (warp == 0) {
         const long long tc0 = sm_clock();
-        double By = 0.0;  // bound of |y| (real units)
+        if (k <= 1 || (k & (kChebHeld - 1)) == 0) {  // coefficients of the terms from here on
+          const int kb = k & ~(kChebHeld - 1);
+          for (int i = lane; i < kChebHeld; i += 32) S.rk[i] = kb + i <= K ? rk[kb + i] : 0.0;
+          __syncwarp();
+        }
+        const double r_cur = k == 0 ? 0.0 : S.rk[k & (kChebHeld - 1)];
+        UpB By{0.f, 0};  // bound of |y| (real units)
         if (k >= 1)
           By = cheb_term_const<FAMILY>(S, first ? 0 : 1, op, first ? 0 : 1, S.Av[scur], S.Ev[scur],
                                        first ? 0 : S.Av[sdst], first ? 0 : S.Ev[sdst]);
         if (lane == 0) {
           const int Ey = S.c.Eu;
-          S.py = fx_norm_shift(k >= 1 ? fx_scale2(By, -Ey) : 0.0);
+          S.py = By.m > 0.f ? min(max(61 - (By.e - Ey), 0), 61) : 0;
           // the sum: old part (measured) plus this term's bound
-          double Bacc;
+          UpB Bacc = sb_upb_mul(sb_upb(r_cur), By);
           int Eacc;
           if (first) {
-            const double A0r = fx_scale2((double)S.Av[sA], S.Ev[sA]);
-            Bacc = fabs(rk[0]) * A0r + (k >= 1 ? fabs(rk[1]) * By : 0.0);
-            Eacc = fx_exp_for(Bacc, kFxBits);
+            const double r_0 = S.rk[0];
+            Bacc = sb_upb_add(Bacc, sb_upb_mul(sb_upb(r_0), sb_upb_scale2(sb_upb_ll(S.Av[sA]), S.Ev[sA])));
+            Eacc = sb_upb_exp_for(Bacc, kFxBits);
             S.sa = 0;
-            S.p0 = fx_norm_shift((double)S.Av[sA]);
-            S.m_r0 = cheb_coef(rk[0], Eacc, S.Ev[sA], S.p0);
+            S.p0 = sb_norm_shift_ll(S.Av[sA]);
+            S.m_r0 = cheb_coef(r_0, Eacc, S.Ev[sA], S.p0);
           } else {
-            Bacc = fx_scale2((double)S.accmax, S.E_acc) + fabs(rk[k]) * By;
-            Eacc = max(S.E_acc, fx_exp_for(Bacc, kFxBits));
+            Bacc = sb_upb_add(Bacc, sb_upb_scale2(sb_upb_ll(S.accmax), S.E_acc));
+            Eacc = max(S.E_acc, sb_upb_exp_for(Bacc, kFxBits));
             S.sa = Eacc - S.E_acc;
           }
-          S.m_r = k >= 1 ? cheb_coef(rk[k], Eacc, Ey, S.py) : 0;
+          S.m_r = k >= 1 ? cheb_coef(r_cur, Eacc, Ey, S.py) : 0;
           S.E_acc = Eacc;
           if (last) {
             // v_0 of the next exponential: (cos - i sin) sum, |component| <= sqrt(2) Bacc
-            const int E0 = fx_exp_for(1.4142135623730951 * Bacc * (1.0 + 1e-12), kFxBits);
+            const int E0 = sb_upb_exp_for(sb_upb_mul(Bacc, UpB{1.4142137f, 0}), kFxBits);
             S.E_out = E0;
             const Mant mc = fx_mant(R[5]), ms = fx_mant(R[6]);
             // fx_mulhi(m, sum << 4) << L = value at E0
