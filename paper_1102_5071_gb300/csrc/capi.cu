@@ -143,7 +143,7 @@ namespace {
 
 // Reduction / exchange scratch per CTA (8-byte words): the FP64 kernel uses 3
 // partials, the control-warp kernels the two slots of the record exchange.
-constexpr size_t kPartialWordsPerCta = 8;
+constexpr size_t kPartialWordsPerCta = kExchWords;
 constexpr int kMaxCtlGrid = 256;  // 32 lanes x 8 records per lane of the exchange
 // FP64 kernel with full re-orthogonalisation: 3 slots + 2 m_max Gram-Schmidt coefficients per CTA
 static size_t partial_words_per_cta(const cfet_ctx* ctx) {

@@ -22,6 +22,15 @@ constexpr int kSmallTaylorTerms = 18;
 #define CFET_CTL_MAX_THREADS 800
 #endif
 
+// Record exchange (ctl_exchange): words from one CTA's record to the next, and
+// words of both slots per CTA.  Records 256 bytes apart spread the polls of all
+// CTAs over more L2 slices: two exchanges of 152 CTAs take 4.3 us per Lanczos
+// iteration of the grid atom, at 128 bytes 4.7, at 64 5.6, at 32 (the record's
+// size) 7.3 to 8.2 depending on the buffer's address; 512 and 1024 bytes gain
+// 0.1 us more.
+constexpr int kExchStride = 32;
+constexpr int kExchWords = 2 * kExchStride;
+
 // ---------------------------------------------------------------- schemes
 struct SchemeData {
   int id, order, s, M;

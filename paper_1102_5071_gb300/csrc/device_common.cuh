@@ -95,7 +95,6 @@ static __device__ bool warp_grid_barrier(unsigned* bar, unsigned& gen, int* stat
 // reported an error.  The two slots need kExchWords G words.
 constexpr int kExchMaxPerLane = 8;  // grids of at most 256 CTAs
 constexpr int kExchHeld = 5;        // records per lane kept in registers (grids of at most 160 CTAs)
-constexpr int kExchWords = 8;
 
 __device__ __forceinline__ void st_relaxed_v2(unsigned long long* p, unsigned long long a, unsigned long long b) {
   asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
@@ -120,7 +119,7 @@ static __device__ __forceinline__ bool ctl_exchange(unsigned long long* rec, con
     return true;
   }
   const long long c0 = sm_clock();
-  rec += (size_t)(tag & 1u) * (kExchWords / 2) * G;
+  rec += (size_t)(tag & 1u) * kExchStride * G;
   const unsigned t16 = tag & 0xffffu;
   if (lane == 0) {
     if (fence) __threadfence();
@@ -129,7 +128,7 @@ static __device__ __forceinline__ bool ctl_exchange(unsigned long long* rec, con
       const unsigned v0 = mine[3 * j], v1 = 3 * j + 1 < W ? mine[3 * j + 1 < W ? 3 * j + 1 : 0] : 0u;
       const unsigned v2 = 3 * j + 2 < W ? mine[3 * j + 2 < W ? 3 * j + 2 : 0] : 0u;
       const unsigned long long t = (unsigned long long)t16 << 48;
-      st_relaxed_v2(rec + (size_t)blockIdx.x * 4 + 2 * j, t | ((unsigned long long)(v1 & 0xffffu) << 32) | v0,
+      st_relaxed_v2(rec + (size_t)blockIdx.x * kExchStride + 2 * j, t | ((unsigned long long)(v1 & 0xffffu) << 32) | v0,
                     t | ((unsigned long long)v2 << 16) | (v1 >> 16));
     }
   }
@@ -137,31 +136,40 @@ static __device__ __forceinline__ bool ctl_exchange(unsigned long long* rec, con
   int ok = 1;
   const long long t0 = global_timer_ns();
   unsigned rounds = 0;
+  // a lane loads again only what did not carry the tag yet (records do not
+  // change once they do): the repeated polls compete with the passes of the CTAs
+  // that are waited for
   unsigned long long x0[kExchHeld], x1[kExchHeld], x2[kExchHeld], x3[kExchHeld];
+  const unsigned long long want = (unsigned long long)t16 << 48, none = want ^ (1ULL << 48);
+  auto wrong = [&](int k) {
+    return ((unsigned)(x0[k] >> 48) ^ t16) | ((unsigned)(x1[k] >> 48) ^ t16) | ((unsigned)(x2[k] >> 48) ^ t16) |
+           ((unsigned)(x3[k] >> 48) ^ t16);
+  };
+#pragma unroll
+  for (int k = 0; k < kExchHeld; ++k) {
+    x0[k] = x1[k] = lane + 32 * k < G ? none : want;
+    x2[k] = x3[k] = NP > 1 ? x0[k] : want;
+  }
   while (true) {
     unsigned bad = 0;
 #pragma unroll
     for (int k = 0; k < kExchHeld; ++k) {
-      x0[k] = x1[k] = x2[k] = x3[k] = (unsigned long long)t16 << 48;
-      if (32 * k < G) {  // (uniform)
-        const int i = lane + 32 * k < G ? lane + 32 * k : 0;  // (past the end: record 0, not passed on)
-        const ulonglong2 v = ld_relaxed_v2(rec + (size_t)i * 4);
+      if (wrong(k)) {
+        const ulonglong2 v = ld_relaxed_v2(rec + (size_t)(lane + 32 * k) * kExchStride);
         x0[k] = v.x;
         x1[k] = v.y;
         if constexpr (NP > 1) {
-          const ulonglong2 w = ld_relaxed_v2(rec + (size_t)i * 4 + 2);
+          const ulonglong2 w = ld_relaxed_v2(rec + (size_t)(lane + 32 * k) * kExchStride + 2);
           x2[k] = w.x;
           x3[k] = w.y;
         }
       }
     }
 #pragma unroll
-    for (int k = 0; k < kExchHeld; ++k)
-      bad |= ((unsigned)(x0[k] >> 48) ^ t16) | ((unsigned)(x1[k] >> 48) ^ t16) | ((unsigned)(x2[k] >> 48) ^ t16) |
-             ((unsigned)(x3[k] >> 48) ^ t16);
+    for (int k = 0; k < kExchHeld; ++k) bad |= wrong(k);
 #pragma unroll 1
     for (int i = lane + 32 * kExchHeld; i < G; i += 32) {
-      const ulonglong2 v = ld_relaxed_v2(rec + (size_t)i * 4), w = NP > 1 ? ld_relaxed_v2(rec + (size_t)i * 4 + 2) : v;
+      const ulonglong2 v = ld_relaxed_v2(rec + (size_t)i * kExchStride), w = NP > 1 ? ld_relaxed_v2(rec + (size_t)i * kExchStride + 2) : v;
       bad |= ((unsigned)(v.x >> 48) ^ t16) | ((unsigned)(v.y >> 48) ^ t16) | ((unsigned)(w.x >> 48) ^ t16) |
              ((unsigned)(w.y >> 48) ^ t16);
     }
@@ -197,7 +205,7 @@ static __device__ __forceinline__ bool ctl_exchange(unsigned long long* rec, con
       if (lane + 32 * k < G) take(x0[k], x1[k], x2[k], x3[k]);
 #pragma unroll 1
     for (int i = lane + 32 * kExchHeld; i < G; i += 32) {  // complete: the words no longer change
-      const ulonglong2 v = ld_relaxed_v2(rec + (size_t)i * 4), w = NP > 1 ? ld_relaxed_v2(rec + (size_t)i * 4 + 2) : v;
+      const ulonglong2 v = ld_relaxed_v2(rec + (size_t)i * kExchStride), w = NP > 1 ? ld_relaxed_v2(rec + (size_t)i * kExchStride + 2) : v;
       take(v.x, v.y, w.x, w.y);
     }
   }
