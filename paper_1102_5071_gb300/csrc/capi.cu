@@ -46,6 +46,7 @@ struct cfet_ctx {
   // control warp)
   bool small_fx = false;
   int small_block = 0;
+  bool cluster_fx = false;  // fixed-point chains of middle size: the grid is one cluster
   int precision = CFET_PREC_FX;
   std::string err;
   // drives
@@ -266,7 +267,7 @@ cfet_status launch_chunk(cfet_ctx* ctx, const PropParams& base, long long e0, lo
         : ctx->family == kFamilyCsr ? launch_cheb_csr_fx(p, ctx->csr_fx, ctx->grid, cheb_threads(ctx->block - 32), s)
                                     : launch_cheb_dia_fx(p, ctx->dia_fx, ctx->grid, cheb_threads(ctx->block - 32), s);
   else if (ctx->precision == CFET_PREC_FX) {
-    const int b = ctx->small_fx ? ctx->small_block : ctx->block;
+    const int b = ctx->small_fx || ctx->cluster_fx ? ctx->small_block : ctx->block;
     e = ctx->family == kFamilySpin  ? launch_propagate_spin_fx(p, ctx->spin_fx, ctx->grid, b, s)
         : ctx->family == kFamilyCsr ? launch_propagate_csr_fx(p, ctx->csr_fx, ctx->grid, b, s)
                                     : launch_propagate_dia_fx(p, ctx->dia_fx, ctx->grid, b, s);
@@ -335,6 +336,7 @@ PropParams base_params(cfet_ctx* ctx, double2* psi, double tau, double tol) {
   p.tmaps = ctx->d_tmaps;
   p.reorth = ctx->opt.reorth;
   p.small = ctx->small_fx ? 1 : 0;
+  p.cluster = ctx->cluster_fx ? 1 : 0;
   return p;
 }
 
@@ -1248,6 +1250,19 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
     if (sb > 0 && fx_small_prepare(sb) == 0) {
       ctx->small_fx = true;
       ctx->small_block = 32 + std::min(ctx->block - 32, ((dim << lane_bits) + 31) / 32 * 32);
+    }
+  }
+  if (ctx->precision == CFET_PREC_FX && family == kFamilySpin && o.expm == CFET_EXPM_KRYLOV && !ctx->small_fx &&
+      !ctx->tiled && o.grid_size == 0 && nsites <= kFxClusterMaxSites) {
+    // one cluster of at most 16 CTAs with at least 256 elements each
+    int most = 2;
+    while (most < 16 && dim / (2 * most) >= 256) most *= 2;
+    const int part_threads = 32 + std::min(ctx->block - 32, std::max(256, dim / most));
+    const int cs = fx_cluster_prepare(dim, most, part_threads);
+    if (cs > 0) {
+      ctx->cluster_fx = true;
+      ctx->grid = cs;
+      ctx->small_block = 32 + std::min(ctx->block - 32, std::max(256, dim / cs));
     }
   }
   if (ctx->precision == CFET_PREC_FX)  // basis q_1..q_{m_max+1}; the Chebyshev kernel's three vectors

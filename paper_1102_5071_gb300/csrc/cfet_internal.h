@@ -208,6 +208,7 @@ struct PropParams {
   int tiled;             // spin chains: window-tiled apply (complex64 and fixed-point kernels)
   int reorth;            // FP64 kernel: full re-orthogonalisation of every Lanczos vector
   int small;             // fixed-point kernel, one CTA: the Krylov basis lives in shared memory
+  int cluster;           // fixed-point spin kernel: the grid is one thread-block cluster
   // decisions (device arrays, nullable)
   const int* f_nsub; const int* f_k; const int* f_h;
   int* r_nsub; int* r_k; int* r_h; long long r_cap;
@@ -315,6 +316,9 @@ int max_coresident_blocks_fx(int family, int block, bool tiled);
 constexpr size_t kFxSmallSmemMax = 200 * 1024;
 size_t fx_small_smem_bytes(int dim, int m_max);
 int fx_small_prepare(size_t bytes);
+constexpr int kFxClusterMaxSites = 13;
+size_t fx_cluster_smem_bytes(int part);
+int fx_cluster_prepare(int dim, int most, int block);
 int launch_propagate_spin_c64(const PropParams& p, const OpSpinC& op, int grid, int block, void* stream);
 int launch_propagate_dia_c64(const PropParams& p, const OpDiaC& op, int grid, int block, void* stream);
 int launch_propagate_csr_c64(const PropParams& p, const OpCsrC& op, int grid, int block, void* stream);

@@ -11,6 +11,7 @@
 #include <cstdint>
 
 #include "cfet_internal.h"
+#include "device_common.cuh"
 #include "scalar_bounds.cuh"
 
 namespace cfet {
@@ -213,6 +214,78 @@ __device__ __forceinline__ longlong2 fx_apply_spin(const longlong2* q, const lon
     const longlong2 w = qm[x];
     ur += fx_mulhi(c.m_p, w.x << c.pp);
     ui += fx_mulhi(c.m_p, w.y << c.pp);
+  }
+  return make_longlong2(ur, ui);
+}
+
+// One element of a chain whose applied vector is staged in the shared memory of
+// the cluster's CTAs, 2^lc elements each (x = rank 2^lc + j): flips and hops of
+// bits below lc read this CTA's part, those of the rank's bits the same (or, for
+// the bond across, a neighbouring) element of another CTA's part.
+__device__ __forceinline__ longlong2 fx_ld_cluster(unsigned base, int j) {
+  longlong2 v;
+  asm volatile("ld.shared::cluster.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(base + 16u * (unsigned)j));
+  return v;
+}
+__device__ __forceinline__ longlong2 fx_apply_spin_cluster(const longlong2* sq, const longlong2* qm, int j, int rank,
+                                                           int lc, const OpSpinFx& op, const FxConstA& c,
+                                                           const long long* mb, longlong2& v) {
+  const int N = op.N, L = op.lo_bits;
+  const int x = (rank << lc) | j;
+  longlong2 wp = make_longlong2(0, 0);
+  if (c.use_prev) wp = qm[x];  // global memory: issued ahead of the neighbour sums
+  const long long dz = __ldg(op.DZ_lo + (x & ((1 << L) - 1))) + __ldg(op.DZ_hi + (x >> (L - 1)));
+  v = sq[j];
+  long long hr = 0, hi = 0;
+  const unsigned anti = ((unsigned)x ^ ((unsigned)x >> 1)) & ((1u << (N - 1)) - 1u);
+  for (int i = lc - 1; i < N - 1; ++i)
+    if ((anti >> i) & 1u) {  // bond across (i = lc - 1) and bonds of the rank's bits
+      const unsigned other = i == lc - 1 ? 1u : 3u << (i - lc);
+      const longlong2 w = fx_ld_cluster(cluster_addr(sq, (unsigned)rank ^ other), i == lc - 1 ? j ^ (1 << i) : j);
+      hr += w.x;
+      hi += w.y;
+    }
+#pragma unroll 4
+  for (int i = 0; i < lc - 1; ++i)
+    if ((anti >> i) & 1u) {
+      const longlong2 w = sq[j ^ (3 << i)];
+      hr += w.x;
+      hi += w.y;
+    }
+  const long long Dp = fx_mulhi(c.m_cz, dz << 1) << 3;
+  long long ur = fx_mulhi(Dp, v.x << c.pk) + fx_mulhi(c.m_hop, hr << c.ph);
+  long long ui = fx_mulhi(Dp, v.y << c.pk) + fx_mulhi(c.m_hop, hi << c.ph);
+  if (op.uniform) {
+    long long xr = 0, xi = 0;
+    for (int i = lc; i < N; ++i) {
+      const longlong2 w = fx_ld_cluster(cluster_addr(sq, (unsigned)rank ^ (1u << (i - lc))), j);
+      xr += w.x;
+      xi += w.y;
+    }
+#pragma unroll 4
+    for (int i = 0; i < lc; ++i) {
+      const longlong2 w = sq[j ^ (1 << i)];
+      xr += w.x;
+      xi += w.y;
+    }
+    ur += fx_mulhi(c.m_x, xr << c.px);
+    ui += fx_mulhi(c.m_x, xi << c.px);
+  } else {
+    for (int i = lc; i < N; ++i) {
+      const longlong2 w = fx_ld_cluster(cluster_addr(sq, (unsigned)rank ^ (1u << (i - lc))), j);
+      ur += fx_mulhi(mb[i], w.x << c.pk);
+      ui += fx_mulhi(mb[i], w.y << c.pk);
+    }
+#pragma unroll 4
+    for (int i = 0; i < lc; ++i) {
+      const longlong2 w = sq[j ^ (1 << i)];
+      ur += fx_mulhi(mb[i], w.x << c.pk);
+      ui += fx_mulhi(mb[i], w.y << c.pk);
+    }
+  }
+  if (c.use_prev) {
+    ur += fx_mulhi(c.m_p, wp.x << c.pp);
+    ui += fx_mulhi(c.m_p, wp.y << c.pp);
   }
   return make_longlong2(ur, ui);
 }

@@ -49,6 +49,15 @@
 
 namespace cfet {
 
+// Forms of the kernel (separate instantiations, so that none carries the code of
+// the others and the vectors keep their address space).
+enum FxMode {
+  kFxGrid = 0,     // element-wise, vectors in global memory, exchange through L2
+  kFxTiled = 1,    // long spin chains: window-tiled apply
+  kFxSmall = 2,    // one CTA with the Krylov basis in shared memory
+  kFxCluster = 3,  // spin chains on one thread-block cluster, applied vector in its shared memory
+};
+
 // ------------------------------------------------------------------ shared state
 struct SmemFx {
   // per-warp partials of the workers
@@ -134,8 +143,9 @@ struct FxAcc {
 
 // Control warp: combine the workers' per-warp partials into this CTA's record,
 // exchange records with every CTA (the grid barrier), and return the exact
-// global sum (as FP64) and the global max to all lanes.  ONE: the only CTA.
-template <bool ONE>
+// global sum (as FP64) and the global max to all lanes (FxMode; kFxCluster: part
+// is the cluster's exchange slots in shared memory).
+template <int MODE>
 __device__ __forceinline__ bool fx_ctl_reduce(SmemFx& S, int NW, unsigned long long* part, unsigned tag, bool fence, int* status,
                               long long timeout_ns, double& sum, long long& mxi, long long& spin) {
   const int lane = threadIdx.x & 31;
@@ -143,7 +153,7 @@ __device__ __forceinline__ bool fx_ctl_reduce(SmemFx& S, int NW, unsigned long l
   long long hi = 0, m = 0;
   if (lane < NW) { lo = S.wlo[lane]; hi = S.whi[lane]; m = S.wmx[lane]; }
   fx_warp_reduce(lo, hi, m);
-  if constexpr (ONE) {
+  if constexpr (MODE == kFxSmall) {
     sum = fx_i128_to_double(lo, hi);
     mxi = m;
     return true;
@@ -152,7 +162,11 @@ __device__ __forceinline__ bool fx_ctl_reduce(SmemFx& S, int NW, unsigned long l
                             (unsigned)((unsigned long long)hi >> 32), (unsigned)m,
                             (unsigned)((unsigned long long)m >> 32)};
   FxAcc acc;
-  if (!ctl_exchange<6>(part, mine, tag, fence, status, timeout_ns, spin, acc)) return false;
+  if constexpr (MODE == kFxCluster) {
+    if (!cluster_exchange<6>(part, mine, tag, status, timeout_ns, spin, acc)) return false;
+  } else {
+    if (!ctl_exchange<6>(part, mine, tag, fence, status, timeout_ns, spin, acc)) return false;
+  }
   lo = acc.lo;
   hi = acc.hi;
   m = acc.m;
@@ -164,12 +178,12 @@ __device__ __forceinline__ bool fx_ctl_reduce(SmemFx& S, int NW, unsigned long l
 
 // The same out of line, for the passes that run once per launch or substep:
 // results in S.rsum and S.rmx.
-template <bool ONE>
+template <int MODE>
 __device__ __noinline__ bool fx_ctl_reduce_cold(SmemFx& S, int NW, unsigned long long* part, unsigned tag, int* status,
                                                 long long timeout_ns) {
   double sum;
   long long mxi;
-  const bool ok = fx_ctl_reduce<ONE>(S, NW, part, tag, true, status, timeout_ns, sum, mxi, S.tacc[5]);
+  const bool ok = fx_ctl_reduce<MODE>(S, NW, part, tag, true, status, timeout_ns, sum, mxi, S.tacc[5]);
   if (ok && (threadIdx.x & 31) == 0) {
     S.rsum = sum;
     S.rmx = mxi;
@@ -566,13 +580,10 @@ enum FxCmd { kFxExit = 0, kFxMax, kFxConvert, kFxApply, kFxOrth, kFxRec };
 
 __device__ __forceinline__ void fx_cta_sync() { __syncthreads(); }  // by workers and control warp, each from its loop
 
-// TILED: the window-tiled apply of long spin chains (a separate instantiation,
-// so that the element-wise kernel carries none of its code).  SMALL: one CTA
-// with the Krylov basis in shared memory (separate too, so that the other
-// instantiations keep global-memory loads for the vectors).
-template <int FAMILY, class Op, bool TILED, bool SMALL>
+template <int FAMILY, class Op, int MODE>
 __device__ __forceinline__ void fx_worker(const PropParams& p, const Op& op, SmemFx& S, unsigned char* tiles_base,
                                           int wstep) {
+  constexpr bool TILED = MODE == kFxTiled, SMALL = MODE == kFxSmall, CLUSTER = MODE == kFxCluster;
   const int tid = threadIdx.x;
   const int dim = p.dim;
   // each CTA walks one contiguous chunk of the vectors, so that the
@@ -589,6 +600,9 @@ __device__ __forceinline__ void fx_worker(const PropParams& p, const Op& op, Sme
   // one-CTA launches of small problems keep the basis in shared memory
   longlong2* const qb = SMALL ? reinterpret_cast<longlong2*>(tiles_base) : p.qbasis;
   auto Q = [&](int i) -> longlong2* { return qb + (size_t)(i - 1) * dim; };
+  // kFxCluster: this CTA's part of the applied vector, behind the exchange slots
+  longlong2* const sq = reinterpret_cast<longlong2*>(tiles_base + kClusterSlotWords * 8);
+  const int xb = wx0 - tid;
   TileWin win[kTiledMaxWindows] = {};
   int nwin = 1;
   if constexpr (TILED) nwin = tiled_windows<kFxTileBits>(op.N, win);
@@ -631,6 +645,15 @@ __device__ __forceinline__ void fx_worker(const PropParams& p, const Op& op, Sme
             window_written_sync();    // all threads: window w written
             window_exchanged_sync();  // all threads: the grid exchange passed
           }
+        }
+      } else if constexpr (CLUSTER) {
+        const int lc = 31 - __clz(wxe - xb), rank = blockIdx.x;
+        for (; x < wxe; x += wstep) {
+          longlong2 v;
+          const longlong2 hv = fx_apply_spin_cluster(sq, qm, x - xb, rank, lc, op, c, S.mb, v);
+          u[x] = hv;
+          a2 += (__int128)v.x * hv.x + (__int128)v.y * hv.y;
+          mx = max(mx, fx_absmax(hv.x, hv.y));
         }
       } else {
         if constexpr (FAMILY == kFamilySpin) {
@@ -695,6 +718,10 @@ __device__ __forceinline__ void fx_worker(const PropParams& p, const Op& op, Sme
         const long long wi1 = fx_rshr(u1.y, sh_u) + fx_mulhi(m_a, v1.y << pk);
         u[x] = make_longlong2(wr0, wi0);
         u[x + wstep] = make_longlong2(wr1, wi1);
+        if constexpr (CLUSTER) {
+          sq[x - xb] = make_longlong2(wr0, wi0);
+          sq[x + wstep - xb] = make_longlong2(wr1, wi1);
+        }
         b2 += (__int128)wr0 * wr0 + (__int128)wi0 * wi0;
         b2 += (__int128)wr1 * wr1 + (__int128)wi1 * wi1;
         mx = max(mx, max(fx_absmax(wr0, wi0), fx_absmax(wr1, wi1)));
@@ -705,6 +732,7 @@ __device__ __forceinline__ void fx_worker(const PropParams& p, const Op& op, Sme
         const long long wr = fx_rshr(uu.x, sh_u) + fx_mulhi(m_a, v.x << pk);
         const long long wi = fx_rshr(uu.y, sh_u) + fx_mulhi(m_a, v.y << pk);
         u[x] = make_longlong2(wr, wi);
+        if constexpr (CLUSTER) sq[x - xb] = make_longlong2(wr, wi);
         b2 += (__int128)wr * wr + (__int128)wi * wi;
         mx = max(mx, fx_absmax(wr, wi));
       }
@@ -740,6 +768,7 @@ __device__ __forceinline__ void fx_worker(const PropParams& p, const Op& op, Sme
         }
         for (; i < acc_k; ++i) term(i, Q(i + 1)[x], re, im);
         Q(1)[x] = make_longlong2(re, im);
+        if constexpr (CLUSTER) sq[x - xb] = make_longlong2(re, im);
         if (final_rec) p.psi[x] = make_double2(__ll2double_rn(re) * outscale, __ll2double_rn(im) * outscale);
         a2 += (__int128)re * re + (__int128)im * im;
         mx = max(mx, fx_absmax(re, im));
@@ -765,6 +794,7 @@ __device__ __forceinline__ void fx_worker(const PropParams& p, const Op& op, Sme
         const double2 v = p.psi[x];
         const longlong2 qv = make_longlong2(__double2ll_rn(v.x * sc), __double2ll_rn(v.y * sc));
         Q(1)[x] = qv;
+        if constexpr (CLUSTER) sq[x - xb] = qv;
         a2 += (__int128)qv.x * qv.x + (__int128)qv.y * qv.y;
         mx = max(mx, fx_absmax(qv.x, qv.y));
       }
@@ -828,15 +858,19 @@ __device__ __noinline__ int fx_check(SmemFx& S, int it, double tol, double tau, 
   return acc;
 }
 
-template <int FAMILY, class Op, bool TILED, bool SMALL>
-__device__ __forceinline__ void fx_control(const PropParams& p, const Op& op, SmemFx& S, int NW) {
+template <int FAMILY, class Op, int MODE>
+__device__ __forceinline__ void fx_control(const PropParams& p, const Op& op, SmemFx& S, unsigned char* tiles_base,
+                                           int NW) {
+  constexpr bool TILED = MODE == kFxTiled;
   const int lane = threadIdx.x & 31;
   const int G = gridDim.x;
   const int ncoef = 1 + p.nV;
   // record exchange (ctl_exchange): tags continue across launches
   DevStatus* const st = p.st;
-  unsigned tag = (unsigned)ld_volatile_i32((const int*)&st->tag_base);
-  unsigned long long* const rec = reinterpret_cast<unsigned long long*>(p.partials);
+  // (kFxCluster: the launch's own slots in shared memory, tags from 1)
+  unsigned tag = MODE == kFxCluster ? 0u : (unsigned)ld_volatile_i32((const int*)&st->tag_base);
+  unsigned long long* const rec =
+      reinterpret_cast<unsigned long long*>(MODE == kFxCluster ? (void*)tiles_base : (void*)p.partials);
   const bool glead = blockIdx.x == 0 && lane == 0;
   const bool fixed_k = p.tol <= 0.0;
   const bool forced = p.f_nsub != nullptr;
@@ -864,7 +898,7 @@ __device__ __forceinline__ void fx_control(const PropParams& p, const Op& op, Sm
   // ---------------- psi (complex128) -> q_1
   start(kFxMax, 0);
   fx_cta_sync();
-  if (!fx_ctl_reduce_cold<SMALL>(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
+  if (!fx_ctl_reduce_cold<MODE>(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
   if (S.rmx >= 0x7FF0000000000000LL) {
     if (lane == 0) atomicCAS(&st->status, 0, (int)CFET_ENAN);
     return;
@@ -872,7 +906,7 @@ __device__ __forceinline__ void fx_control(const PropParams& p, const Op& op, Sm
   if (lane == 0) S.E[1] = fx_exp_for(__longlong_as_double(S.rmx), kFxBits);
   start(kFxConvert, 0);
   fx_cta_sync();
-  if (!fx_ctl_reduce_cold<SMALL>(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
+  if (!fx_ctl_reduce_cold<MODE>(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
   if (lane == 0) {
     S.nsum = S.rsum;
     S.A[1] = S.rmx;
@@ -943,7 +977,7 @@ __device__ __forceinline__ void fx_control(const PropParams& p, const Op& op, Sm
           {
             const long long sp0 = S.tacc[5];
             // (the tiled apply leaves u written by other CTAs: fence)
-            if (!fx_ctl_reduce<SMALL>(S, NW, rec, ++tag, TILED, &st->status, p.timeout_ns, sum, mxi, S.tacc[5]))
+            if (!fx_ctl_reduce<MODE>(S, NW, rec, ++tag, TILED, &st->status, p.timeout_ns, sum, mxi, S.tacc[5]))
               return;
             if (stop_prev) {  // the deferred check accepted it-1
               it -= 1;
@@ -980,7 +1014,7 @@ __device__ __forceinline__ void fx_control(const PropParams& p, const Op& op, Sm
           fx_cta_sync();
           {
             const long long sp0 = S.tacc[5];
-            if (!fx_ctl_reduce<SMALL>(S, NW, rec, ++tag, true, &st->status, p.timeout_ns, sum, mxi,
+            if (!fx_ctl_reduce<MODE>(S, NW, rec, ++tag, true, &st->status, p.timeout_ns, sum, mxi,
                                       S.tacc[5]))
               return;
             if (lane == 0) {
@@ -1041,7 +1075,7 @@ __device__ __forceinline__ void fx_control(const PropParams& p, const Op& op, Sm
         }
         start(kFxRec, acc_k);
         fx_cta_sync();
-        if (!fx_ctl_reduce_cold<SMALL>(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
+        if (!fx_ctl_reduce_cold<MODE>(S, NW, rec, ++tag, &st->status, p.timeout_ns)) return;
         if (lane == 0) {
           S.nsum = S.rsum;
           S.E[1] = S.Epsi;
@@ -1075,7 +1109,7 @@ __device__ __forceinline__ void fx_control(const PropParams& p, const Op& op, Sm
     __syncwarp();
   }
   if (glead) {
-    st->tag_base = tag;
+    if (MODE != kFxCluster) st->tag_base = tag;
     st->forced_pos = S.fpos;
     st->rec_pos = S.rpos;
     st->n_exp += p.nexp;
@@ -1091,50 +1125,76 @@ __device__ __forceinline__ void fx_control(const PropParams& p, const Op& op, Sm
   }
 }
 
-template <int FAMILY, class Op, bool TILED = false, bool SMALL = false>
+template <int FAMILY, class Op, int MODE>
 __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_fx(PropParams p, Op op) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmemFx& S = *reinterpret_cast<SmemFx*>(smem_raw);
   const int NW = (int)(blockDim.x >> 5) - 1;  // worker warps
-  // behind SmemFx: the shared-memory basis of one-CTA launches, or the tiled
-  // apply's stage mbarriers (128 bytes) and tile buffers
+  // behind SmemFx: the shared-memory basis of one-CTA launches, the tiled
+  // apply's stage mbarriers (128 bytes) and tile buffers, or a cluster's
+  // exchange slots and part of the applied vector
   unsigned char* const tiles_base = smem_raw + ((sizeof(SmemFx) + 127) & ~size_t(127));
-  if constexpr (TILED) {
+  if constexpr (MODE == kFxTiled) {
     if (threadIdx.x == 0) {  // ordered before any use by the CTA barriers of the conversion pass
       for (int s2 = 0; s2 < kTmaStages; ++s2) mbar_init(reinterpret_cast<unsigned long long*>(tiles_base) + s2, 1);
       S.tma_fail = 0;
       mbar_init_fence();
     }
   }
+  if constexpr (MODE == kFxCluster) {
+    for (int i = threadIdx.x; i < kClusterSlotWords; i += blockDim.x)
+      reinterpret_cast<unsigned long long*>(tiles_base)[i] = 0;
+    __syncwarp();
+    cluster_sync_all();  // every CTA runs, with its slots cleared
+  }
   if ((int)(threadIdx.x >> 5) < NW) {
-    fx_worker<FAMILY, Op, TILED, SMALL>(p, op, S, tiles_base, NW * 32);
+    fx_worker<FAMILY, Op, MODE>(p, op, S, tiles_base, NW * 32);
   } else {
-    fx_control<FAMILY, Op, TILED, SMALL>(p, op, S, NW);
+    fx_control<FAMILY, Op, MODE>(p, op, S, tiles_base, NW);
     __syncwarp();
     if ((threadIdx.x & 31) == 0) S.cmd = kFxExit;  // also after an error
     __syncwarp();
     fx_cta_sync();
   }
+  if constexpr (MODE == kFxCluster) {
+    __syncwarp();
+    cluster_sync_all();  // no CTA leaves while another may access its shared memory
+  }
 }
 
 // ------------------------------------------------------------------ launchers
+size_t fx_cluster_smem_bytes(int part) {
+  return ((sizeof(SmemFx) + 127) & ~size_t(127)) + kClusterSlotWords * 8 + (size_t)part * sizeof(longlong2);
+}
+
 template <int FAMILY, class Op>
 static int launch_prop_fx(const PropParams& p, const Op& op, int grid, int block, void* stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = p.tiled ? fx_tiled_smem_bytes() : p.small ? fx_small_smem_bytes(p.dim, p.m_max) : sizeof(SmemFx);
+  cfg.dynamicSmemBytes = p.tiled     ? fx_tiled_smem_bytes()
+                         : p.small   ? fx_small_smem_bytes(p.dim, p.m_max)
+                         : p.cluster ? fx_cluster_smem_bytes(p.dim / grid)
+                                     : sizeof(SmemFx);
   cfg.stream = (cudaStream_t)stream;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeCooperative;
-  at[0].val.cooperative = 1;
+  if (p.cluster) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = grid;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if constexpr (FAMILY == kFamilySpin) {
-    if (p.tiled) return (int)cudaLaunchKernelEx(&cfg, k_propagate_fx<FAMILY, Op, true>, p, op);
+    if (p.tiled) return (int)cudaLaunchKernelEx(&cfg, k_propagate_fx<FAMILY, Op, kFxTiled>, p, op);
+    if (p.cluster) return (int)cudaLaunchKernelEx(&cfg, k_propagate_fx<FAMILY, Op, kFxCluster>, p, op);
   }
-  if (p.small) return (int)cudaLaunchKernelEx(&cfg, k_propagate_fx<FAMILY, Op, false, true>, p, op);
-  return (int)cudaLaunchKernelEx(&cfg, k_propagate_fx<FAMILY, Op>, p, op);
+  if (p.small) return (int)cudaLaunchKernelEx(&cfg, k_propagate_fx<FAMILY, Op, kFxSmall>, p, op);
+  return (int)cudaLaunchKernelEx(&cfg, k_propagate_fx<FAMILY, Op, kFxGrid>, p, op);
 }
 
 int launch_propagate_spin_fx(const PropParams& p, const OpSpinFx& op, int grid, int block, void* stream) {
@@ -1159,15 +1219,45 @@ size_t fx_small_smem_bytes(int dim, int m_max) {
 }
 
 int fx_small_prepare(size_t bytes) {
-  cudaError_t e = cudaFuncSetAttribute(k_propagate_fx<kFamilySpin, OpSpinFx, false, true>,
+  cudaError_t e = cudaFuncSetAttribute(k_propagate_fx<kFamilySpin, OpSpinFx, kFxSmall>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_propagate_fx<kFamilyDia, OpDiaFx, false, true>,
+    e = cudaFuncSetAttribute(k_propagate_fx<kFamilyDia, OpDiaFx, kFxSmall>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_propagate_fx<kFamilyCsr, OpCsrFx, false, true>,
+    e = cudaFuncSetAttribute(k_propagate_fx<kFamilyCsr, OpCsrFx, kFxSmall>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   return (int)e;
+}
+
+// Largest cluster of at most `most` CTAs (a power of two) of `block` threads that
+// holds a vector of dim elements in its shared memory; 0 when there is none.
+int fx_cluster_prepare(int dim, int most, int block) {
+  const void* k = (const void*)k_propagate_fx<kFamilySpin, OpSpinFx, kFxCluster>;
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
+  for (int cs = most; cs >= 2; cs /= 2) {
+    const size_t bytes = fx_cluster_smem_bytes(dim / cs);
+    if (bytes > kFxSmallSmemMax) return 0;  // smaller clusters need more
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cs);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = bytes;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cs;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n >= 1) return cs;
+    cudaGetLastError();
+  }
+  return 0;
 }
 
 int max_coresident_blocks_fx(int family, int block, bool tiled) {
@@ -1177,21 +1267,21 @@ int max_coresident_blocks_fx(int family, int block, bool tiled) {
   // the element-wise kernel needs only a few KB of shared memory: leave the
   // rest of the unified L1/shared storage to L1, which holds each CTA's chunk
   // (a tiled launch asks for its tile buffers and gets the split it needs)
-  cudaFuncSetAttribute(k_propagate_fx<kFamilySpin, OpSpinFx>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-  cudaFuncSetAttribute(k_propagate_fx<kFamilyDia, OpDiaFx>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-  cudaFuncSetAttribute(k_propagate_fx<kFamilyCsr, OpCsrFx>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-  cudaFuncSetAttribute(k_propagate_fx<kFamilySpin, OpSpinFx, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_propagate_fx<kFamilySpin, OpSpinFx, kFxGrid>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+  cudaFuncSetAttribute(k_propagate_fx<kFamilyDia, OpDiaFx, kFxGrid>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+  cudaFuncSetAttribute(k_propagate_fx<kFamilyCsr, OpCsrFx, kFxGrid>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+  cudaFuncSetAttribute(k_propagate_fx<kFamilySpin, OpSpinFx, kFxTiled>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)fx_tiled_smem_bytes());
   cudaError_t e;
   if (family == kFamilySpin)
-    e = tiled ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_fx<kFamilySpin, OpSpinFx, true>, block,
+    e = tiled ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_fx<kFamilySpin, OpSpinFx, kFxTiled>, block,
                                                               fx_tiled_smem_bytes())
-              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_fx<kFamilySpin, OpSpinFx>, block, sizeof(SmemFx));
+              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_fx<kFamilySpin, OpSpinFx, kFxGrid>, block, sizeof(SmemFx));
   else if (family == kFamilyCsr)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_fx<kFamilyCsr, OpCsrFx>, block,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_fx<kFamilyCsr, OpCsrFx, kFxGrid>, block,
                                                       sizeof(SmemFx));
   else
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_fx<kFamilyDia, OpDiaFx>, block,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_fx<kFamilyDia, OpDiaFx, kFxGrid>, block,
                                                       sizeof(SmemFx));
   if (e != cudaSuccess) return -1;
   return per * nsm;
