@@ -667,17 +667,18 @@ cfet_status csr_upload(cfet_ctx* ctx, const cfet_op* H0, int nV, const cfet_op* 
   fx.VR = reinterpret_cast<const long long*>(b + o_VR);
   fx.VI = cplx ? reinterpret_cast<const long long*>(b + o_VI) : nullptr;
   ctx->csr_c = OpCsrC{nops, d_rp, d_col, reinterpret_cast<const float*>(b + o_v32),
-                      cplx ? reinterpret_cast<const float*>(b + o_i32) : nullptr, nullptr, 0};
+                      cplx ? reinterpret_cast<const float*>(b + o_i32) : nullptr, nullptr};
   fx.rb = nullptr;
-  // threads per row of the fixed-point and complex64 applies
+  // threads per row of the fixed-point apply (its sums are exact; the complex64
+  // sums keep one thread per row and the order of the entries)
   // eight or more entries of a row of one operator per thread (mean over the
   // rows): with 10 entries two threads a row take 35.2 us per Lanczos iteration
   // of 60 001 rows, one 46.5, four 36.2 and eight 47.7
   const double per = (double)nnz / ((double)dim * nops);
   int lb = 0;
   while (lb < 4 && per >= 8.0 * (1 << lb)) ++lb;
-  fx.cplx = ctx->csr_c.cplx = cplx;
-  fx.lane_bits = ctx->csr_c.lane_bits = lb;
+  fx.cplx = cplx;
+  fx.lane_bits = lb;
   ctx->csr_rp.swap(rp);
   return CFET_OK;
 }
@@ -1236,7 +1237,7 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
   }
   // element threads per CTA (the fixed-point kernel adds one control warp)
   const int workers = ctl_warp ? ctx->block - 32 : ctx->block;
-  int lane_bits = ctl_warp && family == kFamilyCsr ? ctx->csr_fx.lane_bits : 0;  // 2^lane_bits threads per element
+  int lane_bits = ctx->precision == CFET_PREC_FX && family == kFamilyCsr ? ctx->csr_fx.lane_bits : 0;  // 2^lane_bits threads per element
   int want = (dim + workers - 1) / workers;
   if (want > 1) want = (int)std::min((((long long)dim << lane_bits) + workers - 1) / workers, 1LL << 30);
   if (o.grid_size > 0) want = o.grid_size;
@@ -1291,7 +1292,7 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
     // exact sums: a thread takes at most 4096 rows
     auto cap = [&] { return (4096LL * workers >> lane_bits) * (ctx->precision == CFET_PREC_FX ? 1 : 1 << 20); };
     while (lane_bits > 0 && cap() * ctx->grid < dim) --lane_bits;
-    ctx->csr_fx.lane_bits = ctx->csr_c.lane_bits = lane_bits;
+    ctx->csr_fx.lane_bits = lane_bits;
     const std::vector<int> rb = csr_row_split(ctx->csr_rp, 1 + nV, dim, ctx->grid, cap());
     CKC(cudaMalloc(&ctx->d_csr_rb, rb.size() * sizeof(int)), "cudaMalloc(row split)");
     CKC(cudaMemcpy(ctx->d_csr_rb, rb.data(), rb.size() * sizeof(int), cudaMemcpyHostToDevice), "upload row split");

@@ -191,8 +191,6 @@ struct OpCsrC {
   const float* vr;
   const float* vi;        // NULL for real operators
   const int* rb;          // as OpCsrFx
-  int lane_bits;
-  unsigned cplx;
 };
 
 struct PropParams {

@@ -262,42 +262,33 @@ __device__ __forceinline__ float2 c_apply_dia(const float2* __restrict__ q, cons
 }
 
 // CSR: per operator the row's sum of val * q in FP32 (complex values of
-// Hermitian operators), then the operator's scalar.  2^op.lane_bits
-// neighbouring threads share the row as in fx_apply_csr: each sums every
-// 2^lane_bits-th entry, the partial sums are added by shuffles.
+// Hermitian operators) in the order of the entries, then the operator's scalar.
 __device__ __forceinline__ float2 c_apply_csr(const float2* __restrict__ q, const float2* __restrict__ qm, int r,
-                                              bool on, int dim, const OpCsrC& op, const CConst& c) {
-  const int T = 1 << op.lane_bits, sub = threadIdx.x & (T - 1);
+                                              int dim, const OpCsrC& op, const CConst& c) {
   float ur = 0.f, ui = 0.f;
   for (int o = 0; o < op.nops; ++o) {
     const int* rp = op.rp + (size_t)o * (dim + 1);
-    const int e0 = on ? __ldg(rp + r) + sub : 0, e1 = on ? __ldg(rp + r + 1) : 0;
+    const int e0 = __ldg(rp + r), e1 = __ldg(rp + r + 1);
     float ar = 0.f, ai = 0.f;
-    if ((op.cplx >> o) & 1u) {
-#pragma unroll 2
-      for (int e = e0; e < e1; e += T) {
+    if (op.vi) {
+      for (int e = e0; e < e1; ++e) {
         const float a = __ldg(op.vr + e), b = __ldg(op.vi + e);
         const float2 w = q[__ldg(op.col + e)];
         ar = fmaf(a, w.x, fmaf(-b, w.y, ar));
         ai = fmaf(a, w.y, fmaf(b, w.x, ai));
       }
     } else {
-#pragma unroll 2
-      for (int e = e0; e < e1; e += T) {
+      for (int e = e0; e < e1; ++e) {
         const float a = __ldg(op.vr + e);
         const float2 w = q[__ldg(op.col + e)];
         ar = fmaf(a, w.x, ar);
         ai = fmaf(a, w.y, ai);
       }
     }
-    for (int b = 0; b < op.lane_bits; ++b) {
-      ar += __shfl_xor_sync(0xffffffffu, ar, 1 << b);
-      ai += __shfl_xor_sync(0xffffffffu, ai, 1 << b);
-    }
     ur = fmaf(c.co[o], ar, ur);
     ui = fmaf(c.co[o], ai, ui);
   }
-  if (c.use_prev && on && sub == 0) {
+  if (c.use_prev) {
     const float2 w = qm[r];
     ur = fmaf(c.cp, w.x, ur);
     ui = fmaf(c.cp, w.y, ui);
@@ -827,33 +818,17 @@ __device__ __forceinline__ void c_worker(const PropParams& p, const Op& op, Smem
             ff_add_prod(s1, c1, h2.y, h2.y);
           }
         }
-        if constexpr (FAMILY == kFamilyCsr) {
-          const int lb = op.lane_bits;
-          for (int r0 = wx0 - tid; r0 < wxe; r0 += wstep >> lb) {
-            const int r = r0 + (tid >> lb);
-            const bool on = r < wxe;
-            const float2 hv = c_apply_csr(q, qm, r, on, dim, op, c);
-            if (on && (tid & ((1 << lb) - 1)) == 0) {
-              u[r] = hv;
-              const float2 v = q[r];
-              ff_add_prod(s0, c0, v.x, hv.x);
-              ff_add_prod(s0, c0, v.y, hv.y);
-              ff_add_prod(s1, c1, hv.x, hv.x);
-              ff_add_prod(s1, c1, hv.y, hv.y);
-            }
-          }
-        } else {
-          for (; x < wxe; x += wstep) {
-            float2 hv;
-            if constexpr (FAMILY == kFamilySpin) hv = c_apply_spin(q, qm, x, op, c, S.bx);
-            else hv = c_apply_dia(q, qm, x, dim, op, c);
-            u[x] = hv;
-            const float2 v = q[x];
-            ff_add_prod(s0, c0, v.x, hv.x);
-            ff_add_prod(s0, c0, v.y, hv.y);
-            ff_add_prod(s1, c1, hv.x, hv.x);
-            ff_add_prod(s1, c1, hv.y, hv.y);
-          }
+        for (; x < wxe; x += wstep) {
+          float2 hv;
+          if constexpr (FAMILY == kFamilySpin) hv = c_apply_spin(q, qm, x, op, c, S.bx);
+          else if constexpr (FAMILY == kFamilyDia) hv = c_apply_dia(q, qm, x, dim, op, c);
+          else hv = c_apply_csr(q, qm, x, dim, op, c);
+          u[x] = hv;
+          const float2 v = q[x];
+          ff_add_prod(s0, c0, v.x, hv.x);
+          ff_add_prod(s0, c0, v.y, hv.y);
+          ff_add_prod(s1, c1, hv.x, hv.x);
+          ff_add_prod(s1, c1, hv.y, hv.y);
         }
       }
       c_worker_partial(S, s0, c0, 0);
