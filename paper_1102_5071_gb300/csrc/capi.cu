@@ -47,6 +47,7 @@ struct cfet_ctx {
   bool small_fx = false;
   int small_block = 0;
   bool cluster_fx = false;  // fixed-point chains of middle size: the grid is one cluster
+  int cluster = 0;          // CTAs per cluster (0: none)
   int precision = CFET_PREC_FX;
   std::string err;
   // drives
@@ -336,7 +337,7 @@ PropParams base_params(cfet_ctx* ctx, double2* psi, double tau, double tol) {
   p.tmaps = ctx->d_tmaps;
   p.reorth = ctx->opt.reorth;
   p.small = ctx->small_fx ? 1 : 0;
-  p.cluster = ctx->cluster_fx ? 1 : 0;
+  p.cluster = ctx->cluster;
   return p;
 }
 
@@ -1262,9 +1263,16 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
     const int cs = fx_cluster_prepare(dim, most, part_threads);
     if (cs > 0) {
       ctx->cluster_fx = true;
-      ctx->grid = cs;
+      ctx->grid = ctx->cluster = cs;
       ctx->small_block = 32 + std::min(ctx->block - 32, std::max(256, dim / cs));
     }
+  }
+  // complex64 chains staged in the shared memory of all CTAs
+  if (family == kFamilySpin && ctx->precision == CFET_PREC_C64 && !ctx->tiled && o.grid_size == 0 &&
+      o.apply_form == CFET_APPLY_AUTO && nsites >= kC64StagedMinSites && nsites <= kC64StagedMaxSites &&
+      ctx->grid >= kStagedGrid && c64_staged_prepare(dim, ctx->block)) {
+    ctx->cluster = kStagedCluster;
+    ctx->grid = kStagedGrid;
   }
   if (ctx->precision == CFET_PREC_FX)  // basis q_1..q_{m_max+1}; the Chebyshev kernel's three vectors
     CKC(cudaMalloc(&ctx->d_qbasis, (size_t)std::max(o.m_max + 1, 3) * dim * sizeof(longlong2)),

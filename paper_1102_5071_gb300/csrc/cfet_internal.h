@@ -206,7 +206,7 @@ struct PropParams {
   int tiled;             // spin chains: window-tiled apply (complex64 and fixed-point kernels)
   int reorth;            // FP64 kernel: full re-orthogonalisation of every Lanczos vector
   int small;             // fixed-point kernel, one CTA: the Krylov basis lives in shared memory
-  int cluster;           // fixed-point spin kernel: the grid is one thread-block cluster
+  int cluster;           // spin kernels: CTAs per thread-block cluster (fixed point: the whole grid; 0: none)
   // decisions (device arrays, nullable)
   const int* f_nsub; const int* f_k; const int* f_h;
   int* r_nsub; int* r_k; int* r_h; long long r_cap;
@@ -317,6 +317,12 @@ int fx_small_prepare(size_t bytes);
 constexpr int kFxClusterMaxSites = 13;
 size_t fx_cluster_smem_bytes(int part);
 int fx_cluster_prepare(int dim, int most, int block);
+bool staged_fits(const void* kernel, int grid, int cs, int block, size_t bytes);
+constexpr int kStagedGrid = 128, kStagedCluster = 4;  // CTAs and cluster size of a staged launch
+bool c64_staged_prepare(int dim, int block);
+// Chains of these sizes take the staged complex64 form: below, the parts of 128
+// CTAs are too short (16 sites: 512 elements, no gain), above they leave shared memory.
+constexpr int kC64StagedMinSites = 17, kC64StagedMaxSites = 21;
 int launch_propagate_spin_c64(const PropParams& p, const OpSpinC& op, int grid, int block, void* stream);
 int launch_propagate_dia_c64(const PropParams& p, const OpDiaC& op, int grid, int block, void* stream);
 int launch_propagate_csr_c64(const PropParams& p, const OpCsrC& op, int grid, int block, void* stream);

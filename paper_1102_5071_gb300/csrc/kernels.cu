@@ -844,6 +844,31 @@ int launch_wait_selftest(int which, unsigned long long* rec, unsigned* bar, int*
   k_wait_selftest<<<2, 32>>>(which, rec, bar, status, timeout_ns);
   return (int)cudaGetLastError();
 }
+// Whether `grid` CTAs of `block` threads and `bytes` of dynamic shared memory of
+// the kernel, in clusters of cs, are all resident at once.
+bool staged_fits(const void* kernel, int grid, int cs, int block, size_t bytes) {
+  if (bytes > kFxSmallSmemMax ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = bytes;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  const bool ok = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n * cs >= grid;
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+
 // ||a - b||_2^2 partial sums: block j writes the sum over its grid-stride
 // elements (tree in shared memory, fixed order) to part[j]; the host adds the
 // partials in block order.  Used by the time-step selection (Sec. 6.6).

@@ -29,7 +29,8 @@
 // small exponential (the estimate of iteration k runs while the workers
 // already apply H for iteration k+1, as in the fixed-point kernel).
 //
-// Long chains: the TILED instantiation applies H in window passes over
+// Chains of 17 to 21 sites: the staged form keeps the applied vector in the shared
+// memory of 128 CTAs (clusters of four).  Long chains: the tiled form applies H in window passes over
 // shared-memory tiles moved by TMA (tiled_common.cuh) instead of element by
 // element; its window 0 also does the previous iteration's orthogonalisation
 // step, so it has one grid exchange per iteration less.
@@ -233,6 +234,107 @@ __device__ __forceinline__ void c_apply_spin2(const float2* __restrict__ q, cons
   }
   r1 = make_float2(ur1, ui1);
   r2 = make_float2(ur2, ui2);
+}
+
+// Element pair (x, x + 1) of a chain staged over 128 CTAs, as fx_apply_spin_staged:
+// bits below N - 7 from this CTA's shared memory, the next two from the cluster's,
+// the five highest from global memory (issued ahead); any bit above bit 0 maps the
+// pair onto a pair, one 16-byte access.  Every sum runs in the order of the
+// element-wise form, so the results are the same bits.  The far gathers bound it: 4.5 TB/s over
+// the L2 fabric, where the element-wise form gathers twice as many bytes.  Lanczos
+// iteration 12.1 us at 17 sites (element-wise 13.6), 15.2 at 18 (16.8), 30.8 at 20
+// (32.4), 53.6 at 21 (58.0).  Near loops unrolled by 6 and 12 instead of 4: 3 and
+// 8 % slower.  Fixed-point vectors (twice the bytes, on 128 of 152 SMs) were slower
+// staged, 59.6 against 52.8 us at 20 sites.
+constexpr int kCStagedBits = 7, kCStagedClusterBits = 2, kCStagedFar = kCStagedBits - kCStagedClusterBits;
+__device__ __forceinline__ float4 c_ld_cluster(unsigned base, int j) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(base + 8u * (unsigned)j));
+  return v;
+}
+__device__ __forceinline__ void c_apply_spin_staged2(const float2* sq, const float2* __restrict__ q,
+                                                     const float2* __restrict__ qm, int j, unsigned rank,
+                                                     const OpSpinC& op, const CConst& c, const float* bx, float4& r,
+                                                     float4& v) {
+  const int N = op.N, L = op.lo_bits, lc = N - kCStagedBits, lg = N - kCStagedFar;
+  const int x = (int)(blockIdx.x << lc) | j;
+  const unsigned anti = ((unsigned)x ^ ((unsigned)x >> 1)) & ((1u << (N - 1)) - 1u);
+  auto add = [](float4& s, const float4 w) {
+    s.x += w.x;
+    s.y += w.y;
+    s.z += w.z;
+    s.w += w.w;
+  };
+  auto near4 = [&](int jj) { return *reinterpret_cast<const float4*>(sq + jj); };
+  auto far4 = [&](int xx) { return *reinterpret_cast<const float4*>(q + xx); };
+  float4 f[kCStagedFar], pv = make_float4(0.f, 0.f, 0.f, 0.f);
+  // far hops under way during the near ones (antiparallel bonds, uniform over the CTA)
+#pragma unroll
+  for (int k = 0; k < kCStagedFar; ++k) {
+    f[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if ((anti >> (lg - 1 + k)) & 1u) f[k] = far4(x ^ (3 << (lg - 1 + k)));
+  }
+  if (c.use_prev) pv = *reinterpret_cast<const float4*>(qm + x);
+  v = near4(j);
+  const float2 dlo = __ldg(reinterpret_cast<const float2*>(op.dz_lo + (x & ((1 << L) - 1))));
+  const float dhi = __ldg(op.dz_hi + (x >> (L - 1)));
+  const float d0 = c.cz * (dlo.x + dhi), d1 = c.cz * (dlo.y + dhi);
+  float4 u = make_float4(d0 * v.x, d0 * v.y, d1 * v.z, d1 * v.w);
+  auto madd = [&](float a, const float4 w) {
+    u.x = fmaf(a, w.x, u.x);
+    u.y = fmaf(a, w.y, u.y);
+    u.z = fmaf(a, w.z, u.z);
+    u.w = fmaf(a, w.w, u.w);
+  };
+  float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
+  {  // bond (0, 1): one element of the pair j ^ 2
+    const float4 w = near4(j ^ 2);
+    if ((j >> 1) & 1) {
+      h.x += w.z;
+      h.y += w.w;
+    } else {
+      h.z += w.x;
+      h.w += w.y;
+    }
+  }
+#pragma unroll 4
+  for (int i = 1; i < lc - 1; ++i)
+    if ((anti >> i) & 1u) add(h, near4(j ^ (3 << i)));
+  if ((anti >> (lc - 1)) & 1u) add(h, c_ld_cluster(cluster_addr(sq, rank ^ 1u), j ^ (1 << (lc - 1))));
+  if ((anti >> lc) & 1u) add(h, c_ld_cluster(cluster_addr(sq, rank ^ 3u), j));
+#pragma unroll
+  for (int k = 0; k < kCStagedFar; ++k)
+    if ((anti >> (lg - 1 + k)) & 1u) add(h, f[k]);
+  // far flips under way during the near ones
+#pragma unroll
+  for (int k = 0; k < kCStagedFar; ++k) f[k] = far4(x ^ (1 << (lg + k)));
+  madd(c.ch, h);
+  float4 g[kCStagedClusterBits];
+#pragma unroll
+  for (int k = 0; k < kCStagedClusterBits; ++k) g[k] = c_ld_cluster(cluster_addr(sq, rank ^ (1u << k)), j);
+  const float4 swap = make_float4(v.z, v.w, v.x, v.y);  // bit 0
+  if (op.uniform) {
+    float4 s = swap;
+#pragma unroll 4
+    for (int i = 1; i < lc; ++i) add(s, near4(j ^ (1 << i)));
+#pragma unroll
+    for (int k = 0; k < kCStagedClusterBits; ++k) add(s, g[k]);
+#pragma unroll
+    for (int k = 0; k < kCStagedFar; ++k) add(s, f[k]);
+    madd(c.cx, s);
+  } else {
+    madd(bx[0], swap);
+#pragma unroll 4
+    for (int i = 1; i < lc; ++i) madd(bx[i], near4(j ^ (1 << i)));
+#pragma unroll
+    for (int k = 0; k < kCStagedClusterBits; ++k) madd(bx[lc + k], g[k]);
+#pragma unroll
+    for (int k = 0; k < kCStagedFar; ++k) madd(bx[lg + k], f[k]);
+  }
+  if (c.use_prev) madd(c.cp, pv);
+  r = u;
 }
 
 __device__ __forceinline__ float2 c_apply_dia(const float2* __restrict__ q, const float2* __restrict__ qm, int r,
@@ -725,11 +827,14 @@ __device__ __noinline__ void c_rec_consts(SmemC& S, int acc_k, double ts) {
 // fx_control): the control warp publishes one element pass at a time.
 enum CCmd { kCExit = 0, kCConvert, kCApply, kCOrth, kCRec };
 
-// TILED: the window-tiled apply of long spin chains (a separate instantiation,
-// so that the element-wise kernel carries none of its code).
-template <int FAMILY, class Op, bool TILED>
+// Forms of the kernel, separate instantiations: element-wise; the window-tiled
+// apply of long spin chains; spin chains staged in the shared memory of all CTAs.
+enum CMode { kCGrid = 0, kCTiled, kCStaged };
+
+template <int FAMILY, class Op, int MODE>
 __device__ __forceinline__ void c_worker(const PropParams& p, const Op& op, SmemC& S, unsigned char* tiles_base,
                                          int wstep) {
+  constexpr bool TILED = MODE == kCTiled, STAGED = MODE == kCStaged;
   const int tid = threadIdx.x, lane = tid & 31;
   const int dim = p.dim;
   int wx0, wxe;  // one contiguous chunk per CTA
@@ -742,6 +847,9 @@ __device__ __forceinline__ void c_worker(const PropParams& p, const Op& op, Smem
     wxe = min(dim, ((int)blockIdx.x + 1) * chunk);
   }
   auto Q = [&](int i) -> float2* { return p.qbasis32 + (size_t)(i - 1) * dim; };
+  // staged: this CTA's part of the applied vector
+  float2* const sq = reinterpret_cast<float2*>(tiles_base);
+  const int xb = wx0 - tid;
   TileWin win[kTiledMaxWindows] = {};
   int nwin = 1;
   if constexpr (TILED) nwin = tiled_windows<kTileBits>(op.N, win);
@@ -797,6 +905,21 @@ __device__ __forceinline__ void c_worker(const PropParams& p, const Op& op, Smem
             window_written_sync();    // all threads: window w written
             window_exchanged_sync();  // all threads: the grid exchange passed
           }
+        }
+      } else if constexpr (STAGED) {
+        const unsigned rank = cluster_rank();
+        for (int j = 2 * tid; j < wxe - xb; j += 2 * wstep) {
+          float4 h, v;
+          c_apply_spin_staged2(sq, q, qm, j, rank, op, c, S.bx, h, v);
+          *reinterpret_cast<float4*>(u + xb + j) = h;
+          ff_add_prod(s0, c0, v.x, h.x);
+          ff_add_prod(s0, c0, v.y, h.y);
+          ff_add_prod(s0, c0, v.z, h.z);
+          ff_add_prod(s0, c0, v.w, h.w);
+          ff_add_prod(s1, c1, h.x, h.x);
+          ff_add_prod(s1, c1, h.y, h.y);
+          ff_add_prod(s1, c1, h.z, h.z);
+          ff_add_prod(s1, c1, h.w, h.w);
         }
       } else {
         // spin apply on two elements per thread and loop iteration (twice the
@@ -857,6 +980,7 @@ __device__ __forceinline__ void c_worker(const PropParams& p, const Op& op, Smem
         for (int j = 0; j < 4; ++j) {
           const float2 w = make_float2(fmaf(am, v[j].x, uu[j].x), fmaf(am, v[j].y, uu[j].y));
           u[x + j * wstep] = w;
+          if constexpr (STAGED) sq[x + j * wstep - xb] = w;
           ff_add_prod(s0, c0, w.x, w.x);
           ff_add_prod(s0, c0, w.y, w.y);
         }
@@ -866,6 +990,7 @@ __device__ __forceinline__ void c_worker(const PropParams& p, const Op& op, Smem
         const float2 uu = u[x];
         const float2 w = make_float2(fmaf(am, v.x, uu.x), fmaf(am, v.y, uu.y));
         u[x] = w;
+        if constexpr (STAGED) sq[x - xb] = w;
         ff_add_prod(s0, c0, w.x, w.x);
         ff_add_prod(s0, c0, w.y, w.y);
       }
@@ -897,6 +1022,7 @@ __device__ __forceinline__ void c_worker(const PropParams& p, const Op& op, Smem
           im = fmaf(cr, v.y, fmaf(ci, v.x, im));
         }
         Q(1)[x] = make_float2(re, im);
+        if constexpr (STAGED) sq[x - xb] = make_float2(re, im);
         if (final_rec) p.psi[x] = make_double2((double)re, (double)im);
         ff_add_prod(s, cc, re, re);
         ff_add_prod(s, cc, im, im);
@@ -912,6 +1038,7 @@ __device__ __forceinline__ void c_worker(const PropParams& p, const Op& op, Smem
         bad |= !(isfinite(v.x) && isfinite(v.y));
         const float2 f = make_float2((float)v.x, (float)v.y);
         Q(1)[x] = f;
+        if constexpr (STAGED) sq[x - xb] = f;
         ff_add_prod(s, c, f.x, f.x);
         ff_add_prod(s, c, f.y, f.y);
       }
@@ -922,8 +1049,9 @@ __device__ __forceinline__ void c_worker(const PropParams& p, const Op& op, Smem
   }
 }
 
-template <int FAMILY, class Op, bool TILED>
+template <int FAMILY, class Op, int MODE>
 __device__ __forceinline__ void c_control(const PropParams& p, const Op& op, SmemC& S, int NW) {
+  constexpr bool TILED = MODE == kCTiled;
   const int lane = threadIdx.x & 31;
   const int G = gridDim.x;
   const int ncoef = 1 + p.nV;
@@ -1175,14 +1303,14 @@ __device__ __forceinline__ void c_control(const PropParams& p, const Op& op, Sme
   }
 }
 
-template <int FAMILY, class Op, bool TILED = false>
+template <int FAMILY, class Op, int MODE>
 __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_c64(PropParams p, Op op) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmemC& S = *reinterpret_cast<SmemC*>(smem_raw);
   const int NW = (int)(blockDim.x >> 5) - 1;
   // tiled apply: the stages' mbarriers and tile buffers behind SmemC
   unsigned char* const tiles_base = smem_raw + ((sizeof(SmemC) + 127) & ~size_t(127));
-  if constexpr (TILED) {
+  if constexpr (MODE == kCTiled) {
     if (threadIdx.x == 0) {  // ordered before any use by the CTA barriers of the conversion pass
       for (int s2 = 0; s2 < kTmaStages; ++s2) mbar_init(reinterpret_cast<unsigned long long*>(tiles_base) + s2, 1);
       S.tma_fail = 0;
@@ -1190,13 +1318,17 @@ __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_c64(PropP
     }
   }
   if ((int)(threadIdx.x >> 5) < NW) {
-    c_worker<FAMILY, Op, TILED>(p, op, S, tiles_base, NW * 32);
+    c_worker<FAMILY, Op, MODE>(p, op, S, tiles_base, NW * 32);
   } else {
-    c_control<FAMILY, Op, TILED>(p, op, S, NW);
+    c_control<FAMILY, Op, MODE>(p, op, S, NW);
     __syncwarp();
     if ((threadIdx.x & 31) == 0) S.cmd = kCExit;  // also after an error
     __syncwarp();
     __syncthreads();
+  }
+  if constexpr (MODE == kCStaged) {
+    __syncwarp();
+    cluster_sync_all();  // no CTA leaves while another may read its shared memory
   }
 }
 
@@ -1205,22 +1337,38 @@ size_t c64_tiled_smem_bytes() {
   return ((sizeof(SmemC) + 127) & ~size_t(127)) + 128 + (size_t)kTmaStages * 2 * kTileBytes;
 }
 
+static size_t c64_staged_smem_bytes(int part) {
+  return ((sizeof(SmemC) + 127) & ~size_t(127)) + (size_t)part * sizeof(float2);
+}
+
 template <int FAMILY, class Op>
 static int launch_prop_c64(const PropParams& p, const Op& op, int grid, int block, void* stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = p.tiled ? c64_tiled_smem_bytes() : sizeof(SmemC);
+  cfg.dynamicSmemBytes = p.tiled     ? c64_tiled_smem_bytes()
+                         : p.cluster ? c64_staged_smem_bytes(p.dim / grid)
+                                     : sizeof(SmemC);
   cfg.stream = (cudaStream_t)stream;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = p.cluster;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = p.cluster ? 2 : 1;
   if constexpr (FAMILY == kFamilySpin) {
-    if (p.tiled) return (int)cudaLaunchKernelEx(&cfg, k_propagate_c64<FAMILY, Op, true>, p, op);
+    if (p.tiled) return (int)cudaLaunchKernelEx(&cfg, k_propagate_c64<FAMILY, Op, kCTiled>, p, op);
+    if (p.cluster) return (int)cudaLaunchKernelEx(&cfg, k_propagate_c64<FAMILY, Op, kCStaged>, p, op);
   }
-  return (int)cudaLaunchKernelEx(&cfg, k_propagate_c64<FAMILY, Op>, p, op);
+  return (int)cudaLaunchKernelEx(&cfg, k_propagate_c64<FAMILY, Op, kCGrid>, p, op);
+}
+
+bool c64_staged_prepare(int dim, int block) {
+  return staged_fits((const void*)k_propagate_c64<kFamilySpin, OpSpinC, kCStaged>, kStagedGrid, kStagedCluster, block,
+                     c64_staged_smem_bytes(dim / kStagedGrid));
 }
 
 int launch_propagate_spin_c64(const PropParams& p, const OpSpinC& op, int grid, int block, void* stream) {
@@ -1239,21 +1387,21 @@ int max_coresident_blocks_c64(int family, int block, bool tiled) {
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   // a few KB of shared memory: leave the unified storage to L1 (a tiled launch
   // asks for its tile buffers and gets the shared-memory split it needs)
-  cudaFuncSetAttribute(k_propagate_c64<kFamilySpin, OpSpinC>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-  cudaFuncSetAttribute(k_propagate_c64<kFamilyDia, OpDiaC>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-  cudaFuncSetAttribute(k_propagate_c64<kFamilyCsr, OpCsrC>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-  cudaFuncSetAttribute(k_propagate_c64<kFamilySpin, OpSpinC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_propagate_c64<kFamilySpin, OpSpinC, kCGrid>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+  cudaFuncSetAttribute(k_propagate_c64<kFamilyDia, OpDiaC, kCGrid>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+  cudaFuncSetAttribute(k_propagate_c64<kFamilyCsr, OpCsrC, kCGrid>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+  cudaFuncSetAttribute(k_propagate_c64<kFamilySpin, OpSpinC, kCTiled>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)c64_tiled_smem_bytes());
   cudaError_t e;
   if (family == kFamilySpin)
-    e = tiled ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_c64<kFamilySpin, OpSpinC, true>, block,
+    e = tiled ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_c64<kFamilySpin, OpSpinC, kCTiled>, block,
                                                               c64_tiled_smem_bytes())
-              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_c64<kFamilySpin, OpSpinC>, block, sizeof(SmemC));
+              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_c64<kFamilySpin, OpSpinC, kCGrid>, block, sizeof(SmemC));
   else if (family == kFamilyCsr)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_c64<kFamilyCsr, OpCsrC>, block,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_c64<kFamilyCsr, OpCsrC, kCGrid>, block,
                                                       sizeof(SmemC));
   else
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_c64<kFamilyDia, OpDiaC>, block,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_propagate_c64<kFamilyDia, OpDiaC, kCGrid>, block,
                                                       sizeof(SmemC));
   if (e != cudaSuccess) return -1;
   return per * nsm;
