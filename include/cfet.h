@@ -183,7 +183,9 @@ typedef struct cfet_options {
   int32_t m_max;             /* Krylov dimension limit (default 16, <= 64)    */
   int32_t m_min;             /* first dimension tested (default 2, >= 1)      */
   int32_t max_substeps;      /* per stage exponential (default 64)            */
-  int32_t block_size;        /* 0 = auto; FP64 kernel: threads per CTA (256);
+  int32_t block_size;        /* 0 = auto; FP64 kernel: 2 x block_size threads
+                                per CTA (256 -> 512, the largest allowed;
+                                auto: as many as a CTA has elements, <= 512);
                                 fixed-point and mixed-precision kernels:
                                 2 x block_size worker threads + one control
                                 warp (384 -> 800, the largest allowed)        */
@@ -521,7 +523,7 @@ cfet_status cfet_batch_propagate(cfet_batch* b, void* const* psi, double t0, dou
 
 /* Autotuner: runs nsteps steps of the given propagation on internal states
  * (normalised pseudo-random vectors, reset before every candidate) for every
- * candidate plan (cluster size 1, 2, 4, 8 x 128, 256, 512 threads x three
+ * candidate plan (cluster size 1, 2, 4, 8 x 128, 256, 512 threads x four
  * thresholds) that fits on the device, keeps the fastest as the batch's plan
  * and returns it in `chosen` (may be NULL).  Caller states are not touched. */
 cfet_status cfet_batch_tune(cfet_batch* b, double t0, double dt, int32_t order, double krylov_tol, int64_t nsteps,

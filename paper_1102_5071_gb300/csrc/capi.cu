@@ -143,14 +143,12 @@ struct cfet_ctx {
 
 namespace {
 
-// Reduction / exchange scratch per CTA (8-byte words): the FP64 kernel uses 3
-// partials, the control-warp kernels the two slots of the record exchange.
+// Exchange scratch per CTA (8-byte words): the two slots of the record exchange.
 constexpr size_t kPartialWordsPerCta = kExchWords;
 constexpr int kMaxCtlGrid = 256;  // 32 lanes x 8 records per lane of the exchange
-// FP64 kernel with full re-orthogonalisation: 3 slots + 2 m_max Gram-Schmidt coefficients per CTA
+// (FP64 kernel with full re-orthogonalisation: 2 m_max Gram-Schmidt coefficients behind them.)
 static size_t partial_words_per_cta(const cfet_ctx* ctx) {
-  const size_t need = ctx->opt.reorth ? 3 + 2 * (size_t)ctx->opt.m_max : 0;
-  return need > kPartialWordsPerCta ? need : kPartialWordsPerCta;
+  return kPartialWordsPerCta + (ctx->opt.reorth ? 2 * (size_t)ctx->opt.m_max : 0);
 }
 
 thread_local std::string g_create_err;
@@ -801,9 +799,10 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
     return fail(nullptr, CFET_EINVAL, "reorth requires CFET_PREC_F64 and CFET_EXPM_KRYLOV");
   if (o.apply_form != CFET_APPLY_AUTO && o.apply_form != CFET_APPLY_ELEMENTWISE && o.apply_form != CFET_APPLY_TILED)
     return fail(nullptr, CFET_EINVAL, "apply_form must be CFET_APPLY_AUTO, CFET_APPLY_ELEMENTWISE or CFET_APPLY_TILED");
+  const bool auto_block = o.block_size == 0;
   if (o.block_size == 0) o.block_size = (o.precision == CFET_PREC_F64) ? 256 : 384;
   {
-    // FP64 kernel: block_size threads (<= 256); fixed-point and mixed-precision
+    // FP64 kernel: 2 * block_size threads (<= 512); fixed-point and mixed-precision
     // kernels: 2 * block_size workers + one control warp (<= 1024 threads)
     // (the latter are compiled for at most CFET_CTL_MAX_THREADS threads per CTA)
     const int lim = (o.precision == CFET_PREC_F64) ? 256 : ((CFET_CTL_MAX_THREADS - 32) / 2) & ~31;
@@ -930,11 +929,11 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
   ctx->dim = dim;
   ctx->nV = nV;
   ctx->opt = o;
-  // FP64 kernel: block_size threads; fixed-point and mixed-precision kernels:
+  // FP64 kernel: 2 * block_size threads; fixed-point and mixed-precision kernels:
   // 2 * block_size worker threads plus one control warp (default 768 + 32,
   // one CTA per SM)
   const bool ctl_warp = o.precision != CFET_PREC_F64;
-  ctx->block = ctl_warp ? 2 * o.block_size + 32 : o.block_size;
+  ctx->block = ctl_warp ? 2 * o.block_size + 32 : 2 * o.block_size;
   ctx->precision = o.precision;
   for (int k = 0; k < nV; ++k) {
     ctx->f.push_back(f[k]);
@@ -1243,8 +1242,17 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
   if (want > 1) want = (int)std::min((((long long)dim << lane_bits) + workers - 1) / workers, 1LL << 30);
   if (o.grid_size > 0) want = o.grid_size;
   ctx->grid = want < maxg ? want : maxg;
-  if (ctl_warp && ctx->grid > kMaxCtlGrid) ctx->grid = kMaxCtlGrid;  // record exchange limit
+  if (ctx->grid > kMaxCtlGrid) ctx->grid = kMaxCtlGrid;  // record exchange limit
   if (ctx->grid < 1) ctx->grid = 1;
+  // FP64 kernel: an SM needs four warps for its FP64 pipes, and every further one
+  // lengthens the apply, so 128 elements per CTA up to one CTA per SM and one
+  // thread per element up to 512.  Against 512 threads for 512 elements, 30 steps of
+  // CF4:2 in ms: 9 sites 4.8 (5.9), 12 sites 5.7 (7.8), 14 sites 7.1 (9.7); a chain of
+  // 8 sites stays in one CTA (3.9, 4.4 over two).
+  if (!ctl_warp && auto_block && o.grid_size == 0) {
+    ctx->grid = dim <= 256 ? 1 : std::min(std::min(maxg, kMaxCtlGrid), (dim + 127) / 128);
+    ctx->block = std::min(ctx->block, std::max(64, ((dim + ctx->grid - 1) / ctx->grid + 31) & ~31));
+  }
 
   if (ctx->precision == CFET_PREC_FX && o.expm == CFET_EXPM_KRYLOV && ctx->grid == 1 && !ctx->tiled) {
     // a single CTA: the basis fits in its shared memory for small problems

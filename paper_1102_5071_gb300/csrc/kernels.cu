@@ -8,13 +8,12 @@
 // sparsity pattern).
 //
 // Structure: one persistent cooperative kernel per launch runs a sequence of
-// stage exponentials.  Every CTA walks a grid-stride slice of the vectors;
-// the two scalar reductions of a Lanczos iteration (alpha, beta) go through a
-// per-CTA warp-shuffle/shared-memory tree, one partial per CTA in global
-// memory, and a bounded grid barrier; every CTA then sums the partials in the
-// same fixed order, so all CTAs hold bit-identical alpha/beta and take the
-// same adaptive decisions without a broadcast.  Warp 0 of each CTA evaluates
-// the small exponential exp(-i tau T_k) e_1 of the tridiagonal Lanczos matrix.
+// stage exponentials.  Every CTA walks one contiguous chunk of the vectors; the
+// two scalar reductions of a Lanczos iteration (alpha, beta) go through a CTA
+// tree, one record per CTA (ctl_exchange) and a fixed-order sum, so all CTAs hold
+// bit-identical alpha/beta and take the same adaptive decisions without a
+// broadcast.  Warp 0 of each CTA evaluates the small exponential
+// exp(-i tau T_k) e_1 of the tridiagonal Lanczos matrix.
 // Operator families: XXZ chain with X fields, DIA, CSR, general Pauli sums,
 // and the chain in the interaction picture; optionally every Lanczos vector is
 // re-orthogonalised against all earlier ones (classical Gram-Schmidt).
@@ -191,31 +190,118 @@ struct SmemLayout {
   double bsite_raw[kMaxSites];  // spin: sum_k c_k a_{k,i} for the current exponential
   double copf[1 + kMaxDrives];  // dia: scaled per-operator coefficients
   double scal[1 + kMaxDrives];  // current stage scalars
+  double sum;                   // f64_reduce
   double bcast[4];
-  int dec[4];                   // decision broadcast: accepted, k, h, pad
+  int dec[4];                   // decision broadcast: accepted, y ready, h, pad
   int ok;
 };
 
+// ------------------------------------------------------------------ reduction
+struct SumAcc {  // one double per CTA record
+  double s;
+  __device__ void reset() { s = 0.0; }
+  __device__ void add(const unsigned (&v)[2]) {
+    s += __longlong_as_double((long long)(((unsigned long long)v[1] << 32) | v[0]));
+  }
+};
+// Grid sum of one double per thread into S.sum (every thread of every CTA holds
+// the same value), which is also the grid barrier: the CTA tree, one record per
+// CTA (ctl_exchange, warp 0), a fixed-order sum.  `fence`: vectors written before
+// it are read by other CTAs after it.  False in every thread on a timeout or when
+// another CTA reported an error.
+__device__ __noinline__ bool f64_reduce(SmemLayout& S, double acc, bool fence, unsigned tag, const PropParams& p) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) S.red[warp] = acc;
+  __syncthreads();
+  if (warp == 0) {
+    double c = lane < (int)(blockDim.x >> 5) ? S.red[lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(c);
+    const unsigned mine[2] = {(unsigned)b, (unsigned)(b >> 32)};
+    SumAcc a;
+    long long spin = 0;
+    const bool ok = ctl_exchange<2>(reinterpret_cast<unsigned long long*>(p.partials), mine, tag, fence, &p.st->status,
+                                    p.timeout_ns, spin, a);
+    double t = a.s;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) {
+      S.sum = t;
+      S.ok = ok;
+    }
+  }
+  __syncthreads();
+  return S.ok != 0;
+}
+
+// Decision of iteration it (warp 0): beta, breakdown, gate and estimate into S.
+__device__ __noinline__ void f64_decide(SmemLayout& S, int it, double beta0, double remaining, int kf,
+                                        const PropParams& p) {
+  const int tid = threadIdx.x;
+  const bool fixed_k = p.tol <= 0.0;
+  const double b = sqrt(S.sum);
+  const double prev_b = it > 1 ? S.beta[it - 1] : 0.0;
+  const bool breakdown =
+      sb_no_breakdown(b, S.alpha[it], prev_b) != 1 && b <= 1e-13 * (fabs(S.alpha[it]) + prev_b + 1.0);
+  int acc_flag = 0;
+  double err = 0.0;
+  if (kf > 0) {
+    acc_flag = (it == kf);
+  } else if (fixed_k) {
+    acc_flag = (it == p.m_max) || breakdown;
+  } else if (breakdown) {
+    acc_flag = 1;
+  } else if (it >= p.m_min && gersh_gate(it, S.alpha + 1, S.beta + 1, remaining)) {
+    // T_it: diagonal alpha[1..it], off-diagonal beta[1..it-1]; the
+    // estimate is evaluated only where Eq. (KryErr) applies
+    const double thr = p.tol * remaining / p.tau;
+    if (krylov_lead_rejects(it, S.alpha + 1, S.beta + 1, remaining, beta0 * b, thr)) {
+      err = 2.0 * thr + 1e-300;
+    } else {
+      small_expm_e1(it, S.alpha + 1, S.beta + 1, remaining, S.yr, S.yi, S.tr, S.ti);
+      err = beta0 * b * hypot(S.yr[it - 1], S.yi[it - 1]);
+      acc_flag = err <= thr;
+    }
+  }
+  __syncwarp();
+  if (tid == 0) {
+    S.beta[it] = b;
+    S.scale[it + 1] = div_call(1.0, b);
+    S.dec[0] = acc_flag;
+    S.dec[1] = acc_flag && kf == 0 && !fixed_k && !breakdown;  // yr / yi hold exp(-i remaining T) e_1
+    S.bcast[1] = err;
+  }
+}
+
 // ------------------------------------------------------------------ the persistent kernel
+// The FP64 pipe is the limit of an apply (about 75 FP64 instructions per element
+// at 64 cycles a warp), so every SM gets the same number of elements: contiguous
+// chunks, one element per thread while that is at most 512 threads (the host picks
+// the grid).  Chunks of more than eight elements per thread are interleaved over
+// the CTAs instead, so that the SMs gather from the same part of the vector at a
+// time (20 sites: 8.16 against 8.32 ms; 19 sites 4.30, 18 sites 2.46).  CTAs of
+// 256 threads, three per SM, that met at a counter barrier took 8.24, 4.45 and
+// 2.74 ms (three steps of CF4:2; FP64 pipe 0.6 to 0.7 of its rate).
 template <int FAMILY, class Op>
-__global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
+__global__ void __launch_bounds__(512, 1) k_propagate(PropParams p, Op op) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmemLayout& S = *reinterpret_cast<SmemLayout*>(smem_raw);
   const int tid = threadIdx.x;
   const int dim = p.dim;
-  const int stride = gridDim.x * blockDim.x;
-  const int x0 = blockIdx.x * blockDim.x + tid;
   const int G = gridDim.x;
+  const int chunk = ((dim + G - 1) / G + 31) & ~31;
+  const bool wide = chunk > 8 * (int)blockDim.x;
+  const int stride = wide ? G * (int)blockDim.x : (int)blockDim.x;
+  const int x0 = (wide ? (int)blockDim.x : chunk) * (int)blockIdx.x + tid;
+  const int xe = wide ? dim : min(dim, ((int)blockIdx.x + 1) * chunk);
   const int ncoef = 1 + p.nV;
-  unsigned gen = 0;
-  // three partial slots (phase A, phase B, norm): two uses of one slot are
-  // always separated by a grid barrier on another slot
-  double* part0 = p.partials;
-  double* part1 = p.partials + G;
-  double* part2 = p.partials + 2 * G;
+  unsigned gen = 0;  // barriers of the re-orthogonalisation
   DevStatus* st = p.st;
+  unsigned tag = (unsigned)ld_volatile_i32((const int*)&st->tag_base);
   const bool lead = (blockIdx.x == 0 && tid == 0);
-  const bool fixed_k = p.tol <= 0.0;
   const bool forced = p.f_nsub != nullptr;
 
   long long fpos = st->forced_pos;
@@ -229,19 +315,14 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
   // initial norm of psi
   {
     double acc = 0.0;
-    for (int x = x0; x < dim; x += stride) {
+    for (int x = x0; x < xe; x += stride) {
       const double2 v = p.psi[x];
       acc = fma(v.x, v.x, fma(v.y, v.y, acc));
     }
-    const double s = block_sum(acc, S.red);
-    if (tid == 0) part2[blockIdx.x] = s;
-    if (!grid_barrier(p.bar, gen, &st->status, p.timeout_ns, &S.ok)) return;
-    if (tid < 32) {
-      const double t = sum_partials(part2);
-      if (tid == 0) S.bcast[0] = sqrt(t);
-    }
-    __syncthreads();
+    if (!f64_reduce(S, acc, false, ++tag, p)) return;
   }
+  if (tid == 0) S.bcast[0] = sqrt(S.sum);
+  __syncthreads();
   double beta0 = S.bcast[0];
 
   for (long long e = 0; e < p.nexp; ++e) {
@@ -314,7 +395,7 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
             SpinScaled sc;
             sc.cz = S.scal[0] * s_it;
             sc.cxx = S.scal[0] * s_it * op.J2;
-            for (int x = x0; x < dim; x += stride) {
+            for (int x = x0; x < xe; x += stride) {
               double2 hv = apply_spin_at(q, x, op, sc, S.bsite);
               if (qm) {
                 const double2 w = qm[x];
@@ -327,7 +408,7 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
             }
           } else if constexpr (FAMILY == kFamilyPauli) {
             const double* pc = reinterpret_cast<const double*>(smem_raw + ip_table_offset<SmemLayout>());
-            for (int x = x0; x < dim; x += stride) {
+            for (int x = x0; x < xe; x += stride) {
               double2 hv = apply_pauli_at(q, x, op, pc, S.scal);
               hv.x *= s_it;
               hv.y *= s_it;
@@ -342,7 +423,7 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
             }
           } else if constexpr (FAMILY == kFamilySpinIP) {
             const double2* Wt = reinterpret_cast<const double2*>(smem_raw + ip_table_offset<SmemLayout>());
-            for (int x = x0; x < dim; x += stride) {
+            for (int x = x0; x < xe; x += stride) {
               double2 hv = apply_spin_ip_at(q, x, op.N, Wt);
               hv.x *= s_it;
               hv.y *= s_it;
@@ -356,7 +437,7 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
               acc = fma(v.x, hv.x, fma(v.y, hv.y, acc));
             }
           } else {
-            for (int x = x0; x < dim; x += stride) {
+            for (int x = x0; x < xe; x += stride) {
               double2 hv = apply_sparse_at(q, x, dim, op, S.copf);
               if (qm) {
                 const double2 w = qm[x];
@@ -368,20 +449,13 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
               acc = fma(v.x, hv.x, fma(v.y, hv.y, acc));
             }
           }
-          {
-            const double s = block_sum(acc, S.red);
-            if (tid == 0) part0[blockIdx.x] = s;
-          }
-          if (!grid_barrier(p.bar, gen, &st->status, p.timeout_ns, &S.ok)) return;
-          if (tid < 32) {
-            const double t = sum_partials(part0);
-            if (tid == 0) S.alpha[it] = t * s_it;
-          }
-          __syncthreads();
+          if (!f64_reduce(S, acc, false, ++tag, p)) return;
           // ---------------- phase B: w = u - alpha s_it q_it, beta = ||w||
-          const double am = S.alpha[it] * s_it;
+          const double alpha = S.sum * s_it;
+          if (tid == 0) S.alpha[it] = alpha;
+          const double am = alpha * s_it;
           acc = 0.0;
-          for (int x = x0; x < dim; x += stride) {
+          for (int x = x0; x < xe; x += stride) {
             const double2 v = q[x];
             double2 w = u[x];
             w.x = fma(-am, v.x, w.x);
@@ -389,20 +463,16 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
             u[x] = w;
             acc = fma(w.x, w.x, fma(w.y, w.y, acc));
           }
-          {
-            const double s = block_sum(acc, S.red);
-            if (tid == 0) part1[blockIdx.x] = s;
-          }
-          if (!grid_barrier(p.bar, gen, &st->status, p.timeout_ns, &S.ok)) return;
+          if (!f64_reduce(S, acc, true, ++tag, p)) return;
           if (p.reorth) {
             // ---------------- full re-orthogonalisation (option): one classical
             // Gram-Schmidt sweep w <- w - sum_i v_i <v_i, w> over the stored
-            // q_i = v_i / scale[i]; ||w||^2 is then taken again into part1
-            double* partQ = p.partials + 3 * (size_t)G;  // 2 it doubles per CTA
+            // q_i = v_i / scale[i]; ||w||^2 is then taken again
+            double* partQ = p.partials + kExchWords * (size_t)G;  // 2 it doubles per CTA
             for (int i = 1; i <= it; ++i) {
               const double2* qi = vec(i);
               double ar = 0.0, ai = 0.0;
-              for (int x = x0; x < dim; x += stride) {
+              for (int x = x0; x < xe; x += stride) {
                 const double2 a = qi[x], w = u[x];
                 ar = fma(a.x, w.x, fma(a.y, w.y, ar));   // conj(q_i) w
                 ai = fma(a.x, w.y, fma(-a.y, w.x, ai));
@@ -430,7 +500,7 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
             }
             __syncthreads();
             acc = 0.0;
-            for (int x = x0; x < dim; x += stride) {
+            for (int x = x0; x < xe; x += stride) {
               double2 w = u[x];
               for (int i = 1; i <= it; ++i) {
                 const double2 a = vec(i)[x];
@@ -441,47 +511,10 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
               u[x] = w;
               acc = fma(w.x, w.x, fma(w.y, w.y, acc));
             }
-            {
-              const double s2 = block_sum(acc, S.red);
-              if (tid == 0) part1[blockIdx.x] = s2;
-            }
-            if (!grid_barrier(p.bar, gen, &st->status, p.timeout_ns, &S.ok)) return;
+            if (!f64_reduce(S, acc, true, ++tag, p)) return;
           }
           // ---------------- decision (warp 0)
-          if (tid < 32) {
-            const double t = sum_partials(part1);
-            const double b = sqrt(t);
-            const double prev_b = it > 1 ? S.beta[it - 1] : 0.0;
-            const bool breakdown =
-                sb_no_breakdown(b, S.alpha[it], prev_b) != 1 && b <= 1e-13 * (fabs(S.alpha[it]) + prev_b + 1.0);
-            int acc_flag = 0;
-            double err = 0.0;
-            if (forced) {
-              acc_flag = (it == kf);
-            } else if (fixed_k) {
-              acc_flag = (it == p.m_max) || breakdown;
-            } else if (breakdown) {
-              acc_flag = 1;
-            } else if (it >= p.m_min && gersh_gate(it, S.alpha + 1, S.beta + 1, remaining)) {
-              // T_it: diagonal alpha[1..it], off-diagonal beta[1..it-1]; the
-              // estimate is evaluated only where Eq. (KryErr) applies
-              const double thr = p.tol * remaining / p.tau;
-              if (krylov_lead_rejects(it, S.alpha + 1, S.beta + 1, remaining, beta0 * b, thr)) {
-                err = 2.0 * thr + 1e-300;
-              } else {
-                small_expm_e1(it, S.alpha + 1, S.beta + 1, remaining, S.yr, S.yi, S.tr, S.ti);
-                const double yk = hypot(S.yr[it - 1], S.yi[it - 1]);
-                err = beta0 * b * yk;
-                acc_flag = err <= thr;
-              }
-            }
-            if (tid == 0) {
-              S.beta[it] = b;
-              S.scale[it + 1] = 1.0 / b;
-              S.dec[0] = acc_flag;
-              S.bcast[1] = err;
-            }
-          }
+          if (tid < 32) f64_decide(S, it, beta0, remaining, forced ? kf : 0, p);
           __syncthreads();
           if (S.dec[0]) {
             accepted = true;
@@ -508,7 +541,7 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
               err = beta0 * S.beta[it] * hypot(S.yr[it - 1], S.yi[it - 1]);
               if (err <= p.tol * ts / p.tau) { hh = h; break; }
             }
-            if (tid == 0) { S.dec[2] = hh; S.bcast[1] = err; }
+            if (tid == 0) { S.dec[1] = hh > 0; S.dec[2] = hh; S.bcast[1] = err; }
           }
           __syncthreads();
           acc_h = S.dec[2];
@@ -524,7 +557,8 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
       if (acc_k > 0) {
         // ---------------- reconstruct psi <- beta0 sum_i y_i q_i / ||q_i||
         if (tid < 32) {
-          small_expm_e1(acc_k, S.alpha + 1, S.beta + 1, ts, S.yr, S.yi, S.tr, S.ti);
+          if (!S.dec[1]) small_expm_e1(acc_k, S.alpha + 1, S.beta + 1, ts, S.yr, S.yi, S.tr, S.ti);
+          __syncwarp();
           for (int i = tid; i < acc_k; i += 32) {
             const double f = beta0 * S.scale[i + 1];
             S.cre[i] = f * S.yr[i];
@@ -533,7 +567,7 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
         }
         __syncthreads();
         double acc = 0.0;
-        for (int x = x0; x < dim; x += stride) {
+        for (int x = x0; x < xe; x += stride) {
           double re = 0.0, im = 0.0;
           for (int i = 0; i < acc_k; ++i) {
             const double2 v = vec(i + 1)[x];
@@ -546,15 +580,8 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
           p.psi[x] = make_double2(re, im);
           acc = fma(re, re, fma(im, im, acc));
         }
-        {
-          const double s = block_sum(acc, S.red);
-          if (tid == 0) part2[blockIdx.x] = s;
-        }
-        if (!grid_barrier(p.bar, gen, &st->status, p.timeout_ns, &S.ok)) return;
-        if (tid < 32) {
-          const double t = sum_partials(part2);
-          if (tid == 0) S.bcast[0] = sqrt(t);
-        }
+        if (!f64_reduce(S, acc, true, ++tag, p)) return;
+        if (tid == 0) S.bcast[0] = sqrt(S.sum);
         __syncthreads();
         beta0 = S.bcast[0];
       }
@@ -581,6 +608,7 @@ __global__ void __launch_bounds__(256) k_propagate(PropParams p, Op op) {
     if (lead && p.r_nsub != nullptr) p.r_nsub[eg] = nsub_e;
   }
   if (lead) {
+    st->tag_base = tag;
     st->forced_pos = fpos;
     st->rec_pos = rpos;
     st->n_exp += p.nexp;

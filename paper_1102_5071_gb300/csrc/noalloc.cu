@@ -14,6 +14,7 @@
 // holds it (kStaticBytes, about 2.1 MiB) until the process exits.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -26,9 +27,10 @@ namespace {
 
 constexpr int kStaticMaxSites = 12;     // dim <= 4096
 constexpr int kStaticMaxKrylov = 32;    // m_max <= 32
-constexpr int kStaticBlock = 256;
+constexpr int kStaticBlock = 256;       // one CTA up to this dimension
+constexpr int kStaticPart = 128;        // elements per CTA above it (four warps feed an SM's FP64 pipes)
 constexpr int kStaticMaxDim = 1 << kStaticMaxSites;
-constexpr int kStaticMaxGrid = kStaticMaxDim / kStaticBlock;  // one element per thread at most
+constexpr int kStaticMaxGrid = kStaticMaxDim / kStaticPart;  // one element per thread
 
 constexpr size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
 
@@ -40,7 +42,7 @@ constexpr size_t kOffH = kOffDzHi + align256(sizeof(double) * (1 << (kStaticMaxS
 constexpr size_t kOffXf = kOffH + align256(sizeof(double) * kStaticMaxSites);
 constexpr size_t kOffScal = kOffXf + align256(sizeof(double) * kStaticMaxSites);
 constexpr size_t kOffPart = kOffScal + align256(sizeof(double) * 2);
-constexpr size_t kOffBar = kOffPart + align256(sizeof(double) * 3 * kStaticMaxGrid);
+constexpr size_t kOffBar = kOffPart + align256(sizeof(double) * kExchWords * kStaticMaxGrid);
 constexpr size_t kOffSt = kOffBar + align256(sizeof(unsigned) * 2);
 constexpr size_t kStaticBytes = kOffSt + align256(sizeof(DevStatus));
 
@@ -122,6 +124,7 @@ extern "C" cfet_status cfet_expv_chain_static(int32_t nsites, double J, double D
       cudaMemcpyAsync(d_xf, a, sizeof(double) * N, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
       cudaMemcpyAsync(d_scal, scal, sizeof(scal), cudaMemcpyHostToDevice, cs) != cudaSuccess ||
       cudaMemsetAsync(d_st, 0, sizeof(DevStatus), cs) != cudaSuccess ||
+      cudaMemsetAsync(d_part, 0, sizeof(double) * kExchWords * kStaticMaxGrid, cs) != cudaSuccess ||
       cudaMemsetAsync(d_bar, 0, sizeof(unsigned) * 2, cs) != cudaSuccess)
     return CFET_ECUDA;
   if (launch_spin_tables(N, L, J, Delta, d_h, dz_lo, dz_hi, cs) != cudaSuccess) return CFET_ECUDA;
@@ -150,9 +153,10 @@ extern "C" cfet_status cfet_expv_chain_static(int32_t nsites, double J, double D
   p.bar = d_bar;
   p.st = d_st;
   p.timeout_ns = 2000000000LL;
-  int grid = (dim + kStaticBlock - 1) / kStaticBlock;
+  int grid = dim <= kStaticBlock ? 1 : dim / kStaticPart;
   if (grid > s->max_grid) grid = s->max_grid;
-  if (launch_propagate_spin(p, op, grid, kStaticBlock, cs) != cudaSuccess) return CFET_ECUDA;
+  const int block = grid == 1 ? std::max(64, std::min(dim, kStaticBlock)) : kStaticPart;
+  if (launch_propagate_spin(p, op, grid, block, cs) != cudaSuccess) return CFET_ECUDA;
 
   DevStatus hs;
   if (cudaMemcpyAsync(&hs, d_st, sizeof(DevStatus), cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
