@@ -100,6 +100,7 @@ struct FmtF64 {
   static __device__ __forceinline__ Acc shfl_down(const Acc& a, int o) {
     return Acc{__shfl_down_sync(0xffffffffu, a.s, o)};
   }
+  static __device__ __forceinline__ Acc shfl(const Acc& a, int l) { return Acc{__shfl_sync(0xffffffffu, a.s, l)}; }
   static __device__ __forceinline__ double value(const Acc& a) { return a.s; }
   static __device__ __forceinline__ void ld2(const V* p, V& a, V& b) { a = p[0]; b = p[1]; }
   static __device__ __forceinline__ void st2(V* p, V a, V b) { p[0] = a; p[1] = b; }
@@ -135,6 +136,9 @@ struct FmtC64 {
   }
   static __device__ __forceinline__ Acc shfl_down(const Acc& a, int o) {
     return Acc{__shfl_down_sync(0xffffffffu, a.s, o), __shfl_down_sync(0xffffffffu, a.c, o)};
+  }
+  static __device__ __forceinline__ Acc shfl(const Acc& a, int l) {
+    return Acc{__shfl_sync(0xffffffffu, a.s, l), __shfl_sync(0xffffffffu, a.c, l)};
   }
   static __device__ __forceinline__ double value(const Acc& a) { return (double)a.s + (double)a.c; }
   // element pairs (even index): one 16-byte access
@@ -181,37 +185,55 @@ constexpr int kBatchStageMax = 200 * 1024;   // staged bytes of one CTA, at most
 constexpr int kBatchStageHalf = 100 * 1024;  // two CTAs per SM
 
 // ------------------------------------------------------------------ reductions
-// Sum over the CTA (and over the cluster when coop) of per-thread partials;
-// the result is returned to every thread of the CTA.  Every CTA of a cluster
-// adds the partials in rank order, so all hold the same value.
+// Sum over the CTA (and over the cluster when coop) of the per-thread partials of
+// its first nact warps (the others hold none).  The result is returned to warp 0
+// only, which publishes what the other warps need of it before the barrier that
+// the caller adds.  Every CTA of a cluster adds the partials in rank order, so all
+// hold the same value; they are loaded side by side, one peer per lane.
+// Only the steps that can hold something are taken: an FP64 addition occupies the
+// pipe of a quarter SM for 64 cycles, and the error-free additions of the other
+// format are ten dependent instructions.
 template <class Fmt>
-__device__ double batch_reduce(SmemB<Fmt>& S, typename Fmt::Acc a, int& slot, bool coop, cg::cluster_group& cl) {
+__device__ __forceinline__ double batch_sum_in(SmemB<Fmt>& S, typename Fmt::Acc a, int nact, int slot, bool coop) {
+  using Acc = typename Fmt::Acc;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nw = (int)(blockDim.x >> 5);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) Fmt::add(a, Fmt::shfl_down(a, o));
-  if (lane == 0) S.wacc[warp] = a;
-  __syncthreads();
-  if (warp == 0) {
-    a = lane < nw ? S.wacc[lane] : Fmt::zero();
+  if (warp < nact) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) Fmt::add(a, Fmt::shfl_down(a, o));
-    if (lane == 0) S.cta[slot] = a;
+    if (lane == 0 && nact > 1) S.wacc[warp] = a;
+  }
+  if (nact > 1) {
+    __syncthreads();
+    if (warp == 0) {
+      a = lane < nact ? S.wacc[lane] : Fmt::zero();
+#pragma unroll 1
+      for (int o = nact > 8 ? 8 : nact > 4 ? 4 : nact > 2 ? 2 : 1; o > 0; o >>= 1) Fmt::add(a, Fmt::shfl_down(a, o));
+    }
   }
   if (coop) {
+    cg::cluster_group cl = cg::this_cluster();
+    if (threadIdx.x == 0) S.cta[slot] = a;
     cl.sync();  // release / acquire at cluster scope: partials and vector stores
-    if (threadIdx.x == 0) {
-      typename Fmt::Acc t = Fmt::zero();
+    if (warp == 0) {
       const int nb = (int)cl.num_blocks();
-      for (int r = 0; r < nb; ++r) Fmt::add(t, *cl.map_shared_rank(&S.cta[slot], r));
-      S.result = Fmt::value(t);
+      const Acc r = lane < nb ? *cl.map_shared_rank(&S.cta[slot], lane) : Fmt::zero();
+      a = Fmt::zero();
+      for (int i = 0; i < nb; ++i) Fmt::add(a, Fmt::shfl(r, i));
     }
-  } else if (threadIdx.x == 0) {
-    S.result = Fmt::value(S.cta[slot]);
   }
-  __syncthreads();
-  slot ^= 1;
-  return S.result;
+  return warp == 0 ? __shfl_sync(0xffffffffu, Fmt::value(a), 0) : 0.0;
+}
+template <class Fmt>
+__device__ __noinline__ double batch_sum_call(SmemB<Fmt>& S, typename Fmt::Acc a, int nact, int slot, bool coop) {
+  return batch_sum_in<Fmt>(S, a, nact, slot, coop);
+}
+// In line where registers allow it (one CTA per SM at least: 128 of them): 206 chains
+// of 7 sites take 0.224 ms against 0.238.  Out of line in the 64-register form, whose
+// scalar warp spilled 470 bytes otherwise: 256 chains of 10..16 sites 6.9 against 7.2.
+template <class Fmt, int PER_SM>
+__device__ __forceinline__ double batch_sum(SmemB<Fmt>& S, typename Fmt::Acc a, int nact, int slot, bool coop) {
+  if constexpr (PER_SM == 1) return batch_sum_in<Fmt>(S, a, nact, slot, coop);
+  else return batch_sum_call<Fmt>(S, a, nact, slot, coop);
 }
 
 // ------------------------------------------------------------------ apply
@@ -268,14 +290,15 @@ __device__ __forceinline__ typename Fmt::V batch_apply(const typename Fmt::V* __
 // the element passes keep few enough registers for two CTAs of 512 threads per SM)
 // beta and the decision of iteration it.  kf: the forced Krylov dimension, 0 for none.
 template <class Fmt>
-__device__ __noinline__ void batch_decide(SmemB<Fmt>& S, int it, double bsum, double beta0, const BParams& P, int kf) {
+__device__ __noinline__ void batch_decide(SmemB<Fmt>& S, int it, double bsum, double beta0, double tol, double tau,
+                                          int m_min, int m_max, int kf) {
   const double remaining = S.remaining;
   const int lane = threadIdx.x & 31;
   const double b = sqrt(bsum);
   const double prev_b = it > 1 ? S.beta[it - 1] : 0.0;
   const bool breakdown =
       sb_no_breakdown(b, S.alpha[it], prev_b) != 1 && b <= 1e-13 * (fabs(S.alpha[it]) + prev_b + 1.0);
-  const bool fixed_k = P.tol <= 0.0;
+  const bool fixed_k = tol <= 0.0;
   if (lane == 0) {
     S.beta[it] = b;
     S.scale[it + 1] = div_call(1.0, b);
@@ -286,11 +309,11 @@ __device__ __noinline__ void batch_decide(SmemB<Fmt>& S, int it, double bsum, do
   if (kf > 0) {
     acc_flag = (it == kf);
   } else if (fixed_k) {
-    acc_flag = (it == P.m_max) || breakdown;
+    acc_flag = (it == m_max) || breakdown;
   } else if (breakdown) {
     acc_flag = 1;
-  } else if (it >= P.m_min && gersh_gate(it, S.alpha + 1, S.beta + 1, remaining)) {
-    const double thr = P.tol * remaining / P.tau;
+  } else if (it >= m_min && gersh_gate(it, S.alpha + 1, S.beta + 1, remaining)) {
+    const double thr = tol * remaining / tau;
     if (krylov_lead_rejects(it, S.alpha + 1, S.beta + 1, remaining, beta0 * b, thr)) {
       err = 2.0 * thr + 1e-300;
     } else {
@@ -440,7 +463,7 @@ __device__ __forceinline__ void batch_apply2(const typename Fmt::V* sq, const ty
 // (every pass that forms it writes it there and to the basis): the neighbour sums
 // then read shared memory instead of gathering through L1 from L2, which served
 // most of a large instance's flips and hops.
-template <class Fmt>
+template <class Fmt, int PER_SM>
 __device__ void run_instance(const BParams& P, int ii, int part, int nparts, bool coop, SmemB<Fmt>& S,
                              cg::cluster_group& cl) {
   using V = typename Fmt::V;
@@ -466,6 +489,9 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
   const int x0 = part * chunk + tid, xe = min(dim, (part + 1) * chunk);
   const int step = blockDim.x;
   const int jn = part * chunk < dim ? chunk : 0;  // staged passes: pairs j = 2 tid, 2 tid + 2 step, ...
+  // warps that hold elements in the element-wise passes and in those over pairs
+  const int nact_x = max(1, min(step, (xe - part * chunk) + 31) >> 5);
+  const int nact = staged ? max(1, min(step, (jn >> 1) + 31) >> 5) : nact_x;
   V* const sq = reinterpret_cast<V*>(reinterpret_cast<unsigned char*>(&S) + stage_offset<Fmt>());
   const int xb = part * chunk;
   const T* dz_lo = reinterpret_cast<const T*>(I.dz);
@@ -487,9 +513,11 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
       Fmt::add_prod(a, f.x, f.x);
       Fmt::add_prod(a, f.y, f.y);
     }
-    const double s = batch_reduce<Fmt>(S, a, slot, coop, cl);
-    if (!isfinite(s)) status = CFET_ENAN;
-    beta0 = sqrt(s);
+    const double s = batch_sum<Fmt, PER_SM>(S, a, nact_x, slot ^= 1, coop);
+    if (w0) S.result = sqrt(s);
+    __syncthreads();
+    beta0 = S.result;
+    if (!isfinite(beta0)) status = CFET_ENAN;
   }
 
   for (long long e = 0; e < P.nexp && status == 0; ++e) {
@@ -515,13 +543,10 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
       double acc_err = 0.0;
       if (beta0 != 0.0) {
         const int klimit = forced ? kf : P.m_max;
-        if (tid == 0) S.scale[1] = 1.0 / beta0;
-        int it = 1;
-        bool accepted = false;
-        for (;; ++it) {
-          // constants of u = s_it H_j q_it - beta_{it-1} s_{it-1} q_{it-1}
-          if (tid == 0) {
-            const double sk = S.scale[it];
+        // constants of u = s_it H_j q_it - beta_{it-1} s_{it-1} q_{it-1} (warp 0)
+        auto consts = [&](int it) {
+          const double sk = S.scale[it];
+          if (lane == 0) {
             const double cz = c0 * sk;
             S.cz = (T)cz;
             S.ch = (T)(cz * I.J2);
@@ -529,8 +554,17 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
             S.cp = it > 1 ? (T)(-S.beta[it - 1] * S.scale[it - 1]) : (T)0;
             S.use_prev = it > 1;
           }
-          if (!I.uniform && tid < N) S.bx[tid] = (T)(S.bsite[tid] * S.scale[it]);
-          __syncthreads();
+          if (!I.uniform && lane < N) S.bx[lane] = (T)(S.bsite[lane] * sk);
+        };
+        if (w0) {
+          if (lane == 0) S.scale[1] = 1.0 / beta0;
+          __syncwarp();
+          consts(1);
+        }
+        __syncthreads();
+        int it = 1;
+        bool accepted = false;
+        for (;; ++it) {
           Acc a = Fmt::zero();
           {
             const V* q = Q(it);
@@ -555,9 +589,10 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
               Fmt::add_prod(a, v.y, hv.y);
             }
           }
-          const double s_it = S.scale[it];
-          const double alpha = batch_reduce<Fmt>(S, a, slot, coop, cl) * s_it;
+          const double asum = batch_sum<Fmt, PER_SM>(S, a, nact, slot ^= 1, coop);
           if (tid == 0) {
+            const double s_it = S.scale[it];
+            const double alpha = asum * s_it;
             S.alpha[it] = alpha;
             S.am = (T)(-alpha * s_it);
           }
@@ -591,8 +626,12 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
               Fmt::add_prod(a, w.y, w.y);
             }
           }
-          const double bsum = batch_reduce<Fmt>(S, a, slot, coop, cl);
-          if (w0) batch_decide<Fmt>(S, it, bsum, beta0, P, forced ? kf : 0);
+          const double bsum = batch_sum<Fmt, PER_SM>(S, a, nact, slot ^= 1, coop);
+          if (w0) {
+            batch_decide<Fmt>(S, it, bsum, beta0, P.tol, P.tau, P.m_min, P.m_max, forced ? kf : 0);
+            __syncwarp();
+            if (!S.accept_now && it < klimit) consts(it + 1);
+          }
           __syncthreads();
           if (S.accept_now) {
             accepted = true;
@@ -636,7 +675,10 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
           Fmt::add_prod(a, re, re);
           Fmt::add_prod(a, im, im);
         }
-        beta0 = sqrt(batch_reduce<Fmt>(S, a, slot, coop, cl));
+        const double s = batch_sum<Fmt, PER_SM>(S, a, nact_x, slot ^= 1, coop);
+        if (w0) S.result = sqrt(s);
+        __syncthreads();
+        beta0 = S.result;
       }
       __syncthreads();  // everyone has read the step's state
       if (tid == 0) {
@@ -675,8 +717,12 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
 }
 
 // ------------------------------------------------------------------ the kernel
-template <class Fmt>
-__global__ void __launch_bounds__(512, 2) k_batch_propagate(BParams P) {
+// PER_SM = 1: 128 registers, for launches whose items are all resident at once that
+// way (latency-bound: the scalar work and the sums keep their values in registers,
+// 206 chains of 7 sites 0.32 ms FP64 / 0.224 complex64 against 0.34 / 0.25); PER_SM = 2:
+// 64 registers, two CTAs of 512 threads per SM.
+template <class Fmt, int PER_SM>
+__global__ void __launch_bounds__(512, PER_SM) k_batch_propagate(BParams P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmemB<Fmt>& S = *reinterpret_cast<SmemB<Fmt>*>(smem_raw);
   cg::cluster_group cl = cg::this_cluster();
@@ -688,9 +734,9 @@ __global__ void __launch_bounds__(512, 2) k_batch_propagate(BParams P) {
     if (item >= P.nitems) break;
     const BItem& it = P.items[item];
     if (it.coop) {
-      run_instance<Fmt>(P, it.inst[0], rank, (int)cl.num_blocks(), true, S, cl);
+      run_instance<Fmt, PER_SM>(P, it.inst[0], rank, (int)cl.num_blocks(), true, S, cl);
     } else if (rank < it.n) {
-      run_instance<Fmt>(P, it.inst[rank], 0, 1, false, S, cl);
+      run_instance<Fmt, PER_SM>(P, it.inst[rank], 0, 1, false, S, cl);
     }
     cl.sync();  // the item is done in every CTA before rank 0 takes the next
   }
@@ -698,7 +744,7 @@ __global__ void __launch_bounds__(512, 2) k_batch_propagate(BParams P) {
 }
 
 template <class Fmt>
-int launch_batch(const BParams& p, int clusters, int cluster_size, int threads, void* stream) {
+int launch_batch(const BParams& p, int clusters, int cluster_size, int threads, bool roomy, void* stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(clusters * cluster_size);
   cfg.blockDim = dim3(threads);
@@ -711,12 +757,13 @@ int launch_batch(const BParams& p, int clusters, int cluster_size, int threads, 
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return (int)cudaLaunchKernelEx(&cfg, k_batch_propagate<Fmt>, p);
+  return (int)cudaLaunchKernelEx(&cfg, roomy ? k_batch_propagate<Fmt, 1> : k_batch_propagate<Fmt, 2>, p);
 }
 
 template <class Fmt>
-int max_clusters(int cluster_size, int threads, int stage_bytes) {
-  if (cudaFuncSetAttribute(k_batch_propagate<Fmt>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+int max_clusters(int cluster_size, int threads, int stage_bytes, bool roomy) {
+  auto* const kernel = roomy ? k_batch_propagate<Fmt, 1> : k_batch_propagate<Fmt, 2>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            stage_offset<Fmt>() + kBatchStageMax) != cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -733,7 +780,7 @@ int max_clusters(int cluster_size, int threads, int stage_bytes) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, k_batch_propagate<Fmt>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -881,7 +928,9 @@ int stage_bytes_for(const cfet_batch* b, const cfet_batch_plan& pl) {
 // (bound by the FP64 units, vectors twice as large): clusters of 4 from 13
 // sites, 25.9 ms a step (31.4 with the former default, 31.4 with clusters of 8).
 // CTAs of 256 threads where the spread instances give each SM more than two
-// CTAs of short parts (100 chains of 12..14 sites: 1.93 against 2.34 ms); the
+// CTAs of short parts (100 chains of 12..14 sites: 1.93 against 2.34 ms), and of
+// 256 or 128 where no part reaches 1024 or 256 elements (206 FP64 chains of 7
+// sites: 0.32 ms with 128 threads, 0.35 with 512); the
 // part of a spread instance is at least 256 elements.
 cfet_batch_plan default_plan(const cfet_batch* b) {
   const bool c64 = b->precision == CFET_PREC_C64;
@@ -892,8 +941,17 @@ cfet_batch_plan default_plan(const cfet_batch* b) {
   pl.coop_min_sites = std::max(11, std::min(c64 ? 14 : 13, nmax - 1));
   long long spread = 0;
   for (int i = 0; i < b->n; ++i) spread += b->chains[i].nsites >= pl.coop_min_sites;
-  const bool short_parts = (1LL << nmax) / pl.cluster_size < 4096;
-  pl.threads = short_parts && spread * pl.cluster_size > 304 ? 256 : 512;
+  int lg = 0;
+  while ((1 << lg) < pl.cluster_size) ++lg;
+  int lc = 0;  // log2 of the largest part of a CTA
+  for (int i = 0; i < b->n; ++i) {
+    const int N = b->chains[i].nsites;
+    lc = std::max(lc, N >= pl.coop_min_sites ? N - lg : N);
+  }
+  if (lc < 10)
+    pl.threads = lc < 8 ? 128 : 256;
+  else
+    pl.threads = nmax - lg < 12 && spread * pl.cluster_size > 304 ? 256 : 512;
   pl.tuned_ms = 0.f;
   return pl;
 }
@@ -1029,8 +1087,14 @@ cfet_status run_batch(cfet_batch* b, const cfet_batch_plan& pl, double2* const* 
   const std::vector<BItem> items = make_items(b, pl);
   const int stage = stage_bytes_for(b, pl);
   p.stage_bytes = stage;
-  const int maxc = b->precision == CFET_PREC_C64 ? max_clusters<FmtC64>(pl.cluster_size, pl.threads, stage)
-                                                 : max_clusters<FmtF64>(pl.cluster_size, pl.threads, stage);
+  auto resident = [&](bool roomy) {
+    return b->precision == CFET_PREC_C64 ? max_clusters<FmtC64>(pl.cluster_size, pl.threads, stage, roomy)
+                                         : max_clusters<FmtF64>(pl.cluster_size, pl.threads, stage, roomy);
+  };
+  // the 128-register form where its CTAs hold all items at once
+  int maxc = resident(true);
+  const bool roomy = maxc >= (int)items.size();
+  if (!roomy) maxc = resident(false);
   if (maxc < 1) return bfail(b, CFET_EINVAL, "plan cannot be launched (no cluster fits on the device)");
   const int clusters = std::min<int>((int)items.size(), maxc);
   // the previous launch may still read the tables: order on the stream
@@ -1055,8 +1119,8 @@ cfet_status run_batch(cfet_batch* b, const cfet_batch_plan& pl, double2* const* 
   p.stat = b->d_stat;
   BCK(cudaEventRecord(b->ev0, s), "event");
   const int e = b->precision == CFET_PREC_C64
-                    ? launch_batch<FmtC64>(p, clusters, pl.cluster_size, pl.threads, s)
-                    : launch_batch<FmtF64>(p, clusters, pl.cluster_size, pl.threads, s);
+                    ? launch_batch<FmtC64>(p, clusters, pl.cluster_size, pl.threads, roomy, s)
+                    : launch_batch<FmtF64>(p, clusters, pl.cluster_size, pl.threads, roomy, s);
   if (e != cudaSuccess) return bcuda(b, (cudaError_t)e, "batch kernel launch");
   BCK(cudaEventRecord(b->ev1, s), "event");
   BCK(cudaMemcpyAsync(b->h_stat, b->d_stat, (size_t)b->n * sizeof(BStat), cudaMemcpyDeviceToHost, s),
