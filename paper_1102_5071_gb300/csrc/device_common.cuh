@@ -30,42 +30,6 @@ static __device__ __forceinline__ long long sm_clock() {
   asm volatile("mov.u64 %0, %%clock64;" : "=l"(t) : : "memory");
   return t;
 }
-// Bounded grid barrier executed by one warp of each CTA (lane 0 arrives and
-// spins; `spin` accumulates its SM cycles).  Returns false in every lane when
-// the wait limit expired or another CTA reported an error.
-static __device__ bool warp_grid_barrier(unsigned* bar, unsigned& gen, int* status, long long timeout_ns, long long& spin) {
-  const int lane = threadIdx.x & 31;
-  int ok = 1;
-  if (gridDim.x > 1 && lane == 0) {
-    const long long c0 = sm_clock();
-    const unsigned target = gen + 1;
-    __threadfence();
-    const unsigned arrived = atomicAdd(&bar[0], 1u) + 1u;
-    if (arrived == gridDim.x) {
-      atomicExch(&bar[0], 0u);
-      __threadfence();
-      atomicExch(&bar[1], target);
-    } else {
-      const long long t0 = global_timer_ns();
-      unsigned spins = 0;
-      while (ld_volatile_u32(&bar[1]) != target) {
-        if ((++spins & 63u) == 0u) {
-          if (ld_volatile_i32(status) != 0) { ok = 0; break; }
-          if (global_timer_ns() - t0 > timeout_ns) {
-            atomicCAS(status, 0, (int)CFET_ETIMEOUT);
-            ok = 0;
-            break;
-          }
-        }
-      }
-    }
-    __threadfence();
-    spin += sm_clock() - c0;
-  }
-  gen += 1;
-  ok = __shfl_sync(0xffffffffu, ok, 0);
-  return ok != 0;
-}
 
 // ------------------------------------------------------------------ tagged exchange
 // Grid-wide exchange of small per-CTA records, executed by one warp of each
@@ -377,31 +341,6 @@ __device__ __forceinline__ double sum_partials(const double* part) {
   for (int i = lane; i < (int)gridDim.x; i += 32) s += part[i];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
-}
-
-// Maximum over the CTA of one double per thread; result valid in thread 0.
-__device__ __forceinline__ double block_max(double v, double* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0) {
-    const int nw = blockDim.x >> 5;
-    for (int i = 0; i < nw; ++i) s = fmax(s, red[i]);
-  }
-  return s;
-}
-
-// Maximum of the per-CTA partials (warp 0, result in all lanes of warp 0).
-__device__ __forceinline__ double max_partials(const double* part) {
-  const int lane = threadIdx.x & 31;
-  double s = 0.0;
-  for (int i = lane; i < (int)gridDim.x; i += 32) s = fmax(s, part[i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
   return s;
 }
 

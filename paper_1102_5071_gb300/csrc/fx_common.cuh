@@ -44,12 +44,6 @@ __device__ __forceinline__ int fx_exp_for(double bound, int bits) {
   if (b <= 0 || ex < 1023 - 963 || ex > 1023 + 963) return -960;
   return fx_ilog2_up(bound) - (bits - 1);
 }
-// Left shift that brings a value of magnitude <= a (a >= 1) to < 2^62.
-__device__ __forceinline__ int fx_norm_shift(double a) {
-  if (__double_as_longlong(a) < 0x3FF0000000000000LL) return 0;  // a < 1 (or negative)
-  const int p = 61 - fx_ilog2_up(a);
-  return p < 0 ? 0 : (p > 61 ? 61 : p);
-}
 // x * 2^e exactly, by exponent arithmetic when the result stays normal.
 __device__ __forceinline__ double fx_scale2(double x, int e) {
   const long long b = __double_as_longlong(x);

@@ -30,10 +30,10 @@
 // already apply H for iteration k+1, as in the fixed-point kernel).
 //
 // Chains of 17 to 21 sites: the staged form keeps the applied vector in the shared
-// memory of 128 CTAs (clusters of four).  Long chains: the tiled form applies H in window passes over
-// shared-memory tiles moved by TMA (tiled_common.cuh) instead of element by
-// element; its window 0 also does the previous iteration's orthogonalisation
-// step, so it has one grid exchange per iteration less.
+// memory of 128 CTAs (clusters of four).  Long chains: the tiled form applies H in
+// window passes over shared-memory tiles moved by TMA (tiled_common.cuh) instead
+// of element by element; its window 0 also does the previous iteration's
+// orthogonalisation step, so it has one grid exchange per iteration less.
 #include <cuda_runtime.h>
 
 #include <cmath>

@@ -32,11 +32,11 @@
 // iteration k+1; if it accepts k, that apply is discarded.  The accepted
 // estimate's y = exp(-i tau T_k) e_1 is reused for the reconstruction.
 //
-// Long chains.  The TILED instantiation replaces the element-wise spin apply
+// Long chains.  The kFxTiled instantiation replaces the element-wise spin apply
 // by window passes over shared-memory tiles moved by TMA (tiled_common.cuh)
 // separated by grid exchanges, for chains whose vectors leave L2.  Small
-// problems.  The SMALL instantiation runs one CTA with the whole Krylov basis
-// in shared memory.
+// problems.  kFxSmall runs one CTA with the whole Krylov basis in shared memory,
+// kFxCluster one thread-block cluster with the applied vector staged in it.
 #include <cuda_runtime.h>
 
 #include <cmath>

@@ -49,12 +49,6 @@ __host__ __device__ __forceinline__ int tile_x(const TileWin& W, int t, int j) {
   return (j & ((1 << W.c) - 1)) | (tl << W.c) | ((j >> W.c) << W.b0) | (th << (W.b0 + W.width));
 }
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 // Barrier of the n worker threads only (named barrier 1).
 __device__ __forceinline__ void workers_sync(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
 // Hand-over between the workers and the control warp around a window exchange
