@@ -485,7 +485,14 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
   int lc = N - (31 - __clz(nparts));
   if (lc < 6) lc = min(N, 6);
   const int chunk = 1 << lc;
-  const bool staged = chunk * (int)sizeof(V) <= P.stage_bytes;
+  // parts of at most four warps of elements: one element per thread (pairs would
+  // leave the FP64 pipes of half the SM idle), from the staged vector as well: 206
+  // FP64 chains of 7 sites 0.310 ms (0.324 in pairs).  Only where registers allow
+  // it; the 64-register form would spill more in its paths for larger instances
+  // (256 chains of 10..16 sites complex64 8.4 ms a pass against 7.9).
+  const bool fits = chunk * (int)sizeof(V) <= P.stage_bytes;
+  const bool single = PER_SM == 1 && fits && nparts == 1 && chunk <= 128;
+  const bool staged = fits && !single;
   const int x0 = part * chunk + tid, xe = min(dim, (part + 1) * chunk);
   const int step = blockDim.x;
   const int jn = part * chunk < dim ? chunk : 0;  // staged passes: pairs j = 2 tid, 2 tid + 2 step, ...
@@ -509,7 +516,7 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
     for (int x = x0; x < xe; x += step) {
       const V f = Fmt::from64(I.psi[x]);
       Q(1)[x] = f;
-      if (staged) sq[x - xb] = f;
+      if (fits) sq[x - xb] = f;
       Fmt::add_prod(a, f.x, f.x);
       Fmt::add_prod(a, f.y, f.y);
     }
@@ -567,7 +574,7 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
         for (;; ++it) {
           Acc a = Fmt::zero();
           {
-            const V* q = Q(it);
+            const V* q = single ? sq : Q(it);
             const V* qm = it > 1 ? Q(it - 1) : q;
             V* u = Q(it + 1);
             if (staged) {
@@ -600,7 +607,7 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
           a = Fmt::zero();
           {
             const T am = S.am;
-            const V* q = Q(it);
+            const V* q = single ? sq : Q(it);
             V* u = Q(it + 1);
             if (staged) {
               for (int j = 2 * tid; j < jn; j += 2 * step) {
@@ -622,6 +629,7 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
               const V uu = u[x];
               const V w = Fmt::make(fma(am, v.x, uu.x), fma(am, v.y, uu.y));
               u[x] = w;
+              if (single) sq[x] = w;
               Fmt::add_prod(a, w.x, w.x);
               Fmt::add_prod(a, w.y, w.y);
             }
@@ -670,7 +678,7 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
             im = fma(cr, v.y, fma(ci, v.x, im));
           }
           Q(1)[x] = Fmt::make(re, im);
-          if (staged) sq[x - xb] = Fmt::make(re, im);
+          if (fits) sq[x - xb] = Fmt::make(re, im);
           if (final_rec) I.psi[x] = make_double2((double)re, (double)im);
           Fmt::add_prod(a, re, re);
           Fmt::add_prod(a, im, im);
@@ -719,7 +727,7 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
 // ------------------------------------------------------------------ the kernel
 // PER_SM = 1: 128 registers, for launches whose items are all resident at once that
 // way (latency-bound: the scalar work and the sums keep their values in registers,
-// 206 chains of 7 sites 0.32 ms FP64 / 0.224 complex64 against 0.34 / 0.25); PER_SM = 2:
+// 206 chains of 7 sites 0.31 ms FP64 / 0.224 complex64 against 0.34 / 0.25); PER_SM = 2:
 // 64 registers, two CTAs of 512 threads per SM.
 template <class Fmt, int PER_SM>
 __global__ void __launch_bounds__(512, PER_SM) k_batch_propagate(BParams P) {
@@ -930,7 +938,7 @@ int stage_bytes_for(const cfet_batch* b, const cfet_batch_plan& pl) {
 // CTAs of 256 threads where the spread instances give each SM more than two
 // CTAs of short parts (100 chains of 12..14 sites: 1.93 against 2.34 ms), and of
 // 256 or 128 where no part reaches 1024 or 256 elements (206 FP64 chains of 7
-// sites: 0.32 ms with 128 threads, 0.35 with 512); the
+// sites: 0.31 ms with 128 threads, 0.35 with 512); the
 // part of a spread instance is at least 256 elements.
 cfet_batch_plan default_plan(const cfet_batch* b) {
   const bool c64 = b->precision == CFET_PREC_C64;
