@@ -1257,7 +1257,7 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
   if (ctx->precision == CFET_PREC_FX && o.expm == CFET_EXPM_KRYLOV && ctx->grid == 1 && !ctx->tiled) {
     // a single CTA: the basis fits in its shared memory for small problems
     const size_t sb = fx_small_smem_bytes(dim, o.m_max);
-    if (sb > 0 && fx_small_prepare(sb) == 0) {
+    if (sb > 0 && fx_small_prepare() == 0) {
       ctx->small_fx = true;
       ctx->small_block = 32 + std::min(ctx->block - 32, ((dim << lane_bits) + 31) / 32 * 32);
     }

@@ -310,10 +310,12 @@ int launch_propagate_spin_fx(const PropParams& p, const OpSpinFx& op, int grid, 
 int launch_propagate_dia_fx(const PropParams& p, const OpDiaFx& op, int grid, int block, void* stream);
 int launch_propagate_csr_fx(const PropParams& p, const OpCsrFx& op, int grid, int block, void* stream);
 int max_coresident_blocks_fx(int family, int block, bool tiled);
+// Dynamic shared memory of a CTA that keeps vectors in it, at most: the limit that
+// those kernels are given (a kernel has one, shared by every context).
+constexpr size_t kStagedSmemMax = 200 * 1024;
 // One-CTA fixed-point launches with the Krylov basis in shared memory.
-constexpr size_t kFxSmallSmemMax = 200 * 1024;
 size_t fx_small_smem_bytes(int dim, int m_max);
-int fx_small_prepare(size_t bytes);
+int fx_small_prepare();
 constexpr int kFxClusterMaxSites = 13;
 size_t fx_cluster_smem_bytes(int part);
 int fx_cluster_prepare(int dim, int most, int block);

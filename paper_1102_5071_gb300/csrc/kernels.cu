@@ -873,10 +873,12 @@ int launch_wait_selftest(int which, unsigned long long* rec, unsigned* bar, int*
   return (int)cudaGetLastError();
 }
 // Whether `grid` CTAs of `block` threads and `bytes` of dynamic shared memory of
-// the kernel, in clusters of cs, are all resident at once.
+// the kernel, in clusters of cs, are all resident at once.  The kernel's limit is
+// one value for all contexts of the process, so it is the largest that any asks
+// for, whatever this one needs.
 bool staged_fits(const void* kernel, int grid, int cs, int block, size_t bytes) {
-  if (bytes > kFxSmallSmemMax ||
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
+  if (bytes > kStagedSmemMax ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmemMax) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }

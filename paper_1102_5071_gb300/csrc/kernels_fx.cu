@@ -1215,18 +1215,18 @@ size_t fx_tiled_smem_bytes() {
 // does not fit in an SM's shared memory).
 size_t fx_small_smem_bytes(int dim, int m_max) {
   const size_t b = ((sizeof(SmemFx) + 127) & ~size_t(127)) + (size_t)(m_max + 1) * dim * sizeof(longlong2);
-  return b <= kFxSmallSmemMax ? b : 0;
+  return b <= kStagedSmemMax ? b : 0;
 }
 
-int fx_small_prepare(size_t bytes) {
+int fx_small_prepare() {
   cudaError_t e = cudaFuncSetAttribute(k_propagate_fx<kFamilySpin, OpSpinFx, kFxSmall>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_propagate_fx<kFamilyDia, OpDiaFx, kFxSmall>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_propagate_fx<kFamilyCsr, OpCsrFx, kFxSmall>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmemMax);
   return (int)e;
 }
 
@@ -1235,13 +1235,13 @@ int fx_small_prepare(size_t bytes) {
 int fx_cluster_prepare(int dim, int most, int block) {
   const void* k = (const void*)k_propagate_fx<kFamilySpin, OpSpinFx, kFxCluster>;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) cudaGetLastError();
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmemMax) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
   for (int cs = most; cs >= 2; cs /= 2) {
     const size_t bytes = fx_cluster_smem_bytes(dim / cs);
-    if (bytes > kFxSmallSmemMax) return 0;  // smaller clusters need more
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
+    if (bytes > kStagedSmemMax) return 0;  // smaller clusters need more
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs);
     cfg.blockDim = dim3(block);
