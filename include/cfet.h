@@ -637,6 +637,15 @@ cfet_status cfet_selftest_ll_to_double_up(const int64_t* v, int64_t n, double* o
 cfet_status cfet_selftest_krylov_bounds(int32_t k, const double* a, const double* b, double ts, double* log2_bounds,
                                         int32_t* gate);
 
+/* Self-check of the record exchange of the persistent kernels (device): n
+ * exchanges over `grid` CTAs (2 to 256) in one launch, with the record widths
+ * of the kernels mixed, tags counted from first_tag (16 bits of which are
+ * stored; first_tag mod 65536 in [1, 65534]).  wrong[0]: sums that differ from
+ * the exact ones; wrong[1]: words of a CTA's record that do not carry the tag of
+ * their slot's last exchange.  Both 0 when all is well; CFET_EINVAL for
+ * arguments outside the ranges, CFET_ETIMEOUT when a wait gave up.            */
+cfet_status cfet_selftest_exchange(int32_t grid, uint32_t first_tag, int32_t n, int64_t* wrong);
+
 /* Dimension and drive-operator count of ctx (for bindings).                 */
 int64_t cfet_dim(const cfet_ctx* ctx);
 int32_t cfet_num_drives(const cfet_ctx* ctx);

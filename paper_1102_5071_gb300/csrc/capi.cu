@@ -145,7 +145,7 @@ namespace {
 
 // Exchange scratch per CTA (8-byte words): the two slots of the record exchange.
 constexpr size_t kPartialWordsPerCta = kExchWords;
-constexpr int kMaxCtlGrid = 256;  // 32 lanes x 8 records per lane of the exchange
+constexpr int kMaxCtlGrid = 256;  // CTAs of a record exchange, at most: each polls the records of all
 // (FP64 kernel with full re-orthogonalisation: 2 m_max Gram-Schmidt coefficients behind them.)
 static size_t partial_words_per_cta(const cfet_ctx* ctx) {
   return kPartialWordsPerCta + (ctx->opt.reorth ? 2 * (size_t)ctx->opt.m_max : 0);
@@ -1873,6 +1873,36 @@ cfet_status cfet_selftest_wait_timeout(int32_t which, double timeout_s, int32_t*
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "wait self test");
   *device_status = h;
   return h == CFET_ETIMEOUT ? CFET_OK : fail(nullptr, CFET_ECUDA, "wait self test: the wait did not time out");
+}
+
+cfet_status cfet_selftest_exchange(int32_t grid, uint32_t first_tag, int32_t n, int64_t* wrong) {
+  if (grid < 2 || grid > kMaxCtlGrid || n < 1 || n > 200000 || (first_tag & 0xffffu) < 1 ||
+      (first_tag & 0xffffu) > 0xfffeu || !wrong)
+    return fail(nullptr, CFET_EINVAL, "selftest: grid in [2, 256], n in [1, 200000], first_tag mod 65536 in [1, 65534]");
+  cfet_status s = device_available(nullptr);
+  if (s != CFET_OK) return s;
+  unsigned long long *rec = nullptr, *out = nullptr;
+  int* st = nullptr;
+  const size_t bytes = kPartialWordsPerCta * (size_t)grid * sizeof(unsigned long long);
+  unsigned long long h[2] = {0, 0};
+  int hs = 0;
+  cudaError_t e = cudaMalloc(&rec, bytes);
+  if (e == cudaSuccess) e = cudaMalloc(&out, sizeof(h));
+  if (e == cudaSuccess) e = cudaMalloc(&st, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(rec, 0, bytes);
+  if (e == cudaSuccess) e = cudaMemset(out, 0, sizeof(h));
+  if (e == cudaSuccess) e = cudaMemset(st, 0, sizeof(int));
+  if (e == cudaSuccess) e = (cudaError_t)launch_exchange_selftest(rec, first_tag, n, grid, st, out);
+  if (e == cudaSuccess) e = cudaMemcpy(h, out, sizeof(h), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(&hs, st, sizeof(int), cudaMemcpyDeviceToHost);
+  cudaFree(rec);
+  cudaFree(out);
+  cudaFree(st);
+  if (e != cudaSuccess) return cuda_fail(nullptr, e, "exchange self test");
+  if (hs != 0) return fail(nullptr, (cfet_status)hs, "exchange self test: a wait gave up");
+  wrong[0] = (int64_t)h[0];
+  wrong[1] = (int64_t)h[1];
+  return CFET_OK;
 }
 
 cfet_status cfet_probe_copy_gbs(void* a, void* b, int64_t bytes, int32_t reps, void* stream, double* gbs) {

@@ -42,12 +42,18 @@ static __device__ __forceinline__ long long sm_clock() {
 // 64-bit element of a 16-byte store or load is single-copy atomic); readers wait
 // until the words of every CTA carry `tag`.  No atomics and no last-arriver step:
 // one store and one round of loads per exchange.  Two slots alternate by the
-// parity of the tag, which counts the exchanges of a call from 1, so a stale
-// word always carries the tag of two exchanges before (the slots are cleared
-// per call), and a slot is rewritten only after every CTA has published in the
-// other one, that is, has read this one.  Lane l reads the records of CTAs l,
-// l + 32, ..., l + 32 (kExchMaxPerLane - 1); the loads of a polling round (one
-// or two 16-byte loads per record) are all in flight together, and only the
+// parity of the tag, which counts the exchanges of a call from 1 (the slots are
+// cleared per call), and a slot is rewritten only after every CTA has published
+// in the other one, that is, has read this one.  Every exchange writes both pairs
+// of a record, also when its payload fits in the first, and polls the pairs that
+// hold its payload.  So the words of a slot carry the tag of its last exchange,
+// and what a reader can still see of an older one is at most as old as the last
+// exchange with `fence` (every word stored before that one is visible after it):
+// a few exchanges, never the 65 536 after which 16 bits of tag repeat.  With the
+// second pair left as it was by short payloads, a slot that saw only those for a
+// whole launch kept a tag of any age.  (cfet_selftest_exchange checks the words.)
+// Lane l reads the records of CTAs l, l + 32, ...; the loads of a polling round
+// (one or two 16-byte loads per record) are all in flight together, and only the
 // complete round is passed to acc.add(), in that order.  (One tagged 64-bit word
 // per payload word, six 8-byte loads per record accumulated inside the polling
 // loop, took 4.0 us per exchange of six words over 152 CTAs where registers were
@@ -57,9 +63,7 @@ static __device__ __forceinline__ long long sm_clock() {
 // CTAs will read vectors written before the exchange.  Returns false in every
 // lane when the wait limit expired (CFET_ETIMEOUT recorded) or another CTA
 // reported an error.  The two slots need kExchWords G words.
-constexpr int kExchMaxPerLane = 8;  // grids of at most 256 CTAs
-constexpr int kExchHeld = 5;        // records per lane kept in registers (grids of at most 160 CTAs)
-
+constexpr int kExchHeld = 5;  // records per lane kept in registers (grids of at most 160 CTAs)
 
 __device__ __forceinline__ void st_relaxed_v2(unsigned long long* p, unsigned long long a, unsigned long long b) {
   asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
@@ -89,9 +93,9 @@ static __device__ __forceinline__ bool ctl_exchange(unsigned long long* rec, con
   if (lane == 0) {
     if (fence) __threadfence();
 #pragma unroll
-    for (int j = 0; j < NP; ++j) {
-      const unsigned v0 = mine[3 * j], v1 = 3 * j + 1 < W ? mine[3 * j + 1 < W ? 3 * j + 1 : 0] : 0u;
-      const unsigned v2 = 3 * j + 2 < W ? mine[3 * j + 2 < W ? 3 * j + 2 : 0] : 0u;
+    for (int j = 0; j < 2; ++j) {
+      auto word = [&](int i) { return i < W ? mine[i < W ? i : 0] : 0u; };
+      const unsigned v0 = word(3 * j), v1 = word(3 * j + 1), v2 = word(3 * j + 2);
       const unsigned long long t = (unsigned long long)t16 << 48;
       st_relaxed_v2(rec + (size_t)blockIdx.x * kExchStride + 2 * j, t | ((unsigned long long)(v1 & 0xffffu) << 32) | v0,
                     t | ((unsigned long long)v2 << 16) | (v1 >> 16));

@@ -866,7 +866,80 @@ __global__ void k_wait_selftest(int which, unsigned long long* rec, unsigned* ba
     grid_barrier(bar, gen, status, timeout_ns, &s_ok);
   }
 }
+
+// One exchange of W words: every CTA's payload is a hash of its index, the word and
+// the tag; out[0] counts the sums that come out wrong, out[1] the words of this
+// CTA's record in the exchange's slot that do not carry its tag.
+template <int W>
+__device__ bool exchange_step(unsigned long long* rec, unsigned tag, bool fence, int* status, unsigned long long* out) {
+  const int lane = threadIdx.x & 31;
+  auto payload = [&](unsigned cta, int w) { return (cta * 2654435761u + (unsigned)w * 40503u) ^ (tag * 2246822519u); };
+  struct SumAcc {
+    unsigned long long s[W];
+    __device__ void reset() {
+      for (int w = 0; w < W; ++w) s[w] = 0;
+    }
+    __device__ void add(const unsigned (&v)[W]) {
+      for (int w = 0; w < W; ++w) s[w] += v[w];
+    }
+  } acc;
+  unsigned mine[W];
+  for (int w = 0; w < W; ++w) mine[w] = payload(blockIdx.x, w);
+  long long spin = 0;
+  if (!ctl_exchange<W>(rec, mine, tag, fence, status, 2000000000LL, spin, acc)) return false;
+  for (int w = 0; w < W; ++w) {
+    unsigned long long want = 0, got = acc.s[w];
+    for (int i = lane; i < (int)gridDim.x; i += 32) want += payload(i, w);
+    for (int o = 16; o > 0; o >>= 1) {
+      want += __shfl_xor_sync(0xffffffffu, want, o);
+      got += __shfl_xor_sync(0xffffffffu, got, o);
+    }
+    if (lane == 0 && got != want) atomicAdd(out, 1ULL);
+  }
+  if (lane == 0) {
+    const unsigned long long* r = rec + (size_t)(tag & 1u) * kExchStride * gridDim.x + (size_t)blockIdx.x * kExchStride;
+    for (int j = 0; j < 4; j += 2) {
+      const ulonglong2 v = ld_relaxed_v2(r + j);
+      const int bad = (int)((unsigned)(v.x >> 48) != (tag & 0xffffu)) + (int)((unsigned)(v.y >> 48) != (tag & 0xffffu));
+      if (bad) atomicAdd(out + 1, (unsigned long long)bad);
+    }
+  }
+  __syncwarp();
+  return true;
+}
+// n exchanges from tag first on, the record widths of the kernels mixed.
+__global__ void k_exchange_selftest(unsigned long long* rec, unsigned first, int n, int* status,
+                                    unsigned long long* out) {
+  for (int i = 0; i < n; ++i) {
+    const unsigned tag = first + (unsigned)i;
+    const bool fence = i & 1;
+    bool ok;
+    switch (i % 7) {
+      case 0: ok = exchange_step<4>(rec, tag, fence, status, out); break;
+      case 1: ok = exchange_step<2>(rec, tag, fence, status, out); break;
+      case 2: ok = exchange_step<2>(rec, tag, fence, status, out); break;
+      case 3: ok = exchange_step<6>(rec, tag, fence, status, out); break;
+      case 4: ok = exchange_step<1>(rec, tag, fence, status, out); break;
+      case 5: ok = exchange_step<1>(rec, tag, fence, status, out); break;
+      default: ok = exchange_step<3>(rec, tag, fence, status, out); break;
+    }
+    if (!ok) return;
+  }
+}
 }  // namespace
+
+int launch_exchange_selftest(unsigned long long* rec, unsigned first, int n, int grid, int* status,
+                             unsigned long long* out) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(32);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return (int)cudaLaunchKernelEx(&cfg, k_exchange_selftest, rec, first, n, status, out);
+}
 
 int launch_wait_selftest(int which, unsigned long long* rec, unsigned* bar, int* status, long long timeout_ns) {
   k_wait_selftest<<<2, 32>>>(which, rec, bar, status, timeout_ns);
