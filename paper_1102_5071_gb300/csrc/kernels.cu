@@ -298,7 +298,10 @@ __global__ void __launch_bounds__(512, 1) k_propagate(PropParams p, Op op) {
   const int x0 = (wide ? (int)blockDim.x : chunk) * (int)blockIdx.x + tid;
   const int xe = wide ? dim : min(dim, ((int)blockIdx.x + 1) * chunk);
   const int ncoef = 1 + p.nV;
-  unsigned gen = 0;  // barriers of the re-orthogonalisation
+  // barriers of the re-orthogonalisation: the generation goes on from the launch
+  // before (it cannot move before this CTA arrives).  Counted from 0 again, a launch
+  // after one with a single barrier found its first generation already there.
+  unsigned gen = ld_volatile_u32(p.bar + 1);
   DevStatus* st = p.st;
   unsigned tag = (unsigned)ld_volatile_i32((const int*)&st->tag_base);
   const bool lead = (blockIdx.x == 0 && tid == 0);
