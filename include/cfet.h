@@ -183,9 +183,9 @@ typedef struct cfet_options {
   int32_t m_max;             /* Krylov dimension limit (default 16, <= 64)    */
   int32_t m_min;             /* first dimension tested (default 2, >= 1)      */
   int32_t max_substeps;      /* per stage exponential (default 64)            */
-  int32_t block_size;        /* 0 = auto; FP64 kernel: 2 x block_size threads
-                                per CTA (256 -> 512, the largest allowed;
-                                auto: as many as a CTA has elements, <= 512);
+  int32_t block_size;        /* 0 = auto; FP64 kernel: threads per CTA (256 the
+                                largest allowed; auto: as many as a CTA has
+                                elements, at most 512);
                                 fixed-point and mixed-precision kernels:
                                 2 x block_size worker threads + one control
                                 warp (384 -> 800, the largest allowed)        */
@@ -636,6 +636,10 @@ cfet_status cfet_selftest_i128_to_double(const uint64_t* lo, const int64_t* hi, 
 cfet_status cfet_selftest_ll_to_double_up(const int64_t* v, int64_t n, double* out);
 cfet_status cfet_selftest_krylov_bounds(int32_t k, const double* a, const double* b, double ts, double* log2_bounds,
                                         int32_t* gate);
+
+/* CTAs and threads per CTA of ctx's propagation kernel, for checks of what
+ * block_size and grid_size give.  CFET_EINVAL for NULL pointers.            */
+cfet_status cfet_selftest_launch_shape(const cfet_ctx* ctx, int32_t* grid, int32_t* block);
 
 /* Self-check of the record exchange of the persistent kernels (device): n
  * exchanges over `grid` CTAs (2 to 256) in one launch, with the record widths

@@ -251,6 +251,12 @@ void fill_stats(const DevStatus& s, cfet_stats* out) {
   }
 }
 
+// Threads per CTA of the propagation kernel.
+int launch_block(const cfet_ctx* ctx) {
+  if (ctx->opt.expm == CFET_EXPM_CHEBYSHEV) return cheb_threads(ctx->block - 32);
+  return ctx->small_fx || ctx->cluster_fx ? ctx->small_block : ctx->block;
+}
+
 // One persistent launch over exponentials [e0, e0 + ne).
 cfet_status launch_chunk(cfet_ctx* ctx, const PropParams& base, long long e0, long long ne, cudaStream_t s) {
   PropParams p = base;
@@ -262,11 +268,11 @@ cfet_status launch_chunk(cfet_ctx* ctx, const PropParams& base, long long e0, lo
     OpSpinIP op{ctx->spin.N, p.ip_nw, p.ip_w};
     e = launch_propagate_spin_ip(p, op, ctx->grid, ctx->block, s);
   } else if (ctx->opt.expm == CFET_EXPM_CHEBYSHEV)
-    e = ctx->family == kFamilySpin  ? launch_cheb_spin_fx(p, ctx->spin_fx, ctx->grid, cheb_threads(ctx->block - 32), s)
-        : ctx->family == kFamilyCsr ? launch_cheb_csr_fx(p, ctx->csr_fx, ctx->grid, cheb_threads(ctx->block - 32), s)
-                                    : launch_cheb_dia_fx(p, ctx->dia_fx, ctx->grid, cheb_threads(ctx->block - 32), s);
+    e = ctx->family == kFamilySpin  ? launch_cheb_spin_fx(p, ctx->spin_fx, ctx->grid, launch_block(ctx), s)
+        : ctx->family == kFamilyCsr ? launch_cheb_csr_fx(p, ctx->csr_fx, ctx->grid, launch_block(ctx), s)
+                                    : launch_cheb_dia_fx(p, ctx->dia_fx, ctx->grid, launch_block(ctx), s);
   else if (ctx->precision == CFET_PREC_FX) {
-    const int b = ctx->small_fx || ctx->cluster_fx ? ctx->small_block : ctx->block;
+    const int b = launch_block(ctx);
     e = ctx->family == kFamilySpin  ? launch_propagate_spin_fx(p, ctx->spin_fx, ctx->grid, b, s)
         : ctx->family == kFamilyCsr ? launch_propagate_csr_fx(p, ctx->csr_fx, ctx->grid, b, s)
                                     : launch_propagate_dia_fx(p, ctx->dia_fx, ctx->grid, b, s);
@@ -802,8 +808,8 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
   const bool auto_block = o.block_size == 0;
   if (o.block_size == 0) o.block_size = (o.precision == CFET_PREC_F64) ? 256 : 384;
   {
-    // FP64 kernel: 2 * block_size threads (<= 512); fixed-point and mixed-precision
-    // kernels: 2 * block_size workers + one control warp (<= 1024 threads)
+    // FP64 kernel: block_size threads (<= 256; 512 by default); fixed-point and
+    // mixed-precision kernels: 2 * block_size workers + one control warp (<= 1024 threads)
     // (the latter are compiled for at most CFET_CTL_MAX_THREADS threads per CTA)
     const int lim = (o.precision == CFET_PREC_F64) ? 256 : ((CFET_CTL_MAX_THREADS - 32) / 2) & ~31;
     if (o.block_size < 32 || o.block_size > lim || o.block_size % 32)
@@ -929,11 +935,11 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
   ctx->dim = dim;
   ctx->nV = nV;
   ctx->opt = o;
-  // FP64 kernel: 2 * block_size threads; fixed-point and mixed-precision kernels:
+  // FP64 kernel: block_size threads, 512 by default; fixed-point and mixed-precision kernels:
   // 2 * block_size worker threads plus one control warp (default 768 + 32,
   // one CTA per SM)
   const bool ctl_warp = o.precision != CFET_PREC_F64;
-  ctx->block = ctl_warp ? 2 * o.block_size + 32 : 2 * o.block_size;
+  ctx->block = ctl_warp ? 2 * o.block_size + 32 : auto_block ? 512 : o.block_size;
   ctx->precision = o.precision;
   for (int k = 0; k < nV; ++k) {
     ctx->f.push_back(f[k]);
@@ -1242,15 +1248,15 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
   if (want > 1) want = (int)std::min((((long long)dim << lane_bits) + workers - 1) / workers, 1LL << 30);
   if (o.grid_size > 0) want = o.grid_size;
   ctx->grid = want < maxg ? want : maxg;
-  if (ctx->grid > kMaxCtlGrid) ctx->grid = kMaxCtlGrid;  // record exchange limit
+  if (ctl_warp && ctx->grid > kMaxCtlGrid) ctx->grid = kMaxCtlGrid;  // record exchange limit
   if (ctx->grid < 1) ctx->grid = 1;
   // FP64 kernel: an SM needs four warps for its FP64 pipes, and every further one
   // lengthens the apply, so 128 elements per CTA up to one CTA per SM and one
   // thread per element up to 512.  Against 512 threads for 512 elements, 30 steps of
   // CF4:2 in ms: 9 sites 4.8 (5.9), 12 sites 5.7 (7.8), 14 sites 7.1 (9.7); a chain of
   // 8 sites stays in one CTA (3.9, 4.4 over two).
-  if (!ctl_warp && auto_block && o.grid_size == 0) {
-    ctx->grid = dim <= 256 ? 1 : std::min(std::min(maxg, kMaxCtlGrid), (dim + 127) / 128);
+  if (!ctl_warp && auto_block) {
+    if (o.grid_size == 0) ctx->grid = dim <= 256 ? 1 : std::min(std::min(maxg, kMaxCtlGrid), (dim + 127) / 128);
     ctx->block = std::min(ctx->block, std::max(64, ((dim + ctx->grid - 1) / ctx->grid + 31) & ~31));
   }
 
@@ -1803,6 +1809,13 @@ static cfet_status build_tile_maps(cfet_ctx* ctx, int N, int nvec, bool fx) {
   return CFET_OK;
 }
 }  // extern "C++"
+
+cfet_status cfet_selftest_launch_shape(const cfet_ctx* ctx, int32_t* grid, int32_t* block) {
+  if (!ctx || !grid || !block) return CFET_EINVAL;
+  *grid = ctx->grid;
+  *block = launch_block(ctx);
+  return CFET_OK;
+}
 
 cfet_status cfet_selftest_tiling(int32_t nsites, int32_t tile_bits, int64_t* checked) {
   if (!checked) return fail(nullptr, CFET_EINVAL, "checked is NULL");

@@ -209,30 +209,51 @@ struct SumAcc {  // one double per CTA record
 // CTA (ctl_exchange, warp 0), a fixed-order sum.  `fence`: vectors written before
 // it are read by other CTAs after it.  False in every thread on a timeout or when
 // another CTA reported an error.
+// Grids of more than 224 CTAs (only with an explicit block or grid size: the default
+// has one CTA per SM) leave one partial per CTA and meet at the counter barrier, since
+// in an exchange every CTA polls the records of all.  20 stage exponentials of 14
+// sites, 128 threads per CTA: 200 CTAs 3.26 ms with the exchange, 3.64 at the barrier;
+// 256 CTAs 3.50 and 3.37.  Three slots by the tag: two uses of one lie two barriers
+// apart.
+constexpr int kF64ExchGrid = 224;
+__device__ __forceinline__ void f64_meet(SmemLayout& S, double c, unsigned tag, const PropParams& p) {  // c: thread 0's CTA sum
+  double* const part = p.partials + (size_t)(tag % 3u) * gridDim.x;
+  if (threadIdx.x == 0) part[blockIdx.x] = c;
+  unsigned gen = threadIdx.x == 0 ? ld_volatile_u32(p.bar + 1) : 0u;  // (it cannot move before this CTA arrives)
+  if (grid_barrier(p.bar, gen, &p.st->status, p.timeout_ns, &S.ok) && threadIdx.x < 32) {
+    const double t = sum_partials(part);
+    if (threadIdx.x == 0) S.sum = t;
+  }
+}
 __device__ __noinline__ bool f64_reduce(SmemLayout& S, double acc, bool fence, unsigned tag, const PropParams& p) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) S.red[warp] = acc;
   __syncthreads();
+  double c = 0.0;
   if (warp == 0) {
-    double c = lane < (int)(blockDim.x >> 5) ? S.red[lane] : 0.0;
+    c = lane < (int)(blockDim.x >> 5) ? S.red[lane] : 0.0;
+    const int nw = (int)(blockDim.x >> 5);  // (lane 0 holds the sum of lanes 0 .. nw - 1; the others are 0)
+#pragma unroll 1
+    for (int o = nw > 8 ? 8 : nw > 4 ? 4 : nw > 2 ? 2 : nw >> 1; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (gridDim.x <= kF64ExchGrid) {
+      const unsigned long long b = (unsigned long long)__double_as_longlong(c);
+      const unsigned mine[2] = {(unsigned)b, (unsigned)(b >> 32)};
+      SumAcc a;
+      long long spin = 0;
+      const bool ok = ctl_exchange<2>(reinterpret_cast<unsigned long long*>(p.partials), mine, tag, fence,
+                                      &p.st->status, p.timeout_ns, spin, a);
+      double t = a.s;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    const unsigned long long b = (unsigned long long)__double_as_longlong(c);
-    const unsigned mine[2] = {(unsigned)b, (unsigned)(b >> 32)};
-    SumAcc a;
-    long long spin = 0;
-    const bool ok = ctl_exchange<2>(reinterpret_cast<unsigned long long*>(p.partials), mine, tag, fence, &p.st->status,
-                                    p.timeout_ns, spin, a);
-    double t = a.s;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) {
-      S.sum = t;
-      S.ok = ok;
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) {
+        S.sum = t;
+        S.ok = ok;
+      }
     }
   }
+  if (gridDim.x > kF64ExchGrid) f64_meet(S, c, tag, p);
   __syncthreads();
   return S.ok != 0;
 }
@@ -283,7 +304,7 @@ __device__ __noinline__ void f64_decide(SmemLayout& S, int it, double beta0, dou
 // the grid).  Chunks of more than eight elements per thread are interleaved over
 // the CTAs instead, so that the SMs gather from the same part of the vector at a
 // time (20 sites: 8.16 against 8.32 ms; 19 sites 4.30, 18 sites 2.46).  CTAs of
-// 256 threads, three per SM, that met at a counter barrier took 8.24, 4.45 and
+// 256 threads, two per SM, that met at a counter barrier took 8.24, 4.45 and
 // 2.74 ms (three steps of CF4:2; FP64 pipe 0.6 to 0.7 of its rate).
 template <int FAMILY, class Op>
 __global__ void __launch_bounds__(512, 1) k_propagate(PropParams p, Op op) {
@@ -298,10 +319,6 @@ __global__ void __launch_bounds__(512, 1) k_propagate(PropParams p, Op op) {
   const int x0 = (wide ? (int)blockDim.x : chunk) * (int)blockIdx.x + tid;
   const int xe = wide ? dim : min(dim, ((int)blockIdx.x + 1) * chunk);
   const int ncoef = 1 + p.nV;
-  // barriers of the re-orthogonalisation: the generation goes on from the launch
-  // before (it cannot move before this CTA arrives).  Counted from 0 again, a launch
-  // after one with a single barrier found its first generation already there.
-  unsigned gen = ld_volatile_u32(p.bar + 1);
   DevStatus* st = p.st;
   unsigned tag = (unsigned)ld_volatile_i32((const int*)&st->tag_base);
   const bool lead = (blockIdx.x == 0 && tid == 0);
@@ -489,6 +506,10 @@ __global__ void __launch_bounds__(512, 1) k_propagate(PropParams p, Op op) {
               }
               __syncthreads();
             }
+            // (the generation goes on from the launch before; it cannot move before this CTA
+            // arrives.  Counted from 0 again, a launch after one with a single barrier
+            // found its first generation already there)
+            unsigned gen = tid == 0 ? ld_volatile_u32(p.bar + 1) : 0u;
             if (!grid_barrier(p.bar, gen, &st->status, p.timeout_ns, &S.ok)) return;
             if (tid < 32) {
               for (int i = 1; i <= it; ++i) {
