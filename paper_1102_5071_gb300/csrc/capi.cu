@@ -1270,12 +1270,16 @@ cfet_status cfet_create(cfet_ctx** out, const cfet_op* H0, int32_t nV, const cfe
   }
   if (ctx->precision == CFET_PREC_FX && family == kFamilySpin && o.expm == CFET_EXPM_KRYLOV && !ctx->small_fx &&
       !ctx->tiled && o.grid_size == 0 && nsites <= kFxClusterMaxSites) {
-    // one cluster of at most 16 CTAs with at least 256 elements each
+    // one cluster of at most 16 CTAs with at least 256 elements each, where these are at
+    // most two per thread: with small explicit blocks the grid of independent CTAs,
+    // which has more of them, is faster (10 CF4:2 steps of 13 sites, 64 threads per CTA,
+    // 2.14 ms on 128 CTAs, 4.22 on the cluster; 128 threads 2.01 and 2.71; 192 threads,
+    // 2.7 per thread, 2.06 and 2.41; 256 threads on the cluster 2.12)
     int most = 2;
     while (most < 16 && dim / (2 * most) >= 256) most *= 2;
     const int part_threads = 32 + std::min(ctx->block - 32, std::max(256, dim / most));
     const int cs = fx_cluster_prepare(dim, most, part_threads);
-    if (cs > 0) {
+    if (cs > 0 && dim / cs <= 2 * (ctx->block - 32)) {
       ctx->cluster_fx = true;
       ctx->grid = ctx->cluster = cs;
       ctx->small_block = 32 + std::min(ctx->block - 32, std::max(256, dim / cs));
