@@ -44,9 +44,9 @@ static __device__ __forceinline__ long long sm_clock() {
 // one store and one round of loads per exchange.  Two slots alternate by the
 // parity of the tag, which counts the exchanges of a call from 1 (the slots are
 // cleared per call), and a slot is rewritten only after every CTA has published
-// in the other one, that is, has read this one.  Every exchange writes both pairs
-// of a record, also when its payload fits in the first, and polls the pairs that
-// hold its payload.  So the words of a slot carry the tag of its last exchange,
+// in the other one, that is, has read this one.  Every exchange writes the PAIRS
+// pairs that the widest exchange of its kernel needs, also when its own payload fits
+// in the first, and polls those that hold its payload.  So the words of a slot carry the tag of its last exchange,
 // and what a reader can still see of an older one is at most as old as the last
 // exchange with `fence` (every word stored before that one is visible after it):
 // a few exchanges, never the 65 536 after which 16 bits of tag repeat.  With the
@@ -74,12 +74,13 @@ __device__ __forceinline__ ulonglong2 ld_relaxed_v2(const unsigned long long* p)
   return v;
 }
 
-template <int W, class Acc>
+template <int W, int PAIRS = 2, class Acc>
 static __device__ __forceinline__ bool ctl_exchange(unsigned long long* rec, const unsigned (&mine)[W], unsigned tag,
                                                     bool fence, int* status, long long timeout_ns, long long& spin,
                                                     Acc& acc) {
   static_assert(W >= 1 && W <= 6, "two pairs of words hold six payload words");
   constexpr int NP = (W + 2) / 3;
+  static_assert(NP <= PAIRS && PAIRS <= 2, "PAIRS is for the kernel's widest exchange");
   const int lane = threadIdx.x & 31;
   const int G = gridDim.x;
   if (G == 1) {  // a single CTA: its own record is the total; nothing to publish or wait for
@@ -93,7 +94,7 @@ static __device__ __forceinline__ bool ctl_exchange(unsigned long long* rec, con
   if (lane == 0) {
     if (fence) __threadfence();
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
+    for (int j = 0; j < PAIRS; ++j) {
       auto word = [&](int i) { return i < W ? mine[i < W ? i : 0] : 0u; };
       const unsigned v0 = word(3 * j), v1 = word(3 * j + 1), v2 = word(3 * j + 2);
       const unsigned long long t = (unsigned long long)t16 << 48;

@@ -216,7 +216,7 @@ struct SumAcc {  // one double per CTA record
 // 256 CTAs 3.50 and 3.37.  Three slots by the tag: two uses of one lie two barriers
 // apart.
 constexpr int kF64ExchGrid = 224;
-__device__ __forceinline__ void f64_meet(SmemLayout& S, double c, unsigned tag, const PropParams& p) {  // c: thread 0's CTA sum
+__device__ __noinline__ void f64_meet(SmemLayout& S, double c, unsigned tag, const PropParams& p) {  // c: thread 0's CTA sum
   double* const part = p.partials + (size_t)(tag % 3u) * gridDim.x;
   if (threadIdx.x == 0) part[blockIdx.x] = c;
   unsigned gen = threadIdx.x == 0 ? ld_volatile_u32(p.bar + 1) : 0u;  // (it cannot move before this CTA arrives)
@@ -235,15 +235,17 @@ __device__ __noinline__ bool f64_reduce(SmemLayout& S, double acc, bool fence, u
   if (warp == 0) {
     c = lane < (int)(blockDim.x >> 5) ? S.red[lane] : 0.0;
     const int nw = (int)(blockDim.x >> 5);  // (lane 0 holds the sum of lanes 0 .. nw - 1; the others are 0)
-#pragma unroll 1
-    for (int o = nw > 8 ? 8 : nw > 4 ? 4 : nw > 2 ? 2 : nw >> 1; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+      if (nw > o) c += __shfl_xor_sync(0xffffffffu, c, o);
     if (gridDim.x <= kF64ExchGrid) {
       const unsigned long long b = (unsigned long long)__double_as_longlong(c);
       const unsigned mine[2] = {(unsigned)b, (unsigned)(b >> 32)};
       SumAcc a;
       long long spin = 0;
-      const bool ok = ctl_exchange<2>(reinterpret_cast<unsigned long long*>(p.partials), mine, tag, fence,
-                                      &p.st->status, p.timeout_ns, spin, a);
+      // (one pair: every exchange of this kernel is of these two words)
+      const bool ok = ctl_exchange<2, 1>(reinterpret_cast<unsigned long long*>(p.partials), mine, tag, fence,
+                                         &p.st->status, p.timeout_ns, spin, a);
       double t = a.s;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
@@ -319,6 +321,10 @@ __global__ void __launch_bounds__(512, 1) k_propagate(PropParams p, Op op) {
   const int x0 = (wide ? (int)blockDim.x : chunk) * (int)blockIdx.x + tid;
   const int xe = wide ? dim : min(dim, ((int)blockIdx.x + 1) * chunk);
   const int ncoef = 1 + p.nV;
+  // barriers of the re-orthogonalisation: the generation goes on from the launch
+  // before (it cannot move before this CTA arrives).  Counted from 0 again, a launch
+  // after one with a single barrier found its first generation already there.
+  unsigned gen = ld_volatile_u32(p.bar + 1);
   DevStatus* st = p.st;
   unsigned tag = (unsigned)ld_volatile_i32((const int*)&st->tag_base);
   const bool lead = (blockIdx.x == 0 && tid == 0);
@@ -506,10 +512,7 @@ __global__ void __launch_bounds__(512, 1) k_propagate(PropParams p, Op op) {
               }
               __syncthreads();
             }
-            // (the generation goes on from the launch before; it cannot move before this CTA
-            // arrives.  Counted from 0 again, a launch after one with a single barrier
-            // found its first generation already there)
-            unsigned gen = tid == 0 ? ld_volatile_u32(p.bar + 1) : 0u;
+            if (G > kF64ExchGrid) gen = ld_volatile_u32(p.bar + 1);  // (f64_meet has moved it)
             if (!grid_barrier(p.bar, gen, &st->status, p.timeout_ns, &S.ok)) return;
             if (tid < 32) {
               for (int i = 1; i <= it; ++i) {
