@@ -644,9 +644,9 @@ cfet_status cfet_selftest_launch_shape(const cfet_ctx* ctx, int32_t* grid, int32
 /* Self-check of the record exchange of the persistent kernels (device): n
  * exchanges over `grid` CTAs (2 to 256) in one launch, with the record widths
  * of the kernels mixed, tags counted from first_tag (16 bits of which are
- * stored; first_tag mod 65536 in [1, 65534]).  wrong[0]: sums that differ from
- * the exact ones; wrong[1]: words of a CTA's record that do not carry the tag of
- * their slot's last exchange.  Both 0 when all is well; CFET_EINVAL for
+ * stored; 1 to 2^30).  wrong[0]: sums that differ from the exact ones; wrong[1]:
+ * words of a CTA's record that do not carry the exchange's tag or, where a short
+ * record leaves them as they were, are over 2048 exchanges old.  Both 0 when all is well; CFET_EINVAL for
  * arguments outside the ranges, CFET_ETIMEOUT when a wait gave up.            */
 cfet_status cfet_selftest_exchange(int32_t grid, uint32_t first_tag, int32_t n, int64_t* wrong);
 

@@ -1893,9 +1893,8 @@ cfet_status cfet_selftest_wait_timeout(int32_t which, double timeout_s, int32_t*
 }
 
 cfet_status cfet_selftest_exchange(int32_t grid, uint32_t first_tag, int32_t n, int64_t* wrong) {
-  if (grid < 2 || grid > kMaxCtlGrid || n < 1 || n > 200000 || (first_tag & 0xffffu) < 1 ||
-      (first_tag & 0xffffu) > 0xfffeu || !wrong)
-    return fail(nullptr, CFET_EINVAL, "selftest: grid in [2, 256], n in [1, 200000], first_tag mod 65536 in [1, 65534]");
+  if (grid < 2 || grid > kMaxCtlGrid || n < 1 || n > 200000 || first_tag < 1 || first_tag > 1u << 30 || !wrong)
+    return fail(nullptr, CFET_EINVAL, "selftest: grid in [2, 256], n in [1, 200000], first_tag in [1, 2^30], wrong required");
   cfet_status s = device_available(nullptr);
   if (s != CFET_OK) return s;
   unsigned long long *rec = nullptr, *out = nullptr;
@@ -1906,7 +1905,12 @@ cfet_status cfet_selftest_exchange(int32_t grid, uint32_t first_tag, int32_t n, 
   cudaError_t e = cudaMalloc(&rec, bytes);
   if (e == cudaSuccess) e = cudaMalloc(&out, sizeof(h));
   if (e == cudaSuccess) e = cudaMalloc(&st, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(rec, 0, bytes);
+  // the slots as first_tag - 1 exchanges left them (cleared before the first)
+  std::vector<unsigned long long> init(bytes / sizeof(unsigned long long), 0);
+  for (uint32_t t = first_tag > 2 ? first_tag - 2 : 0; t < first_tag; ++t)
+    std::fill_n(init.begin() + (size_t)(t & 1u) * kExchStride * grid, (size_t)kExchStride * grid,
+                (unsigned long long)(t & 0xffffu) << 48);
+  if (e == cudaSuccess) e = cudaMemcpy(rec, init.data(), bytes, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(out, 0, sizeof(h));
   if (e == cudaSuccess) e = cudaMemset(st, 0, sizeof(int));
   if (e == cudaSuccess) e = (cudaError_t)launch_exchange_selftest(rec, first_tag, n, grid, st, out);

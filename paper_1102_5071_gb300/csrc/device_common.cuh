@@ -44,14 +44,16 @@ static __device__ __forceinline__ long long sm_clock() {
 // one store and one round of loads per exchange.  Two slots alternate by the
 // parity of the tag, which counts the exchanges of a call from 1 (the slots are
 // cleared per call), and a slot is rewritten only after every CTA has published
-// in the other one, that is, has read this one.  Every exchange writes the PAIRS
-// pairs that the widest exchange of its kernel needs, also when its own payload fits
-// in the first, and polls those that hold its payload.  So the words of a slot carry the tag of its last exchange,
-// and what a reader can still see of an older one is at most as old as the last
-// exchange with `fence` (every word stored before that one is visible after it):
-// a few exchanges, never the 65 536 after which 16 bits of tag repeat.  With the
-// second pair left as it was by short payloads, a slot that saw only those for a
-// whole launch kept a tag of any age.  (cfet_selftest_exchange checks the words.)
+// in the other one, that is, has read this one.  So the pairs that hold an
+// exchange's payload carry, until they are rewritten, the tag of two exchanges
+// before.  In a kernel whose widest exchange has two pairs (PAIRS = 2) shorter ones
+// leave the second as it was, possibly for a whole launch: it is given the exchange's
+// tag once in kExchRefresh exchanges of a slot.  A reader then never meets a word as
+// old as the 65 536 exchanges after which 16 bits of tag repeat: at most 2
+// kExchRefresh, and the few since the last exchange with `fence`, which makes every
+// word stored before it visible.  (cfet_selftest_exchange checks the ages.  Written
+// with every exchange the second pair cost up to 5 % of a complex64 call: 2000 x 100
+// atom 0.271 ms against 0.257, 17 sites 1.70 against 1.65.)
 // Lane l reads the records of CTAs l, l + 32, ...; the loads of a polling round
 // (one or two 16-byte loads per record) are all in flight together, and only the
 // complete round is passed to acc.add(), in that order.  (One tagged 64-bit word
@@ -64,6 +66,7 @@ static __device__ __forceinline__ long long sm_clock() {
 // lane when the wait limit expired (CFET_ETIMEOUT recorded) or another CTA
 // reported an error.  The two slots need kExchWords G words.
 constexpr int kExchHeld = 5;  // records per lane kept in registers (grids of at most 160 CTAs)
+constexpr unsigned kExchRefresh = 1024;  // a power of two
 
 __device__ __forceinline__ void st_relaxed_v2(unsigned long long* p, unsigned long long a, unsigned long long b) {
   asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
@@ -93,13 +96,17 @@ static __device__ __forceinline__ bool ctl_exchange(unsigned long long* rec, con
   const unsigned t16 = tag & 0xffffu;
   if (lane == 0) {
     if (fence) __threadfence();
+    const unsigned long long t = (unsigned long long)t16 << 48;
+    unsigned long long* const out = rec + (size_t)blockIdx.x * kExchStride;
 #pragma unroll
-    for (int j = 0; j < PAIRS; ++j) {
+    for (int j = 0; j < NP; ++j) {
       auto word = [&](int i) { return i < W ? mine[i < W ? i : 0] : 0u; };
       const unsigned v0 = word(3 * j), v1 = word(3 * j + 1), v2 = word(3 * j + 2);
-      const unsigned long long t = (unsigned long long)t16 << 48;
-      st_relaxed_v2(rec + (size_t)blockIdx.x * kExchStride + 2 * j, t | ((unsigned long long)(v1 & 0xffffu) << 32) | v0,
+      st_relaxed_v2(out + 2 * j, t | ((unsigned long long)(v1 & 0xffffu) << 32) | v0,
                     t | ((unsigned long long)v2 << 16) | (v1 >> 16));
+    }
+    if constexpr (NP < PAIRS) {
+      if (((tag >> 1) & (kExchRefresh - 1u)) == 0u) st_relaxed_v2(out + 2, t, t);
     }
   }
   __syncwarp();

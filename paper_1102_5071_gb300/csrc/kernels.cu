@@ -896,7 +896,8 @@ __global__ void k_wait_selftest(int which, unsigned long long* rec, unsigned* ba
 
 // One exchange of W words: every CTA's payload is a hash of its index, the word and
 // the tag; out[0] counts the sums that come out wrong, out[1] the words of this
-// CTA's record in the exchange's slot that do not carry its tag.
+// CTA's record in the exchange's slot that do not carry its tag or, in the second
+// pair, are too old.
 template <int W>
 __device__ bool exchange_step(unsigned long long* rec, unsigned tag, bool fence, int* status, unsigned long long* out) {
   const int lane = threadIdx.x & 31;
@@ -927,21 +928,25 @@ __device__ bool exchange_step(unsigned long long* rec, unsigned tag, bool fence,
     const unsigned long long* r = rec + (size_t)(tag & 1u) * kExchStride * gridDim.x + (size_t)blockIdx.x * kExchStride;
     for (int j = 0; j < 4; j += 2) {
       const ulonglong2 v = ld_relaxed_v2(r + j);
-      const int bad = (int)((unsigned)(v.x >> 48) != (tag & 0xffffu)) + (int)((unsigned)(v.y >> 48) != (tag & 0xffffu));
+      const unsigned most = j == 0 || W > 3 ? 0u : 2u * kExchRefresh;
+      const int bad = (int)(((tag - (unsigned)(v.x >> 48)) & 0xffffu) > most) +
+                      (int)(((tag - (unsigned)(v.y >> 48)) & 0xffffu) > most);
       if (bad) atomicAdd(out + 1, (unsigned long long)bad);
     }
   }
   __syncwarp();
   return true;
 }
-// n exchanges from tag first on, the record widths of the kernels mixed.
+// n exchanges from tag first on, the record widths of the kernels mixed: by turns
+// every width on either slot, and for 3000 exchanges long records on one slot and
+// short ones on the other, as within a launch of the complex64 kernel.
 __global__ void k_exchange_selftest(unsigned long long* rec, unsigned first, int n, int* status,
                                     unsigned long long* out) {
   for (int i = 0; i < n; ++i) {
     const unsigned tag = first + (unsigned)i;
     const bool fence = i & 1;
     bool ok;
-    switch (i % 7) {
+    switch ((i / 3000) & 1 ? i & 1 : i % 7) {
       case 0: ok = exchange_step<4>(rec, tag, fence, status, out); break;
       case 1: ok = exchange_step<2>(rec, tag, fence, status, out); break;
       case 2: ok = exchange_step<2>(rec, tag, fence, status, out); break;

@@ -1,7 +1,8 @@
 """Record exchange of the persistent kernels: sums over all CTAs' records are exact
-and every word of a record carries the tag of its slot's last exchange, with the
-kernels' record widths mixed (short records leave no older tag in the second pair of
-words) and across the point where the stored 16 bits of the tag repeat."""
+and every word of a record carries the exchange's tag or, where a short record leaves
+the second pair of words as it was, one not so old that the stored 16 bits of it could
+repeat, with the kernels' record widths mixed, with one slot left to short records for
+thousands of exchanges, and across the repetition."""
 
 import ctypes as C
 
@@ -11,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("grid", [2, 31, 33, 152, 160, 161, 200])  # 160 records are held in registers
-@pytest.mark.parametrize("first,n", [(1, 40), (65510, 60), (3 * 65536 + 65533, 20), (1, 66000)])
+@pytest.mark.parametrize("first,n", [(1, 40), (65510, 60), (3 * 65536 + 65533, 20), (4 * 65536, 9), (1, 68000)])
 def test_exchange_words_and_sums(grid, first, n):
     pytest.importorskip("torch")
     from paper_1102_5071_gb300 import _capi
