@@ -31,6 +31,8 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <functional>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -804,6 +806,7 @@ using namespace cfet;
 
 struct cfet_batch {
   int device = 0;
+  int sms = 1;                             // SMs of the device
   int n = 0;
   int precision = CFET_PREC_F64;
   cfet_options opt{};
@@ -902,15 +905,49 @@ std::vector<BItem> make_items(const cfet_batch* b, const cfet_batch_plan& pl) {
   return out;
 }
 
-// Shared memory of a CTA for the staged vector under plan pl: the largest part
-// of an instance (as run_instance splits it) within kBatchStageMax; parts above
-// kBatchStageHalf, which leave room for one CTA per SM only, count when they are
-// at least half of the work that can be staged.
-int stage_bytes_for(const cfet_batch* b, const cfet_batch_plan& pl) {
-  const int esz = b->precision == CFET_PREC_C64 ? (int)sizeof(float2) : (int)sizeof(double2);
+// Whether the longest item of a launch decides how long it takes, on CTAs of 128
+// registers a thread (512 such threads per SM): all items together fill those
+// clusters for at most 1.3 times the longest, and handed out longest first they end
+// within 1.5 times.  `items` in order of decreasing work.
+bool longest_decides(const cfet_batch* b, const cfet_batch_plan& pl, const std::vector<BItem>& items) {
+  const size_t slots = (size_t)std::max(1, b->sms * (512 / pl.threads) / pl.cluster_size);
+  if (items.size() <= slots) return true;
+  auto work = [&](const BItem& it) {  // a group takes as long as its first, largest instance
+    return (double)b->dims[it.inst[0]] / (it.coop ? pl.cluster_size : 1);
+  };
+  double all = 0.0;
+  for (const BItem& it : items) all += work(it);
+  const double longest = work(items[0]);
+  if (all > 1.3 * longest * (double)slots) return false;
+  std::priority_queue<double, std::vector<double>, std::greater<double>> busy(
+      std::greater<double>(), std::vector<double>(slots, 0.0));
+  double end = 0.0;
+  for (const BItem& it : items) {
+    const double t = busy.top() + work(it);
+    busy.pop();
+    busy.push(t);
+    end = std::max(end, t);
+  }
+  return end <= 1.5 * longest;
+}
+
+// Shared memory of a CTA for the staged vector under plan pl: the largest part of an
+// instance (as run_instance splits it) within kBatchStageMax.  Parts above
+// kBatchStageHalf leave room for one CTA per SM only: where the longest item does not
+// decide, complex64 launches make room for them when they are at least half of the
+// work that can be staged (FP64 ones always: its units are the limit either way).
+// Where it decides and its part cannot be staged, nothing is (but with 512 threads in
+// FP64, whose units are busy either way): its gathers need the L1 cache that staged
+// parts of the others would take.  24 chains of 10..16 sites,
+// complex64, one CTA of 128 threads each: 10.3 ms a step without, 14.4 with 64 KB;
+// where it can be staged, 300 chains of 10..14 sites: 2.5 ms with its 128 KB, 4.4
+// with 64 KB.
+int stage_bytes_for(const cfet_batch* b, const cfet_batch_plan& pl, bool longest_first) {
+  const bool c64 = b->precision == CFET_PREC_C64;
+  const int esz = c64 ? (int)sizeof(float2) : (int)sizeof(double2);
   int lg = 0;
   while ((1 << lg) < pl.cluster_size) ++lg;
-  long long most = 0, most_half = 0;
+  long long most = 0, most_half = 0, largest = 0;
   double big = 0.0, all = 0.0;
   for (int i = 0; i < b->n; ++i) {
     const int N = b->chains[i].nsites;
@@ -918,13 +955,16 @@ int stage_bytes_for(const cfet_batch* b, const cfet_batch_plan& pl) {
     int lc = coop ? N - lg : N;
     if (lc < 6) lc = std::min(N, 6);
     const long long bytes = (1LL << lc) * esz;
+    largest = std::max(largest, bytes);
     if (bytes > kBatchStageMax) continue;
     most = std::max(most, bytes);
     if (bytes <= kBatchStageHalf) most_half = std::max(most_half, bytes);
     else big += b->dims[i];
     all += b->dims[i];
   }
-  return ((int)(2.0 * big >= all ? most : most_half) + 127) & ~127;
+  if (longest_first && largest > kBatchStageMax && (c64 || pl.threads < 512)) return 0;
+  const bool large = longest_first || !c64 || 2.0 * big >= all;
+  return ((int)(large ? most : most_half) + 127) & ~127;
 }
 
 // Plan before any tuning, by what the instances are (256 chains of 10..16 sites,
@@ -1093,15 +1133,20 @@ cfet_status run_batch(cfet_batch* b, const cfet_batch_plan& pl, double2* const* 
     inst[i].r_cap = r_cap[i];
   }
   const std::vector<BItem> items = make_items(b, pl);
-  const int stage = stage_bytes_for(b, pl);
+  const bool longest_first = longest_decides(b, pl, items);
+  const int stage = stage_bytes_for(b, pl, longest_first);
   p.stage_bytes = stage;
   auto resident = [&](bool roomy) {
     return b->precision == CFET_PREC_C64 ? max_clusters<FmtC64>(pl.cluster_size, pl.threads, stage, roomy)
                                          : max_clusters<FmtF64>(pl.cluster_size, pl.threads, stage, roomy);
   };
-  // the 128-register form where its CTAs hold all items at once
+  // the 128-register form where its CTAs hold all items at once; and where the longest
+  // item decides and two CTAs on an SM would slow it down: FP64 (its units are the
+  // limit; 100 chains of 8..13 sites, default plan, 1.26 ms a step, 1.92 with 64
+  // registers) and launches without staged vectors
   int maxc = resident(true);
-  const bool roomy = maxc >= (int)items.size();
+  const bool roomy = maxc >= (int)items.size() ||
+                     (maxc >= 1 && longest_first && (b->precision != CFET_PREC_C64 || stage == 0));
   if (!roomy) maxc = resident(false);
   if (maxc < 1) return bfail(b, CFET_EINVAL, "plan cannot be launched (no cluster fits on the device)");
   const int clusters = std::min<int>((int)items.size(), maxc);
@@ -1213,6 +1258,7 @@ cfet_status cfet_batch_create(cfet_batch** out, int32_t n, const cfet_chain* cha
   }
   cfet_batch* b = new cfet_batch();
   cudaGetDevice(&b->device);
+  cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device);
   b->n = n;
   b->precision = o.precision;
   b->opt = o;
