@@ -975,9 +975,13 @@ int stage_bytes_for(const cfet_batch* b, const cfet_batch_plan& pl, bool longest
 // the largest size spread) 20.9, and 21.2 before vectors were staged.  FP64
 // (bound by the FP64 units, vectors twice as large): clusters of 4 from 13
 // sites, 25.9 ms a step (31.4 with the former default, 31.4 with clusters of 8).
-// CTAs of 256 threads where the spread instances give each SM more than two
-// CTAs of short parts (100 chains of 12..14 sites: 1.93 against 2.34 ms), and of
-// 256 or 128 where no part reaches 1024 or 256 elements (206 FP64 chains of 7
+// Chains of 11 sites are not spread (16 of them 0.114 ms a CF4:2 step on one CTA each,
+// 0.120 spread; 256 of them 0.15 and 0.54), and up to 13 sites, which one CTA can stage
+// as well, only as many as give each SM 2.7 CTAs (48 chains of 12 sites 0.149 spread,
+// 0.158 not; 100 of them 0.29 and 0.16, 256 of 10..12 sites 0.41 and 0.23).
+// CTAs of 256 threads where the spread instances give each SM more than 1.5
+// CTAs of short parts (100 chains of 12..14 sites: 1.93 against 2.34 ms; 100 of 8..13
+// sites 0.19 against 0.26), and of 256 or 128 where no part reaches 1024 or 256 elements (206 FP64 chains of 7
 // sites: 0.31 ms with 128 threads, 0.35 with 512); the
 // part of a spread instance is at least 256 elements.
 cfet_batch_plan default_plan(const cfet_batch* b) {
@@ -986,9 +990,18 @@ cfet_batch_plan default_plan(const cfet_batch* b) {
   for (int i = 0; i < b->n; ++i) nmax = std::max(nmax, b->chains[i].nsites);
   cfet_batch_plan pl{};
   pl.cluster_size = c64 ? 8 : 4;
-  pl.coop_min_sites = std::max(11, std::min(c64 ? 14 : 13, nmax - 1));
+  pl.coop_min_sites = std::max(c64 ? 12 : 11, std::min(c64 ? 14 : 13, nmax - 1));
   long long spread = 0;
-  for (int i = 0; i < b->n; ++i) spread += b->chains[i].nsites >= pl.coop_min_sites;
+  auto count = [&] {
+    spread = 0;
+    for (int i = 0; i < b->n; ++i) spread += b->chains[i].nsites >= pl.coop_min_sites;
+  };
+  count();
+  if (c64 && nmax <= 13)
+    while (3 * spread * pl.cluster_size > 8 * b->sms) {
+      ++pl.coop_min_sites;
+      count();
+    }
   int lg = 0;
   while ((1 << lg) < pl.cluster_size) ++lg;
   int lc = 0;  // log2 of the largest part of a CTA
@@ -999,7 +1012,7 @@ cfet_batch_plan default_plan(const cfet_batch* b) {
   if (lc < 10)
     pl.threads = lc < 8 ? 128 : 256;
   else
-    pl.threads = nmax - lg < 12 && spread * pl.cluster_size > 304 ? 256 : 512;
+    pl.threads = nmax - lg < 12 && 2 * spread * pl.cluster_size > 3 * b->sms ? 256 : 512;
   pl.tuned_ms = 0.f;
   return pl;
 }
