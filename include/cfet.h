@@ -634,6 +634,18 @@ cfet_status cfet_selftest_i128_to_double(const uint64_t* lo, const int64_t* hi, 
  * kernels' int64 maxima, which enter the exponent bounds and must not round
  * down.  CFET_EINVAL for NULL pointers or n < 0.                            */
 cfet_status cfet_selftest_ll_to_double_up(const int64_t* v, int64_t n, double* out);
+/* cfet_selftest_upper_bounds: the upper bounds mant 2^expo (FP32 mantissa, 0 or
+ * in [1, 2]) from which the exponents of the fixed-point vectors follow, of
+ * |a[i]| (op 0), v[i] (op 1; 0 for v[i] <= 0), |a[i]| |b[i]| (op 2) and
+ * |a[i]| + |b[i]| (op 3), for i < n; never below the value, and above it by less
+ * than 2^-21 relative per operation (subnormals count as 2^-1022).  exp57[i]: the
+ * exponent E with bound < 2^(57 + E), -960 for zero and for bounds outside
+ * 2^-963 .. 2^964.  a, b finite; inputs that op does not use may be NULL.
+ * cfet_selftest_norm_shift: the left shift that brings v[i] into [2^61, 2^62) (0
+ * for v[i] <= 0 or at or above 2^62).  CFET_EINVAL for other arguments.        */
+cfet_status cfet_selftest_upper_bounds(int32_t op, const double* a, const double* b, const int64_t* v, int64_t n,
+                                       float* mant, int32_t* expo, int32_t* exp57);
+cfet_status cfet_selftest_norm_shift(const int64_t* v, int64_t n, int32_t* shift);
 cfet_status cfet_selftest_krylov_bounds(int32_t k, const double* a, const double* b, double ts, double* log2_bounds,
                                         int32_t* gate);
 

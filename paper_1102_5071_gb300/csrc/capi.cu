@@ -1845,6 +1845,28 @@ cfet_status cfet_selftest_ll_to_double_up(const int64_t* v, int64_t n, double* o
   return CFET_OK;
 }
 
+cfet_status cfet_selftest_upper_bounds(int32_t op, const double* a, const double* b, const int64_t* v, int64_t n,
+                                       float* mant, int32_t* expo, int32_t* exp57) {
+  if (op < 0 || op > 3 || n < 0 || !mant || !expo || !exp57 || (op == 1 ? !v : !a) || (op > 1 && !b))
+    return fail(nullptr, CFET_EINVAL, "selftest: op in [0, 3], n >= 0, its inputs and mant, expo, exp57 required");
+  for (int64_t i = 0; i < n; ++i) {
+    const UpB u = op == 0   ? sb_upb(a[i])
+                  : op == 1 ? sb_upb_ll(v[i])
+                  : op == 2 ? sb_upb_mul(sb_upb(a[i]), sb_upb(b[i]))
+                            : sb_upb_add(sb_upb(a[i]), sb_upb(b[i]));
+    mant[i] = u.m;
+    expo[i] = u.e;
+    exp57[i] = sb_upb_exp_for(u, 57);
+  }
+  return CFET_OK;
+}
+
+cfet_status cfet_selftest_norm_shift(const int64_t* v, int64_t n, int32_t* shift) {
+  if (!v || !shift || n < 0) return fail(nullptr, CFET_EINVAL, "selftest: v, shift required, n >= 0");
+  for (int64_t i = 0; i < n; ++i) shift[i] = sb_norm_shift_ll(v[i]);
+  return CFET_OK;
+}
+
 cfet_status cfet_selftest_krylov_bounds(int32_t k, const double* a, const double* b, double ts, double* log2_bounds,
                                         int32_t* gate) {
   if (k < 1 || k > kMaxKrylov || !a || (k > 1 && !b) || !log2_bounds || !gate)

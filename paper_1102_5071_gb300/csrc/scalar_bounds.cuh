@@ -8,8 +8,9 @@
 // arithmetic with explicit error margins: a helper either returns the FP64
 // decision for certain or says that it cannot, and the caller then evaluates
 // the FP64 form.  Everything here also compiles for the host, where
-// cfet_selftest_i128_to_double, cfet_selftest_ll_to_double_up and
-// cfet_selftest_krylov_bounds expose it to tests against exact arithmetic.
+// cfet_selftest_i128_to_double, cfet_selftest_ll_to_double_up,
+// cfet_selftest_krylov_bounds, cfet_selftest_upper_bounds and
+// cfet_selftest_norm_shift expose it to tests against exact arithmetic.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -343,7 +344,7 @@ __host__ __device__ __forceinline__ int sb_gersh_gate(const GershAcc& s, int k, 
 // (m = 0, or 1 <= m < 2 up to the operations' own normalisation): the
 // fixed-point exponents only need bounds, and FP64 arithmetic for them costs 64
 // cycles per operation on the control warp.  Every operation rounds up; one
-// loses at most 2^-22 relative.
+// loses at most 2^-21 relative (its factor of 2^-22 and two FP32 roundings).
 struct UpB {
   float m;
   int e;
