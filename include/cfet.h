@@ -602,6 +602,14 @@ cfet_status cfet_probe_copy_gbs(void* a, void* b, int64_t bytes, int32_t reps, v
  * is inconsistent.                                                          */
 cfet_status cfet_selftest_tiling(int32_t nsites, int32_t tile_bits, int64_t* checked);
 
+/* Host-only self-check of the row split of CSR operators over the CTAs of a
+ * launch: row_ptr holds nops row pointers of dim + 1 entries each; CTA b takes
+ * the rows [rb[b], rb[b + 1]) (rb: grid + 1 entries), at most cap of them
+ * (cap * grid >= dim), about the same number of entries each.  CFET_EINVAL for
+ * other arguments.                                                          */
+cfet_status cfet_selftest_row_split(const int32_t* row_ptr, int32_t nops, int32_t dim, int32_t grid, int64_t cap,
+                                    int32_t* rb);
+
 /* Host-only checks (no device needed) of the scalar helpers that the
  * control warps of the persistent kernels use instead of FP64 instructions
  * (the same source compiled for the host).

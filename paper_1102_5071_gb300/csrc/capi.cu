@@ -1831,6 +1831,16 @@ cfet_status cfet_selftest_tiling(int32_t nsites, int32_t tile_bits, int64_t* che
   return CFET_OK;
 }
 
+cfet_status cfet_selftest_row_split(const int32_t* row_ptr, int32_t nops, int32_t dim, int32_t grid, int64_t cap,
+                                    int32_t* rb) {
+  if (!row_ptr || !rb || nops < 1 || dim < 1 || grid < 1 || cap < 1 || cap > (1LL << 40) || cap * grid < dim)
+    return fail(nullptr, CFET_EINVAL, "selftest: nops, dim, grid >= 1, cap in [1, 2^40], cap * grid >= dim");
+  const std::vector<int> s =
+      csr_row_split(std::vector<int>(row_ptr, row_ptr + (size_t)nops * (dim + 1)), nops, dim, grid, cap);
+  std::copy(s.begin(), s.end(), rb);
+  return CFET_OK;
+}
+
 cfet_status cfet_selftest_i128_to_double(const uint64_t* lo, const int64_t* hi, int64_t n, int32_t shift,
                                          double* out) {
   if (!lo || !hi || !out || n < 0 || shift < -200 || shift > 200)
