@@ -676,7 +676,7 @@ cfet_status csr_upload(cfet_ctx* ctx, const cfet_op* H0, int nV, const cfet_op* 
   fx.rb = nullptr;
   // threads per row of the fixed-point apply (its sums are exact; the complex64
   // sums keep one thread per row and the order of the entries)
-  // eight or more entries of a row of one operator per thread (mean over the
+  // at least four entries of a row of one operator per thread (mean over the
   // rows): with 10 entries two threads a row take 35.2 us per Lanczos iteration
   // of 60 001 rows, one 46.5, four 36.2 and eight 47.7
   const double per = (double)nnz / ((double)dim * nops);
