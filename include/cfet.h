@@ -232,8 +232,12 @@ enum { CFET_PREC_DEFAULT = 0, CFET_PREC_F64 = 1, CFET_PREC_FX = 2, CFET_PREC_C64
 
 /* cfet_options.apply_form: the form of the XXZ-chain apply in the fixed-point
  * and complex64 Krylov kernels.
- *  AUTO        : element-wise below 23 sites, window-tiled from 23 sites.
- *  ELEMENTWISE : every element gathers its neighbours from global memory.
+ *  AUTO        : element-wise below 23 sites, window-tiled from 23 sites; complex64
+ *                chains of 17..21 sites element-wise from a vector staged in the
+ *                shared memory of 128 CTAs.
+ *  ELEMENTWISE : every element gathers its neighbours, from global memory or, in
+ *                fixed point up to 13 sites, from the shared memory of the one CTA
+ *                or the cluster that holds the vector (the same states).
  *  TILED       : window passes over shared-memory tiles; chains of 13..30
  *                sites (other sizes, operators and precisions keep the
  *                element-wise form).  Any other value: CFET_EINVAL.         */

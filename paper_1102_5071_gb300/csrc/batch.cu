@@ -589,13 +589,14 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
                 Fmt::add_prod(a, v1.x, h1.x);
                 Fmt::add_prod(a, v1.y, h1.y);
               }
-            } else
-            for (int x = x0; x < xe; x += step) {
-              const V hv = batch_apply<Fmt>(q, qm, x, N, I.L, I.uniform, dz_lo, dz_hi, S);
-              u[x] = hv;
-              const V v = q[x];
-              Fmt::add_prod(a, v.x, hv.x);
-              Fmt::add_prod(a, v.y, hv.y);
+            } else {
+              for (int x = x0; x < xe; x += step) {
+                const V hv = batch_apply<Fmt>(q, qm, x, N, I.L, I.uniform, dz_lo, dz_hi, S);
+                u[x] = hv;
+                const V v = q[x];
+                Fmt::add_prod(a, v.x, hv.x);
+                Fmt::add_prod(a, v.y, hv.y);
+              }
             }
           }
           const double asum = batch_sum<Fmt, PER_SM>(S, a, nact, slot ^= 1, coop);
@@ -625,15 +626,16 @@ __device__ void run_instance(const BParams& P, int ii, int part, int nparts, boo
                 Fmt::add_prod(a, w1_.x, w1_.x);
                 Fmt::add_prod(a, w1_.y, w1_.y);
               }
-            } else
-            for (int x = x0; x < xe; x += step) {
-              const V v = q[x];
-              const V uu = u[x];
-              const V w = Fmt::make(fma(am, v.x, uu.x), fma(am, v.y, uu.y));
-              u[x] = w;
-              if (single) sq[x] = w;
-              Fmt::add_prod(a, w.x, w.x);
-              Fmt::add_prod(a, w.y, w.y);
+            } else {
+              for (int x = x0; x < xe; x += step) {
+                const V v = q[x];
+                const V uu = u[x];
+                const V w = Fmt::make(fma(am, v.x, uu.x), fma(am, v.y, uu.y));
+                u[x] = w;
+                if (single) sq[x] = w;
+                Fmt::add_prod(a, w.x, w.x);
+                Fmt::add_prod(a, w.y, w.y);
+              }
             }
           }
           const double bsum = batch_sum<Fmt, PER_SM>(S, a, nact, slot ^= 1, coop);

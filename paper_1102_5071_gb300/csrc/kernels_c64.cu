@@ -102,8 +102,7 @@ struct SmemC {
   // commands to the workers
   int cmd, it;                   // CCmd; the iteration, or the number of basis vectors (kCRec)
   int final_rec;
-  // control flow (in shared memory: a register spill would go to local memory,
-  // whose lines the workers' loops sweep out of L1)
+  // control flow
   long long e, fpos;             // stage exponential of the launch; next forced decision
   double remaining;              // of the stage exponential
   double acc_err;                // estimate of the accepted substep
@@ -236,11 +235,13 @@ __device__ __forceinline__ void c_apply_spin2(const float2* __restrict__ q, cons
   r2 = make_float2(ur2, ui2);
 }
 
-// Element pair (x, x + 1) of a chain staged over 128 CTAs, as fx_apply_spin_staged:
+// Element pair (x, x + 1) of a chain whose applied vector is staged in the shared
+// memory of 128 CTAs, 2^(N - 7) elements each, in clusters of four: flips and hops of
 // bits below N - 7 from this CTA's shared memory, the next two from the cluster's,
 // the five highest from global memory (issued ahead); any bit above bit 0 maps the
-// pair onto a pair, one 16-byte access.  Every sum runs in the order of the
-// element-wise form, so the results are the same bits.  The far gathers bound it: 4.5 TB/s over
+// pair onto a pair, one 16-byte access.  Every element's sum runs in the order of the
+// element-wise form, so an apply gives the same bits (the compensated sums over the
+// vector run over 128 parts instead of 152).  The far gathers bound it: 4.5 TB/s over
 // the L2 fabric, where the element-wise form gathers twice as many bytes.  Lanczos
 // iteration 12.1 us at 17 sites (element-wise 13.6), 15.2 at 18 (16.8), 30.8 at 20
 // (32.4), 53.6 at 21 (58.0).  Near loops unrolled by 6 and 12 instead of 4: 3 and

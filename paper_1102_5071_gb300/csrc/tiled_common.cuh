@@ -4,7 +4,7 @@
 // The element-wise apply gathers 2N - 1 neighbours of every element; for
 // vectors beyond the 129 MB L2 the far-bit gathers read DRAM.  The tiled form
 // splits the bits of the index into windows and runs one pass per window over
-// tiles of 2^B elements staged in shared memory (cp.async, double-buffered):
+// tiles of 2^B elements staged in shared memory (TMA, three stages of two tiles):
 //   window 0 takes contiguous tiles (bits 0..B-1): diagonal, previous Krylov
 //     vector, flips of bits 0..B-1, hops of bonds (i, i+1) for i <= B-2;
 //   window w >= 1 takes strided tiles made of 2^c contiguous elements times
