@@ -665,6 +665,12 @@ cfet_status cfet_selftest_krylov_bounds(int32_t k, const double* a, const double
  * block_size and grid_size give.  CFET_EINVAL for NULL pointers.            */
 cfet_status cfet_selftest_launch_shape(const cfet_ctx* ctx, int32_t* grid, int32_t* block);
 
+/* Self-check of the test that the cluster kernels make before they touch a peer's
+ * shared memory (device): *device_status is 0 when a launch in clusters of
+ * cluster_size (1, 2, 4 or 8) CTAs has the expected size, CFET_ECUDA otherwise.
+ * CFET_EINVAL for other arguments.                                          */
+cfet_status cfet_selftest_cluster_check(int32_t cluster_size, int32_t expected, int32_t* device_status);
+
 /* Self-check of the record exchange of the persistent kernels (device): n
  * exchanges over `grid` CTAs (2 to 256) in one launch, with the record widths
  * of the kernels mixed, tags counted from first_tag (16 bits of which are

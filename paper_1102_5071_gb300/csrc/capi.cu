@@ -1924,6 +1924,24 @@ cfet_status cfet_selftest_wait_timeout(int32_t which, double timeout_s, int32_t*
   return h == CFET_ETIMEOUT ? CFET_OK : fail(nullptr, CFET_ECUDA, "wait self test: the wait did not time out");
 }
 
+cfet_status cfet_selftest_cluster_check(int32_t cluster_size, int32_t expected, int32_t* device_status) {
+  if ((cluster_size != 1 && cluster_size != 2 && cluster_size != 4 && cluster_size != 8) || expected < 1 ||
+      !device_status)
+    return fail(nullptr, CFET_EINVAL, "selftest: cluster_size in {1, 2, 4, 8}, expected >= 1, device_status required");
+  cfet_status s = device_available(nullptr);
+  if (s != CFET_OK) return s;
+  int* st = nullptr;
+  int h = 0;
+  cudaError_t e = cudaMalloc(&st, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(st, 0, sizeof(int));
+  if (e == cudaSuccess) e = (cudaError_t)launch_cluster_selftest(cluster_size, expected, st);
+  if (e == cudaSuccess) e = cudaMemcpy(&h, st, sizeof(int), cudaMemcpyDeviceToHost);
+  cudaFree(st);
+  if (e != cudaSuccess) return cuda_fail(nullptr, e, "cluster self test");
+  *device_status = h;
+  return CFET_OK;
+}
+
 cfet_status cfet_selftest_exchange(int32_t grid, uint32_t first_tag, int32_t n, int64_t* wrong) {
   if (grid < 2 || grid > kMaxCtlGrid || n < 1 || n > 200000 || first_tag < 1 || first_tag > 1u << 30 || !wrong)
     return fail(nullptr, CFET_EINVAL, "selftest: grid in [2, 256], n in [1, 200000], first_tag in [1, 2^30], wrong required");

@@ -339,6 +339,7 @@ constexpr int kFxTiledMinSites = 23;
 constexpr int kTiledMinSites = 13;  // tiles of up to 2^12 elements
 constexpr int kTiledMaxSites = 30;  // four windows cover 32 sites at 2^11-element tiles
 int launch_adjoint_spin(const AdjParams& p, const OpSpin& op, int grid, void* stream);
+int launch_cluster_selftest(int cluster_size, int expected, int* status);
 int launch_exchange_selftest(unsigned long long* rec, unsigned first, int n, int grid, int* status,
                              unsigned long long* out);
 int launch_wait_selftest(int which, unsigned long long* rec, unsigned* bar, int* status, long long timeout_ns);

@@ -207,6 +207,17 @@ __device__ __forceinline__ unsigned cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+// Whether the launch's clusters are of n CTAs.  Checked before any access to a
+// peer's shared memory: a launch that lost its cluster attribute (a profiler that
+// replays a graph's kernel node by itself, for one) would address CTAs that do not
+// exist.  False in every thread, with CFET_ECUDA recorded.
+__device__ __forceinline__ bool cluster_is(unsigned n, int* status) {
+  unsigned c;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(c));
+  if (c == n) return true;
+  if (threadIdx.x == 0) atomicCAS(status, 0, (int)CFET_ECUDA);
+  return false;
+}
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }

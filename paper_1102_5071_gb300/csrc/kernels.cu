@@ -958,7 +958,23 @@ __global__ void k_exchange_selftest(unsigned long long* rec, unsigned first, int
     if (!ok) return;
   }
 }
+// The check of the cluster size by itself.
+__global__ void k_cluster_selftest(unsigned expected, int* status) { cluster_is(expected, status); }
 }  // namespace
+
+int launch_cluster_selftest(int cluster_size, int expected, int* status) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(8);
+  cfg.blockDim = dim3(32);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cluster_size;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster_size > 1 ? 1 : 0;
+  return (int)cudaLaunchKernelEx(&cfg, k_cluster_selftest, (unsigned)expected, status);
+}
 
 int launch_exchange_selftest(unsigned long long* rec, unsigned first, int n, int grid, int* status,
                              unsigned long long* out) {

@@ -1309,6 +1309,9 @@ __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_c64(PropP
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmemC& S = *reinterpret_cast<SmemC*>(smem_raw);
   const int NW = (int)(blockDim.x >> 5) - 1;
+  if constexpr (MODE == kCStaged) {
+    if (!cluster_is(kStagedCluster, &p.st->status)) return;
+  }
   // tiled apply: the stages' mbarriers and tile buffers behind SmemC
   unsigned char* const tiles_base = smem_raw + ((sizeof(SmemC) + 127) & ~size_t(127));
   if constexpr (MODE == kCTiled) {

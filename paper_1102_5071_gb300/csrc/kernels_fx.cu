@@ -1141,6 +1141,7 @@ __global__ void __launch_bounds__(CFET_CTL_MAX_THREADS, 1) k_propagate_fx(PropPa
     }
   }
   if constexpr (MODE == kFxCluster) {
+    if (!cluster_is(gridDim.x, &p.st->status)) return;
     for (int i = threadIdx.x; i < kClusterSlotWords; i += blockDim.x)
       reinterpret_cast<unsigned long long*>(tiles_base)[i] = 0;
     __syncwarp();
